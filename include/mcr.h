@@ -13,14 +13,13 @@
  *
  * Calls are asynchronous on `stream` (a cudaStream_t passed as void*; NULL = legacy default
  * stream) unless a `stats` pointer is given, in which case the call synchronises that stream
- * to fill it, or the run takes the sorted-record deposit (one problem whose fixed-point tally
- * exceeds 256 MB, see mcr_launch.deposit), which synchronises once per chunk of packets.  Every call returns MCR_OK (0) or a negative status; no C++ exception crosses the
+ * to fill it.  Every call returns MCR_OK (0) or a negative status; no C++ exception crosses the
  * ABI.  Errors found on the device (negative or NaN mu, a packet that hit its event cap, a tally
  * near overflow) are latched per device and returned by the next call that synchronises
  * (a call with stats != NULL, or mc_check).
  *
  * The library keeps one grow-only workspace per device (fixed-point tallies, packed medium,
- * source CDF, counters), allocated with cudaMalloc on first use and freed by
+ * source CDF, counters, and two record buffers of up to 4 GB each, see mcr_launch.deposit), allocated with cudaMalloc on first use and freed by
  * mc_release_workspace().  Calls that share a device share that workspace: calls on different
  * streams of one device must not overlap in time.
  */
@@ -243,20 +242,21 @@ typedef struct {
                                 pixel tiles; other kinds keep their order), so that the packets in flight
                                 start close together and their tally rows stay in L2.  The tally does not
                                 depend on the order (bit-identical).  Default: on once the tallies of the
-                                launch exceed 96 MB (mc_forward and mc_adjoint always use the default) */
-  int32_t deposit;           /* 0 default, 1 direct, 2 sorted records (a batch of one harmonic problem):
-                                the transport writes one 16-byte record per pixel segment instead of its
-                                deposit, the records are sorted by pixel and each pixel's run is summed in
-                                registers before one reduction -- the same rounded products, so the tally is
-                                bit-identical, with far less HBM traffic when the tally does not fit in L2.
-                                Default: on for one problem whose tally exceeds 256 MB (mc_forward and
-                                mc_adjoint included).  It reads the record count back once per chunk of
-                                packets (a stream synchronisation), so it is never used while the stream is
-                                being captured into a graph. */
-  int64_t record_capacity;   /* records per chunk of the sorted-record deposit (0: 2^30, two 16 GB buffers;
-                                if they cannot be allocated the run deposits directly); chunks are sized
-                                from the records per packet seen so far, and a chunk that overflows the
-                                buffer is run again with the direct deposit */
+                                launch exceed 96 MB (mc_forward and mc_adjoint always use the default).  An
+                                option of the direct deposit: the record deposit keeps the packets' order */
+  int32_t deposit;           /* 0 default, 1 direct, 2 records: the transport writes one 16-byte record per
+                                pixel segment instead of its deposit, the records are sorted by pixel and each
+                                pixel's records are summed in registers before one reduction -- the same
+                                rounded products, so the tally is bit-identical.  Default: records (mc_forward
+                                and mc_adjoint included) unless merge_collisions, shared_tally or launch_order
+                                is 2 (options of the direct deposit).  Nothing is read back, and the call can be
+                                captured into a graph; during a capture records are used if the workspace
+                                already holds buffers of the needed size (after one call outside capture) */
+  int64_t record_capacity;   /* records per launch of the record deposit (0: 1024 per packet, at least 2^22 and
+                                at most 2^28: two buffers of 64 MB to 4 GB; if they cannot be allocated the
+                                run deposits directly).  A launch whose buffer is full pauses and the next one
+                                goes on with its packets; packets left after all launches (some 4096 records per
+                                packet, at most 1024 launches) are finished by the direct deposit */
 } mcr_launch;
 
 /*

@@ -43,7 +43,7 @@ int grow(void **ptr, size_t *cap, size_t need) {
 // Sizes the workspace of one launch needs (all problems together).
 struct Need {
   size_t tally = 0, acc = 0, mu = 0, cdf = 0, block_sums = 0, order = 0, order_hist = 0;
-  size_t records = 0, rec_hist = 0;  // sorted-record deposit (records: each of the two buffers)
+  size_t records = 0, rec_scratch = 0;  // record deposit (records: each of the two buffers)
 };
 
 // Workspace of the current device, grown to `need`.
@@ -74,11 +74,18 @@ int workspace(const Need &need, Workspace **out) {
   if (need.records) {
     if ((rc = grow((void **)&w.records, &w.records_bytes, need.records))) return rc;
     if ((rc = grow((void **)&w.sorted, &w.sorted_bytes, need.records))) return rc;
-    if ((rc = grow((void **)&w.rec_hdr, &w.rec_hdr_bytes, sizeof(RecordHeader)))) return rc;
-    if ((rc = grow((void **)&w.rec_hist, &w.rec_hist_bytes, need.rec_hist))) return rc;
+    if ((rc = grow((void **)&w.rec_scratch, &w.rec_scratch_bytes, need.rec_scratch))) return rc;
   }
   *out = &w;
   return MCR_OK;
+}
+
+// Whether the current device's workspace already has room for `need`'s record buffers.
+bool holds_records(const Need &need) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+  const Workspace &w = g_ws[dev];
+  return w.records_bytes >= need.records && w.sorted_bytes >= need.records && w.rec_scratch_bytes >= need.rec_scratch;
 }
 
 void fill_stats(const DevStats &d, mcr_stats *s) {
@@ -134,12 +141,15 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
   const bool chunked = np == 1 && probs[0].n_packets > kChunkPackets;
   Need need;
   std::vector<size_t> mu_off(np), tally_off(np), cdf_off(np), bs_off(np);
+  int64_t rows = 0;  // the problems' tallies are one array of rows
+  uint64_t launch_packets = 0;
   for (int i = 0; i < np; ++i) {
     const int64_t npix = (int64_t)probs[i].med->nx * probs[i].med->nz;
     mu_off[i] = need.mu / sizeof(float4);
     need.mu += ((size_t)npix * sizeof(float4) + 255) & ~size_t(255);
-    tally_off[i] = need.tally / 8 + roff;
-    need.tally += ((size_t)npix * Cpad * 8 + 255) & ~size_t(255);
+    tally_off[i] = (size_t)rows * Cpad + roff;
+    rows += npix;
+    launch_packets += chunked ? kChunkPackets : probs[i].n_packets;
     if (probs[i].qstar) {
       cdf_off[i] = need.cdf / 8;
       need.cdf += ((size_t)npix * 8 + 255) & ~size_t(255);
@@ -148,58 +158,58 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
     }
     if (chunked) need.acc = (size_t)npix * C * sizeof(double);
   }
+  need.tally = (size_t)rows * Cpad * 8;
   // launch order: by default once the tallies no longer fit in L2, for the kinds it orders
   bool ordered = false;
   unsigned total_bins = 0;
   {
     bool orderable = false;
-    uint64_t packets = 0;
     for (int i = 0; i < np; ++i) {
       orderable |= probs[i].qstar != nullptr || (probs[i].src && probs[i].src->kind == MCR_LINE);
-      packets += chunked ? kChunkPackets : probs[i].n_packets;
       ProblemDesc d{};
       d.kind = probs[i].qstar ? kVolume : probs[i].src->kind;
       d.nx = probs[i].med->nx;
       d.nz = probs[i].med->nz;
       total_bins += order_bins(d);
     }
-    ordered = orderable && packets > 0 && packets <= 0xFFFFFFFFull && !common->sectors && !common->time_bins &&
+    ordered = orderable && launch_packets > 0 && launch_packets <= 0xFFFFFFFFull && !common->sectors && !common->time_bins &&
               (cfg.launch_order == 2 || (cfg.launch_order == 0 && (double)need.tally > kOrderTallyBytes));
     if (ordered) {
-      need.order = (size_t)packets * sizeof(unsigned);
+      need.order = (size_t)launch_packets * sizeof(unsigned);
       need.order_hist = (size_t)total_bins * sizeof(unsigned);
     }
   }
-  // sorted-record deposit: one harmonic problem whose tally does not fit in L2 (not while a graph
-  // is being captured: the chunk sizes are read back from the device)
-  cudaStreamCaptureStatus cap0 = cudaStreamCaptureStatusNone;
-  MCR_TRY_CUDA(cudaStreamIsCapturing(s, &cap0));
-  bool rec_mode = np == 1 && !common->sectors && !common->time_bins && cap0 == cudaStreamCaptureStatusNone &&
-                        probs[0].n_packets > 0 &&
-                        (cfg.deposit == 2 || (cfg.deposit == 0 && (double)need.tally > kRecordTallyBytes));
-  const unsigned long long rec_cap = cfg.record_capacity > 0 ? (unsigned long long)cfg.record_capacity : kRecordCapacity;
+  TransportParams p;
+  memset(&p, 0, sizeof(p));
+  p.n_problems = np;
+  // record deposit: the harmonic tallies, unless an option of the direct deposit is asked for (256 x 256,
+  // 2e6 packets, direct / records: K = 0 38.1 / 26.9 ms, K = 16 47.9 / 32.7, K = 64 134 / 74; 1e3 packets
+  // at K = 16: 6.6 / 3.1 ms -- there is no size at which the direct deposit is the faster one).  While a
+  // graph is being captured nothing may be allocated: then only if the workspace holds the buffers.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  MCR_TRY_CUDA(cudaStreamIsCapturing(s, &cap));
+  const bool timed = cap == cudaStreamCaptureStatusNone;
+  RecordPlan plan{};
+  bool rec_mode = !common->sectors && !common->time_bins && launch_packets > 0 &&
+                  (cfg.deposit == 2 ||
+                   (cfg.deposit == 0 && cfg.merge != 2 && cfg.shared_tally != 2 && cfg.launch_order != 2));
+  if (rec_mode) rec_mode = rec_plan(p, cfg, rows, launch_packets, &plan) == cudaSuccess;
   if (rec_mode) {
-    const int64_t npix = (int64_t)probs[0].med->nx * probs[0].med->nz;
-    need.records = (size_t)rec_cap * sizeof(float4);
-    need.rec_hist = ((size_t)npix * 2 + (npix + 255) / 256 + 1) * sizeof(unsigned);
+    need.records = rec_buffer_bytes(plan);
+    need.rec_scratch = rec_scratch_bytes(plan);
   }
   Workspace *w = nullptr;
+  if (rec_mode && !timed && !holds_records(need)) rec_mode = false;
+  if (!rec_mode) need.records = need.rec_scratch = 0;
   int rc = workspace(need, &w);
   if (rc == MCR_ERR_NOMEM && rec_mode) {  // no room for the record buffers: deposit directly
     rec_mode = false;
-    need.records = need.rec_hist = 0;
+    need.records = need.rec_scratch = 0;
     rc = workspace(need, &w);
   }
   if (rc) return rc;
 
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  MCR_TRY_CUDA(cudaStreamIsCapturing(s, &cap));
-  const bool timed = cap == cudaStreamCaptureStatusNone;
-
   MCR_TRY_CUDA(cudaMemsetAsync(w->stats(slot), 0, sizeof(DevStats), s));
-  TransportParams p;
-  memset(&p, 0, sizeof(p));
-  p.n_problems = np;
   p.K = common->K;
   p.C = C;
   p.Cpad = Cpad;
@@ -257,86 +267,37 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
     end += chunked ? 0 : h.n_packets;
     d.end = end;
     d.bin_base = bin_base;
+    d.row_base = (unsigned)(tally_off[i] / Cpad);
     bin_base += order_bins(d);
   }
   p.order = ordered ? w->order : nullptr;
   MCR_TRY_CUDA(cudaMemsetAsync(w->tally, 0, need.tally, s));
   if (chunked) MCR_TRY_CUDA(cudaMemsetAsync(w->acc, 0, need.acc, s));
   if (timed) MCR_TRY_CUDA(cudaEventRecord(w->ev_start[slot], s));
-  // one problem's packets [first, first + count) added into the tally: directly ...
-  auto direct = [&](uint64_t first, uint64_t count) -> int {
-    MCR_TRY_CUDA(cudaMemsetAsync(w->work(), 0, 8, s));
-    p.prob[0].first_packet = first;
-    p.prob[0].end = count;
+  // the launch's packets (p.prob[].end and .first_packet set) added into the tallies
+  auto run_packets = [&](uint64_t count) -> int {
     p.total_packets = count;
+    if (!count) return MCR_OK;
+    MCR_TRY_CUDA(cudaMemsetAsync(w->work(), 0, 8, s));
+    if (rec_mode) {
+      MCR_TRY_CUDA(launch_records(p, cfg, plan, w->records, w->sorted, w->rec_scratch, w->tally + roff, s));
+      return MCR_OK;
+    }
     if (ordered) MCR_TRY_CUDA(launch_order(p, total_bins, w->order_hist, w->order, s));
     MCR_TRY_CUDA(launch_transport(p, cfg, s));
     return MCR_OK;
   };
-  // ... or by sorted records, in chunks sized so that their records fit the buffer (from the most
-  // records per packet seen so far); a chunk whose records overflow runs again directly
-  double rec_per_packet = 0.0;
-  auto by_records = [&](uint64_t first, uint64_t count) -> int {
-    const int64_t npix = (int64_t)probs[0].med->nx * probs[0].med->nz;
-    unsigned *hist = w->rec_hist, *cursor = w->rec_hist + npix, *bsums = w->rec_hist + 2 * npix;
-    for (uint64_t done = 0; done < count;) {
-      // first chunk: room for 2048 records per packet; then from the most records per packet seen
-      uint64_t chunk = rec_per_packet > 0.0 ? (uint64_t)((double)rec_cap / (1.25 * rec_per_packet)) : rec_cap / 2048;
-      chunk = chunk < 1 ? 1 : (chunk > kChunkPackets ? kChunkPackets : chunk);
-      const uint64_t this_n = count - done < chunk ? count - done : chunk;
-      TransportParams q = p;
-      q.prob[0].first_packet = first + done;
-      q.prob[0].end = this_n;
-      q.total_packets = this_n;
-      q.order = nullptr;
-      q.records = w->records;
-      q.rec_count = &w->rec_hdr->count;
-      q.rec_overflow = &w->rec_hdr->overflow;
-      q.rec_capacity = rec_cap;
-      q.rec_hist = hist;
-      q.stats = &w->rec_hdr->stats;
-      MCR_TRY_CUDA(cudaMemsetAsync(w->work(), 0, 8, s));
-      MCR_TRY_CUDA(cudaMemsetAsync(w->rec_hdr, 0, sizeof(RecordHeader), s));
-      MCR_TRY_CUDA(cudaMemsetAsync(hist, 0, (size_t)npix * sizeof(unsigned), s));
-      MCR_TRY_CUDA(launch_transport_records(q, cfg, s));
-      RecordHeader hdr;
-      MCR_TRY_CUDA(cudaMemcpyAsync(&hdr, w->rec_hdr, sizeof(hdr), cudaMemcpyDeviceToHost, s));
-      MCR_TRY_CUDA(cudaStreamSynchronize(s));
-      if (hdr.overflow) {
-        int rc2 = direct(first + done, this_n);
-        if (rc2) return rc2;
-      } else {
-        // slots reserved past the capacity (a warp's last block may straddle it) were never written
-        const unsigned long long n_slots = hdr.count < rec_cap ? hdr.count : rec_cap;
-        MCR_TRY_CUDA(launch_sort_and_deposit(w->records, n_slots, hist, cursor, bsums, (int)npix, w->sorted,
-                                             common->K, Cpad, w->tally + tally_off[0], w->flags(), s));
-        MCR_TRY_CUDA(launch_add_stats(p.stats, &w->rec_hdr->stats, s));
-      }
-      const double r = (double)hdr.count / (double)this_n;
-      if (r > rec_per_packet) rec_per_packet = r;
-      done += this_n;
-    }
-    return MCR_OK;
-  };
-  auto run_range = [&](uint64_t first, uint64_t count) -> int {
-    return rec_mode ? by_records(first, count) : direct(first, count);
-  };
   if (!chunked) {
-    p.total_packets = end;
-    if (rec_mode) {
-      if ((rc = run_range(probs[0].first_packet, probs[0].n_packets))) return rc;
-    } else {
-      MCR_TRY_CUDA(cudaMemsetAsync(w->work(), 0, 8, s));
-      if (end && ordered) MCR_TRY_CUDA(launch_order(p, total_bins, w->order_hist, w->order, s));
-      if (end) MCR_TRY_CUDA(launch_transport(p, cfg, s));
-    }
+    if ((rc = run_packets(end))) return rc;
   } else {
     const HostProblem &h = probs[0];
     const int64_t npix = (int64_t)h.med->nx * h.med->nz;
     for (uint64_t done = 0; done < h.n_packets;) {
       const uint64_t this_n = h.n_packets - done < kChunkPackets ? h.n_packets - done : kChunkPackets;
       if (done) MCR_TRY_CUDA(cudaMemsetAsync(w->tally, 0, need.tally, s));
-      if ((rc = run_range(h.first_packet + done, this_n))) return rc;
+      p.prob[0].first_packet = h.first_packet + done;
+      p.prob[0].end = this_n;
+      if ((rc = run_packets(this_n))) return rc;
       MCR_TRY_CUDA(launch_accumulate(w->tally + tally_off[0], npix, C, Cpad, ldexp(1.0, -qexp[0]), w->acc, s));
       done += this_n;
     }
@@ -587,7 +548,7 @@ int mc_release_workspace(void) {
   MCR_TRY_CUDA(cudaDeviceSynchronize());
   Workspace &w = g_ws[dev];
   void *ptrs[] = {w.tally, w.acc, w.mu, w.cdf, w.block_sums, w.partials, w.small, w.order, w.order_hist,
-                  w.records, w.sorted, w.rec_hdr, w.rec_hist};
+                  w.records, w.sorted, w.rec_scratch};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   for (int k = 0; k < 3; ++k) {

@@ -64,7 +64,10 @@ struct ProblemDesc {
   float ang_c[MCR_MAX_ANG], ang_s[MCR_MAX_ANG];
   unsigned key0, key1;
   unsigned bin_base;  // launch order: the problem's first bin in the launch's bin space
+  unsigned row_base;  // record deposit: the problem's first row in the launch's row space (all tallies)
 };
+
+struct RecordHeader;
 
 struct TransportParams {
   int n_problems;
@@ -78,12 +81,17 @@ struct TransportParams {
   unsigned long long total_packets;  // = prob[n_problems-1].end
   unsigned long long *work;          // packet counter
   const unsigned *order;             // launch order: the launch index taken at step g (nullptr: g)
-  // sorted-record deposit (transport variant RECS): one record per segment instead of deposits
-  float4 *records;                   // (pixel bits, track weight x 2^q, s_x, s_z), capacity rec_capacity
-  unsigned long long *rec_count;     // records written (may pass the capacity: then rec_overflow is set)
-  unsigned *rec_overflow;
-  unsigned long long rec_capacity;
-  unsigned *rec_hist;                // records per pixel
+  // record deposit (mcr_records.cu): one record per segment instead of deposits, in launches that
+  // pause when their record buffer is full and hand their packets to the next launch
+  float4 *records;                   // (global row bits, track weight x 2^q, s_x, s_z), rec_blocks x kRecBlock
+  unsigned rec_blocks;
+  RecordHeader *rec_hdr;             // this launch's counters
+  const RecordHeader *rec_prev;      // the previous launch's (nullptr: the first)
+  unsigned *rec_hist;                // records per tile of 2^tile_shift rows
+  int tile_shift, n_tiles;
+  uint4 *saved;                      // packets under way between launches, n_saved slots (one per lane of the
+  unsigned n_saved;                  // record launches); the direct transport adopts them when set
+  unsigned *saved_work;              // direct transport: the next slot to adopt
   DevStats *stats;
   unsigned *flags;                   // error bits: transport does nothing if kFlagMedium is set; it
                                      // latches kFlagEventLimit when a packet reached max_events
@@ -97,36 +105,44 @@ struct TransportLaunch {
   int merge;         // collision merge: 0 library default, 1 off, 2 on
   int shared_tally;  // 0 default (global), 1 global, 2 per-block shared-memory copy where it applies
   int launch_order;  // 0 library default (on above kOrderTallyBytes of tallies), 1 off, 2 on
-  int deposit;       // 0 library default (sorted records above kRecordTallyBytes), 1 direct, 2 sorted records
-  long long record_capacity;  // records per chunk of the sorted-record deposit (0: kRecordCapacity)
+  int deposit;       // 0 library default (records for the harmonic tallies), 1 direct, 2 records
+  long long record_capacity;  // records per launch of the record deposit (0: by the packet count)
 };
 
-// Sorted-record deposit (single problems whose tally lives in HBM): the transport writes one
-// record per pixel segment, the records are sorted by pixel (one counting-sort pass) and a
-// deposit kernel sums each pixel's run in registers before one reduction per run.  The integer
-// tally is bit-identical to the direct deposit.
-constexpr double kRecordTallyBytes = 256.0 * 1024 * 1024;
-// Records per chunk (16 GB per buffer, two buffers): a chunk must hold several times the packets
-// in flight (~1.2e5 lanes), or the transport spends it waiting for the last, longest packets.
-constexpr unsigned long long kRecordCapacity = 1ull << 30;
-constexpr unsigned kRecBlock = 1024;            // record slots a warp reserves at a time
-constexpr unsigned kRecSentinel = 0xFFFFFFFFu;  // pixel field of an unused slot
-struct RecordHeader {
-  unsigned long long count;
-  unsigned overflow;
-  unsigned pad[13];
-  DevStats stats;  // counters of the record-mode launch, added to the run's once its records are deposited
+// Record deposit (mcr_records.cu).  The transport writes one 16-byte record per pixel segment, the
+// records are sorted into tiles of neighbouring tally rows, and a deposit kernel sums each row's
+// records in registers before one reduction per coefficient.  The integer tally is bit-identical
+// to the direct deposit.
+constexpr unsigned kRecBlock = 256;             // record slots a warp reserves at a time
+constexpr unsigned kRecSentinel = 0xFFFFFFFFu;  // row field of an unused slot
+struct RecordHeader {                           // one per record launch of a call, zeroed at its start
+  unsigned blocks;                              // blocks reserved (may pass the capacity)
+  unsigned paused;                              // 1: the launch ended with packets left
+  unsigned n_units, n_coarse_units;             // work units of the deposit and of the second sorting pass
+  unsigned pad[4];
 };
-// dst += src (run counters)
-cudaError_t launch_add_stats(DevStats *dst, const DevStats *src, cudaStream_t s);
-// Launch the transport in record mode (p.records etc. set; single harmonic problem).
-cudaError_t launch_transport_records(const TransportParams &p, const TransportLaunch &cfg, cudaStream_t s);
-// cursor[i] = sum_{k<i} hist[k] (exclusive scan of the per-pixel counts), then the records in
-// pixel order into `sorted` (cursor consumed), then the runs of each pixel deposited into the tally.
-// n: the written slots to read (at most the records buffer's capacity; sentinels are skipped).
-cudaError_t launch_sort_and_deposit(const float4 *records, unsigned long long n, const unsigned *hist,
-                                    unsigned *cursor, unsigned *block_sums, int npix, float4 *sorted, int K, int Cpad,
-                                    unsigned long long *tally, unsigned *flags, cudaStream_t s);
+// How a call's records are laid out and sorted (rec_plan).
+struct RecordPlan {
+  int64_t rows;           // tally rows of all problems
+  unsigned blocks;        // capacity of each record buffer, in blocks
+  unsigned launches;      // record launches enqueued
+  int tile_shift;         // rows per tile = 2^tile_shift
+  int n_tiles;
+  int coarse_shift;       // > 0: two sorting passes, 2^coarse_shift tiles per coarse bin
+  int n_coarse;
+  int threads;            // of the transport's blocks
+  unsigned lanes;         // lanes of the transport's grid (saved packet slots)
+};
+// capacity_records: 0 for the default.  Device limits are read from the current device.
+cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64_t rows, uint64_t packets,
+                     RecordPlan *out);
+size_t rec_buffer_bytes(const RecordPlan &pl);   // of each of the two record buffers
+size_t rec_scratch_bytes(const RecordPlan &pl);  // headers, counts, cursors, saved packets
+// Runs p's packets (p.prob[].row_base set, all tallies one array of rows from `tally`) through record
+// launches and a closing direct transport launch that takes over whatever packets they leave.
+// Asynchronous on s: nothing is read back.
+cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg, const RecordPlan &pl, float4 *buf_a,
+                           float4 *buf_b, unsigned char *scratch, unsigned long long *tally, cudaStream_t s);
 
 // Launch order: packets processed in the order of their launch position (line sources: bins of
 // 1/4096 of the line; volumetric sources: 32 x 32-pixel tiles of the launch pixel; other kinds
@@ -158,15 +174,13 @@ struct Workspace {
   size_t order_bytes = 0;
   unsigned *order_hist = nullptr;
   size_t order_hist_bytes = 0;
-  // sorted-record deposit: records and their pixel-sorted copy, header, per-pixel counts / cursors
+  // record deposit: two record buffers, and headers, counts, cursors and saved packets
   float4 *records = nullptr;
   size_t records_bytes = 0;
   float4 *sorted = nullptr;
   size_t sorted_bytes = 0;
-  RecordHeader *rec_hdr = nullptr;
-  size_t rec_hdr_bytes = 0;
-  unsigned *rec_hist = nullptr;  // [npix] counts, then [npix] cursors, then block sums
-  size_t rec_hist_bytes = 0;
+  unsigned char *rec_scratch = nullptr;
+  size_t rec_scratch_bytes = 0;
   double *partials = nullptr;
   size_t partials_bytes = 0;
   // small block: packet counter, run counters per call kind (0 forward, 1 adjoint, 2 batch),

@@ -1,0 +1,908 @@
+// mcr_records.cu -- the record deposit of the 2D harmonic tally (Sec. 3.1, Eqs. 9-11).
+//
+// The direct deposit (mcr_transport.cu) adds every segment's 2K+1 products to the pixel's tally row
+// at once: 8 (2K+1) bytes of 64-bit reductions per segment through the SM's request interface to L2,
+// which bounds it.  Here the transport only writes one 16-byte record per segment -- tally row, track
+// weight x 2^q, direction -- and the products are made later, row by row, and summed in registers:
+//   1. k_transport_rec follows the packets and appends records to blocks of slots that each warp
+//      reserves; it counts them per tile (2^tile_shift neighbouring tally rows) in shared memory.
+//      When the record buffer is full it pauses: every lane's packet is saved and the next launch
+//      takes it up, so that no launch waits for its longest packets.
+//   2. k_rec_scan turns the tile counts into offsets and lists the work units.
+//   3. k_rec_sort (one pass, or two for many tiles) moves the records into tile order: a block sorts
+//      a batch in shared memory and writes each bin's run to its place in one go.
+//   4. k_rec_deposit takes a batch of one tile's records, sorts their indices by row in shared memory,
+//      and gives each group of four lanes a run of one row's records: every lane rebuilds the harmonic
+//      row of two records at a time (the same complex products as harmonic_row, as packed FP32 pairs)
+//      and sums the rounded products in registers; one reduction per coefficient and run follows.
+// Every product is rounded exactly as in the direct deposit and integer addition is exact, so the
+// tally is bit-identical to it.
+//
+// Nothing is read back: a call enqueues more record launches than it is likely to need (one that finds
+// nothing to do ends at once) and then one direct transport launch that adopts whatever packets are
+// left, so the call stays asynchronous and can be captured into a graph.
+#include <math_constants.h>
+
+#include <mutex>
+
+#include "mcr_packet.cuh"
+
+namespace mcr {
+namespace {
+
+constexpr int kMaxTiles = 12288;    // tile counters of one transport block (48 KB of shared memory)
+constexpr int kMaxBins = 2048;      // bins of one sorting pass
+constexpr int kSortThreads = 512;
+constexpr int kSortBatch = 4096;    // records a block sorts at a time
+constexpr int kDepThreads = 128;
+constexpr int kItem = 64;           // most records of one run (a group of four lanes, two records each)
+constexpr int kCurStride = 8;       // words between cursors: one 32-byte sector each
+constexpr unsigned kMaxLaunches = 1024;
+constexpr unsigned kSegmentsPerPacket = 4096;  // record launches are enqueued for this many per packet
+
+// ------------------------------------------------------------------------------------- transport
+// Lanes that stopped at a collision wait (`pend`) until fewer than kFlyMin of the warp's lanes are still
+// flying; the scatter, the new flight's random numbers and the launch of new packets then run for all
+// waiting lanes together.
+constexpr int kFlyMin = 16;
+constexpr int kFewLanes = 4;
+
+// A sum of FP32 weights and, apart, of its rounding errors (Knuth's two-sum): FP64's accuracy for a
+// lane's few thousand terms without the FP64 pipe, which is narrow on this part.
+struct WeightSum {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float t = s + v, b = t - s;
+    e += (s - (t - b)) + (v - b);
+    s = t;
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+
+template <bool BATCH>
+__global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __grid_constant__ TransportParams p) {
+  extern __shared__ unsigned hist[];  // records per tile of this block
+  if (*p.flags & kFlagMedium) return;
+  if (p.rec_prev && p.rec_prev->paused == 0u) return;  // every packet has ended
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < p.n_tiles; i += blockDim.x) hist[i] = 0u;
+  __syncthreads();
+
+  bool alive = false, exhausted = false, pend = false;
+  unsigned long long pid = 0;
+  // the lane's problem: per-lane registers in a batch, uniform kernel parameters for a single problem
+  const float4 *mu = nullptr;
+  int prob = 0, nx = 1, nz = 1;
+  float dx = 1.f, hg_c = 1.f, qscale = 1.f;
+  unsigned key0 = 0, key1 = 0, row_base = 0;
+  auto NX = [&]() { return BATCH ? nx : p.prob[0].nx; };
+  auto NZ = [&]() { return BATCH ? nz : p.prob[0].nz; };
+  auto DX = [&]() { return BATCH ? dx : p.prob[0].dx; };
+  auto HGC = [&]() { return BATCH ? hg_c : p.prob[0].hg_c; };
+  auto QS = [&]() { return BATCH ? qscale : p.prob[0].qscale; };
+  auto KEY0 = [&]() { return BATCH ? key0 : p.prob[0].key0; };
+  auto KEY1 = [&]() { return BATCH ? key1 : p.prob[0].key1; };
+  auto MU = [&]() { return BATCH ? mu : p.prob[0].mu; };
+  auto ROW = [&]() { return BATCH ? row_base : p.prob[0].row_base; };
+  auto take_problem = [&](int pi) {
+    if (!BATCH) return;
+    const ProblemDesc &P = p.prob[pi];
+    prob = pi;
+    mu = P.mu;
+    nx = P.nx;
+    nz = P.nz;
+    dx = P.dx;
+    hg_c = P.hg_c;
+    qscale = P.qscale;
+    key0 = P.key0;
+    key1 = P.key1;
+    row_base = P.row_base;
+  };
+  // packet state; (ox, oz): the offset of the edge ahead, (inv_ax, inv_az): 1 / |s| per axis, and
+  // (mu_a, mu_s, 1/mu_a, 1/mu_s) of the current pixel
+  float fx = 0.f, fz = 0.f, sx = 0.f, sz = 1.f, W = 0.f, tau = 0.f;
+  float inv_ax = 0.f, inv_az = 0.f, ox = 0.f, oz = 0.f;
+  int ix = 0, iz = 0;
+  float4 m = make_float4(0.f, 0.f, CUDART_INF_F, CUDART_INF_F);
+  unsigned flight = 0, nscat = 0, cu1 = 0, cu2 = 0;
+  unsigned n_launch = 0, n_flight = 0, n_coll = 0, n_seg = 0, n_esc = 0, n_rrk = 0, n_rrs = 0, n_scl = 0, n_evl = 0;
+  int w_launch = 0;  // |W0| = 1
+  WeightSum w_esc, w_rr, w_kill;
+
+  auto load_mu = [&]() {
+    if (MCR_GUARD(p.flags, (unsigned)ix < (unsigned)NX() && (unsigned)iz < (unsigned)NZ())) m = __ldg(MU() + iz * NX() + ix);
+  };
+  // Per-flight geometry.  A nonzero component keeps a finite reciprocal (so that 0 x it is 0); a zero
+  // one gets infinity, and 0 x infinity = NaN loses every comparison below.
+  auto set_direction = [&]() {
+    inv_ax = __frcp_rn(fabsf(sx));
+    inv_az = __frcp_rn(fabsf(sz));
+    if (sx != 0.f) inv_ax = fminf(inv_ax, 3.402823466e38f);
+    if (sz != 0.f) inv_az = fminf(inv_az, 3.402823466e38f);
+    ox = sx > 0.f ? DX() : 0.f;
+    oz = sz > 0.f ? DX() : 0.f;
+  };
+
+  const size_t slot = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (p.rec_prev) {
+    const SavedPacket s = load_packet(p.saved, p.n_saved, slot);
+    alive = s.alive, exhausted = s.exhausted;
+    if (alive) {
+      take_problem(s.prob);
+      pid = s.pid, fx = s.fx, fz = s.fz, sx = s.sx, sz = s.sz, W = s.W, tau = s.tau, ix = s.ix, iz = s.iz;
+      flight = s.flight, nscat = s.nscat, cu1 = s.cu1, cu2 = s.cu2;
+      set_direction();
+      load_mu();
+    }
+  }
+
+  float4 *out = nullptr;     // the warp's block of record slots, filled to `fill`
+  unsigned fill = kRecBlock;
+  bool stop = false;         // warp-uniform: the record buffer is full
+  auto pad = [&]() {
+    for (unsigned j = fill + lane; j < kRecBlock; j += 32) out[j] = make_float4(__uint_as_float(kRecSentinel), 0.f, 0.f, 1.f);
+  };
+
+  // One pixel segment of a flying packet: advances it, sets pend at a collision, ends the packet at the
+  // grid's edge; returns whether there is a record (row, ts and the flight's direction).
+  auto segment = [&](unsigned &row, float &ts) -> bool {
+    const float dist_x = fabsf(ox - fx) * inv_ax, dist_z = fabsf(oz - fz) * inv_az;
+    const float d_edge = fminf(dist_x, dist_z);
+    const float d_coll = tau * m.w;  // +inf when mu_s = 0 (NaN when tau is 0 too: an edge segment)
+    pend = d_coll < d_edge;
+    const float l = fminf(d_coll, d_edge);
+    // track weight of the segment: W (1 - e^{-mu_a l}) / mu_a, then W <- W e^{-mu_a l}
+    const float em1 = expm1f(-m.x * l);
+    const float t = m.x > 0.f ? (-W * em1) * m.z : W * l;
+    W = fmaf(W, em1, W);
+    ++n_seg;
+    ts = t * QS();
+    row = ROW() + (unsigned)(iz * NX() + ix);
+    tau = fmaxf(fmaf(-m.y, l, tau), 0.f);  // (a collision draws a new one)
+    fx = clamp_dx(fmaf(l, sx, fx), DX());
+    fz = clamp_dx(fmaf(l, sz, fz), DX());
+    if (!pend) {  // step over the edge ahead; ties: x first, z follows as a zero-length segment
+      const bool cx = dist_x == d_edge;
+      ix += cx ? (sx > 0.f ? 1 : -1) : 0;
+      iz += cx ? 0 : (sz > 0.f ? 1 : -1);
+      fx = cx ? DX() - ox : fx;
+      fz = cx ? fz : DX() - oz;
+      if ((unsigned)ix >= (unsigned)NX() || (unsigned)iz >= (unsigned)NZ()) {
+        ++n_esc;
+        w_esc.add(W);
+        alive = false;
+      } else {
+        m = __ldg(MU() + iz * NX() + ix);
+      }
+    }
+    return t != 0.f && MCR_GUARD(p.flags, isfinite(t));
+  };
+  // The random numbers of free flight f (event f + 1): tau = -ln U, the scatter and roulette uniforms.
+  auto draw_flight = [&](unsigned f) {
+    const uint4 r = philox4x32_10(pid, f + 1u, KEY0(), KEY1());
+    tau = -logf(u01(r.x));
+    cu1 = r.y;
+    cu2 = r.z;
+  };
+  // The collision of a packet that stopped at one: scatter, roulette, and the next flight.  The next
+  // flight's numbers depend on nothing here and are drawn first, beside the scatter's own chain.
+  auto collide = [&]() {
+    pend = false;
+    ++n_coll;
+    if (nscat >= p.max_scatter) {
+      ++n_scl;
+      w_kill.add(W);
+      alive = false;
+      return;
+    }
+    const unsigned u1 = cu1, u2 = cu2;
+    draw_flight(flight + 1u);
+    scatter_hg(HGC(), u01(u1), sx, sz);
+    set_direction();
+    ++nscat;
+    if (fabsf(W) < p.w_threshold) {  // |W0| = 1
+      if (u01(u2) < p.rr_p) {
+        const float Wn = W * p.rr_inv_p;
+        w_rr.add(Wn);
+        w_rr.add(-W);
+        W = Wn;
+        ++n_rrs;
+      } else {
+        w_rr.add(-W);
+        ++n_rrk;
+        alive = false;
+        return;
+      }
+    }
+    if (flight >= p.max_events) {
+      ++n_evl;
+      w_kill.add(W);
+      alive = false;
+      return;
+    }
+    ++flight;
+    ++n_flight;
+  };
+
+  for (;;) {
+    if (fill + 32 > kRecBlock) {  // room for one step's records
+      pad();
+      unsigned b = 0;
+      if (lane == 0) b = atomicAdd(&p.rec_hdr->blocks, 1u);
+      b = __shfl_sync(kFull, b, 0);
+      stop = b >= p.rec_blocks;
+      fill = stop ? kRecBlock : 0u;
+      if (!stop) out = p.records + (size_t)b * kRecBlock;
+    }
+    unsigned flying = __ballot_sync(kFull, alive && !pend);
+    if (stop || __popc(flying) < kFlyMin) {
+      if (pend) collide();
+      if (stop) break;
+      // ------------------------------------------------------------- refill / launch
+      const unsigned need = __ballot_sync(kFull, !alive && !exhausted);
+      if (need) {
+        const int leader = __ffs(need) - 1;
+        unsigned long long base = 0;
+        if (lane == leader) base = atomicAdd(p.work, (unsigned long long)__popc(need));
+        base = __shfl_sync(kFull, base, leader);
+        if (!alive && !exhausted) {
+          const unsigned long long g = base + __popc(need & ((1u << lane) - 1u));
+          if (g >= p.total_packets) {
+            exhausted = true;
+          } else {
+            int lo = 0;  // the problem owning launch packet g: smallest pi with prob[pi].end > g
+            if (BATCH) {
+              int hi = p.n_problems - 1;
+              while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (p.prob[mid].end > g)
+                  hi = mid;
+                else
+                  lo = mid + 1;
+              }
+            }
+            const ProblemDesc &P = p.prob[lo];
+            pid = P.first_packet + (g - (lo ? p.prob[lo - 1].end : 0ull));
+            take_problem(lo);
+            ++n_launch;
+            float W0;
+            const bool inside = launch_packet(P, pid, NX(), NZ(), DX(), KEY0(), KEY1(), ix, iz, fx, fz, sx, sz, W0);
+            W = W0;
+            w_launch += (int)W0;
+            nscat = 0;
+            flight = 0;
+            if (!inside) {
+              ++n_esc;
+              w_esc.add(W);
+            } else if (p.max_events == 0u) {
+              ++n_evl;
+              w_kill.add(W);
+            } else {
+              flight = 1;
+              ++n_flight;
+              alive = true;
+              draw_flight(1u);
+              set_direction();
+              load_mu();
+            }
+          }
+        }
+      }
+      flying = __ballot_sync(kFull, alive);
+      if (!flying) {
+        if (__all_sync(kFull, exhausted)) break;
+        continue;
+      }
+      // The last packets of a run: a warp with few packets left and none to come lets each of them run
+      // on its own share of the block, with no vote per segment -- what then counts is the latency of
+      // one packet's chain.
+      const int n = __popc(flying);
+      if (n <= kFewLanes && __all_sync(kFull, alive || exhausted)) {
+        const unsigned per = (kRecBlock - fill) / n;
+        unsigned k = 0;
+        float4 *const own = out + fill + __popc(flying & ((1u << lane) - 1u)) * per;
+        while (alive && k < per) {
+          unsigned row;
+          float ts;
+          const float ux = sx, uz = sz;
+          if (segment(row, ts) && MCR_GUARD(p.flags, (row >> p.tile_shift) < (unsigned)p.n_tiles)) {
+            own[k++] = make_float4(__uint_as_float(row), ts, ux, uz);
+            atomicAdd(&hist[row >> p.tile_shift], 1u);
+          }
+          if (pend) collide();
+        }
+        if ((flying >> lane) & 1u)
+          for (; k < per; ++k) own[k] = make_float4(__uint_as_float(kRecSentinel), 0.f, 0.f, 1.f);
+        fill += n * per;
+        __syncwarp();
+        continue;
+      }
+    }
+
+    // ---------------------------------------------------------------- one pixel segment
+    bool has = false;
+    unsigned row = 0u;
+    float ts = 0.f;
+    if (alive && !pend) has = segment(row, ts);
+    const unsigned who = __ballot_sync(kFull, has);
+    if (has && MCR_GUARD(p.flags, (row >> p.tile_shift) < (unsigned)p.n_tiles)) {
+      out[fill + __popc(who & ((1u << lane) - 1u))] = make_float4(__uint_as_float(row), ts, sx, sz);
+      atomicAdd(&hist[row >> p.tile_shift], 1u);
+    }
+    fill += __popc(who);
+  }
+  if (fill < kRecBlock) pad();  // slots left empty hold a sentinel that the sort skips
+
+  SavedPacket s;
+  s.pid = pid, s.fx = fx, s.fz = fz, s.sx = sx, s.sz = sz, s.W = W, s.tau = tau, s.ix = ix, s.iz = iz, s.prob = prob;
+  s.flight = flight, s.nscat = nscat, s.cu1 = cu1, s.cu2 = cu2, s.alive = alive, s.exhausted = exhausted;
+  save_packet(p.saved, p.n_saved, slot, s);
+  if (__any_sync(kFull, alive || !exhausted) && lane == 0) p.rec_hdr->paused = 1u;
+  // ---------------------------------------------------------------- counters
+  const unsigned c_launch = __reduce_add_sync(kFull, n_launch), c_flight = __reduce_add_sync(kFull, n_flight),
+                 c_coll = __reduce_add_sync(kFull, n_coll), c_seg = __reduce_add_sync(kFull, n_seg),
+                 c_esc = __reduce_add_sync(kFull, n_esc), c_rrk = __reduce_add_sync(kFull, n_rrk),
+                 c_rrs = __reduce_add_sync(kFull, n_rrs), c_scl = __reduce_add_sync(kFull, n_scl),
+                 c_evl = __reduce_add_sync(kFull, n_evl);
+  const double s_launch = (double)__reduce_add_sync(kFull, w_launch), s_esc = warp_sum(w_esc.value()),
+               s_rr = warp_sum(w_rr.value()), s_kill = warp_sum(w_kill.value());
+  if (lane == 0) {
+    DevStats *st = p.stats;
+    auto add = [](unsigned long long *dst, unsigned v) {
+      if (v) atomicAdd(dst, (unsigned long long)v);
+    };
+    auto addw = [](double *dst, double v) {
+      if (v != 0.0) atomicAdd(dst, v);
+    };
+    if (c_evl) atomicOr(p.flags, kFlagEventLimit);
+    add(&st->launched, c_launch);
+    add(&st->flights, c_flight);
+    add(&st->collisions, c_coll);
+    add(&st->segments, c_seg);
+    add(&st->escapes, c_esc);
+    add(&st->rr_kill, c_rrk);
+    add(&st->rr_survive, c_rrs);
+    add(&st->scatter_limit, c_scl);
+    add(&st->event_limit, c_evl);
+    addw(&st->launched_w, s_launch);
+    addw(&st->escaped_w, s_esc);
+    addw(&st->rr_net_w, s_rr);
+    addw(&st->killed_w, s_kill);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < p.n_tiles; i += blockDim.x)
+    if (hist[i]) atomicAdd(p.rec_hist + i, hist[i]);
+}
+
+// ------------------------------------------------------------------------------------- offsets
+// Inclusive scan of v over the block (1024 threads); warp_tot: 32 words of shared memory.
+__device__ unsigned block_scan(unsigned v, unsigned *warp_tot) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned t = __shfl_up_sync(kFull, v, o);
+    if (lane >= o) v += t;
+  }
+  __syncthreads();
+  if (lane == 31) warp_tot[wid] = v;
+  __syncthreads();
+  if (wid == 0) {
+    unsigned t = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned u = __shfl_up_sync(kFull, t, o);
+      if (lane >= o) t += u;
+    }
+    warp_tot[lane] = t;
+  }
+  __syncthreads();
+  return v + (wid ? warp_tot[wid - 1] : 0u);
+}
+
+// Exclusive scan of f(i), i < n, into off[0, n] by one block of 1024 threads; returns the total.
+template <typename F>
+__device__ unsigned scan_into(int n, unsigned *off, unsigned *warp_tot, F f) {
+  unsigned carry = 0;
+  __shared__ unsigned total;
+  for (int base = 0; base < n; base += 1024) {
+    const int i = base + threadIdx.x;
+    const unsigned x = i < n ? f(i) : 0u;
+    const unsigned incl = block_scan(x, warp_tot);
+    if (i < n) off[i] = carry + incl - x;
+    if (threadIdx.x == 1023) total = incl;
+    __syncthreads();
+    carry += total;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) off[n] = carry;
+  __syncthreads();
+  return carry;
+}
+
+// Tile counts -> tile offsets and cursors, and the unit offsets of the deposit (batches of dep_batch
+// records per tile) and of the second sorting pass (batches of kSortBatch per coarse bin); clears the
+// counts for the next launch.
+__global__ void __launch_bounds__(1024) k_rec_scan(RecordHeader *hdr, unsigned *hist, int n_tiles, int coarse_shift,
+                                                   int n_coarse, int dep_batch, unsigned *tile_off, unsigned *tile_cur,
+                                                   unsigned *unit_off, unsigned *coarse_cur, unsigned *coarse_unit_off) {
+  __shared__ unsigned warp_tot[32];
+  if (hdr->blocks == 0u) return;
+  scan_into(n_tiles, tile_off, warp_tot, [&](int i) { return hist[i]; });
+  const unsigned units = scan_into(n_tiles, unit_off, warp_tot, [&](int i) { return (hist[i] + dep_batch - 1) / dep_batch; });
+  for (int i = threadIdx.x; i < n_tiles; i += 1024) {
+    tile_cur[i * kCurStride] = tile_off[i];
+    hist[i] = 0u;
+  }
+  unsigned coarse_units = 0;
+  if (coarse_shift) {
+    auto first = [&](int c) { return tile_off[min(c << coarse_shift, n_tiles)]; };
+    coarse_units = scan_into(n_coarse, coarse_unit_off, warp_tot,
+                             [&](int c) { return (first(c + 1) - first(c) + kSortBatch - 1) / kSortBatch; });
+    for (int c = threadIdx.x; c < n_coarse; c += 1024) coarse_cur[c * kCurStride] = first(c);
+  }
+  if (threadIdx.x == 0) {
+    hdr->n_units = units;
+    hdr->n_coarse_units = coarse_units;
+  }
+}
+
+// The last i < n with off[i] <= u (off nondecreasing, off[0] = 0), found by the whole block in two
+// rounds of probes; n <= blockDim.x^2.
+__device__ int block_find(const unsigned *__restrict__ off, int n, unsigned u) {
+  const int t = threadIdx.x, step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int a = (__syncthreads_count(t * step < n && __ldg(off + t * step) <= u) - 1) * step;
+  return a + __syncthreads_count(t < step && a + t < n && __ldg(off + a + t) <= u) - 1;
+}
+
+// ------------------------------------------------------------------------------------- sort
+// One sorting pass: batches of records into bins.  FIRST: the transport's slots (sentinels skipped) into
+// bins of 2^shift rows.  Otherwise: one coarse bin's records into its tiles.
+// The batch is sorted in shared memory first, so that a bin's records leave as one contiguous run and
+// take one cursor update per batch and bin instead of one per record.
+template <bool FIRST>
+__global__ void __launch_bounds__(kSortThreads, 2)
+    k_rec_sort(const float4 *__restrict__ in, float4 *__restrict__ sorted, const RecordHeader *hdr, unsigned max_blocks,
+               int shift, int n_bins, unsigned *cursor, unsigned capacity, const unsigned *__restrict__ tile_off,
+               const unsigned *__restrict__ coarse_unit_off, int n_coarse, int coarse_shift, int n_tiles,
+               unsigned *flags) {
+  constexpr int kPer = kSortBatch / kSortThreads;
+  extern __shared__ float4 srec[];                           // [kSortBatch]
+  unsigned *cnt = reinterpret_cast<unsigned *>(srec + kSortBatch);  // [n_bins] counts, then local starts
+  unsigned *delta = cnt + n_bins;                            // [n_bins] global place minus local place
+  __shared__ unsigned warp_tot[32];
+  const unsigned n = min(hdr->blocks, max_blocks) * kRecBlock;
+  const unsigned units = FIRST ? (n + kSortBatch - 1) / kSortBatch : hdr->n_coarse_units;
+  for (unsigned u = blockIdx.x; u < units; u += gridDim.x) {
+    unsigned lo = u * kSortBatch, hi = min(lo + kSortBatch, n), bin0 = 0;
+    unsigned *cur = cursor;
+    if (!FIRST) {
+      const int c = block_find(coarse_unit_off, n_coarse, u);
+      bin0 = (unsigned)c << coarse_shift;
+      lo = tile_off[bin0] + (u - coarse_unit_off[c]) * kSortBatch;
+      hi = min(lo + kSortBatch, tile_off[min((c + 1) << coarse_shift, n_tiles)]);
+      cur += bin0 * kCurStride;
+    }
+    for (int i = threadIdx.x; i < n_bins; i += kSortThreads) cnt[i] = 0u;
+    __syncthreads();
+    float4 r[kPer];
+    unsigned bin[kPer], rank[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const unsigned i = lo + k * kSortThreads + threadIdx.x;
+      r[k] = i < hi ? __ldcs(in + i) : make_float4(__uint_as_float(kRecSentinel), 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const unsigned row = __float_as_uint(r[k].x);
+      bin[k] = row == kRecSentinel ? kRecSentinel : (row >> shift) - bin0;
+      if (bin[k] != kRecSentinel && !MCR_GUARD(flags, bin[k] < (unsigned)n_bins)) bin[k] = kRecSentinel;
+      rank[k] = bin[k] != kRecSentinel ? atomicAdd(&cnt[bin[k]], 1u) : 0u;
+    }
+    __syncthreads();
+    // local starts by a block scan over the bins, and each bin's place from the global cursor
+    constexpr int kBins = kMaxBins / kSortThreads;  // neighbouring bins of one thread
+    const int b0 = threadIdx.x * kBins;
+    unsigned c[kBins], at[kBins], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kBins; ++k) {
+      c[k] = b0 + k < n_bins ? cnt[b0 + k] : 0u;
+      sum += c[k];
+    }
+#pragma unroll
+    for (int k = 0; k < kBins; ++k)
+      if (c[k]) at[k] = atomicAdd(cur + (b0 + k) * kCurStride, c[k]);
+    unsigned start = block_scan(sum, warp_tot) - sum;
+#pragma unroll
+    for (int k = 0; k < kBins; ++k) {
+      if (b0 + k < n_bins) {
+        cnt[b0 + k] = start;
+        if (c[k]) delta[b0 + k] = at[k] - start;
+      }
+      start += c[k];
+    }
+    __syncthreads();
+    const unsigned total = warp_tot[(kSortThreads >> 5) - 1];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+      if (bin[k] != kRecSentinel) srec[cnt[bin[k]] + rank[k]] = r[k];
+    __syncthreads();
+    for (unsigned i = threadIdx.x; i < total; i += kSortThreads) {
+      const float4 v = srec[i];
+      const unsigned at = delta[(__float_as_uint(v.x) >> shift) - bin0] + i;
+      if (MCR_GUARD(flags, at < capacity)) sorted[at] = v;
+    }
+    __syncthreads();
+  }
+}
+
+// ------------------------------------------------------------------------------------- deposit
+// The rounded products round(t 2^q h) (below 2^30 in magnitude) are summed exactly in two 32-bit words
+// per coefficient, in two ways that load different pipes (cosines take the first, sines the second):
+// SumX converts (XU pipe, 16 lanes a cycle) and keeps the sum modulo 2^32 and the sum of the high
+// halves x >> 16, which together determine the 64-bit sum of up to 2^16 terms (the low halves' sum is
+// below 2^32);
+struct SumX {
+  unsigned lo = 0u;
+  int hi = 0;
+  __device__ __forceinline__ void add(float a, float b) {
+    const int x = __float2int_rn(a) + __float2int_rn(b);
+    lo += (unsigned)x;
+    hi += x >> 16;
+  }
+  static __device__ __forceinline__ long long value(unsigned lo, unsigned hi) {
+    return ((long long)(int)hi << 16) + (long long)(lo - (hi << 16));
+  }
+};
+// SumF splits by FP32 additions (FMA pipe): y + 1.5 2^31 holds k = round(y / 2^8) in its low mantissa
+// bits, and (y - 2^8 k) + 1.5 2^23 the rest's nearest integer (|rest| <= 2^7; both steps are exact, and
+// ties round to even as y's own rounding does, 2^8 k being even).  The words are the sums of the two bit
+// patterns; n terms carry n times the constants' bits and at most n 2^22 (n < 2^9).
+struct SumF {
+  static constexpr float kHigh = 3221225472.f, kLow = 12582912.f;             // 1.5 2^31, 1.5 2^23
+  static constexpr unsigned kHighBits = 0x4F400000u, kLowBits = 0x4B400000u;  // their bits
+  unsigned lo = 0u, hi = 0u;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float ha = __fadd_rn(a, kHigh), hb = __fadd_rn(b, kHigh);
+    const float la = __fadd_rn(__fadd_rn(a, __fsub_rn(kHigh, ha)), kLow);
+    const float lb = __fadd_rn(__fadd_rn(b, __fsub_rn(kHigh, hb)), kLow);
+    hi += __float_as_uint(ha) + __float_as_uint(hb);
+    lo += __float_as_uint(la) + __float_as_uint(lb);
+  }
+  static __device__ __forceinline__ long long value(unsigned lo, unsigned hi, unsigned n) {
+    return ((long long)(int)(hi - n * kHighBits) << 8) + (long long)(int)(lo - n * kLowBits);
+  }
+};
+
+constexpr int kFlushStride = 32 * 8 + 16;  // bytes per coefficient of a warp's flush buffer
+constexpr int kFlushBytes = 8 * kFlushStride;
+
+struct DepositSmem {  // dynamic shared memory of k_rec_deposit for tiles of T rows and batches of kDepBatch records
+  static size_t bytes(int T, int kDepBatch) {
+    return (size_t)kDepBatch * 16 + (kDepThreads / 32) * kFlushBytes + kDepBatch * 2 + (size_t)T * 8 +
+           (size_t)(kDepBatch / kItem + T) * 4 + 64;
+  }
+};
+
+// Orders n0+1 .. n0+KT per pass (two passes above 32), coefficient 0 with the first.
+template <int KT, int MINB, int kDepBatch>
+__global__ void __launch_bounds__(kDepThreads, MINB)
+    k_rec_deposit(const float4 *__restrict__ rec, const RecordHeader *hdr, const unsigned *__restrict__ tile_off,
+                  const unsigned *__restrict__ unit_off, int n_tiles, int tile_shift, long long n_rows, int K, int Cpad,
+                  unsigned long long *__restrict__ tally, unsigned *flags) {
+  extern __shared__ float4 srec[];  // [kDepBatch]
+  const int T = 1 << tile_shift;
+  unsigned char *flush = reinterpret_cast<unsigned char *>(srec + kDepBatch);
+  unsigned *cnt = reinterpret_cast<unsigned *>(flush + (kDepThreads / 32) * kFlushBytes);  // [T] records per row
+  unsigned *start = cnt + T;                                                               // [T]
+  unsigned *items = start + T;                       // runs: start | length << 12 | row << 19
+  unsigned *bucket = items + kDepBatch / kItem + T;  // [16] runs by their number of steps, then places
+  unsigned short *idx = reinterpret_cast<unsigned short *>(bucket + 16);  // [kDepBatch] record indices by row
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane & 3, g = lane >> 2;
+  unsigned char *const my_flush = flush + warp * kFlushBytes;
+  const int C = 2 * K + 1;
+  const unsigned units = hdr->n_units;
+  for (unsigned u = blockIdx.x; u < units; u += gridDim.x) {
+    const int tile = block_find(unit_off, n_tiles, u);
+    const unsigned lo = tile_off[tile] + (u - unit_off[tile]) * kDepBatch;
+    const int n = (int)min((unsigned)kDepBatch, tile_off[tile + 1] - lo);
+    // ------------------------------------------------------------- the batch, sorted by row
+    for (int i = threadIdx.x; i < n; i += kDepThreads) {
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(srec + i);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(rec + lo + i) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int i = threadIdx.x; i < T; i += kDepThreads) cnt[i] = 0u;
+    if (threadIdx.x < 16) bucket[threadIdx.x] = 0u;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    unsigned short rank[kDepBatch / kDepThreads];
+#pragma unroll
+    for (int k = 0; k < kDepBatch / kDepThreads; ++k) {
+      const int i = threadIdx.x + k * kDepThreads;
+      rank[k] = i < n ? (unsigned short)atomicAdd(&cnt[__float_as_uint(srec[i].x) & (T - 1)], 1u) : 0;
+    }
+    __syncthreads();
+    // starts of the rows, and how many runs of how many steps (8 records a step) they make
+    if (warp == 0) {
+      unsigned carry = 0;
+      for (int b = 0; b < T; b += 32) {
+        const int row = b + lane;
+        const unsigned c = row < T ? cnt[row] : 0u;
+        unsigned v = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned t = __shfl_up_sync(kFull, v, o);
+          if (lane >= o) v += t;
+        }
+        if (row < T) start[row] = carry + v - c;
+        carry += __shfl_sync(kFull, v, 31);
+        if (c) {
+          const unsigned k = (c + kItem - 1) / kItem, len = (c + k - 1) / k;
+          atomicAdd(&bucket[(len + 7) / 8], k);
+        }
+      }
+      __syncwarp();
+      unsigned v = lane < 16 ? bucket[lane] : 0u;  // longest runs first
+      unsigned sum = v;
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const unsigned t = __shfl_down_sync(kFull, sum, o);
+        if (lane + o < 16) sum += t;
+      }
+      if (lane < 16) bucket[lane] = sum - v;
+      if (lane == 0) bucket[15] = sum;  // (no run has 15 steps) their total
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kDepBatch / kDepThreads; ++k) {
+      const int i = threadIdx.x + k * kDepThreads;
+      if (i < n) idx[start[__float_as_uint(srec[i].x) & (T - 1)] + rank[k]] = (unsigned short)i;
+    }
+    const int n_items = (int)bucket[15];
+    __syncthreads();
+    for (int row = threadIdx.x; row < T; row += kDepThreads) {
+      const unsigned c = cnt[row];
+      if (!c) continue;
+      const unsigned k = (c + kItem - 1) / kItem, len = (c + k - 1) / k;
+      const unsigned at = atomicAdd(&bucket[(len + 7) / 8], k);
+      for (unsigned q = 0; q < k; ++q)
+        items[at + q] = (start[row] + q * len) | (min(len, c - q * len) << 12) | ((unsigned)row << 19);
+    }
+    __syncthreads();
+    // ------------------------------------------------------------- eight runs a warp, four lanes each
+    for (int it = warp * 8; it < n_items; it += (kDepThreads / 32) * 8) {
+      const unsigned item = it + g < n_items ? items[it + g] : 0u;
+      const int s0 = item & 0xFFFu, len = (item >> 12) & 0x7Fu;
+      const long long row = ((long long)tile << tile_shift) + (item >> 19);
+      const int steps = (int)__reduce_max_sync(kFull, (unsigned)(len + 7) / 8);
+      const bool ok = len > 0 && MCR_GUARD(flags, row < n_rows);
+      unsigned long long *const dst = tally + (size_t)row * Cpad;
+      for (int n0 = 0; n0 == 0 || n0 < K; n0 += KT) {
+        SumX sum0, sum_c[KT];
+        SumF sum_s[KT];
+        for (int k = 0; k < steps; ++k) {
+          const int ia = k * 8 + j, ib = ia + 4;
+          float4 a = make_float4(0.f, 0.f, 0.f, 1.f), b = a;
+          if (ia < len) a = srec[idx[s0 + ia]];
+          if (ib < len) b = srec[idx[s0 + ib]];
+          if (n0 == 0) sum0.add(a.y, b.y);
+          // (cos n theta, sin n theta) by the complex products of harmonic_row
+          float ca = a.w, sa = a.z, cb = b.w, sb = b.z;
+          auto turn = [](float &c, float &s, float sx, float sz) {
+            const float cn = fmaf(c, sz, -s * sx);
+            s = fmaf(s, sz, c * sx);
+            c = cn;
+          };
+          for (int q = 0; q < n0; ++q) {
+            turn(ca, sa, a.z, a.w);
+            turn(cb, sb, b.z, b.w);
+          }
+#pragma unroll
+          for (int q = 0; q < KT; ++q) {
+            sum_c[q].add(__fmul_rn(a.y, ca), __fmul_rn(b.y, cb));
+            sum_s[q].add(__fmul_rn(a.y, sa), __fmul_rn(b.y, sb));
+            turn(ca, sa, a.z, a.w);
+            turn(cb, sb, b.z, b.w);
+          }
+        }
+        // ----------------------------------------------------------- sums of the four lanes, 16 coefficients a round
+        if (n0 == 0) {
+          sum0.lo += __shfl_xor_sync(kFull, sum0.lo, 1);
+          sum0.hi += __shfl_xor_sync(kFull, sum0.hi, 1);
+          sum0.lo += __shfl_xor_sync(kFull, sum0.lo, 2);
+          sum0.hi += __shfl_xor_sync(kFull, sum0.hi, 2);
+          if (j == 0 && ok) atomicAdd(dst, (unsigned long long)SumX::value(sum0.lo, (unsigned)sum0.hi));
+        }
+        constexpr int kRound = 8;
+#pragma unroll
+        for (int r = 0; r < 2 * KT; r += kRound) {
+          __syncwarp();
+#pragma unroll
+          for (int c = 0; c < kRound; c += 2) {
+            const SumX &x = sum_c[(r + c) / 2];
+            const SumF &f = sum_s[(r + c) / 2];
+            *reinterpret_cast<uint2 *>(my_flush + c * kFlushStride + lane * 8) = make_uint2(x.lo, (unsigned)x.hi);
+            *reinterpret_cast<uint2 *>(my_flush + (c + 1) * kFlushStride + lane * 8) = make_uint2(f.lo, f.hi);
+          }
+          __syncwarp();
+#pragma unroll
+          for (int q = 0; q < kRound; q += 4) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(my_flush + (q + j) * kFlushStride + g * 32);
+            const uint4 w = *reinterpret_cast<const uint4 *>(my_flush + (q + j) * kFlushStride + g * 32 + 16);
+            const unsigned tl = v.x + v.z + w.x + w.z, th = v.y + v.w + w.y + w.w;
+            const long long t = j & 1 ? SumF::value(tl, th, 8u * steps) : SumX::value(tl, th);
+            const int c = 1 + 2 * n0 + r + q + j;
+            if (ok && c < C) atomicAdd(dst + c, (unsigned long long)t);
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// ------------------------------------------------------------------------------------- host side
+std::mutex g_rec_mu;
+
+// Blocks of `threads` with `smem` bytes that fit on one SM, the kernel opted in to that much.
+template <typename K>
+cudaError_t rec_blocks_per_sm(K kernel, int threads, size_t smem, int *per_sm) {
+  std::lock_guard<std::mutex> lock(g_rec_mu);
+  cudaFuncAttributes a;
+  cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  if ((int)smem > a.maxDynamicSharedSizeBytes) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, threads, smem);
+  return e != cudaSuccess ? e : (*per_sm < 1 ? cudaErrorInvalidConfiguration : cudaSuccess);
+}
+
+cudaError_t sm_count(int *sms) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
+size_t sort_smem(int n_bins) { return (size_t)kSortBatch * 16 + (size_t)n_bins * 8; }
+
+struct Scratch {  // rec_scratch, laid out
+  RecordHeader *hdr;
+  unsigned *saved_work, *hist, *tile_off, *tile_cur, *unit_off, *coarse_cur, *coarse_unit_off;
+  uint4 *saved;
+  size_t zeroed, total;
+};
+Scratch layout(unsigned char *base, const RecordPlan &pl) {
+  Scratch s;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    unsigned char *q = base + at;
+    at += (bytes + 255) & ~size_t(255);
+    return q;
+  };
+  s.hdr = reinterpret_cast<RecordHeader *>(take(pl.launches * sizeof(RecordHeader)));
+  s.saved_work = reinterpret_cast<unsigned *>(take(4));
+  s.hist = reinterpret_cast<unsigned *>(take((size_t)pl.n_tiles * 4));
+  s.zeroed = at;
+  s.tile_off = reinterpret_cast<unsigned *>(take((size_t)(pl.n_tiles + 1) * 4));
+  s.tile_cur = reinterpret_cast<unsigned *>(take((size_t)pl.n_tiles * kCurStride * 4));
+  s.unit_off = reinterpret_cast<unsigned *>(take((size_t)(pl.n_tiles + 1) * 4));
+  s.coarse_cur = reinterpret_cast<unsigned *>(take((size_t)pl.n_coarse * kCurStride * 4));
+  s.coarse_unit_off = reinterpret_cast<unsigned *>(take((size_t)(pl.n_coarse + 1) * 4));
+  s.saved = reinterpret_cast<uint4 *>(take((size_t)pl.lanes * 64));
+  s.total = at;
+  return s;
+}
+
+using DepositKernel = void (*)(const float4 *, const RecordHeader *, const unsigned *, const unsigned *, int, int,
+                               long long, int, int, unsigned long long *, unsigned *);
+struct DepositChoice {
+  DepositKernel kernel;
+  int batch;  // records of one unit
+};
+DepositChoice deposit_kernel(int K) {
+  const int per_pass = K > 32 ? (K + 1) / 2 : K;
+  if (per_pass <= 4) return {k_rec_deposit<4, 6, 1536>, 1536};
+  if (per_pass <= 8) return {k_rec_deposit<8, 6, 1536>, 1536};
+  if (per_pass <= 12) return {k_rec_deposit<12, 5, 1536>, 1536};
+  if (per_pass <= 16) return {k_rec_deposit<16, 4, 2048>, 2048};
+  if (per_pass <= 24) return {k_rec_deposit<24, 3, 3072>, 3072};
+  return {k_rec_deposit<32, 3, 3072>, 3072};
+}
+
+}  // namespace
+
+cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64_t rows, uint64_t packets,
+                     RecordPlan *out) {
+  RecordPlan pl{};
+  pl.rows = rows;
+  // Tiles: 32 rows, or as many as keep the tile counters in a transport block's shared memory; more
+  // than kMaxBins tiles are sorted in two passes of about equal width.
+  pl.tile_shift = 5;
+  while (((rows + (1ll << pl.tile_shift) - 1) >> pl.tile_shift) > kMaxTiles) ++pl.tile_shift;
+  if (pl.tile_shift > 12) return cudaErrorInvalidValue;  // (a run's row field has 13 bits)
+  pl.n_tiles = (int)((rows + (1ll << pl.tile_shift) - 1) >> pl.tile_shift);
+  pl.coarse_shift = 0;
+  if (pl.n_tiles > kMaxBins)
+    while ((1 << (2 * pl.coarse_shift)) < pl.n_tiles / 8) ++pl.coarse_shift;
+  pl.n_coarse = pl.coarse_shift ? (pl.n_tiles + (1 << pl.coarse_shift) - 1) >> pl.coarse_shift : 0;
+  // Capacity: 1024 records per packet (one launch holds most runs), 64 MB to 4 GB per buffer.
+  uint64_t cap = cfg.record_capacity > 0 ? (uint64_t)cfg.record_capacity : packets * 1024;
+  if (cfg.record_capacity <= 0) cap = cap < (1ull << 22) ? (1ull << 22) : cap;
+  if (cap > (1ull << 28)) cap = 1ull << 28;
+  pl.blocks = (unsigned)((cap + kRecBlock - 1) / kRecBlock);
+  const uint64_t want = (packets * kSegmentsPerPacket + (uint64_t)pl.blocks * kRecBlock - 1) / ((uint64_t)pl.blocks * kRecBlock) + 1;
+  pl.launches = (unsigned)(want < kMaxLaunches ? want : kMaxLaunches);
+  pl.threads = cfg.threads_per_block > 0 ? cfg.threads_per_block : 256;
+  int sms = 0, per_sm = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)pl.n_tiles * 4;
+  e = p.n_problems > 1 ? rec_blocks_per_sm(k_transport_rec<true>, pl.threads, smem, &per_sm)
+                       : rec_blocks_per_sm(k_transport_rec<false>, pl.threads, smem, &per_sm);
+  if (e != cudaSuccess) return e;
+  if (cfg.blocks_per_sm > 0 && cfg.blocks_per_sm < per_sm) per_sm = cfg.blocks_per_sm;
+  pl.lanes = (unsigned)(sms * per_sm * pl.threads);
+  *out = pl;
+  return cudaSuccess;
+}
+
+size_t rec_buffer_bytes(const RecordPlan &pl) { return (size_t)pl.blocks * kRecBlock * sizeof(float4); }
+size_t rec_scratch_bytes(const RecordPlan &pl) { return layout(nullptr, pl).total; }
+
+cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg, const RecordPlan &pl, float4 *buf_a,
+                           float4 *buf_b, unsigned char *scratch, unsigned long long *tally, cudaStream_t s) {
+  const Scratch sc = layout(scratch, pl);
+  cudaError_t e = cudaMemsetAsync(scratch, 0, sc.zeroed, s);
+  if (e != cudaSuccess) return e;
+  int sms = 0, sort1 = 0, sort2 = 0, dep = 0;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
+  const int first_bins = pl.coarse_shift ? pl.n_coarse : pl.n_tiles;
+  if ((e = rec_blocks_per_sm(k_rec_sort<true>, kSortThreads, sort_smem(first_bins), &sort1)) != cudaSuccess) return e;
+  if (pl.coarse_shift &&
+      (e = rec_blocks_per_sm(k_rec_sort<false>, kSortThreads, sort_smem(1 << pl.coarse_shift), &sort2)) != cudaSuccess)
+    return e;
+  const DepositChoice dc = deposit_kernel(p.K);
+  const size_t dep_smem = DepositSmem::bytes(1 << pl.tile_shift, dc.batch);
+  if ((e = rec_blocks_per_sm(dc.kernel, kDepThreads, dep_smem, &dep)) != cudaSuccess) return e;
+  const unsigned capacity = pl.blocks * kRecBlock;
+  TransportParams q = p;
+  q.order = nullptr;
+  q.records = buf_a;
+  q.rec_blocks = pl.blocks;
+  q.rec_hist = sc.hist;
+  q.tile_shift = pl.tile_shift;
+  q.n_tiles = pl.n_tiles;
+  q.saved = sc.saved;
+  q.n_saved = pl.lanes;
+  q.saved_work = sc.saved_work;
+  const unsigned grid = pl.lanes / pl.threads;
+  const size_t smem = (size_t)pl.n_tiles * 4;
+  for (unsigned i = 0; i < pl.launches; ++i) {
+    q.rec_hdr = sc.hdr + i;
+    q.rec_prev = i ? sc.hdr + i - 1 : nullptr;
+    if (p.n_problems > 1)
+      k_transport_rec<true><<<grid, pl.threads, smem, s>>>(q);
+    else
+      k_transport_rec<false><<<grid, pl.threads, smem, s>>>(q);
+    k_rec_scan<<<1, 1024, 0, s>>>(q.rec_hdr, sc.hist, pl.n_tiles, pl.coarse_shift, pl.n_coarse, dc.batch,
+                                  sc.tile_off, sc.tile_cur, sc.unit_off, sc.coarse_cur, sc.coarse_unit_off);
+    k_rec_sort<true><<<sms * sort1, kSortThreads, sort_smem(first_bins), s>>>(
+        buf_a, buf_b, q.rec_hdr, pl.blocks, pl.tile_shift + pl.coarse_shift, first_bins,
+        pl.coarse_shift ? sc.coarse_cur : sc.tile_cur, capacity, sc.tile_off, sc.coarse_unit_off, pl.n_coarse,
+        pl.coarse_shift, pl.n_tiles, p.flags);
+    if (pl.coarse_shift)
+      k_rec_sort<false><<<sms * sort2, kSortThreads, sort_smem(1 << pl.coarse_shift), s>>>(
+          buf_b, buf_a, q.rec_hdr, pl.blocks, pl.tile_shift, 1 << pl.coarse_shift, sc.tile_cur, capacity, sc.tile_off,
+          sc.coarse_unit_off, pl.n_coarse, pl.coarse_shift, pl.n_tiles, p.flags);
+    dc.kernel<<<sms * dep, kDepThreads, dep_smem, s>>>(pl.coarse_shift ? buf_a : buf_b, q.rec_hdr, sc.tile_off,
+                                                        sc.unit_off, pl.n_tiles, pl.tile_shift, (long long)pl.rows, p.K,
+                                                        p.Cpad, tally, p.flags);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  q.rec_prev = sc.hdr + pl.launches - 1;
+  return launch_transport(q, TransportLaunch{0, 0, 1, 0}, s);
+}
+
+}  // namespace mcr

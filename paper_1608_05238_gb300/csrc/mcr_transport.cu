@@ -42,65 +42,13 @@
 #include <mutex>
 
 #include "mcr_harmonics.cuh"
-#include "mcr_internal.h"
-#include "mcr_rng.cuh"
+#include "mcr_packet.cuh"
 
 namespace mcr {
 namespace {
 
-constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kRowsPerStep = 2;  // independent single-lane rows deposited per step
 constexpr double kL2SpillBytes = 256.0 * 1024 * 1024;  // tallies beyond this live in HBM
-
-// Volumetric source: smallest i with cdf[i] > floor(r48 * total / 2^48).
-__device__ __forceinline__ int pick_pixel(const unsigned long long *__restrict__ cdf, int npix,
-                                          unsigned long long total, unsigned w0, unsigned w1) {
-  const unsigned long long r48 = ((unsigned long long)w0 << 16) | (unsigned long long)(w1 >> 16);
-  const unsigned long long target = __umul64hi(r48 << 16, total);
-  int lo = 0, hi = npix - 1;
-  while (lo < hi) {
-    const int mid = lo + ((hi - lo) >> 1);
-    if (__ldg(cdf + mid) > target)
-      hi = mid;
-    else
-      lo = mid + 1;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ float clamp_dx(float v, float dx) { return fminf(fmaxf(v, 0.f), dx); }
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
-
-// Launch angle (from +z) of an MCR_ANGULAR_POINT source: the theta in [0, 2 pi) at which the
-// integral of its density from 0,
-//   F(theta) = (theta + sum_n [c_n sin n theta + s_n (1 - cos n theta)] / n) / (2 pi),
-// reaches u; 24 bisection steps resolve theta to the FP32 spacing of [0, 2 pi).  Runs once per
-// packet, at launch.
-__device__ __forceinline__ float launch_angle(const ProblemDesc &P, float u) {
-  const float two_pi = 6.28318530717958648f;
-  float lo = 0.f, hi = two_pi;
-  const float target = u * two_pi;
-  for (int it = 0; it < 24; ++it) {
-    const float mid = 0.5f * (lo + hi);
-    float F = mid;
-    for (int n = 1; n <= P.n_ang; ++n) {
-      float sn, cn;
-      sincosf(n * mid, &sn, &cn);
-      F += (P.ang_c[n - 1] * sn + P.ang_s[n - 1] * (1.f - cn)) / n;
-    }
-    if (F < target)
-      lo = mid;
-    else
-      hi = mid;
-  }
-  return 0.5f * (lo + hi);
-}
 
 // NP = 0: the discrete-ordinates variant (Sec. 3.1's alternative to the harmonics): each segment
 // adds its track weight to one of p.sectors equal angular sectors of its pixel, one per-lane
@@ -108,14 +56,11 @@ __device__ __forceinline__ float launch_angle(const ProblemDesc &P, float u) {
 // NP = -1: the time-resolved variant: each segment's track weight is split over the path-length
 // bins [b w, (b+1) w) it spans (the last bin open-ended), one per-lane reduction per piece; the
 // packet's path and weight updates are those of the plain run.
-// RECS: the harmonic tally by sorted records -- each segment with a deposit writes one record
-// (pixel, track weight x 2^q, direction) and counts it for its pixel; the deposit is done later
-// by k_deposit_sorted with the same harmonic rows and products (single problem, no merge).
-template <int NP, bool BATCH, bool MERGE, bool STALLY, bool RECS = false>
+template <int NP, bool BATCH, bool MERGE, bool STALLY>
 __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ TransportParams p) {
   constexpr bool SECT = NP == 0;
   constexpr bool TIMED = NP < 0;
-  constexpr bool ROWLESS = SECT || TIMED || RECS;  // no harmonic rows
+  constexpr bool ROWLESS = SECT || TIMED;  // no harmonic rows
   static_assert(!ROWLESS || (!BATCH && !MERGE && !STALLY), "the sector and time tallies run one plain forward problem");
   extern __shared__ float smem[];
   const int lane = threadIdx.x & 31;
@@ -127,6 +72,7 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
   unsigned long long *const stally =
       reinterpret_cast<unsigned long long *>(smem + (size_t)blockDim.x * (MERGE ? 2 : 1) * p.row_stride);
   if (*p.flags & kFlagMedium) return;
+  if (p.saved && p.rec_prev->paused == 0u) return;  // the record launches ran every packet to its end
   if (STALLY) {
     const size_t nw = (size_t)p.prob[0].nx * p.prob[0].nz * p.Cpad;
     for (size_t i = threadIdx.x; i < nw; i += blockDim.x) stally[i] = 0ull;
@@ -193,15 +139,6 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
     return v;
   };
   unsigned flight = 0, nscat = 0, cu1 = 0, cu2 = 0;
-  // RECS: the warp's block of record slots [rec_block, rec_block + kRecBlock), filled to rec_fill;
-  // slots left empty when a block is closed hold a sentinel that the sort skips
-  unsigned long long rec_block = 0;
-  unsigned rec_fill = kRecBlock;
-  auto rec_pad = [&]() {
-    if (rec_fill >= kRecBlock) return;
-    for (unsigned j = rec_fill + lane; j < kRecBlock; j += 32)
-      if (rec_block + j < p.rec_capacity) p.records[rec_block + j] = make_float4(__uint_as_float(kRecSentinel), 0.f, 0.f, 1.f);
-  };
   int sect = 0;           // SECT: the current flight's angular sector
   float plen = 0.f;       // TIMED: path length since launch
   int rb = 0;             // row of the current flight's harmonics
@@ -229,14 +166,50 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
       float th = atan2f(sx, sz);  // (-pi, pi], from +z
       if (th < 0.f) th += 6.28318530717958648f;
       sect = min((int)(th * p.sector_scale), p.sectors - 1);
-    } else if constexpr (!TIMED && !RECS) {
+    } else if constexpr (!TIMED) {
       write_row();
     }
   };
 
+  bool more_saved = !ROWLESS && !STALLY && p.saved != nullptr;  // warp-uniform
   for (;;) {
     // ---------------------------------------------------------------- refill / launch
     const unsigned need = __ballot_sync(kFull, !alive && !exhausted);
+    if (more_saved && need) {  // the packets that the record launches left under way come first
+      const int leader = __ffs(need) - 1;
+      unsigned base = 0;
+      if (lane == leader) base = atomicAdd(p.saved_work, (unsigned)__popc(need));
+      base = __shfl_sync(kFull, base, leader);
+      const unsigned i = base + __popc(need & ((1u << lane) - 1u));
+      if (((need >> lane) & 1u) && i < p.n_saved) {
+        const SavedPacket sp = load_packet(p.saved, p.n_saved, i);
+        if (sp.alive) {
+          if (BATCH) {
+            const ProblemDesc &P = p.prob[sp.prob];
+            mu = P.mu;
+            prob = sp.prob;
+            nx = P.nx;
+            nz = P.nz;
+            dx = P.dx;
+            hg_c = P.hg_c;
+            qscale = P.qscale;
+            key0 = P.key0;
+            key1 = P.key1;
+          }
+          pid = sp.pid;
+          fx = sp.fx, fz = sp.fz, sx = sp.sx, sz = sp.sz, W = sp.W, tau = sp.tau;
+          ix = sp.ix, iz = sp.iz;
+          flight = sp.flight, nscat = sp.nscat, cu1 = sp.cu1, cu2 = sp.cu2;
+          inv_ax = __frcp_rn(fabsf(sx));
+          inv_az = __frcp_rn(fabsf(sz));
+          if constexpr (!ROWLESS) write_row();
+          if constexpr (!BATCH) mcur = load_mu();
+          alive = true;
+        }
+      }
+      if (base + __popc(need) >= p.n_saved) more_saved = false;
+      continue;
+    }
     if (need) {
       const int leader = __ffs(need) - 1;
       unsigned long long base = 0;
@@ -275,49 +248,8 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
             key1 = P.key1;
           }
           ++n_launch;
-          float W0 = 1.f;
-          bool inside = true;
-          if (P.kind == kVolume) {
-            const int npix = NX() * NZ();
-            const unsigned long long total = __ldg(P.cdf + npix - 1);
-            if (total == 0ull) {  // all-zero source: nothing to launch
-              inside = false;
-              W0 = 0.f;
-            } else {
-              const uint4 r0 = philox4x32_10(pid, 0u, KEY0(), KEY1());
-              const uint4 r1 = philox4x32_10(pid, 1u, KEY0(), KEY1());
-              const int pix = pick_pixel(P.cdf, npix, total, r0.x, r0.y);
-              ix = pix % NX();
-              iz = pix / NX();
-              fx = u01(r1.x) * DX();
-              fz = u01(r1.y) * DX();
-              sincospif(2.f * u01(r0.z), &sx, &sz);
-              W0 = __ldg(P.q + pix) < 0.f ? -1.f : 1.f;
-            }
-          } else {
-            float x = P.x0, z = P.z0;
-            sx = P.dir_x;
-            sz = P.dir_z;
-            if (P.kind == MCR_LINE) {
-              const uint4 r0 = philox4x32_10(pid, 0u, KEY0(), KEY1());
-              const float u = u01(r0.x);
-              x = fmaf(u, P.x1 - P.x0, P.x0);
-              z = fmaf(u, P.z1 - P.z0, P.z0);
-            } else if (P.kind == MCR_ISO_POINT) {
-              const uint4 r0 = philox4x32_10(pid, 0u, KEY0(), KEY1());
-              sincospif(2.f * u01(r0.z), &sx, &sz);
-            } else if (P.kind == MCR_ANGULAR_POINT) {
-              const uint4 r0 = philox4x32_10(pid, 0u, KEY0(), KEY1());
-              sincosf(launch_angle(P, u01(r0.z)), &sx, &sz);
-            }
-            inside = x >= 0.f && x <= NX() * DX() && z >= 0.f && z <= NZ() * DX();
-            if (inside) {
-              ix = min((int)floorf(x / DX()), NX() - 1);
-              iz = min((int)floorf(z / DX()), NZ() - 1);
-              fx = clamp_dx(x - ix * DX(), DX());
-              fz = clamp_dx(z - iz * DX(), DX());
-            }
-          }
+          float W0;
+          const bool inside = launch_packet(P, pid, NX(), NZ(), DX(), KEY0(), KEY1(), ix, iz, fx, fz, sx, sz, W0);
           W = W0;
           w_launch += W0;
           nscat = 0;
@@ -442,30 +374,6 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
           }
           if (s2 >= seg_l || b + 1 == T) break;
         }
-      }
-    }
-    if constexpr (RECS) {
-      const unsigned has = __ballot_sync(kFull, seg_key != 0u);
-      if (has) {  // coalesced 16-byte record stores into the warp's own block of slots
-        const unsigned n = __popc(has);
-        if (rec_fill + n > kRecBlock) {  // warp-uniform: close the block, reserve the next one
-          rec_pad();
-          unsigned long long nb = 0;
-          if (lane == 0) nb = atomicAdd(p.rec_count, (unsigned long long)kRecBlock);
-          rec_block = __shfl_sync(kFull, nb, 0);
-          rec_fill = 0;
-        }
-        if (seg_key != 0u) {
-          const unsigned long long slot = rec_block + rec_fill + __popc(has & ((1u << lane) - 1u));
-          const unsigned pix = (seg_key >> 6) - 1u;
-          if (slot < p.rec_capacity && row_ok(seg_key)) {
-            p.records[slot] = make_float4(__uint_as_float(pix), seg_ts, sx, sz);
-            atomicAdd(p.rec_hist + pix, 1u);
-          } else {
-            atomicOr(p.rec_overflow, 1u);
-          }
-        }
-        rec_fill += n;
       }
     }
     unsigned pend = ROWLESS ? 0u : __ballot_sync(kFull, seg_key != 0u);
@@ -601,18 +509,7 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
           w_kill += W;
           alive = false;
         } else {
-          // 2D HG angle theta_s = 2 atan(c tan(pi U)) (Eq. 7), applied as a rotation with
-          // cos theta_s = (cp^2 - c^2 sp^2)/(cp^2 + c^2 sp^2), sin theta_s = 2 c sp cp/(...),
-          // (sp, cp) = (sin pi U, cos pi U): the same angle without tan's pole at U = 1/2.
-          float sp, cp;
-          sincospif(u01(cu1), &sp, &cp);
-          const float a = cp * cp, b = HGC() * HGC() * sp * sp;
-          const float inv = 1.f / (a + b);
-          const float cs = (a - b) * inv, sn = 2.f * HGC() * sp * cp * inv;
-          const float nsx = fmaf(sx, cs, sz * sn), nsz = fmaf(sz, cs, -sx * sn);
-          const float rn = rsqrtf(fmaf(nsx, nsx, nsz * nsz));
-          sx = nsx * rn;
-          sz = nsz * rn;
+          scatter_hg(HGC(), u01(cu1), sx, sz);
           ++nscat;
           if (fabsf(W) < p.w_threshold) {  // |W0| = 1
             if (u01(cu2) < p.rr_p) {
@@ -642,8 +539,7 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
     __syncwarp();
   }
 
-  if constexpr (RECS) rec_pad();  // the warp's last block
-  if (dense) flush0();            // the lane's last pending coefficient 0
+  if (dense) flush0();  // the lane's last pending coefficient 0
   // ---------------------------------------------------------------- counters
   const unsigned c_launch = __reduce_add_sync(kFull, n_launch), c_flight = __reduce_add_sync(kFull, n_flight),
                  c_coll = __reduce_add_sync(kFull, n_coll), c_seg = __reduce_add_sync(kFull, n_seg),
@@ -655,7 +551,7 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
   w_rr = warp_sum(w_rr);
   w_kill = warp_sum(w_kill);
   if (lane == 0 && c_evl) atomicOr(p.flags, kFlagEventLimit);
-  if (lane == 0 && c_launch) {
+  if (lane == 0 && (c_launch || p.saved)) {
     DevStats *s = p.stats;
     atomicAdd(&s->launched, (unsigned long long)c_launch);
     atomicAdd(&s->flights, (unsigned long long)c_flight);
@@ -779,7 +675,7 @@ size_t shared_tally_bytes(const TransportParams &p) {
 // do not hold the workspace lock (mc_forward_noalloc) reach them from any host thread.
 std::mutex g_attr_mu;
 
-template <int NP, bool BATCH, bool MERGE, bool STALLY = false, bool RECS = false>
+template <int NP, bool BATCH, bool MERGE, bool STALLY = false>
 cudaError_t blocks_per_sm(int threads, size_t smem, int *per_sm) {
   static int configured[64];  // largest dynamic smem opted in, per device
   int dev = 0;
@@ -792,30 +688,30 @@ cudaError_t blocks_per_sm(int threads, size_t smem, int *per_sm) {
   {
     std::lock_guard<std::mutex> lock(g_attr_mu);
     if (dev >= 64 || configured[dev] < (int)smem) {
-      e = cudaFuncSetAttribute(k_transport<NP, BATCH, MERGE, STALLY, RECS>,
+      e = cudaFuncSetAttribute(k_transport<NP, BATCH, MERGE, STALLY>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
       if (dev < 64) configured[dev] = (int)smem;
     }
   }
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_transport<NP, BATCH, MERGE, STALLY, RECS>, threads,
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_transport<NP, BATCH, MERGE, STALLY>, threads,
                                                        smem);
 }
 
-template <int NP, bool BATCH, bool MERGE, bool STALLY = false, bool RECS = false>
+template <int NP, bool BATCH, bool MERGE, bool STALLY = false>
 cudaError_t launch_kernel(const TransportParams &p, int threads, int cap, cudaStream_t s) {
   if (threads % 32 || threads > 256 || threads <= 0) return cudaErrorInvalidValue;
-  const size_t smem = RECS ? 16 : transport_smem_bytes(p.row_stride, threads, MERGE) + (STALLY ? shared_tally_bytes(p) : 0);
+  const size_t smem = transport_smem_bytes(p.row_stride, threads, MERGE) + (STALLY ? shared_tally_bytes(p) : 0);
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  e = blocks_per_sm<NP, BATCH, MERGE, STALLY, RECS>(threads, smem, &per_sm);
+  e = blocks_per_sm<NP, BATCH, MERGE, STALLY>(threads, smem, &per_sm);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   if (cap > 0 && cap < per_sm) per_sm = cap;
-  k_transport<NP, BATCH, MERGE, STALLY, RECS><<<sms * per_sm, threads, smem, s>>>(p);
+  k_transport<NP, BATCH, MERGE, STALLY><<<sms * per_sm, threads, smem, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -894,13 +790,6 @@ size_t transport_smem_bytes(int row_stride, int threads, bool merge) {
   return (size_t)threads * row_stride * sizeof(float) * (merge ? 2 : 1);
 }
 
-
-
-cudaError_t launch_transport_records(const TransportParams &p, const TransportLaunch &cfg, cudaStream_t s) {
-  if (p.n_problems != 1 || p.sectors > 0 || p.time_bins > 0 || !p.records) return cudaErrorInvalidValue;
-  return launch_kernel<1, false, false, false, true>(p, cfg.threads_per_block > 0 ? cfg.threads_per_block : 128,
-                                                    cfg.blocks_per_sm, s);
-}
 
 cudaError_t launch_transport(const TransportParams &p, const TransportLaunch &cfg, cudaStream_t s) {
   if (p.sectors > 0 || p.time_bins > 0) {  // discrete ordinates / time bins: one plain forward problem

@@ -398,8 +398,8 @@ def run_batch(problems: list, common: Run, launch: tuple | None = None, stats: b
     blocks_per_sm[, merge_collisions[, shared_tally[, launch_order]]]) or None for the defaults
     (0 in a field: its default; merge_collisions 1 off, 2 on; shared_tally 2: per-block
     shared-memory tally where it applies; launch_order 1 off, 2 on: packets in the order of their
-    launch position; deposit 1 direct, 2 sorted records (a batch of one harmonic problem);
-    record_capacity: records per chunk of the sorted-record deposit).  The call can be captured in a CUDA graph once a
+    launch position; deposit 1 direct, 2 records; record_capacity: records per launch of the record
+    deposit).  The call can be captured in a CUDA graph once a
     first call has grown the library's workspace to this batch's size.
     """
     lib = load()
