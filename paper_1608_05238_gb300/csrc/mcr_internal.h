@@ -87,8 +87,8 @@ struct TransportParams {
   unsigned rec_blocks;
   RecordHeader *rec_hdr;             // this launch's counters
   const RecordHeader *rec_prev;      // the previous launch's (nullptr: the first)
-  unsigned *rec_hist;                // records per tile of 2^tile_shift rows
-  int tile_shift, n_tiles;
+  unsigned *rec_hist;                // records per bin of 2^bin_shift rows
+  int bin_shift, n_bins;
   uint4 *saved;                      // packets under way between launches, n_saved slots (one per lane of the
   unsigned n_saved;                  // record launches); the direct transport adopts them when set
   unsigned *saved_work;              // direct transport: the next slot to adopt
@@ -129,7 +129,7 @@ struct RecordPlan {
   int tile_shift;         // rows per tile = 2^tile_shift
   int n_tiles;
   int coarse_shift;       // > 0: two sorting passes, 2^coarse_shift tiles per coarse bin
-  int n_coarse;
+  int n_coarse;           // bins of the first pass (= n_tiles with one)
   int threads;            // of the transport's blocks
   unsigned lanes;         // lanes of the transport's grid (saved packet slots)
 };

@@ -30,8 +30,8 @@
 namespace mcr {
 namespace {
 
-constexpr int kMaxTiles = 12288;    // tile counters of one transport block (48 KB of shared memory)
-constexpr int kMaxBins = 2048;      // bins of one sorting pass
+constexpr int kMaxBins = 2048;      // bins of one sorting pass (and counters of one transport block)
+constexpr int kMaxTiles = 1 << 17;  // tiles of two passes
 constexpr int kSortThreads = 512;
 constexpr int kSortBatch = 4096;    // records a block sorts at a time
 constexpr int kDepThreads = 128;
@@ -61,11 +61,11 @@ struct WeightSum {
 
 template <bool BATCH>
 __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __grid_constant__ TransportParams p) {
-  extern __shared__ unsigned hist[];  // records per tile of this block
+  extern __shared__ unsigned hist[];  // records per bin of this block
   if (*p.flags & kFlagMedium) return;
   if (p.rec_prev && p.rec_prev->paused == 0u) return;  // every packet has ended
   const int lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < p.n_tiles; i += blockDim.x) hist[i] = 0u;
+  for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x) hist[i] = 0u;
   __syncthreads();
 
   bool alive = false, exhausted = false, pend = false;
@@ -305,9 +305,9 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
           unsigned row;
           float ts;
           const float ux = sx, uz = sz;
-          if (segment(row, ts) && MCR_GUARD(p.flags, (row >> p.tile_shift) < (unsigned)p.n_tiles)) {
+          if (segment(row, ts) && MCR_GUARD(p.flags, (row >> p.bin_shift) < (unsigned)p.n_bins)) {
             own[k++] = make_float4(__uint_as_float(row), ts, ux, uz);
-            atomicAdd(&hist[row >> p.tile_shift], 1u);
+            atomicAdd(&hist[row >> p.bin_shift], 1u);
           }
           if (pend) collide();
         }
@@ -325,9 +325,9 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
     float ts = 0.f;
     if (alive && !pend) has = segment(row, ts);
     const unsigned who = __ballot_sync(kFull, has);
-    if (has && MCR_GUARD(p.flags, (row >> p.tile_shift) < (unsigned)p.n_tiles)) {
+    if (has && MCR_GUARD(p.flags, (row >> p.bin_shift) < (unsigned)p.n_bins)) {
       out[fill + __popc(who & ((1u << lane) - 1u))] = make_float4(__uint_as_float(row), ts, sx, sz);
-      atomicAdd(&hist[row >> p.tile_shift], 1u);
+      atomicAdd(&hist[row >> p.bin_shift], 1u);
     }
     fill += __popc(who);
   }
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
     addw(&st->killed_w, s_kill);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < p.n_tiles; i += blockDim.x)
+  for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x)
     if (hist[i]) atomicAdd(p.rec_hist + i, hist[i]);
 }
 
@@ -419,39 +419,30 @@ __device__ unsigned scan_into(int n, unsigned *off, unsigned *warp_tot, F f) {
   return carry;
 }
 
-// Tile counts -> tile offsets and cursors, and the unit offsets of the deposit (batches of dep_batch
-// records per tile) and of the second sorting pass (batches of kSortBatch per coarse bin); clears the
-// counts for the next launch.
-__global__ void __launch_bounds__(1024) k_rec_scan(RecordHeader *hdr, unsigned *hist, int n_tiles, int coarse_shift,
-                                                   int n_coarse, int dep_batch, unsigned *tile_off, unsigned *tile_cur,
-                                                   unsigned *unit_off, unsigned *coarse_cur, unsigned *coarse_unit_off) {
+// Counts per bin -> offsets, cursors and the offsets of the bins' work units (batches of `batch`
+// records); clears the counts for the next launch.  n_units: the launch's word for their number.
+__global__ void __launch_bounds__(1024) k_rec_scan(const RecordHeader *hdr, unsigned *n_units, unsigned *hist, int n,
+                                                   int batch, unsigned *off, unsigned *cur, unsigned *unit_off) {
   __shared__ unsigned warp_tot[32];
   if (hdr->blocks == 0u) return;
-  scan_into(n_tiles, tile_off, warp_tot, [&](int i) { return hist[i]; });
-  const unsigned units = scan_into(n_tiles, unit_off, warp_tot, [&](int i) { return (hist[i] + dep_batch - 1) / dep_batch; });
-  for (int i = threadIdx.x; i < n_tiles; i += 1024) {
-    tile_cur[i * kCurStride] = tile_off[i];
+  scan_into(n, off, warp_tot, [&](int i) { return hist[i]; });
+  const unsigned units = scan_into(n, unit_off, warp_tot, [&](int i) { return (hist[i] + batch - 1) / batch; });
+  for (int i = threadIdx.x; i < n; i += 1024) {
+    cur[i * kCurStride] = off[i];
     hist[i] = 0u;
   }
-  unsigned coarse_units = 0;
-  if (coarse_shift) {
-    auto first = [&](int c) { return tile_off[min(c << coarse_shift, n_tiles)]; };
-    coarse_units = scan_into(n_coarse, coarse_unit_off, warp_tot,
-                             [&](int c) { return (first(c + 1) - first(c) + kSortBatch - 1) / kSortBatch; });
-    for (int c = threadIdx.x; c < n_coarse; c += 1024) coarse_cur[c * kCurStride] = first(c);
-  }
-  if (threadIdx.x == 0) {
-    hdr->n_units = units;
-    hdr->n_coarse_units = coarse_units;
-  }
+  if (threadIdx.x == 0) *n_units = units;
 }
 
 // The last i < n with off[i] <= u (off nondecreasing, off[0] = 0), found by the whole block in two
-// rounds of probes; n <= blockDim.x^2.
+// rounds of probes (three where n > blockDim.x^2).
 __device__ int block_find(const unsigned *__restrict__ off, int n, unsigned u) {
-  const int t = threadIdx.x, step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int a = (__syncthreads_count(t * step < n && __ldg(off + t * step) <= u) - 1) * step;
-  return a + __syncthreads_count(t < step && a + t < n && __ldg(off + a + t) <= u) - 1;
+  const int t = threadIdx.x, nt = (int)blockDim.x;
+  int a = 0;
+  for (int step = n > nt * nt ? nt * nt : (n > nt ? nt : 1);; step = step > nt ? nt : 1) {
+    a += (__syncthreads_count(a + t * step < n && __ldg(off + a + t * step) <= u) - 1) * step;
+    if (step == 1) return a;
+  }
 }
 
 // ------------------------------------------------------------------------------------- sort
@@ -462,13 +453,12 @@ __device__ int block_find(const unsigned *__restrict__ off, int n, unsigned u) {
 template <bool FIRST>
 __global__ void __launch_bounds__(kSortThreads, 2)
     k_rec_sort(const float4 *__restrict__ in, float4 *__restrict__ sorted, const RecordHeader *hdr, unsigned max_blocks,
-               int shift, int n_bins, unsigned *cursor, unsigned capacity, const unsigned *__restrict__ tile_off,
-               const unsigned *__restrict__ coarse_unit_off, int n_coarse, int coarse_shift, int n_tiles,
-               unsigned *flags) {
+               int shift, int n_bins, unsigned *cursor, unsigned capacity, const unsigned *__restrict__ coarse_off, const unsigned *__restrict__ coarse_unit_off,
+               int n_coarse, int coarse_shift, unsigned *flags) {
   constexpr int kPer = kSortBatch / kSortThreads;
-  extern __shared__ float4 srec[];                           // [kSortBatch]
+  extern __shared__ float4 srec[];                                  // [kSortBatch]
   unsigned *cnt = reinterpret_cast<unsigned *>(srec + kSortBatch);  // [n_bins] counts, then local starts
-  unsigned *delta = cnt + n_bins;                            // [n_bins] global place minus local place
+  unsigned *delta = cnt + n_bins;                                   // [n_bins] global place minus local place
   __shared__ unsigned warp_tot[32];
   const unsigned n = min(hdr->blocks, max_blocks) * kRecBlock;
   const unsigned units = FIRST ? (n + kSortBatch - 1) / kSortBatch : hdr->n_coarse_units;
@@ -478,8 +468,8 @@ __global__ void __launch_bounds__(kSortThreads, 2)
     if (!FIRST) {
       const int c = block_find(coarse_unit_off, n_coarse, u);
       bin0 = (unsigned)c << coarse_shift;
-      lo = tile_off[bin0] + (u - coarse_unit_off[c]) * kSortBatch;
-      hi = min(lo + kSortBatch, tile_off[min((c + 1) << coarse_shift, n_tiles)]);
+      lo = coarse_off[c] + (u - coarse_unit_off[c]) * kSortBatch;
+      hi = min(lo + kSortBatch, coarse_off[c + 1]);
       cur += bin0 * kCurStride;
     }
     for (int i = threadIdx.x; i < n_bins; i += kSortThreads) cnt[i] = 0u;
@@ -535,6 +525,34 @@ __global__ void __launch_bounds__(kSortThreads, 2)
   }
 }
 
+// Counts per tile of the coarse-sorted records, before the second pass.
+__global__ void __launch_bounds__(kSortThreads) k_rec_count(const float4 *__restrict__ rec, const RecordHeader *hdr,
+                                                            const unsigned *__restrict__ coarse_off,
+                                                            const unsigned *__restrict__ coarse_unit_off, int n_coarse,
+                                                            int coarse_shift, int tile_shift, unsigned *tile_hist,
+                                                            unsigned *flags) {
+  __shared__ unsigned cnt[kMaxBins];
+  const int nb = 1 << coarse_shift;
+  const unsigned units = hdr->n_coarse_units;
+  for (unsigned u = blockIdx.x; u < units; u += gridDim.x) {
+    for (int i = threadIdx.x; i < nb; i += kSortThreads) cnt[i] = 0u;
+    const int c = block_find(coarse_unit_off, n_coarse, u);
+    const unsigned lo = coarse_off[c] + (u - coarse_unit_off[c]) * kSortBatch;
+    const unsigned hi = min(lo + kSortBatch, coarse_off[c + 1]), bin0 = (unsigned)c << coarse_shift;
+#pragma unroll
+    for (int k = 0; k < kSortBatch / kSortThreads; ++k) {
+      const unsigned i = lo + k * kSortThreads + threadIdx.x;
+      if (i >= hi) continue;
+      const unsigned b = (__float_as_uint(__ldg(&rec[i].x)) >> tile_shift) - bin0;
+      if (MCR_GUARD(flags, b < (unsigned)nb)) atomicAdd(&cnt[b], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nb; i += kSortThreads)
+      if (cnt[i]) atomicAdd(tile_hist + bin0 + i, cnt[i]);
+    __syncthreads();
+  }
+}
+
 // ------------------------------------------------------------------------------------- deposit
 // The rounded products round(t 2^q h) (below 2^30 in magnitude) are summed exactly in two 32-bit words
 // per coefficient, in two ways that load different pipes (cosines take the first, sines the second):
@@ -577,14 +595,16 @@ constexpr int kFlushStride = 32 * 8 + 16;  // bytes per coefficient of a warp's 
 constexpr int kFlushBytes = 8 * kFlushStride;
 
 struct DepositSmem {  // dynamic shared memory of k_rec_deposit for tiles of T rows and batches of kDepBatch records
-  static size_t bytes(int T, int kDepBatch) {
-    return (size_t)kDepBatch * 16 + (kDepThreads / 32) * kFlushBytes + kDepBatch * 2 + (size_t)T * 8 +
-           (size_t)(kDepBatch / kItem + T) * 4 + 64;
+  static size_t bytes(int T, int kDepBatch, bool two) {
+    return (size_t)kDepBatch * 16 + (kDepThreads / 32) * kFlushBytes + (size_t)T * 8 +
+           (size_t)(kDepBatch / kItem + T) * 4 + 64 + kDepBatch * 4 +
+           (two ? (size_t)(kDepThreads / 32) * (kItem / 8) * 32 * 16 : 0);
   }
 };
 
-// Orders n0+1 .. n0+KT per pass (two passes above 32), coefficient 0 with the first.
-template <int KT, int MINB, int kDepBatch>
+// Orders n0+1 .. n0+KT per pass, coefficient 0 with the first; TWO: two passes, the second starting from
+// the powers that the first left in shared memory.
+template <int KT, int MINB, int kDepBatch, bool TWO>
 __global__ void __launch_bounds__(kDepThreads, MINB)
     k_rec_deposit(const float4 *__restrict__ rec, const RecordHeader *hdr, const unsigned *__restrict__ tile_off,
                   const unsigned *__restrict__ unit_off, int n_tiles, int tile_shift, long long n_rows, int K, int Cpad,
@@ -597,6 +617,8 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
   unsigned *items = start + T;                       // runs: start | length << 12 | row << 19
   unsigned *bucket = items + kDepBatch / kItem + T;  // [16] runs by their number of steps, then places
   unsigned short *idx = reinterpret_cast<unsigned short *>(bucket + 16);  // [kDepBatch] record indices by row
+  unsigned short *rank = idx + kDepBatch;                                 // [kDepBatch] place within the row
+  float4 *const powers = reinterpret_cast<float4 *>(rank + kDepBatch) + (threadIdx.x >> 5) * (kItem / 8) * 32 + (threadIdx.x & 31);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane & 3, g = lane >> 2;
   unsigned char *const my_flush = flush + warp * kFlushBytes;
   const int C = 2 * K + 1;
@@ -606,25 +628,27 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
     const unsigned lo = tile_off[tile] + (u - unit_off[tile]) * kDepBatch;
     const int n = (int)min((unsigned)kDepBatch, tile_off[tile + 1] - lo);
     // ------------------------------------------------------------- the batch, sorted by row
+#pragma unroll 4
     for (int i = threadIdx.x; i < n; i += kDepThreads) {
       const unsigned dst = (unsigned)__cvta_generic_to_shared(srec + i);
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(rec + lo + i) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll 1
     for (int i = threadIdx.x; i < T; i += kDepThreads) cnt[i] = 0u;
     if (threadIdx.x < 16) bucket[threadIdx.x] = 0u;
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    unsigned short rank[kDepBatch / kDepThreads];
-#pragma unroll
-    for (int k = 0; k < kDepBatch / kDepThreads; ++k) {
-      const int i = threadIdx.x + k * kDepThreads;
-      rank[k] = i < n ? (unsigned short)atomicAdd(&cnt[__float_as_uint(srec[i].x) & (T - 1)], 1u) : 0;
-    }
+    // (small loops throughout: the blocks of an SM are in different phases of this kernel and share its
+    // instruction cache)
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += kDepThreads)
+      rank[i] = (unsigned short)atomicAdd(&cnt[__float_as_uint(srec[i].x) & (T - 1)], 1u);
     __syncthreads();
     // starts of the rows, and how many runs of how many steps (8 records a step) they make
     if (warp == 0) {
       unsigned carry = 0;
+#pragma unroll 1
       for (int b = 0; b < T; b += 32) {
         const int row = b + lane;
         const unsigned c = row < T ? cnt[row] : 0u;
@@ -653,18 +677,18 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
       if (lane == 0) bucket[15] = sum;  // (no run has 15 steps) their total
     }
     __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kDepBatch / kDepThreads; ++k) {
-      const int i = threadIdx.x + k * kDepThreads;
-      if (i < n) idx[start[__float_as_uint(srec[i].x) & (T - 1)] + rank[k]] = (unsigned short)i;
-    }
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += kDepThreads)
+      idx[start[__float_as_uint(srec[i].x) & (T - 1)] + rank[i]] = (unsigned short)i;
     const int n_items = (int)bucket[15];
     __syncthreads();
+#pragma unroll 1
     for (int row = threadIdx.x; row < T; row += kDepThreads) {
       const unsigned c = cnt[row];
       if (!c) continue;
       const unsigned k = (c + kItem - 1) / kItem, len = (c + k - 1) / k;
       const unsigned at = atomicAdd(&bucket[(len + 7) / 8], k);
+#pragma unroll 1
       for (unsigned q = 0; q < k; ++q)
         items[at + q] = (start[row] + q * len) | (min(len, c - q * len) << 12) | ((unsigned)row << 19);
     }
@@ -677,15 +701,28 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
       const int steps = (int)__reduce_max_sync(kFull, (unsigned)(len + 7) / 8);
       const bool ok = len > 0 && MCR_GUARD(flags, row < n_rows);
       unsigned long long *const dst = tally + (size_t)row * Cpad;
-      for (int n0 = 0; n0 == 0 || n0 < K; n0 += KT) {
-        SumX sum0, sum_c[KT];
-        SumF sum_s[KT];
+      if (TWO)  // the first pass starts from (cos theta, sin theta), found where the second finds its powers
+#pragma unroll 1
         for (int k = 0; k < steps; ++k) {
           const int ia = k * 8 + j, ib = ia + 4;
           float4 a = make_float4(0.f, 0.f, 0.f, 1.f), b = a;
           if (ia < len) a = srec[idx[s0 + ia]];
           if (ib < len) b = srec[idx[s0 + ib]];
-          if (n0 == 0) sum0.add(a.y, b.y);
+          powers[k * 32] = make_float4(a.w, a.z, b.w, b.z);
+        }
+#pragma unroll 1
+      for (int pass = 0; pass < (TWO ? 2 : 1); ++pass) {
+        int n0 = pass * KT;
+        if (TWO) asm volatile("" : "+r"(n0));  // one copy of the loops for both passes
+        SumX sum0, sum_c[KT];
+        SumF sum_s[KT];
+#pragma unroll 1
+        for (int k = 0; k < steps; ++k) {
+          const int ia = k * 8 + j, ib = ia + 4;
+          float4 a = make_float4(0.f, 0.f, 0.f, 1.f), b = a;
+          if (ia < len) a = srec[idx[s0 + ia]];
+          if (ib < len) b = srec[idx[s0 + ib]];
+          sum0.add(a.y, b.y);
           // (cos n theta, sin n theta) by the complex products of harmonic_row
           float ca = a.w, sa = a.z, cb = b.w, sb = b.z;
           auto turn = [](float &c, float &s, float sx, float sz) {
@@ -693,9 +730,9 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
             s = fmaf(s, sz, c * sx);
             c = cn;
           };
-          for (int q = 0; q < n0; ++q) {
-            turn(ca, sa, a.z, a.w);
-            turn(cb, sb, b.z, b.w);
+          if (TWO) {
+            const float4 v = powers[k * 32];
+            ca = v.x, sa = v.y, cb = v.z, sb = v.w;
           }
 #pragma unroll
           for (int q = 0; q < KT; ++q) {
@@ -704,9 +741,10 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
             turn(ca, sa, a.z, a.w);
             turn(cb, sb, b.z, b.w);
           }
+          if (TWO) powers[k * 32] = make_float4(ca, sa, cb, sb);
         }
         // ----------------------------------------------------------- sums of the four lanes, 16 coefficients a round
-        if (n0 == 0) {
+        if (!TWO || n0 == 0) {
           sum0.lo += __shfl_xor_sync(kFull, sum0.lo, 1);
           sum0.hi += __shfl_xor_sync(kFull, sum0.hi, 1);
           sum0.lo += __shfl_xor_sync(kFull, sum0.lo, 2);
@@ -769,7 +807,9 @@ size_t sort_smem(int n_bins) { return (size_t)kSortBatch * 16 + (size_t)n_bins *
 
 struct Scratch {  // rec_scratch, laid out
   RecordHeader *hdr;
-  unsigned *saved_work, *hist, *tile_off, *tile_cur, *unit_off, *coarse_cur, *coarse_unit_off;
+  unsigned *saved_work;
+  unsigned *hist, *off, *cur, *unit_off;                  // bins of the first pass
+  unsigned *tile_hist, *tile_off, *tile_cur, *dep_unit_off;  // tiles (the same arrays after a single pass)
   uint4 *saved;
   size_t zeroed, total;
 };
@@ -783,13 +823,17 @@ Scratch layout(unsigned char *base, const RecordPlan &pl) {
   };
   s.hdr = reinterpret_cast<RecordHeader *>(take(pl.launches * sizeof(RecordHeader)));
   s.saved_work = reinterpret_cast<unsigned *>(take(4));
-  s.hist = reinterpret_cast<unsigned *>(take((size_t)pl.n_tiles * 4));
+  auto words = [&](size_t n) { return reinterpret_cast<unsigned *>(take(n * 4)); };
+  const bool two = pl.coarse_shift > 0;
+  s.hist = words(pl.n_coarse);
+  s.tile_hist = two ? words(pl.n_tiles) : s.hist;
   s.zeroed = at;
-  s.tile_off = reinterpret_cast<unsigned *>(take((size_t)(pl.n_tiles + 1) * 4));
-  s.tile_cur = reinterpret_cast<unsigned *>(take((size_t)pl.n_tiles * kCurStride * 4));
-  s.unit_off = reinterpret_cast<unsigned *>(take((size_t)(pl.n_tiles + 1) * 4));
-  s.coarse_cur = reinterpret_cast<unsigned *>(take((size_t)pl.n_coarse * kCurStride * 4));
-  s.coarse_unit_off = reinterpret_cast<unsigned *>(take((size_t)(pl.n_coarse + 1) * 4));
+  s.off = words(pl.n_coarse + 1);
+  s.cur = words((size_t)pl.n_coarse * kCurStride);
+  s.unit_off = words(pl.n_coarse + 1);
+  s.tile_off = two ? words(pl.n_tiles + 1) : s.off;
+  s.tile_cur = two ? words((size_t)pl.n_tiles * kCurStride) : s.cur;
+  s.dep_unit_off = two ? words(pl.n_tiles + 1) : s.unit_off;
   s.saved = reinterpret_cast<uint4 *>(take((size_t)pl.lanes * 64));
   s.total = at;
   return s;
@@ -800,15 +844,17 @@ using DepositKernel = void (*)(const float4 *, const RecordHeader *, const unsig
 struct DepositChoice {
   DepositKernel kernel;
   int batch;  // records of one unit
+  bool two;
 };
 DepositChoice deposit_kernel(int K) {
-  const int per_pass = K > 32 ? (K + 1) / 2 : K;
-  if (per_pass <= 4) return {k_rec_deposit<4, 6, 1536>, 1536};
-  if (per_pass <= 8) return {k_rec_deposit<8, 6, 1536>, 1536};
-  if (per_pass <= 12) return {k_rec_deposit<12, 5, 1536>, 1536};
-  if (per_pass <= 16) return {k_rec_deposit<16, 4, 2048>, 2048};
-  if (per_pass <= 24) return {k_rec_deposit<24, 3, 3072>, 3072};
-  return {k_rec_deposit<32, 3, 3072>, 3072};
+  if (K <= 4) return {k_rec_deposit<4, 5, 2048, false>, 2048, false};
+  if (K <= 8) return {k_rec_deposit<8, 5, 2048, false>, 2048, false};
+  if (K <= 12) return {k_rec_deposit<12, 5, 2048, false>, 2048, false};
+  if (K <= 16) return {k_rec_deposit<16, 4, 2560, false>, 2560, false};
+  if (K <= 24) return {k_rec_deposit<24, 3, 3072, false>, 3072, false};
+  if (K <= 32) return {k_rec_deposit<32, 3, 3072, false>, 3072, false};
+  if (K <= 48) return {k_rec_deposit<24, 3, 2304, true>, 2304, true};
+  return {k_rec_deposit<32, 3, 2304, true>, 2304, true};
 }
 
 }  // namespace
@@ -817,8 +863,8 @@ cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64
                      RecordPlan *out) {
   RecordPlan pl{};
   pl.rows = rows;
-  // Tiles: 32 rows, or as many as keep the tile counters in a transport block's shared memory; more
-  // than kMaxBins tiles are sorted in two passes of about equal width.
+  // Tiles of 32 rows (more where they would be over kMaxTiles); over kMaxBins of them are sorted in two
+  // passes of about equal width.
   pl.tile_shift = 5;
   while (((rows + (1ll << pl.tile_shift) - 1) >> pl.tile_shift) > kMaxTiles) ++pl.tile_shift;
   if (pl.tile_shift > 12) return cudaErrorInvalidValue;  // (a run's row field has 13 bits)
@@ -826,7 +872,7 @@ cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64
   pl.coarse_shift = 0;
   if (pl.n_tiles > kMaxBins)
     while ((1 << (2 * pl.coarse_shift)) < pl.n_tiles / 8) ++pl.coarse_shift;
-  pl.n_coarse = pl.coarse_shift ? (pl.n_tiles + (1 << pl.coarse_shift) - 1) >> pl.coarse_shift : 0;
+  pl.n_coarse = pl.coarse_shift ? (pl.n_tiles + (1 << pl.coarse_shift) - 1) >> pl.coarse_shift : pl.n_tiles;
   // Capacity: 1024 records per packet (one launch holds most runs), 64 MB to 4 GB per buffer.
   uint64_t cap = cfg.record_capacity > 0 ? (uint64_t)cfg.record_capacity : packets * 1024;
   if (cfg.record_capacity <= 0) cap = cap < (1ull << 22) ? (1ull << 22) : cap;
@@ -838,7 +884,7 @@ cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64
   int sms = 0, per_sm = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
-  const size_t smem = (size_t)pl.n_tiles * 4;
+  const size_t smem = (size_t)pl.n_coarse * 4;
   e = p.n_problems > 1 ? rec_blocks_per_sm(k_transport_rec<true>, pl.threads, smem, &per_sm)
                        : rec_blocks_per_sm(k_transport_rec<false>, pl.threads, smem, &per_sm);
   if (e != cudaSuccess) return e;
@@ -858,13 +904,12 @@ cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg,
   if (e != cudaSuccess) return e;
   int sms = 0, sort1 = 0, sort2 = 0, dep = 0;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  const int first_bins = pl.coarse_shift ? pl.n_coarse : pl.n_tiles;
-  if ((e = rec_blocks_per_sm(k_rec_sort<true>, kSortThreads, sort_smem(first_bins), &sort1)) != cudaSuccess) return e;
-  if (pl.coarse_shift &&
-      (e = rec_blocks_per_sm(k_rec_sort<false>, kSortThreads, sort_smem(1 << pl.coarse_shift), &sort2)) != cudaSuccess)
-    return e;
+  const bool two = pl.coarse_shift > 0;
+  const size_t smem1 = sort_smem(pl.n_coarse), smem2 = sort_smem(1 << pl.coarse_shift);
+  if ((e = rec_blocks_per_sm(k_rec_sort<true>, kSortThreads, smem1, &sort1)) != cudaSuccess) return e;
+  if (two && (e = rec_blocks_per_sm(k_rec_sort<false>, kSortThreads, smem2, &sort2)) != cudaSuccess) return e;
   const DepositChoice dc = deposit_kernel(p.K);
-  const size_t dep_smem = DepositSmem::bytes(1 << pl.tile_shift, dc.batch);
+  const size_t dep_smem = DepositSmem::bytes(1 << pl.tile_shift, dc.batch, dc.two);
   if ((e = rec_blocks_per_sm(dc.kernel, kDepThreads, dep_smem, &dep)) != cudaSuccess) return e;
   const unsigned capacity = pl.blocks * kRecBlock;
   TransportParams q = p;
@@ -872,33 +917,36 @@ cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg,
   q.records = buf_a;
   q.rec_blocks = pl.blocks;
   q.rec_hist = sc.hist;
-  q.tile_shift = pl.tile_shift;
-  q.n_tiles = pl.n_tiles;
+  q.bin_shift = pl.tile_shift + pl.coarse_shift;
+  q.n_bins = pl.n_coarse;
   q.saved = sc.saved;
   q.n_saved = pl.lanes;
   q.saved_work = sc.saved_work;
   const unsigned grid = pl.lanes / pl.threads;
-  const size_t smem = (size_t)pl.n_tiles * 4;
+  const size_t smem = (size_t)pl.n_coarse * 4;
   for (unsigned i = 0; i < pl.launches; ++i) {
-    q.rec_hdr = sc.hdr + i;
-    q.rec_prev = i ? sc.hdr + i - 1 : nullptr;
+    RecordHeader *hdr = sc.hdr + i;
+    q.rec_hdr = hdr;
+    q.rec_prev = i ? hdr - 1 : nullptr;
     if (p.n_problems > 1)
       k_transport_rec<true><<<grid, pl.threads, smem, s>>>(q);
     else
       k_transport_rec<false><<<grid, pl.threads, smem, s>>>(q);
-    k_rec_scan<<<1, 1024, 0, s>>>(q.rec_hdr, sc.hist, pl.n_tiles, pl.coarse_shift, pl.n_coarse, dc.batch,
-                                  sc.tile_off, sc.tile_cur, sc.unit_off, sc.coarse_cur, sc.coarse_unit_off);
-    k_rec_sort<true><<<sms * sort1, kSortThreads, sort_smem(first_bins), s>>>(
-        buf_a, buf_b, q.rec_hdr, pl.blocks, pl.tile_shift + pl.coarse_shift, first_bins,
-        pl.coarse_shift ? sc.coarse_cur : sc.tile_cur, capacity, sc.tile_off, sc.coarse_unit_off, pl.n_coarse,
-        pl.coarse_shift, pl.n_tiles, p.flags);
-    if (pl.coarse_shift)
-      k_rec_sort<false><<<sms * sort2, kSortThreads, sort_smem(1 << pl.coarse_shift), s>>>(
-          buf_b, buf_a, q.rec_hdr, pl.blocks, pl.tile_shift, 1 << pl.coarse_shift, sc.tile_cur, capacity, sc.tile_off,
-          sc.coarse_unit_off, pl.n_coarse, pl.coarse_shift, pl.n_tiles, p.flags);
-    dc.kernel<<<sms * dep, kDepThreads, dep_smem, s>>>(pl.coarse_shift ? buf_a : buf_b, q.rec_hdr, sc.tile_off,
-                                                        sc.unit_off, pl.n_tiles, pl.tile_shift, (long long)pl.rows, p.K,
-                                                        p.Cpad, tally, p.flags);
+    k_rec_scan<<<1, 1024, 0, s>>>(hdr, two ? &hdr->n_coarse_units : &hdr->n_units, sc.hist, pl.n_coarse,
+                                  two ? kSortBatch : dc.batch, sc.off, sc.cur, sc.unit_off);
+    k_rec_sort<true><<<sms * sort1, kSortThreads, smem1, s>>>(buf_a, buf_b, hdr, pl.blocks, q.bin_shift, pl.n_coarse,
+                                                              sc.cur, capacity, nullptr, nullptr, 0, 0, p.flags);
+    if (two) {
+      k_rec_count<<<sms * 4, kSortThreads, 0, s>>>(buf_b, hdr, sc.off, sc.unit_off, pl.n_coarse, pl.coarse_shift,
+                                                   pl.tile_shift, sc.tile_hist, p.flags);
+      k_rec_scan<<<1, 1024, 0, s>>>(hdr, &hdr->n_units, sc.tile_hist, pl.n_tiles, dc.batch, sc.tile_off, sc.tile_cur,
+                                    sc.dep_unit_off);
+      k_rec_sort<false><<<sms * sort2, kSortThreads, smem2, s>>>(
+          buf_b, buf_a, hdr, pl.blocks, pl.tile_shift, 1 << pl.coarse_shift, sc.tile_cur, capacity, sc.off, sc.unit_off, pl.n_coarse, pl.coarse_shift, p.flags);
+    }
+    dc.kernel<<<sms * dep, kDepThreads, dep_smem, s>>>(two ? buf_a : buf_b, hdr, sc.tile_off, sc.dep_unit_off,
+                                                       pl.n_tiles, pl.tile_shift, (long long)pl.rows, p.K, p.Cpad,
+                                                       tally, p.flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   q.rec_prev = sc.hdr + pl.launches - 1;
