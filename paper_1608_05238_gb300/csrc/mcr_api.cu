@@ -145,8 +145,10 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
   uint64_t launch_packets = 0;
   for (int i = 0; i < np; ++i) {
     const int64_t npix = (int64_t)probs[i].med->nx * probs[i].med->nz;
-    mu_off[i] = need.mu / sizeof(float4);
-    need.mu += ((size_t)npix * sizeof(float4) + 255) & ~size_t(255);
+    // a margin of a row and a pixel on both sides: the neighbours of every pixel can be read
+    const size_t margin = (size_t)probs[i].med->nx + 1;
+    mu_off[i] = need.mu / sizeof(float4) + margin;
+    need.mu += ((size_t)(npix + 2 * margin) * sizeof(float4) + 255) & ~size_t(255);
     tally_off[i] = (size_t)rows * Cpad + roff;
     rows += npix;
     launch_packets += chunked ? kChunkPackets : probs[i].n_packets;

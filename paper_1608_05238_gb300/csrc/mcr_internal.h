@@ -89,9 +89,13 @@ struct TransportParams {
   const RecordHeader *rec_prev;      // the previous launch's (nullptr: the first)
   unsigned *rec_hist;                // records per bin of 2^bin_shift rows
   int bin_shift, n_bins;
-  uint4 *saved;                      // packets under way between launches, n_saved slots (one per lane of the
-  unsigned n_saved;                  // record launches); the direct transport adopts them when set
-  unsigned *saved_work;              // direct transport: the next slot to adopt
+  uint4 *saved;                      // packets under way between launches, two buffers of n_saved: rec_prev->n_left
+  unsigned n_saved;                  // packets in buffer rec_prev->buf; the direct transport adopts them when set
+  unsigned *saved_work;              // direct transport: the next one to adopt
+  unsigned *ended;                   // packets that have ended
+  int n_sm;                          // SMs the grid is spread over
+  unsigned tail_max;                 // most packets the tail takes
+  unsigned long long work_base;      // packets launched by place at the start; the counter `work` goes on from there
   DevStats *stats;
   unsigned *flags;                   // error bits: transport does nothing if kFlagMedium is set; it
                                      // latches kFlagEventLimit when a packet reached max_events
@@ -117,9 +121,11 @@ constexpr unsigned kRecBlock = 256;             // record slots a warp reserves 
 constexpr unsigned kRecSentinel = 0xFFFFFFFFu;  // row field of an unused slot
 struct RecordHeader {                           // one per record launch of a call, zeroed at its start
   unsigned blocks;                              // blocks reserved (may pass the capacity)
-  unsigned paused;                              // 1: the launch ended with packets left
+  unsigned n_left;                              // packets the launch left under way
+  unsigned buf;                                 // which of the two buffers holds them
+  unsigned fresh;                               // 1: packets were still to be launched at its end
+  unsigned tail_ran, n_tail_left, tail_next;    // the tail took them over; packets it left; the next to take
   unsigned n_units, n_coarse_units;             // work units of the deposit and of the second sorting pass
-  unsigned pad[4];
 };
 // How a call's records are laid out and sorted (rec_plan).
 struct RecordPlan {
@@ -132,6 +138,7 @@ struct RecordPlan {
   int n_coarse;           // bins of the first pass (= n_tiles with one)
   int threads;            // of the transport's blocks
   unsigned lanes;         // lanes of the transport's grid (saved packet slots)
+  int tail_blocks;
 };
 // capacity_records: 0 for the default.  Device limits are read from the current device.
 cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64_t rows, uint64_t packets,

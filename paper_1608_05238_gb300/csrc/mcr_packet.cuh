@@ -106,19 +106,30 @@ __device__ __forceinline__ bool launch_packet(const ProblemDesc &P, unsigned lon
   return true;
 }
 
-// Scatter a direction by the 2D HG angle theta_s = 2 atan(c tan(pi U)) (Eq. 7), applied as a rotation
-// with cos theta_s = (cp^2 - c^2 sp^2)/(cp^2 + c^2 sp^2), sin theta_s = 2 c sp cp/(...),
-// (sp, cp) = (sin pi U, cos pi U): the same angle without tan's pole at U = 1/2; then renormalise.
-__device__ __forceinline__ void scatter_hg(float hg_c, float u, float &sx, float &sz) {
+// The 2D HG angle theta_s = 2 atan(c tan(pi U)) (Eq. 7) as a rotation: cos theta_s =
+// (cp^2 - c^2 sp^2)/(cp^2 + c^2 sp^2), sin theta_s = 2 c sp cp/(...), (sp, cp) = (sin pi U, cos pi U): the
+// same angle without tan's pole at U = 1/2.
+__device__ __forceinline__ void hg_rotation(float hg_c, float u, float &cs, float &sn) {
   float sp, cp;
   sincospif(u, &sp, &cp);
   const float a = cp * cp, b = hg_c * hg_c * sp * sp;
   const float inv = 1.f / (a + b);
-  const float cs = (a - b) * inv, sn = 2.f * hg_c * sp * cp * inv;
+  cs = (a - b) * inv;
+  sn = 2.f * hg_c * sp * cp * inv;
+}
+
+// Turn a direction and renormalise it.
+__device__ __forceinline__ void rotate(float cs, float sn, float &sx, float &sz) {
   const float nsx = fmaf(sx, cs, sz * sn), nsz = fmaf(sz, cs, -sx * sn);
   const float rn = rsqrtf(fmaf(nsx, nsx, nsz * nsz));
   sx = nsx * rn;
   sz = nsz * rn;
+}
+
+__device__ __forceinline__ void scatter_hg(float hg_c, float u, float &sx, float &sz) {
+  float cs, sn;
+  hg_rotation(hg_c, u, cs, sn);
+  rotate(cs, sn, sx, sz);
 }
 
 // A packet between two launches (record transport -> its next launch, or -> the direct transport):
@@ -128,7 +139,6 @@ struct SavedPacket {
   float fx, fz, sx, sz, W, tau;
   int ix, iz, prob;
   unsigned flight, nscat, cu1, cu2;
-  bool alive, exhausted;
 };
 
 __device__ __forceinline__ void save_packet(uint4 *saved, size_t n, size_t i, const SavedPacket &s) {
@@ -136,7 +146,7 @@ __device__ __forceinline__ void save_packet(uint4 *saved, size_t n, size_t i, co
   saved[i] = make_uint4(f(s.fx), f(s.fz), f(s.sx), f(s.sz));
   saved[n + i] = make_uint4(f(s.W), f(s.tau), (unsigned)s.ix, (unsigned)s.iz);
   saved[2 * n + i] = make_uint4((unsigned)s.pid, (unsigned)(s.pid >> 32), s.flight, s.nscat);
-  saved[3 * n + i] = make_uint4(s.cu1, s.cu2, (unsigned)s.prob, (s.alive ? 1u : 0u) | (s.exhausted ? 2u : 0u));
+  saved[3 * n + i] = make_uint4(s.cu1, s.cu2, (unsigned)s.prob, 0u);
 }
 
 __device__ __forceinline__ SavedPacket load_packet(const uint4 *saved, size_t n, size_t i) {
@@ -147,7 +157,6 @@ __device__ __forceinline__ SavedPacket load_packet(const uint4 *saved, size_t n,
   s.W = f(b.x), s.tau = f(b.y), s.ix = (int)b.z, s.iz = (int)b.w;
   s.pid = (unsigned long long)c.x | ((unsigned long long)c.y << 32);
   s.flight = c.z, s.nscat = c.w, s.cu1 = d.x, s.cu2 = d.y, s.prob = (int)d.z;
-  s.alive = (d.w & 1u) != 0u, s.exhausted = (d.w & 2u) != 0u;
   return s;
 }
 

@@ -33,6 +33,10 @@ namespace {
 constexpr int kMaxBins = 2048;      // bins of one sorting pass (and counters of one transport block)
 constexpr int kMaxTiles = 1 << 17;  // tiles of two passes
 constexpr int kSortThreads = 512;
+constexpr int kTailThreads = 256;
+// The tail takes over at this many packets to one of its warps (256 x 256, K = 16, 1e5 packets, transport:
+// 3.9 ms at 1, 3.8 at 2, 3.5 at 4, 4.1 at 8; the 128 registers of two blocks per SM beat three blocks by 0.3 ms).
+constexpr unsigned kTailPackets = 4;
 constexpr int kSortBatch = 4096;    // records a block sorts at a time
 constexpr int kDepThreads = 128;
 constexpr int kItem = 64;           // most records of one run (a group of four lanes, two records each)
@@ -41,11 +45,11 @@ constexpr unsigned kMaxLaunches = 1024;
 constexpr unsigned kSegmentsPerPacket = 4096;  // record launches are enqueued for this many per packet
 
 // ------------------------------------------------------------------------------------- transport
-// Lanes that stopped at a collision wait (`pend`) until fewer than kFlyMin of the warp's lanes are still
-// flying; the scatter, the new flight's random numbers and the launch of new packets then run for all
-// waiting lanes together.
-constexpr int kFlyMin = 16;
-constexpr int kFewLanes = 4;
+// Bound by instruction issue (80 % of the slots, 9.9 warp instructions and 9.8 ps a segment at 256 x 256
+// with the SMs full).  Lanes that stopped at a collision wait (`pend`) until fewer than kFlyMin of the
+// warp's lanes are still flying; the scatter, the new flight's random numbers and the launch of new packets
+// then run for all waiting lanes together (4e6 packets: 22.0, 21.4, 21.1, 25.4 ms at 8, 10, 12, 20).
+constexpr int kFlyMin = 12;
 
 // A sum of FP32 weights and, apart, of its rounding errors (Knuth's two-sum): FP64's accuracy for a
 // lane's few thousand terms without the FP64 pipe, which is narrow on this part.
@@ -59,12 +63,101 @@ struct WeightSum {
   __device__ __forceinline__ double value() const { return (double)s + (double)e; }
 };
 
+// The warp's record slots: a block of kRecBlock at a time from the launch's buffer.
+struct RecordWriter {
+  float4 *out = nullptr;
+  unsigned fill = kRecBlock;  // slots of the block in use
+  bool stop = false;          // the buffer is full (or the launch should pause): write no more
+  // what is left of the block holds a sentinel that the sort skips
+  __device__ __forceinline__ void pad(int lane) {
+    for (unsigned j = fill + lane; j < kRecBlock; j += 32) out[j] = make_float4(__uint_as_float(kRecSentinel), 0.f, 0.f, 1.f);
+  }
+  __device__ __forceinline__ void room(const TransportParams &p, int lane) {  // for 32 more records; else stop
+    if (stop || fill + 32 <= kRecBlock) return;
+    pad(lane);
+    unsigned b = 0;
+    if (lane == 0) b = atomicAdd(&p.rec_hdr->blocks, 1u);
+    b = __shfl_sync(kFull, b, 0);
+    stop = b >= p.rec_blocks;
+    fill = stop ? kRecBlock : 0u;
+    if (!stop) out = p.records + (size_t)b * kRecBlock;
+  }
+  // the warp's records of one step, in its lanes' order
+  __device__ __forceinline__ void put(const TransportParams &p, unsigned *hist, int lane, bool has, unsigned row,
+                                      float ts, float ux, float uz) {
+    const unsigned who = __ballot_sync(kFull, has);
+    if (has && MCR_GUARD(p.flags, (row >> p.bin_shift) < (unsigned)p.n_bins)) {
+      out[fill + __popc(who & ((1u << lane) - 1u))] = make_float4(__uint_as_float(row), ts, ux, uz);
+      atomicAdd(&hist[row >> p.bin_shift], 1u);
+    }
+    fill += __popc(who);
+  }
+};
+
+// A lane's run counters, added to the run's by the warp at the end.
+struct PacketCounts {
+  unsigned launch = 0, flight = 0, coll = 0, seg = 0, esc = 0, rrk = 0, rrs = 0, scl = 0, evl = 0;
+  int w_launch = 0;  // |W0| = 1
+  WeightSum w_esc, w_rr, w_kill;
+  __device__ void add_to(DevStats *st, unsigned *flags, int lane) const {
+    auto add = [&](unsigned long long *dst, unsigned v) {
+      const unsigned t = __reduce_add_sync(kFull, v);
+      if (lane == 0 && t) atomicAdd(dst, (unsigned long long)t);
+      return t;
+    };
+    auto addw = [&](double *dst, double v) {
+      const double t = warp_sum(v);
+      if (lane == 0 && t != 0.0) atomicAdd(dst, t);
+    };
+    add(&st->launched, launch);
+    add(&st->flights, flight);
+    add(&st->collisions, coll);
+    add(&st->segments, seg);
+    add(&st->escapes, esc);
+    add(&st->rr_kill, rrk);
+    add(&st->rr_survive, rrs);
+    add(&st->scatter_limit, scl);
+    if (add(&st->event_limit, evl) && lane == 0) atomicOr(flags, kFlagEventLimit);
+    addw(&st->launched_w, (double)w_launch);
+    addw(&st->escaped_w, w_esc.value());
+    addw(&st->rr_net_w, w_rr.value());
+    addw(&st->killed_w, w_kill.value());
+  }
+};
+
+// The warps of a grid in an order that spreads the first ones over the SMs and their schedulers (blocks
+// b, b + n_sm, ... run on one SM, and a block's warp w on scheduler w mod 4).
+__device__ __forceinline__ unsigned warp_place(int n_sm) {
+  const unsigned wid = (threadIdx.x >> 5) + blockIdx.x / (unsigned)n_sm;
+  return (wid % (blockDim.x >> 5)) * gridDim.x + blockIdx.x;
+}
+
+// Per-flight geometry of one axis: the offset of the edge ahead and 1 / |s|.  A nonzero component keeps a
+// finite reciprocal (so that 0 x it is 0); a zero one gets infinity, and 0 x infinity = NaN loses every
+// comparison of the segment.
+__device__ __forceinline__ void set_axis(float s, float dx, float &o, float &inv) {
+  inv = __frcp_rn(fabsf(s));
+  if (s != 0.f) inv = fminf(inv, 3.402823466e38f);
+  o = s > 0.f ? dx : 0.f;
+}
+
 template <bool BATCH>
 __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __grid_constant__ TransportParams p) {
   extern __shared__ unsigned hist[];  // records per bin of this block
   if (*p.flags & kFlagMedium) return;
-  if (p.rec_prev && p.rec_prev->paused == 0u) return;  // every packet has ended
+  // packets that the previous launch left, and whether there are new ones to launch
+  const unsigned n_in = p.rec_prev ? p.rec_prev->n_left : 0u;
+  const bool fresh = !p.rec_prev || p.rec_prev->fresh;
+  if (!n_in && !fresh) return;  // every packet has ended
+  const unsigned in_buf = p.rec_prev ? p.rec_prev->buf : 1u;
+  if (threadIdx.x == 0) p.rec_hdr->buf = 1u - in_buf;
   const int lane = threadIdx.x & 31;
+  const unsigned place = warp_place(p.n_sm);
+  // Once no more than `enough` packets are left the launch pauses, so that the next one packs them into
+  // full warps, or the tail runs them.
+  const unsigned lanes = gridDim.x * blockDim.x;
+  const unsigned in_use = fresh ? (unsigned)min(p.total_packets, (unsigned long long)lanes) : n_in;
+  const unsigned enough = max(in_use / 2u, p.tail_max);
   for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x) hist[i] = 0u;
   __syncthreads();
 
@@ -105,43 +198,27 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
   int ix = 0, iz = 0;
   float4 m = make_float4(0.f, 0.f, CUDART_INF_F, CUDART_INF_F);
   unsigned flight = 0, nscat = 0, cu1 = 0, cu2 = 0;
-  unsigned n_launch = 0, n_flight = 0, n_coll = 0, n_seg = 0, n_esc = 0, n_rrk = 0, n_rrs = 0, n_scl = 0, n_evl = 0;
-  int w_launch = 0;  // |W0| = 1
-  WeightSum w_esc, w_rr, w_kill;
+  PacketCounts n;
 
   auto load_mu = [&]() {
     if (MCR_GUARD(p.flags, (unsigned)ix < (unsigned)NX() && (unsigned)iz < (unsigned)NZ())) m = __ldg(MU() + iz * NX() + ix);
   };
-  // Per-flight geometry.  A nonzero component keeps a finite reciprocal (so that 0 x it is 0); a zero
-  // one gets infinity, and 0 x infinity = NaN loses every comparison below.
   auto set_direction = [&]() {
-    inv_ax = __frcp_rn(fabsf(sx));
-    inv_az = __frcp_rn(fabsf(sz));
-    if (sx != 0.f) inv_ax = fminf(inv_ax, 3.402823466e38f);
-    if (sz != 0.f) inv_az = fminf(inv_az, 3.402823466e38f);
-    ox = sx > 0.f ? DX() : 0.f;
-    oz = sz > 0.f ? DX() : 0.f;
+    set_axis(sx, DX(), ox, inv_ax);
+    set_axis(sz, DX(), oz, inv_az);
   };
 
-  const size_t slot = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (p.rec_prev) {
-    const SavedPacket s = load_packet(p.saved, p.n_saved, slot);
-    alive = s.alive, exhausted = s.exhausted;
-    if (alive) {
-      take_problem(s.prob);
-      pid = s.pid, fx = s.fx, fz = s.fz, sx = s.sx, sz = s.sz, W = s.W, tau = s.tau, ix = s.ix, iz = s.iz;
-      flight = s.flight, nscat = s.nscat, cu1 = s.cu1, cu2 = s.cu2;
-      set_direction();
-      load_mu();
-    }
+  // the packets left by the previous launch, 32 to a warp
+  bool carrying = false;  // the lane has a packet, or one whose end is not yet counted
+  if (place * 32u + lane < n_in) {
+    const SavedPacket s = load_packet(p.saved + (size_t)in_buf * 4 * p.n_saved, p.n_saved, place * 32u + lane);
+    take_problem(s.prob);
+    pid = s.pid, fx = s.fx, fz = s.fz, sx = s.sx, sz = s.sz, W = s.W, tau = s.tau, ix = s.ix, iz = s.iz;
+    flight = s.flight, nscat = s.nscat, cu1 = s.cu1, cu2 = s.cu2;
+    set_direction();
+    load_mu();
+    alive = carrying = true;
   }
-
-  float4 *out = nullptr;     // the warp's block of record slots, filled to `fill`
-  unsigned fill = kRecBlock;
-  bool stop = false;         // warp-uniform: the record buffer is full
-  auto pad = [&]() {
-    for (unsigned j = fill + lane; j < kRecBlock; j += 32) out[j] = make_float4(__uint_as_float(kRecSentinel), 0.f, 0.f, 1.f);
-  };
 
   // One pixel segment of a flying packet: advances it, sets pend at a collision, ends the packet at the
   // grid's edge; returns whether there is a record (row, ts and the flight's direction).
@@ -155,7 +232,7 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
     const float em1 = expm1f(-m.x * l);
     const float t = m.x > 0.f ? (-W * em1) * m.z : W * l;
     W = fmaf(W, em1, W);
-    ++n_seg;
+    ++n.seg;
     ts = t * QS();
     row = ROW() + (unsigned)(iz * NX() + ix);
     tau = fmaxf(fmaf(-m.y, l, tau), 0.f);  // (a collision draws a new one)
@@ -168,8 +245,8 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
       fx = cx ? DX() - ox : fx;
       fz = cx ? fz : DX() - oz;
       if ((unsigned)ix >= (unsigned)NX() || (unsigned)iz >= (unsigned)NZ()) {
-        ++n_esc;
-        w_esc.add(W);
+        ++n.esc;
+        n.w_esc.add(W);
         alive = false;
       } else {
         m = __ldg(MU() + iz * NX() + ix);
@@ -188,10 +265,10 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
   // flight's numbers depend on nothing here and are drawn first, beside the scatter's own chain.
   auto collide = [&]() {
     pend = false;
-    ++n_coll;
+    ++n.coll;
     if (nscat >= p.max_scatter) {
-      ++n_scl;
-      w_kill.add(W);
+      ++n.scl;
+      n.w_kill.add(W);
       alive = false;
       return;
     }
@@ -203,50 +280,61 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
     if (fabsf(W) < p.w_threshold) {  // |W0| = 1
       if (u01(u2) < p.rr_p) {
         const float Wn = W * p.rr_inv_p;
-        w_rr.add(Wn);
-        w_rr.add(-W);
+        n.w_rr.add(Wn);
+        n.w_rr.add(-W);
         W = Wn;
-        ++n_rrs;
+        ++n.rrs;
       } else {
-        w_rr.add(-W);
-        ++n_rrk;
+        n.w_rr.add(-W);
+        ++n.rrk;
         alive = false;
         return;
       }
     }
     if (flight >= p.max_events) {
-      ++n_evl;
-      w_kill.add(W);
+      ++n.evl;
+      n.w_kill.add(W);
       alive = false;
       return;
     }
     ++flight;
-    ++n_flight;
+    ++n.flight;
   };
 
-  for (;;) {
-    if (fill + 32 > kRecBlock) {  // room for one step's records
-      pad();
-      unsigned b = 0;
-      if (lane == 0) b = atomicAdd(&p.rec_hdr->blocks, 1u);
-      b = __shfl_sync(kFull, b, 0);
-      stop = b >= p.rec_blocks;
-      fill = stop ? kRecBlock : 0u;
-      if (!stop) out = p.records + (size_t)b * kRecBlock;
+  // Ends of packets, counted for the whole call; true when the launch should pause.  (The count is read
+  // only by warps that have found no more packets to launch: the answer takes a round trip to L2.)
+  auto count_ends = [&]() -> bool {
+    const unsigned ends = __ballot_sync(kFull, carrying && !alive);
+    if (!alive) carrying = false;
+    const bool draining = __any_sync(kFull, exhausted);
+    unsigned ended = 0u;
+    if (lane == 0) {
+      if (ends) atomicAdd(p.ended, (unsigned)__popc(ends));
+      if (draining) ended = *(volatile unsigned *)p.ended;
     }
+    return draining && p.total_packets - __shfl_sync(kFull, ended, 0) <= enough;
+  };
+
+  RecordWriter w;
+  w.stop = in_use <= enough;  // nothing for this kernel to do but launch the first packets
+  bool first = p.rec_prev == nullptr;
+  for (;;) {
+    w.room(p, lane);
     unsigned flying = __ballot_sync(kFull, alive && !pend);
-    if (stop || __popc(flying) < kFlyMin) {
+    if (w.stop || __popc(flying) < kFlyMin) {
       if (pend) collide();
-      if (stop) break;
+      if (count_ends()) w.stop = true;
+      if (w.stop && !first) break;  // (the first packets are launched all the same)
       // ------------------------------------------------------------- refill / launch
       const unsigned need = __ballot_sync(kFull, !alive && !exhausted);
       if (need) {
         const int leader = __ffs(need) - 1;
         unsigned long long base = 0;
-        if (lane == leader) base = atomicAdd(p.work, (unsigned long long)__popc(need));
+        if (lane == leader && !first) base = atomicAdd(p.work, (unsigned long long)__popc(need)) + p.work_base;
         base = __shfl_sync(kFull, base, leader);
         if (!alive && !exhausted) {
-          const unsigned long long g = base + __popc(need & ((1u << lane) - 1u));
+          // the first packets go to the warps by their place
+          const unsigned long long g = first ? place * 32u + lane : base + __popc(need & ((1u << lane) - 1u));
           if (g >= p.total_packets) {
             exhausted = true;
           } else {
@@ -264,22 +352,23 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
             const ProblemDesc &P = p.prob[lo];
             pid = P.first_packet + (g - (lo ? p.prob[lo - 1].end : 0ull));
             take_problem(lo);
-            ++n_launch;
+            ++n.launch;
+            carrying = true;
             float W0;
             const bool inside = launch_packet(P, pid, NX(), NZ(), DX(), KEY0(), KEY1(), ix, iz, fx, fz, sx, sz, W0);
             W = W0;
-            w_launch += (int)W0;
+            n.w_launch += (int)W0;
             nscat = 0;
             flight = 0;
             if (!inside) {
-              ++n_esc;
-              w_esc.add(W);
+              ++n.esc;
+              n.w_esc.add(W);
             } else if (p.max_events == 0u) {
-              ++n_evl;
-              w_kill.add(W);
+              ++n.evl;
+              n.w_kill.add(W);
             } else {
               flight = 1;
-              ++n_flight;
+              ++n.flight;
               alive = true;
               draw_flight(1u);
               set_direction();
@@ -288,33 +377,11 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
           }
         }
       }
+      first = false;
+      if (w.stop) break;
       flying = __ballot_sync(kFull, alive);
       if (!flying) {
         if (__all_sync(kFull, exhausted)) break;
-        continue;
-      }
-      // The last packets of a run: a warp with few packets left and none to come lets each of them run
-      // on its own share of the block, with no vote per segment -- what then counts is the latency of
-      // one packet's chain.
-      const int n = __popc(flying);
-      if (n <= kFewLanes && __all_sync(kFull, alive || exhausted)) {
-        const unsigned per = (kRecBlock - fill) / n;
-        unsigned k = 0;
-        float4 *const own = out + fill + __popc(flying & ((1u << lane) - 1u)) * per;
-        while (alive && k < per) {
-          unsigned row;
-          float ts;
-          const float ux = sx, uz = sz;
-          if (segment(row, ts) && MCR_GUARD(p.flags, (row >> p.bin_shift) < (unsigned)p.n_bins)) {
-            own[k++] = make_float4(__uint_as_float(row), ts, ux, uz);
-            atomicAdd(&hist[row >> p.bin_shift], 1u);
-          }
-          if (pend) collide();
-        }
-        if ((flying >> lane) & 1u)
-          for (; k < per; ++k) own[k] = make_float4(__uint_as_float(kRecSentinel), 0.f, 0.f, 1.f);
-        fill += n * per;
-        __syncwarp();
         continue;
       }
     }
@@ -324,52 +391,225 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
     unsigned row = 0u;
     float ts = 0.f;
     if (alive && !pend) has = segment(row, ts);
-    const unsigned who = __ballot_sync(kFull, has);
-    if (has && MCR_GUARD(p.flags, (row >> p.bin_shift) < (unsigned)p.n_bins)) {
-      out[fill + __popc(who & ((1u << lane) - 1u))] = make_float4(__uint_as_float(row), ts, sx, sz);
-      atomicAdd(&hist[row >> p.bin_shift], 1u);
+    w.put(p, hist, lane, has, row, ts, sx, sz);
+  }
+  if (w.fill < kRecBlock) w.pad(lane);
+  count_ends();
+  // the packets left go to the next launch, close together
+  const unsigned left = __ballot_sync(kFull, alive);
+  if (left) {
+    unsigned at = 0u;
+    if (lane == 0) at = atomicAdd(&p.rec_hdr->n_left, (unsigned)__popc(left));
+    at = __shfl_sync(kFull, at, 0) + __popc(left & ((1u << lane) - 1u));
+    if (alive && MCR_GUARD(p.flags, at < p.n_saved)) {
+      SavedPacket s;
+      s.pid = pid, s.fx = fx, s.fz = fz, s.sx = sx, s.sz = sz, s.W = W, s.tau = tau, s.ix = ix, s.iz = iz, s.prob = prob;
+      s.flight = flight, s.nscat = nscat, s.cu1 = cu1, s.cu2 = cu2;
+      save_packet(p.saved + (size_t)(1u - in_buf) * 4 * p.n_saved, p.n_saved, at, s);
     }
-    fill += __popc(who);
   }
-  if (fill < kRecBlock) pad();  // slots left empty hold a sentinel that the sort skips
-
-  SavedPacket s;
-  s.pid = pid, s.fx = fx, s.fz = fz, s.sx = sx, s.sz = sz, s.W = W, s.tau = tau, s.ix = ix, s.iz = iz, s.prob = prob;
-  s.flight = flight, s.nscat = nscat, s.cu1 = cu1, s.cu2 = cu2, s.alive = alive, s.exhausted = exhausted;
-  save_packet(p.saved, p.n_saved, slot, s);
-  if (__any_sync(kFull, alive || !exhausted) && lane == 0) p.rec_hdr->paused = 1u;
-  // ---------------------------------------------------------------- counters
-  const unsigned c_launch = __reduce_add_sync(kFull, n_launch), c_flight = __reduce_add_sync(kFull, n_flight),
-                 c_coll = __reduce_add_sync(kFull, n_coll), c_seg = __reduce_add_sync(kFull, n_seg),
-                 c_esc = __reduce_add_sync(kFull, n_esc), c_rrk = __reduce_add_sync(kFull, n_rrk),
-                 c_rrs = __reduce_add_sync(kFull, n_rrs), c_scl = __reduce_add_sync(kFull, n_scl),
-                 c_evl = __reduce_add_sync(kFull, n_evl);
-  const double s_launch = (double)__reduce_add_sync(kFull, w_launch), s_esc = warp_sum(w_esc.value()),
-               s_rr = warp_sum(w_rr.value()), s_kill = warp_sum(w_kill.value());
-  if (lane == 0) {
-    DevStats *st = p.stats;
-    auto add = [](unsigned long long *dst, unsigned v) {
-      if (v) atomicAdd(dst, (unsigned long long)v);
-    };
-    auto addw = [](double *dst, double v) {
-      if (v != 0.0) atomicAdd(dst, v);
-    };
-    if (c_evl) atomicOr(p.flags, kFlagEventLimit);
-    add(&st->launched, c_launch);
-    add(&st->flights, c_flight);
-    add(&st->collisions, c_coll);
-    add(&st->segments, c_seg);
-    add(&st->escapes, c_esc);
-    add(&st->rr_kill, c_rrk);
-    add(&st->rr_survive, c_rrs);
-    add(&st->scatter_limit, c_scl);
-    add(&st->event_limit, c_evl);
-    addw(&st->launched_w, s_launch);
-    addw(&st->escaped_w, s_esc);
-    addw(&st->rr_net_w, s_rr);
-    addw(&st->killed_w, s_kill);
-  }
+  n.add_to(p.stats, p.flags, lane);
   __syncthreads();
+  for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x)
+    if (hist[i]) atomicAdd(p.rec_hist + i, hist[i]);
+}
+
+// ------------------------------------------------------------------------------------------ tail
+// The last packets of a run (256 x 256, 1e3 packets: 6.3 ms with the loop of the direct deposit, 3.4 with the
+// one above, 1.2 here; 460 cycles a segment, a chain of dependent instructions).
+// A packet that stays in the medium lives for thousands of segments, and once
+// there are few packets to a warp the run lasts as long as one packet's chain of segments; a warp with
+// one lane in use would take every step of the loop above for it.  So a whole warp follows one packet:
+// all lanes take the same steps (no divergence), the lanes draw the numbers of 32 flights at once, and
+// what does not steer the packet -- track weights, the weight itself -- is computed for 32 segments at
+// once, one per lane, in the same order of operations.  The pixels ahead are loaded a segment early.
+__global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant__ TransportParams p) {
+  extern __shared__ unsigned hist[];  // records per bin of this block
+  if (*p.flags & kFlagMedium) return;
+  const unsigned n_in = p.rec_hdr->n_left;
+  if (n_in == 0u || n_in > p.tail_max || *p.work + p.work_base < p.total_packets) return;
+  for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x) hist[i] = 0u;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const unsigned n_warps = gridDim.x * (blockDim.x >> 5), in_buf = p.rec_hdr->buf;
+  PacketCounts n;
+  RecordWriter w;
+  unsigned i = warp_place(p.n_sm);  // the warp's packet; then the next one not yet taken
+  while (i < n_in) {
+    SavedPacket s = load_packet(p.saved + (size_t)in_buf * 4 * p.n_saved, p.n_saved, i);
+    const ProblemDesc &P = p.prob[s.prob];
+    const float4 *const mu = P.mu;
+    const int nx = P.nx, nz = P.nz;
+    const float dx = P.dx, hg_c = P.hg_c, qscale = P.qscale;
+    const unsigned key0 = P.key0, key1 = P.key1, row_base = P.row_base;
+    const unsigned long long pid = s.pid;
+    float fx = s.fx, fz = s.fz, sx = s.sx, sz = s.sz, W = s.W, tau = s.tau;
+    int ix = s.ix, iz = s.iz;
+    unsigned flight = s.flight, nscat = s.nscat;
+    float inv_ax, inv_az, ox, oz;
+    // this pixel and the next ones in x and z (mu has margins: a pixel's neighbours are always there)
+    const float4 *at = mu + iz * nx + ix;
+    int step_x = 1, step_z = 1, stride_z = nx;
+    float4 m = __ldg(at), mx = m, mz = m;
+    auto look_ahead = [&]() {
+      mx = __ldg(at + step_x);
+      mz = __ldg(at + stride_z);
+    };
+    auto set_direction = [&]() {
+      set_axis(sx, dx, ox, inv_ax);
+      set_axis(sz, dx, oz, inv_az);
+      step_x = sx > 0.f ? 1 : -1;
+      step_z = sz > 0.f ? 1 : -1;
+      stride_z = sz > 0.f ? nx : -nx;
+      look_ahead();
+    };
+    set_direction();
+    unsigned first = 0u;  // lane k holds the numbers of flight first + k: tau, rotation, roulette uniform
+    float n_tau = 0.f, n_cs = 1.f, n_sn = 0.f, n_u = 0.f;
+    auto draw_flights = [&]() {
+      first = flight;
+      const uint4 r = philox4x32_10(pid, flight + lane + 1u, key0, key1);
+      n_tau = -logf(u01(r.x));
+      hg_rotation(hg_c, u01(r.y), n_cs, n_sn);
+      n_u = u01(r.z);
+    };
+    draw_flights();
+    bool ended = false;
+    while (!ended) {
+      w.room(p, lane);  // (before a batch, so that one is never left half written)
+      if (w.stop) break;
+      unsigned row = 0u;  // the lane's segment of the batch
+      float len = 0.f, mua = 0.f, imua = 0.f, ux = 0.f, uz = 1.f;
+      int cnt = 0;
+      float loss = 0.f;  // sum of mu_a l of the batch
+      // the batch's track weights and records; W becomes exact again
+      auto flush = [&]() {
+        const float em1 = lane < cnt ? expm1f(-mua * len) : 0.f;
+        float mine = W;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {  // (past the batch W + W 0)
+          const float e = __shfl_sync(kFull, em1, k);
+          mine = k == lane ? W : mine;
+          W = fmaf(W, e, W);
+        }
+        const float t = mua > 0.f ? (-mine * em1) * imua : mine * len;
+        w.put(p, hist, lane, lane < cnt && t != 0.f && MCR_GUARD(p.flags, isfinite(t)), row, t * qscale, ux, uz);
+        if (lane == 0) n.seg += cnt;
+        cnt = 0;
+      };
+      while (cnt < 32 && !ended) {
+        bool hit, inside = true;
+        do {  // segments up to a collision, the grid's edge or the end of the batch
+          const float dist_x = fabsf(ox - fx) * inv_ax, dist_z = fabsf(oz - fz) * inv_az;
+          const float d_edge = fminf(dist_x, dist_z);
+          const float d_coll = tau * m.w;
+          hit = d_coll < d_edge;
+          const float l = fminf(d_coll, d_edge);
+          if (lane == cnt) {
+            row = row_base + (unsigned)(iz * nx + ix);
+            len = l;
+            mua = m.x;
+            imua = m.z;
+            ux = sx;
+            uz = sz;
+          }
+          ++cnt;
+          loss = fmaf(m.x, l, loss);
+          fx = clamp_dx(fmaf(l, sx, fx), dx);
+          fz = clamp_dx(fmaf(l, sz, fz), dx);
+          if (hit) break;
+          tau = fmaxf(fmaf(-m.y, l, tau), 0.f);
+          const bool cx = dist_x == d_edge;
+          ix += cx ? step_x : 0;
+          iz += cx ? 0 : step_z;
+          at += cx ? step_x : stride_z;
+          fx = cx ? dx - ox : fx;
+          fz = cx ? fz : dx - oz;
+          m = cx ? mx : mz;
+          inside = (unsigned)ix < (unsigned)nx && (unsigned)iz < (unsigned)nz;
+          if (inside) look_ahead();
+        } while (inside && cnt < 32);
+        if (!hit) {
+          if (inside) continue;
+          flush();
+          if (lane == 0) {
+            ++n.esc;
+            n.w_esc.add(W);
+          }
+          ended = true;
+          continue;
+        }
+        if (lane == 0) ++n.coll;
+        if (nscat >= p.max_scatter) {
+          flush();
+          if (lane == 0) {
+            ++n.scl;
+            n.w_kill.add(W);
+          }
+          ended = true;
+          continue;
+        }
+        const int k = (int)(flight - first);
+        rotate(__shfl_sync(kFull, n_cs, k), __shfl_sync(kFull, n_sn, k), sx, sz);
+        ++nscat;
+        // |W| is at least |W at the last flush| (1 - loss): the exact weight is needed only when that does
+        // not settle the threshold
+        if (!(fabsf(W) * (1.f - loss) >= 1.001f * p.w_threshold)) {
+          flush();
+          if (fabsf(W) < p.w_threshold) {
+            if (__shfl_sync(kFull, n_u, k) < p.rr_p) {
+              const float Wn = W * p.rr_inv_p;
+              if (lane == 0) {
+                n.w_rr.add(Wn);
+                n.w_rr.add(-W);
+                ++n.rrs;
+              }
+              W = Wn;
+            } else {
+              if (lane == 0) {
+                n.w_rr.add(-W);
+                ++n.rrk;
+              }
+              ended = true;
+              continue;
+            }
+          }
+        }
+        if (flight >= p.max_events) {
+          flush();
+          if (lane == 0) {
+            ++n.evl;
+            n.w_kill.add(W);
+          }
+          ended = true;
+          continue;
+        }
+        ++flight;
+        if (lane == 0) ++n.flight;
+        if (flight - first == 32u) draw_flights();
+        tau = __shfl_sync(kFull, n_tau, (int)(flight - first));
+        set_direction();
+        if (cnt == 0) break;  // flushed: a new batch needs its own room
+      }
+      if (cnt) flush();
+    }
+    if (lane == 0) {
+      if (ended) {
+        atomicAdd(p.ended, 1u);
+      } else {  // (the buffer is full: the packets still to come pass straight on)
+        const uint4 r = philox4x32_10(pid, flight + 1u, key0, key1);
+        s.fx = fx, s.fz = fz, s.sx = sx, s.sz = sz, s.W = W, s.tau = tau, s.ix = ix, s.iz = iz;
+        s.flight = flight, s.nscat = nscat, s.cu1 = r.y, s.cu2 = r.z;
+        save_packet(p.saved + (size_t)(1u - in_buf) * 4 * p.n_saved, p.n_saved, atomicAdd(&p.rec_hdr->n_tail_left, 1u), s);
+      }
+      i = n_warps + atomicAdd(&p.rec_hdr->tail_next, 1u);
+    }
+    i = __shfl_sync(kFull, i, 0);
+  }
+  if (w.fill < kRecBlock) w.pad(lane);
+  n.add_to(p.stats, p.flags, lane);
+  __syncthreads();
+  if (threadIdx.x == 0) p.rec_hdr->tail_ran = 1u;
   for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x)
     if (hist[i]) atomicAdd(p.rec_hist + i, hist[i]);
 }
@@ -420,10 +660,20 @@ __device__ unsigned scan_into(int n, unsigned *off, unsigned *warp_tot, F f) {
 }
 
 // Counts per bin -> offsets, cursors and the offsets of the bins' work units (batches of `batch`
-// records); clears the counts for the next launch.  n_units: the launch's word for their number.
-__global__ void __launch_bounds__(1024) k_rec_scan(const RecordHeader *hdr, unsigned *n_units, unsigned *hist, int n,
-                                                   int batch, unsigned *off, unsigned *cur, unsigned *unit_off) {
+// records); clears the counts for the next launch.  n_units: the launch's word for their number.  Also
+// settles, for every warp of the next launch alike, what is left to it.
+__global__ void __launch_bounds__(1024) k_rec_scan(RecordHeader *hdr, unsigned *n_units, unsigned *hist, int n,
+                                                   int batch, unsigned *off, unsigned *cur, unsigned *unit_off,
+                                                   const unsigned long long *launched, unsigned long long n_packets) {
   __shared__ unsigned warp_tot[32];
+  if (threadIdx.x == 0) {
+    if (*launched < n_packets) hdr->fresh = 1u;
+    if (hdr->tail_ran == 1u) {  // what the tail left stands in the other buffer
+      hdr->n_left = hdr->n_tail_left;
+      hdr->buf = 1u - hdr->buf;
+      hdr->tail_ran = 2u;
+    }
+  }
   if (hdr->blocks == 0u) return;
   scan_into(n, off, warp_tot, [&](int i) { return hist[i]; });
   const unsigned units = scan_into(n, unit_off, warp_tot, [&](int i) { return (hist[i] + batch - 1) / batch; });
@@ -807,10 +1057,10 @@ size_t sort_smem(int n_bins) { return (size_t)kSortBatch * 16 + (size_t)n_bins *
 
 struct Scratch {  // rec_scratch, laid out
   RecordHeader *hdr;
-  unsigned *saved_work;
+  unsigned *saved_work, *ended;
   unsigned *hist, *off, *cur, *unit_off;                  // bins of the first pass
   unsigned *tile_hist, *tile_off, *tile_cur, *dep_unit_off;  // tiles (the same arrays after a single pass)
-  uint4 *saved;
+  uint4 *saved;  // two buffers, read and written by turns
   size_t zeroed, total;
 };
 Scratch layout(unsigned char *base, const RecordPlan &pl) {
@@ -823,6 +1073,7 @@ Scratch layout(unsigned char *base, const RecordPlan &pl) {
   };
   s.hdr = reinterpret_cast<RecordHeader *>(take(pl.launches * sizeof(RecordHeader)));
   s.saved_work = reinterpret_cast<unsigned *>(take(4));
+  s.ended = reinterpret_cast<unsigned *>(take(4));
   auto words = [&](size_t n) { return reinterpret_cast<unsigned *>(take(n * 4)); };
   const bool two = pl.coarse_shift > 0;
   s.hist = words(pl.n_coarse);
@@ -834,7 +1085,7 @@ Scratch layout(unsigned char *base, const RecordPlan &pl) {
   s.tile_off = two ? words(pl.n_tiles + 1) : s.off;
   s.tile_cur = two ? words((size_t)pl.n_tiles * kCurStride) : s.cur;
   s.dep_unit_off = two ? words(pl.n_tiles + 1) : s.unit_off;
-  s.saved = reinterpret_cast<uint4 *>(take((size_t)pl.lanes * 64));
+  s.saved = reinterpret_cast<uint4 *>(take((size_t)pl.lanes * 128));
   s.total = at;
   return s;
 }
@@ -878,7 +1129,7 @@ cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64
   if (cfg.record_capacity <= 0) cap = cap < (1ull << 22) ? (1ull << 22) : cap;
   if (cap > (1ull << 28)) cap = 1ull << 28;
   pl.blocks = (unsigned)((cap + kRecBlock - 1) / kRecBlock);
-  const uint64_t want = (packets * kSegmentsPerPacket + (uint64_t)pl.blocks * kRecBlock - 1) / ((uint64_t)pl.blocks * kRecBlock) + 1;
+  const uint64_t want = (packets * kSegmentsPerPacket + (uint64_t)pl.blocks * kRecBlock - 1) / ((uint64_t)pl.blocks * kRecBlock) + 7;
   pl.launches = (unsigned)(want < kMaxLaunches ? want : kMaxLaunches);
   pl.threads = cfg.threads_per_block > 0 ? cfg.threads_per_block : 256;
   int sms = 0, per_sm = 0;
@@ -890,6 +1141,8 @@ cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64
   if (e != cudaSuccess) return e;
   if (cfg.blocks_per_sm > 0 && cfg.blocks_per_sm < per_sm) per_sm = cfg.blocks_per_sm;
   pl.lanes = (unsigned)(sms * per_sm * pl.threads);
+  if ((e = rec_blocks_per_sm(k_transport_tail, kTailThreads, smem, &per_sm)) != cudaSuccess) return e;
+  pl.tail_blocks = sms * per_sm;
   *out = pl;
   return cudaSuccess;
 }
@@ -919,9 +1172,15 @@ cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg,
   q.rec_hist = sc.hist;
   q.bin_shift = pl.tile_shift + pl.coarse_shift;
   q.n_bins = pl.n_coarse;
+  q.ended = sc.ended;
+  q.n_sm = sms;
   q.saved = sc.saved;
   q.n_saved = pl.lanes;
   q.saved_work = sc.saved_work;
+  q.tail_max = pl.tail_blocks * (kTailThreads / 32) * kTailPackets;
+  q.work_base = pl.lanes;
+  // the count at which `work` has launched the last packet
+  const unsigned long long to_launch = p.total_packets > q.work_base ? p.total_packets - q.work_base : 0ull;
   const unsigned grid = pl.lanes / pl.threads;
   const size_t smem = (size_t)pl.n_coarse * 4;
   for (unsigned i = 0; i < pl.launches; ++i) {
@@ -932,15 +1191,16 @@ cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg,
       k_transport_rec<true><<<grid, pl.threads, smem, s>>>(q);
     else
       k_transport_rec<false><<<grid, pl.threads, smem, s>>>(q);
+    k_transport_tail<<<pl.tail_blocks, kTailThreads, smem, s>>>(q);
     k_rec_scan<<<1, 1024, 0, s>>>(hdr, two ? &hdr->n_coarse_units : &hdr->n_units, sc.hist, pl.n_coarse,
-                                  two ? kSortBatch : dc.batch, sc.off, sc.cur, sc.unit_off);
+                                  two ? kSortBatch : dc.batch, sc.off, sc.cur, sc.unit_off, p.work, to_launch);
     k_rec_sort<true><<<sms * sort1, kSortThreads, smem1, s>>>(buf_a, buf_b, hdr, pl.blocks, q.bin_shift, pl.n_coarse,
                                                               sc.cur, capacity, nullptr, nullptr, 0, 0, p.flags);
     if (two) {
       k_rec_count<<<sms * 4, kSortThreads, 0, s>>>(buf_b, hdr, sc.off, sc.unit_off, pl.n_coarse, pl.coarse_shift,
                                                    pl.tile_shift, sc.tile_hist, p.flags);
       k_rec_scan<<<1, 1024, 0, s>>>(hdr, &hdr->n_units, sc.tile_hist, pl.n_tiles, dc.batch, sc.tile_off, sc.tile_cur,
-                                    sc.dep_unit_off);
+                                    sc.dep_unit_off, p.work, to_launch);
       k_rec_sort<false><<<sms * sort2, kSortThreads, smem2, s>>>(
           buf_b, buf_a, hdr, pl.blocks, pl.tile_shift, 1 << pl.coarse_shift, sc.tile_cur, capacity, sc.off, sc.unit_off, pl.n_coarse, pl.coarse_shift, p.flags);
     }

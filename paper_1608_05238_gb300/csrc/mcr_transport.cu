@@ -72,7 +72,9 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
   unsigned long long *const stally =
       reinterpret_cast<unsigned long long *>(smem + (size_t)blockDim.x * (MERGE ? 2 : 1) * p.row_stride);
   if (*p.flags & kFlagMedium) return;
-  if (p.saved && p.rec_prev->paused == 0u) return;  // the record launches ran every packet to its end
+  const unsigned n_saved = p.saved ? p.rec_prev->n_left : 0u;
+  // nothing is left when the record launches ran every packet to its end
+  if (p.saved && n_saved == 0u && *p.work + p.work_base >= p.total_packets) return;
   if (STALLY) {
     const size_t nw = (size_t)p.prob[0].nx * p.prob[0].nz * p.Cpad;
     for (size_t i = threadIdx.x; i < nw; i += blockDim.x) stally[i] = 0ull;
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
     }
   };
 
-  bool more_saved = !ROWLESS && !STALLY && p.saved != nullptr;  // warp-uniform
+  bool more_saved = !ROWLESS && !STALLY && n_saved > 0u;  // warp-uniform
   for (;;) {
     // ---------------------------------------------------------------- refill / launch
     const unsigned need = __ballot_sync(kFull, !alive && !exhausted);
@@ -181,39 +183,37 @@ __global__ void __launch_bounds__(256) k_transport(const __grid_constant__ Trans
       if (lane == leader) base = atomicAdd(p.saved_work, (unsigned)__popc(need));
       base = __shfl_sync(kFull, base, leader);
       const unsigned i = base + __popc(need & ((1u << lane) - 1u));
-      if (((need >> lane) & 1u) && i < p.n_saved) {
-        const SavedPacket sp = load_packet(p.saved, p.n_saved, i);
-        if (sp.alive) {
-          if (BATCH) {
-            const ProblemDesc &P = p.prob[sp.prob];
-            mu = P.mu;
-            prob = sp.prob;
-            nx = P.nx;
-            nz = P.nz;
-            dx = P.dx;
-            hg_c = P.hg_c;
-            qscale = P.qscale;
-            key0 = P.key0;
-            key1 = P.key1;
-          }
-          pid = sp.pid;
-          fx = sp.fx, fz = sp.fz, sx = sp.sx, sz = sp.sz, W = sp.W, tau = sp.tau;
-          ix = sp.ix, iz = sp.iz;
-          flight = sp.flight, nscat = sp.nscat, cu1 = sp.cu1, cu2 = sp.cu2;
-          inv_ax = __frcp_rn(fabsf(sx));
-          inv_az = __frcp_rn(fabsf(sz));
-          if constexpr (!ROWLESS) write_row();
-          if constexpr (!BATCH) mcur = load_mu();
-          alive = true;
+      if (((need >> lane) & 1u) && i < n_saved) {
+        const SavedPacket sp = load_packet(p.saved + (size_t)p.rec_prev->buf * 4 * p.n_saved, p.n_saved, i);
+        if (BATCH) {
+          const ProblemDesc &P = p.prob[sp.prob];
+          mu = P.mu;
+          prob = sp.prob;
+          nx = P.nx;
+          nz = P.nz;
+          dx = P.dx;
+          hg_c = P.hg_c;
+          qscale = P.qscale;
+          key0 = P.key0;
+          key1 = P.key1;
         }
+        pid = sp.pid;
+        fx = sp.fx, fz = sp.fz, sx = sp.sx, sz = sp.sz, W = sp.W, tau = sp.tau;
+        ix = sp.ix, iz = sp.iz;
+        flight = sp.flight, nscat = sp.nscat, cu1 = sp.cu1, cu2 = sp.cu2;
+        inv_ax = __frcp_rn(fabsf(sx));
+        inv_az = __frcp_rn(fabsf(sz));
+        if constexpr (!ROWLESS) write_row();
+        if constexpr (!BATCH) mcur = load_mu();
+        alive = true;
       }
-      if (base + __popc(need) >= p.n_saved) more_saved = false;
+      if (base + __popc(need) >= n_saved) more_saved = false;
       continue;
     }
     if (need) {
       const int leader = __ffs(need) - 1;
       unsigned long long base = 0;
-      if (lane == leader) base = atomicAdd(p.work, (unsigned long long)__popc(need));
+      if (lane == leader) base = atomicAdd(p.work, (unsigned long long)__popc(need)) + p.work_base;
       base = __shfl_sync(kFull, base, leader);
       if (!alive && !exhausted) {
         const unsigned long long step = base + __popc(need & ((1u << lane) - 1u));
