@@ -184,7 +184,7 @@ __global__ void k_finalize(const unsigned long long *__restrict__ tally, const d
       if (acc)
         v = acc[(int64_t)c * npix + pix] * scale;
       else
-        v = (double)tile[threadIdx.x * Cpad + c] * quantum * scale;
+        v = (double)tile[threadIdx.x * Cpad + c] * (quantum * scale);
       float *o = coeff + (int64_t)c * npix + pix;
       *o = accumulate ? *o + (float)(sgn * v) : (float)(sgn * v);
     }
@@ -238,38 +238,101 @@ __global__ void k_dot(const float *__restrict__ a, const float *__restrict__ b, 
   }
 }
 
-// eps = 1/2 A sum(partials), summed by one thread in block order (deterministic).
-__global__ void k_eps_final(const double *__restrict__ partials, int n, double half_area, double *eps) {
+// eps = 1/2 A sum(partials) by one block, in an order fixed by n (deterministic).  (One thread took 57 us
+// for 1216 partials: a chain of FP64 additions.)
+__global__ void __launch_bounds__(kThreads) k_eps_final(const double *__restrict__ partials, int n, double half_area,
+                                                        double *eps) {
+  __shared__ double red[kThreads / 32];
   double s = 0.0;
-  for (int i = 0; i < n; ++i) s += partials[i];
-  *eps = half_area * s;
+  for (int i = threadIdx.x; i < n; i += kThreads) s += partials[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < kThreads / 32; ++w) t += red[w];
+    *eps = half_area * t;
+  }
 }
 
+// (the quotient by the reciprocal and one correction from its remainder: three FP64 operations)
 __global__ void k_adjoint_source(const float *__restrict__ mua, const float *__restrict__ dL_dH, int64_t npix,
-                                 double area, float *__restrict__ q) {
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < npix; i += (int64_t)gridDim.x * kThreads)
-    q[i] = (float)(-(double)mua[i] * (double)dL_dH[i] / area);
+                                 double area, double inv_area, float *__restrict__ q) {
+  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < npix; i += (int64_t)gridDim.x * kThreads) {
+    const double x = -(double)mua[i] * (double)dL_dH[i];
+    const double r = x * inv_area;
+    const double d = fma(fma(-r, area, x), inv_area, r);
+    q[i] = (float)(isfinite(r) && r != 0.0 ? d : r);
+  }
+}
+
+// A normal float as a double by integer operations (the conversion itself takes a slot of the FP64 pipe,
+// which does 1/64 of the FP32 rate on this part); `special` is set for zeros, subnormals, infinities and NaN.
+__device__ __forceinline__ double widen_normal(float x, bool &special) {
+  const unsigned u = __float_as_uint(x);
+  special |= ((u + 0x00800000u) & 0x7F000000u) == 0u;  // exponent 0 or 255
+  return __hiloint2double((int)((((int)u >> 3) & 0x8FFFFFFF) + 0x38000000), (int)(u << 29));
 }
 
 // Per pixel, FP64: G_a = a0 a0*/(2pi) + (1/pi) sum (a_n a_n* + b_n b_n*)      (Eq. 22)
 //                  G_s = (1/pi) sum (a_n a_n* + b_n b_n*)(1 - g^n)            (Eq. 28)
+// Bound by the FP64 pipe (1024^2 pixels, K = 64: 1.1 GB take 0.17 ms from memory): four FP64 operations an
+// order -- the weights 1 - g^n come from a table made once per block, the 1/pi is applied to the sums, the
+// coefficients are widened by integer operations -- where per-pixel weights, per-order 1/pi and converted
+// coefficients took eleven (1.46 ms).
 template <typename OutT>
-__global__ void k_gradient(const float *__restrict__ F, const float *__restrict__ Fs, const float *__restrict__ v,
+__global__ void __launch_bounds__(kThreads) k_gradient(const float *__restrict__ F, const float *__restrict__ Fs, const float *__restrict__ v,
                            int64_t npix, int K, double g, double area, OutT *__restrict__ d_mua,
                            OutT *__restrict__ d_mus) {
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < npix; i += (int64_t)gridDim.x * kThreads) {
-    const double a0 = F[i];
-    double Ga = a0 * (double)Fs[i] * (0.5 / CUDART_PI);
-    double Gs = 0.0, gn = 1.0;
+  __shared__ double weight[MCR_MAX_K + 1];
+  if (threadIdx.x == 0) {
+    double gn = 1.0;
     for (int n = 1; n <= K; ++n) {
       gn *= g;
-      const int64_t ca = (int64_t)(2 * n - 1) * npix + i, cb = (int64_t)(2 * n) * npix + i;
-      const double pr = (double)F[ca] * (double)Fs[ca] + (double)F[cb] * (double)Fs[cb];
-      Ga += pr * (1.0 / CUDART_PI);
-      Gs += pr * (1.0 - gn) * (1.0 / CUDART_PI);
+      weight[n] = 1.0 - gn;
     }
+  }
+  __syncthreads();
+  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < npix; i += (int64_t)gridDim.x * kThreads) {
+    const double a0 = F[i];
+    double sum = 0.0, Gs = 0.0;
+    const float *f = F + npix + i, *fs = Fs + npix + i;
+    auto add = [&](double a, double as, double b, double bs, int n) {
+      const double pr = fma(a, as, b * bs);
+      sum += pr;
+      Gs = fma(pr, weight[n], Gs);
+    };
+    constexpr int kOrders = 4;  // loaded, and tested for special values, together
+    int n = 1;
+    for (; n + kOrders <= K + 1; n += kOrders, f += 2 * kOrders * npix, fs += 2 * kOrders * npix) {
+      float x[2 * kOrders], y[2 * kOrders];
+#pragma unroll
+      for (int k = 0; k < 2 * kOrders; ++k) {
+        x[k] = __ldcs(f + k * npix);
+        y[k] = __ldcs(fs + k * npix);
+      }
+      bool special = false;
+      double dx[2 * kOrders], dy[2 * kOrders];
+#pragma unroll
+      for (int k = 0; k < 2 * kOrders; ++k) {
+        dx[k] = widen_normal(x[k], special);
+        dy[k] = widen_normal(y[k], special);
+      }
+      if (special) {
+#pragma unroll
+        for (int k = 0; k < 2 * kOrders; ++k) {
+          dx[k] = (double)x[k];
+          dy[k] = (double)y[k];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kOrders; ++k) add(dx[2 * k], dy[2 * k], dx[2 * k + 1], dy[2 * k + 1], n + k);
+    }
+    for (; n <= K; ++n, f += 2 * npix, fs += 2 * npix) add(f[0], fs[0], f[npix], fs[npix], n);
+    const double Ga = a0 * (double)Fs[i] * (0.5 / CUDART_PI) + sum * (1.0 / CUDART_PI);
     d_mua[i] = (OutT)((double)v[i] * a0 + area * Ga);
-    if (d_mus) d_mus[i] = (OutT)(area * Gs);
+    if (d_mus) d_mus[i] = (OutT)(area * (Gs * (1.0 / CUDART_PI)));
   }
 }
 
@@ -345,7 +408,7 @@ cudaError_t launch_h_eps(const float *mua, const float *a0, const float *Hmeas, 
   int grid = grid_for(npix, kThreads);
   if ((size_t)grid > partials_cap) grid = (int)partials_cap;
   k_h_eps<<<grid, kThreads, 0, s>>>(mua, a0, Hmeas, npix, area, H, dL_dH, (Hmeas && eps) ? partials : nullptr);
-  if (Hmeas && eps) k_eps_final<<<1, 1, 0, s>>>(partials, grid, 0.5 * area, eps);
+  if (Hmeas && eps) k_eps_final<<<1, kThreads, 0, s>>>(partials, grid, 0.5 * area, eps);
   return cudaGetLastError();
 }
 
@@ -354,13 +417,13 @@ cudaError_t launch_dot(const float *a, const float *b, int64_t n, double *partia
   int grid = grid_for(n, kThreads);
   if ((size_t)grid > partials_cap) grid = (int)partials_cap;
   k_dot<<<grid, kThreads, 0, s>>>(a, b, n, partials);
-  k_eps_final<<<1, 1, 0, s>>>(partials, grid, 1.0, out);
+  k_eps_final<<<1, kThreads, 0, s>>>(partials, grid, 1.0, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adjoint_source(const float *mua, const float *dL_dH, int64_t npix, double area, float *q,
                                   cudaStream_t s) {
-  k_adjoint_source<<<grid_for(npix, kThreads), kThreads, 0, s>>>(mua, dL_dH, npix, area, q);
+  k_adjoint_source<<<grid_for(npix, kThreads), kThreads, 0, s>>>(mua, dL_dH, npix, area, 1.0 / area, q);
   return cudaGetLastError();
 }
 
