@@ -11,116 +11,13 @@
 
 #include <mutex>
 
-#include "../../include/mcr3.h"
-#include "mcr_internal.h"
-#include "mcr_rng.cuh"
+#include "mcr3.cuh"
+#include "mcr_fp64.cuh"
 
 namespace mcr {
 namespace {
 
-constexpr unsigned kFull3 = 0xFFFFFFFFu;
-constexpr int kMaxC3 = (MCR3_MAX_L + 1) * (MCR3_MAX_L + 1);
 constexpr int kThreads3 = 128;
-
-struct Transport3Params {
-  int nx, ny, nz;
-  float dx, g;
-  int L, C, Cpad, row_stride;
-  const float4 *mu;  // packed (mu_a, mu_s, 1/mu_a, 1/mu_s) per voxel
-  unsigned long long *tally;
-  const unsigned long long *cdf;  // volumetric source: inclusive prefix of quantised |q|
-  const float *q;
-  int kind;  // MCR_PENCIL, MCR_ISO_POINT, or -1: volumetric
-  float x0, y0, z0, ux0, uy0, uz0;
-  unsigned key0, key1;
-  unsigned long long first_packet, n_packets;
-  unsigned max_scatter, max_events;
-  float w_threshold, rr_p, rr_inv_p, qscale;
-  float nlm[kMaxC3];  // N_lm (times sqrt 2 for m != 0) at index l^2 + l + |m|
-  float rinv[MCR3_MAX_L + 1];  // 1 / k
-  unsigned long long *work;
-  DevStats *stats;
-  unsigned *flags;
-};
-
-// Real orthonormal spherical harmonics of the unit direction u into row[c], c = l^2 + l + m:
-// Y_lm = N_lm Q_l^|m|(u_z) Re/Im[(u_x + i u_y)^|m|], with P_l^m = (1 - u_z^2)^{m/2} Q_l^m and
-// Q_m^m = (2m-1)!!, Q_{m+1}^m = (2m+1) u_z Q_m^m, (l - m) Q_l^m = (2l-1) u_z Q_{l-1}^m - (l+m-1) Q_{l-2}^m.
-__device__ __forceinline__ void sh_row(const Transport3Params &p, float ux, float uy, float uz, float *row) {
-  float cr = 1.f, ci = 0.f;  // (u_x + i u_y)^m
-  float qmm = 1.f;           // Q_m^m
-  for (int m = 0; m <= p.L; ++m) {
-    float q2 = 0.f, q1 = qmm;
-    for (int l = m; l <= p.L; ++l) {
-      float ql;
-      if (l == m)
-        ql = qmm;
-      else if (l == m + 1)
-        ql = (2.f * m + 1.f) * uz * qmm;
-      else
-        ql = ((2.f * l - 1.f) * uz * q1 - (l + m - 1.f) * q2) * p.rinv[l - m];
-      if (l > m) {
-        q2 = q1;
-        q1 = ql;
-      }
-      const int c0 = l * l + l;
-      const float a = p.nlm[c0 + m] * ql;
-      if (m == 0) {
-        row[c0] = a;
-      } else {
-        row[c0 + m] = a * cr;
-        row[c0 - m] = a * ci;
-      }
-    }
-    const float nr = cr * ux - ci * uy, ni = cr * uy + ci * ux;
-    cr = nr;
-    ci = ni;
-    qmm *= 2.f * m + 1.f;
-  }
-}
-
-// cos of a 3D Henyey-Greenstein scattering angle by the inverse CDF at u
-__device__ __forceinline__ float hg3_cos(float g, float u) {
-  if (fabsf(g) < 1e-6f) return 2.f * u - 1.f;
-  const float f = (1.f - g * g) / (1.f - g + 2.f * g * u);
-  return fminf(fmaxf((1.f + g * g - f * f) / (2.f * g), -1.f), 1.f);
-}
-
-// Turn u by polar cos ct and azimuth 2 pi v about itself, in the orthonormal frame of Duff et al.
-// (JCGT 2017), then renormalise.
-__device__ __forceinline__ void turn(float &ux, float &uy, float &uz, float ct, float v) {
-  const float sgn = uz >= 0.f ? 1.f : -1.f;
-  const float a = -1.f / (sgn + uz), b = ux * uy * a;
-  const float t1x = 1.f + sgn * ux * ux * a, t1y = sgn * b, t1z = -sgn * ux;
-  const float t2x = b, t2y = sgn + uy * uy * a, t2z = -uy;
-  const float st = sqrtf(fmaxf(0.f, 1.f - ct * ct));
-  float sp, cp;
-  sincospif(2.f * v, &sp, &cp);
-  float nx = ct * ux + st * (cp * t1x + sp * t2x);
-  float ny = ct * uy + st * (cp * t1y + sp * t2y);
-  float nz = ct * uz + st * (cp * t1z + sp * t2z);
-  const float inv = rsqrtf(nx * nx + ny * ny + nz * nz);
-  ux = nx * inv;
-  uy = ny * inv;
-  uz = nz * inv;
-}
-
-__device__ __forceinline__ int pick_voxel(const unsigned long long *__restrict__ cdf, int n, unsigned long long total,
-                                          unsigned w0, unsigned w1) {
-  const unsigned long long r48 = ((unsigned long long)w0 << 16) | (unsigned long long)(w1 >> 16);
-  const unsigned long long target = __umul64hi(r48 << 16, total);
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = lo + ((hi - lo) >> 1);
-    if (__ldg(cdf + mid) > target)
-      hi = mid;
-    else
-      lo = mid + 1;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ float clamp3(float v, float dx) { return fminf(fmaxf(v, 0.f), dx); }
 
 template <typename T>
 __device__ __forceinline__ T wsum(T v) {
@@ -144,7 +41,9 @@ __global__ void __launch_bounds__(kThreads3, 8) k_transport3(const __grid_consta
   int rb = 0;         // MERGE: which of the lane's two rows holds the current flight's harmonics
   float carry = 0.f;  // MERGE: deferred collision segment (track weight x 2^q), previous row
   if (*p.flags & kFlagMedium) return;
-  const int nvox = p.nx * p.ny * p.nz;
+  // nothing is left when the record launches ran every packet to its end
+  const unsigned n_saved = p.saved ? p.rec_prev->n_left : 0u;
+  if (p.saved && n_saved == 0u && *p.work + p.work_base >= p.n_packets) return;
   const float dx = p.dx;
 
   bool alive = false, exhausted = false;
@@ -210,13 +109,37 @@ __global__ void __launch_bounds__(kThreads3, 8) k_transport3(const __grid_consta
     return true;
   };
 
+  bool more_saved = n_saved > 0u;  // warp-uniform
   for (;;) {
     // ------------------------------------------------------------- refill
     const unsigned need = __ballot_sync(kFull3, !alive && !exhausted);
+    if (more_saved && need) {  // the packets that the record launches left under way come first
+      const int leader = __ffs(need) - 1;
+      unsigned base = 0;
+      if (lane == leader) base = atomicAdd(p.saved_work, (unsigned)__popc(need));
+      base = __shfl_sync(kFull3, base, leader);
+      const unsigned i = base + __popc(need & ((1u << lane) - 1u));
+      if (((need >> lane) & 1u) && i < n_saved) {
+        const SavedPacket3 sp = load_packet3(p.saved + (size_t)p.rec_prev->buf * 4 * p.n_saved, p.n_saved, i);
+        pid = sp.pid;
+        fx = sp.fx, fy = sp.fy, fz = sp.fz, ux = sp.ux, uy = sp.uy, uz = sp.uz, W = sp.W, tau = sp.tau;
+        ix = sp.ix, iy = sp.iy, iz = sp.iz, flight = sp.flight, nscat = sp.nscat;
+        W0 = 1.f;  // (only its magnitude is used)
+        const uint4 r = philox4x32_10(pid, flight + 1u, p.key0, p.key1);
+        cu1 = r.y, cu2 = r.z, cu3 = r.w;
+        inv_ax = __frcp_rn(fabsf(ux));
+        inv_ay = __frcp_rn(fabsf(uy));
+        inv_az = __frcp_rn(fabsf(uz));
+        sh_row(p, ux, uy, uz, myrows + rb * p.row_stride);
+        alive = true;
+      }
+      if (base + __popc(need) >= n_saved) more_saved = false;
+      continue;
+    }
     if (need) {
       const int leader = __ffs(need) - 1;
       unsigned long long base = 0;
-      if (lane == leader) base = atomicAdd(p.work, (unsigned long long)__popc(need));
+      if (lane == leader) base = atomicAdd(p.work, (unsigned long long)__popc(need)) + p.work_base;
       base = __shfl_sync(kFull3, base, leader);
       if (!alive && !exhausted) {
         const unsigned long long g = base + __popc(need & ((1u << lane) - 1u));
@@ -225,64 +148,15 @@ __global__ void __launch_bounds__(kThreads3, 8) k_transport3(const __grid_consta
         } else {
           pid = p.first_packet + g;
           ++n_launch;
-          const uint4 r0 = philox4x32_10(pid, 0u, p.key0, p.key1);
-          float x = p.x0, y = p.y0, z = p.z0;
-          int vx = -1, vy = 0, vz = 0;
-          W0 = 1.f;
-          if (p.kind < 0) {  // volumetric: voxel by |q|, uniform in it, W0 = sign q
-            const unsigned long long total = __ldg(p.cdf + nvox - 1);
-            if (total == 0ull) {  // all-zero source: nothing to launch
-              W0 = 0.f;
-              x = -1.f;
-            } else {
-              const int v = pick_voxel(p.cdf, nvox, total, r0.x, r0.y);
-              const uint4 r1 = philox4x32_10(pid, 1u, p.key0, p.key1);
-              vx = v % p.nx;
-              vy = (v / p.nx) % p.ny;
-              vz = v / (p.nx * p.ny);
-              x = u01(r1.x) * dx;
-              y = u01(r1.y) * dx;
-              z = u01(r1.z) * dx;
-              W0 = __ldg(p.q + v) < 0.f ? -1.f : 1.f;
-            }
-          }
-          if (p.kind == MCR_PENCIL) {
-            ux = p.ux0;
-            uy = p.uy0;
-            uz = p.uz0;
-          } else {  // isotropic: cos th = 2u - 1, ph = 2 pi u'
-            const float ct = 2.f * u01(r0.z) - 1.f, st = sqrtf(fmaxf(0.f, 1.f - ct * ct));
-            float sp, cp;
-            sincospif(2.f * u01(r0.w), &sp, &cp);
-            ux = st * cp;
-            uy = st * sp;
-            uz = ct;
-          }
+          const bool inside = launch3(p, pid, ix, iy, iz, fx, fy, fz, ux, uy, uz, W0);
           W = W0;
           w_launch += W0;
           flight = 0;
           nscat = 0;
-          const bool inside =
-              vx >= 0 || (x >= 0.f && x <= p.nx * dx && y >= 0.f && y <= p.ny * dx && z >= 0.f && z <= p.nz * dx);
           if (!inside) {
             ++n_esc;
             w_esc += W;
           } else {
-            if (vx >= 0) {  // (x, y, z) already the offsets in voxel (vx, vy, vz)
-              ix = vx;
-              iy = vy;
-              iz = vz;
-              fx = x;
-              fy = y;
-              fz = z;
-            } else {
-              ix = min((int)floorf(x / dx), p.nx - 1);
-              iy = min((int)floorf(y / dx), p.ny - 1);
-              iz = min((int)floorf(z / dx), p.nz - 1);
-              fx = clamp3(x - ix * dx, dx);
-              fy = clamp3(y - iy * dx, dx);
-              fz = clamp3(z - iz * dx, dx);
-            }
             alive = begin_flight();
           }
         }
@@ -427,25 +301,40 @@ __global__ void __launch_bounds__(kThreads3, 8) k_transport3(const __grid_consta
 
 // coeff[c][v] (+)= sum * quantum * scale, (-1)^l on odd l when adjoint; scale = fixed_scale or, for
 // a volumetric source, 4 pi qmax total 2^-32 / N_p (S / (N_p V) with S = 4 pi V qmax total 2^-32)
-__global__ void k_finalize3(const unsigned long long *__restrict__ tally, int64_t nvox, int C, int Cpad,
-                            double quantum, double fixed_scale, int volumetric, const unsigned *qmax_bits,
-                            const unsigned long long *cdf_total, double n_packets, int adjoint, int accumulate,
-                            float *__restrict__ coeff, unsigned *flags) {
+// One block = 32 voxels, staged through shared memory so that the voxel-major rows and the channel-major
+// output are both read and written in whole lines (96^3, L = 4: 277 us when each thread took its own word
+// of a row).
+__global__ void __launch_bounds__(256) k_finalize3(const unsigned long long *__restrict__ tally, int64_t nvox, int C,
+                                                   int Cpad, double quantum, double fixed_scale, int volumetric,
+                                                   const unsigned *qmax_bits, const unsigned long long *cdf_total,
+                                                   double n_packets, int adjoint, int accumulate,
+                                                   float *__restrict__ coeff, unsigned *flags) {
+  extern __shared__ long long tile3[];  // [32][C | 1]
   double scale = fixed_scale;
   if (volumetric)
     scale = 4.0 * CUDART_PI * (double)__uint_as_float(*qmax_bits) * (double)(*cdf_total) * (1.0 / 4294967296.0) /
             n_packets;
+  scale *= quantum;  // (a power of two: the product below rounds as it would with the factors in turn)
+  const int stride = C | 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t v0 = (int64_t)blockIdx.x * 32;
+  const int nv = nvox - v0 < 32 ? (int)(nvox - v0) : 32;
   bool near = false;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nvox * C; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i / nvox);
-    const int64_t v = i - (int64_t)c * nvox;
-    const long long s = (long long)tally[v * Cpad + c];
-    near |= (s > (1ll << 61)) || (s < -(1ll << 61));
+  for (int v = warp; v < nv; v += 8)
+    for (int c = lane; c < C; c += 32) {
+      const long long s = (long long)tally[(v0 + v) * Cpad + c];
+      near |= (s > (1ll << 61)) || (s < -(1ll << 61));
+      tile3[v * stride + c] = s;
+    }
+  __syncthreads();
+  for (int c = warp; c < C; c += 8) {
     int l = 0;
     while ((l + 1) * (l + 1) <= c) ++l;
     const double sgn = (adjoint && (l & 1)) ? -1.0 : 1.0;
-    const float val = (float)(sgn * (double)s * quantum * scale);
-    coeff[i] = accumulate ? coeff[i] + val : val;
+    if (lane < nv) {
+      float *o = coeff + (int64_t)c * nvox + v0 + lane;
+      const float val = (float)(sgn * (double)tile3[lane * stride + c] * scale);
+      *o = accumulate ? *o + val : val;
+    }
   }
   if (near) atomicOr(flags, kFlagOverflow);
 }
@@ -483,20 +372,56 @@ __global__ void k_eps3_final(const double *partials, int n, double half_V, doubl
 
 // d_mua = v sqrt(4 pi) c_00 + V sum_c c c*, d_mus = V sum_c (1 - g^l) c c* (FP64, increasing c);
 // OUT double, or float (the FP64 result rounded once)
+// (Three FP64 operations a channel: the weights come from a table, the coefficients are widened by integer
+// operations; with the weights by voxel and FP64 conversions 96^3, L = 4 took 307 us.)
 template <typename OUT>
-__global__ void k_gradient3(const float *__restrict__ co, const float *__restrict__ ca, const float *__restrict__ v,
-                            int64_t n, int C, double g, double V, OUT *d_mua, OUT *d_mus) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double sa = 0.0, ss = 0.0, gl = 1.0;
+__global__ void __launch_bounds__(256) k_gradient3(const float *__restrict__ co, const float *__restrict__ ca,
+                                                   const float *__restrict__ v, int64_t n, int C, double g, double V,
+                                                   OUT *d_mua, OUT *d_mus) {
+  __shared__ double weight[kMaxC3];
+  if (threadIdx.x == 0) {
+    double gl = 1.0;
     int l = 0;
     for (int c = 0; c < C; ++c) {
       if ((l + 1) * (l + 1) <= c) {
         ++l;
         gl *= g;
       }
-      const double p = (double)co[(int64_t)c * n + i] * (double)ca[(int64_t)c * n + i];
-      sa += p;
-      ss += (1.0 - gl) * p;
+      weight[c] = 1.0 - gl;
+    }
+  }
+  __syncthreads();
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    double sa = 0.0, ss = 0.0;
+    constexpr int kGroup = 8;  // channels loaded, and tested for special values, together
+    for (int c = 0; c < C; c += kGroup) {
+      float x[kGroup], y[kGroup];
+#pragma unroll
+      for (int k = 0; k < kGroup; ++k) {
+        x[k] = c + k < C ? __ldcs(co + (int64_t)(c + k) * n + i) : 1.f;
+        y[k] = c + k < C ? __ldcs(ca + (int64_t)(c + k) * n + i) : 1.f;
+      }
+      bool special = false;
+      double dx[kGroup], dy[kGroup];
+#pragma unroll
+      for (int k = 0; k < kGroup; ++k) {
+        dx[k] = widen_normal(x[k], special);
+        dy[k] = widen_normal(y[k], special);
+      }
+      if (special) {
+#pragma unroll
+        for (int k = 0; k < kGroup; ++k) {
+          dx[k] = (double)x[k];
+          dy[k] = (double)y[k];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kGroup; ++k)
+        if (c + k < C) {
+          const double p = dx[k] * dy[k];
+          sa += p;
+          ss += weight[c + k] * p;
+        }
     }
     d_mua[i] = (OUT)((double)v[i] * sqrt(4.0 * CUDART_PI) * (double)co[i] + V * sa);
     d_mus[i] = (OUT)(V * ss);
@@ -511,6 +436,8 @@ struct Work3 {
   size_t cdf_bytes = 0, bs_bytes = 0;
   float4 *mu = nullptr;
   size_t mu_bytes = 0;
+  unsigned char *rec_a = nullptr, *rec_b = nullptr, *rec_scratch = nullptr;  // record deposit
+  size_t rec_a_bytes = 0, rec_b_bytes = 0, rec_scratch_bytes = 0;
   unsigned char *small = nullptr;  // [0,8) counter, [64,192) stats, [448] flags, [512] qmax bits
   double *partials = nullptr;
 };
@@ -532,7 +459,8 @@ int grow3(void **p, size_t *have, size_t need) {
   return MCR_OK;
 }
 
-int work3(size_t tally, size_t nvox, Work3 **out) {
+// (margin: voxels before and after the medium, so that every voxel's neighbours can be read)
+int work3(size_t tally, size_t nvox, size_t margin, Work3 **out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MCR_ERR_CUDA;
   Work3 &w = g_w3[dev];
@@ -544,7 +472,7 @@ int work3(size_t tally, size_t nvox, Work3 **out) {
   }
   if ((rc = grow3((void **)&w.tally, &w.tally_bytes, tally))) return rc;
   if ((rc = grow3((void **)&w.cdf, &w.cdf_bytes, nvox * 8))) return rc;
-  if ((rc = grow3((void **)&w.mu, &w.mu_bytes, nvox * sizeof(float4)))) return rc;
+  if ((rc = grow3((void **)&w.mu, &w.mu_bytes, (nvox + 2 * margin) * sizeof(float4)))) return rc;
   if ((rc = grow3((void **)&w.block_sums, &w.bs_bytes, ((nvox + 255) / 256) * 8))) return rc;
   *out = &w;
   return MCR_OK;
@@ -595,14 +523,16 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
   const int64_t nvox = (int64_t)med->nx * med->ny * med->nz;
   std::lock_guard<std::mutex> lock(g_mu3);
   Work3 *w = nullptr;
-  if ((rc = work3((size_t)nvox * Cpad * 8, (size_t)nvox, &w))) return rc;
+  const size_t margin = (size_t)med->nx * med->ny;
+  if ((rc = work3((size_t)nvox * Cpad * 8, (size_t)nvox, margin, &w))) return rc;
+  float4 *const mu = w->mu + margin;
   unsigned long long *counter = reinterpret_cast<unsigned long long *>(w->small);
   DevStats *dstats = reinterpret_cast<DevStats *>(w->small + 64);
   unsigned *flags = reinterpret_cast<unsigned *>(w->small + 448);
   unsigned *qmax = reinterpret_cast<unsigned *>(w->small + 512);
   MCR3_TRY(cudaMemsetAsync(w->small, 0, 512, s));  // counter, stats, flags
   MCR3_TRY(cudaMemsetAsync(w->tally, 0, (size_t)nvox * Cpad * 8, s));
-  MCR3_TRY(launch_pack_medium(med->mua, med->mus, w->mu, nvox, flags, s));
+  MCR3_TRY(launch_pack_medium(med->mua, med->mus, mu, nvox, flags, s));
   if (qstar) MCR3_TRY(launch_source_cdf(qstar, nvox, w->cdf, w->block_sums, (size_t)((nvox + 255) / 256), qmax, s));
   p.nx = med->nx;
   p.ny = med->ny;
@@ -613,7 +543,7 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
   p.C = C;
   p.Cpad = Cpad;
   p.row_stride = C | 1;  // odd: the lanes' rows fall in distinct banks
-  p.mu = w->mu;
+  p.mu = mu;
   p.tally = w->tally;
   p.cdf = w->cdf;
   p.q = qstar;
@@ -644,6 +574,20 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
   p.work = counter;
   p.stats = dstats;
   p.flags = flags;
+  // The record deposit (mcr3_records.cu), then the direct transport for packets it leaves; the direct
+  // transport alone when the record buffers cannot be allocated or a graph is being captured.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  MCR3_TRY(cudaStreamIsCapturing(s, &cap));
+  RecordPlan plan{};
+  if (run->n_packets && cap == cudaStreamCaptureStatusNone && rec_plan3(p, nvox, &plan) == cudaSuccess) {
+    const size_t bytes = rec_buffer_bytes3(plan);
+    if (grow3((void **)&w->rec_a, &w->rec_a_bytes, bytes) == MCR_OK && grow3((void **)&w->rec_b, &w->rec_b_bytes, bytes) == MCR_OK &&
+        grow3((void **)&w->rec_scratch, &w->rec_scratch_bytes, rec_scratch_bytes(plan)) == MCR_OK) {
+      MCR3_TRY(launch_records3(p, plan, w->rec_a, w->rec_b, w->rec_scratch, &p, s));
+    } else {
+      cudaGetLastError();
+    }
+  }
   if (run->n_packets) {
     int dev = 0, sms = 0, per_sm = 0;
     MCR3_TRY(cudaGetDevice(&dev));
@@ -668,7 +612,7 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
   }
   const double V = (double)med->dx * med->dx * med->dx;
   const double fixed = (!qstar && run->n_packets) ? (double)src->power / ((double)run->n_packets * V) : 0.0;
-  k_finalize3<<<512, 256, 0, s>>>(w->tally, nvox, C, Cpad, ldexp(1.0, -qe), fixed, qstar && run->n_packets ? 1 : 0,
+  k_finalize3<<<(unsigned)((nvox + 31) / 32), 256, (size_t)32 * (C | 1) * 8, s>>>(w->tally, nvox, C, Cpad, ldexp(1.0, -qe), fixed, qstar && run->n_packets ? 1 : 0,
                                   qmax, w->cdf + (nvox - 1), (double)(run->n_packets ? run->n_packets : 1),
                                   qstar ? 1 : 0, run->accumulate ? 1 : 0, coeff, flags);
   MCR3_TRY(cudaGetLastError());
@@ -707,7 +651,7 @@ int release_workspace3(int dev) {
   if (dev < 0 || dev >= 64) return MCR_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mu3);
   Work3 &w = g_w3[dev];
-  void *ptrs[] = {w.tally, w.cdf, w.block_sums, w.mu, w.small, w.partials};
+  void *ptrs[] = {w.tally, w.cdf, w.block_sums, w.mu, w.small, w.partials, w.rec_a, w.rec_b, w.rec_scratch};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   w = Work3{};
@@ -758,7 +702,7 @@ int mc3_h_eps(const mcr3_medium *med, const float *coeff, const float *Hmeas, fl
   cudaStream_t s = (cudaStream_t)stream;
   std::lock_guard<std::mutex> lock(g_mu3);
   Work3 *w = nullptr;
-  if ((rc = work3(0, 1, &w))) return rc;
+  if ((rc = work3(0, 1, 0, &w))) return rc;
   const int grid = (int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
   k_h_eps3<<<grid, 256, 0, s>>>(med->mua, coeff, Hmeas, n, V, H, dL_dH, (Hmeas && eps) ? w->partials : nullptr);
   if (Hmeas && eps) k_eps3_final<<<1, 1, 0, s>>>(w->partials, grid, 0.5 * V, eps);

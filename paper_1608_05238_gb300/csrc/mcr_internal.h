@@ -69,21 +69,11 @@ struct ProblemDesc {
 
 struct RecordHeader;
 
-struct TransportParams {
-  int n_problems;
-  int K, C, Cpad, row_stride;  // C = 2K+1 channels, Cpad = tally_row_words(C), smem row stride
-  int sectors;                 // > 0: discrete-ordinates tally, C = sectors (single forward problem)
-  float sector_scale;          // sectors / (2 pi)
-  int time_bins;               // > 0: path-length (time-of-flight) resolved fluence, C = time_bins
-  float time_bin_mm, inv_time_bin;
-  unsigned max_scatter, max_events;
-  float w_threshold, rr_p, rr_inv_p;
-  unsigned long long total_packets;  // = prob[n_problems-1].end
-  unsigned long long *work;          // packet counter
-  const unsigned *order;             // launch order: the launch index taken at step g (nullptr: g)
-  // record deposit (mcr_records.cu): one record per segment instead of deposits, in launches that
-  // pause when their record buffer is full and hand their packets to the next launch
+// Record deposit (mcr_records.cu): one record per segment instead of deposits, in launches that pause when
+// their record buffer is full and hand their packets to the next launch.
+struct RecordParams {
   float4 *records;                   // (global row bits, track weight x 2^q, s_x, s_z), rec_blocks x kRecBlock
+  float *records_x;                  // 3D: the records' fifth word
   unsigned rec_blocks;
   RecordHeader *rec_hdr;             // this launch's counters
   const RecordHeader *rec_prev;      // the previous launch's (nullptr: the first)
@@ -96,6 +86,20 @@ struct TransportParams {
   int n_sm;                          // SMs the grid is spread over
   unsigned tail_max;                 // most packets the tail takes
   unsigned long long work_base;      // packets launched by place at the start; the counter `work` goes on from there
+};
+
+struct TransportParams : RecordParams {
+  int n_problems;
+  int K, C, Cpad, row_stride;  // C = 2K+1 channels, Cpad = tally_row_words(C), smem row stride
+  int sectors;                 // > 0: discrete-ordinates tally, C = sectors (single forward problem)
+  float sector_scale;          // sectors / (2 pi)
+  int time_bins;               // > 0: path-length (time-of-flight) resolved fluence, C = time_bins
+  float time_bin_mm, inv_time_bin;
+  unsigned max_scatter, max_events;
+  float w_threshold, rr_p, rr_inv_p;
+  unsigned long long total_packets;  // = prob[n_problems-1].end
+  unsigned long long *work;          // packet counter
+  const unsigned *order;             // launch order: the launch index taken at step g (nullptr: g)
   DevStats *stats;
   unsigned *flags;                   // error bits: transport does nothing if kFlagMedium is set; it
                                      // latches kFlagEventLimit when a packet reached max_events

@@ -4,6 +4,7 @@
 // functional gradients (Sec. 5, Eqs. 22 and 28).
 #include <math_constants.h>
 
+#include "mcr_fp64.cuh"
 #include "mcr_internal.h"
 
 namespace mcr {
@@ -265,14 +266,6 @@ __global__ void k_adjoint_source(const float *__restrict__ mua, const float *__r
     const double d = fma(fma(-r, area, x), inv_area, r);
     q[i] = (float)(isfinite(r) && r != 0.0 ? d : r);
   }
-}
-
-// A normal float as a double by integer operations (the conversion itself takes a slot of the FP64 pipe,
-// which does 1/64 of the FP32 rate on this part); `special` is set for zeros, subnormals, infinities and NaN.
-__device__ __forceinline__ double widen_normal(float x, bool &special) {
-  const unsigned u = __float_as_uint(x);
-  special |= ((u + 0x00800000u) & 0x7F000000u) == 0u;  // exponent 0 or 255
-  return __hiloint2double((int)((((int)u >> 3) & 0x8FFFFFFF) + 0x38000000), (int)(u << 29));
 }
 
 // Per pixel, FP64: G_a = a0 a0*/(2pi) + (1/pi) sum (a_n a_n* + b_n b_n*)      (Eq. 22)
