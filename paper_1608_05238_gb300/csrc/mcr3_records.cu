@@ -70,6 +70,7 @@ struct Packet3 {
 // ------------------------------------------------------------------------------------- transport
 __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant__ Transport3Params p) {
   extern __shared__ unsigned hist[];  // records per bin of this block
+  after_previous();
   if (*p.flags & kFlagMedium) return;
   const unsigned n_in = p.rec_prev ? p.rec_prev->n_left : 0u;
   const bool fresh = !p.rec_prev || p.rec_prev->fresh;
@@ -260,6 +261,7 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
 // The last packets of a run, a warp to each (k_transport_tail's scheme).
 __global__ void __launch_bounds__(kTailThreads, 2) k_transport3_tail(const __grid_constant__ Transport3Params p) {
   extern __shared__ unsigned hist[];
+  after_previous();
   if (*p.flags & kFlagMedium) return;
   const unsigned n_in = p.rec_hdr->n_left;
   if (n_in == 0u || n_in > p.tail_max || *p.work + p.work_base < p.n_packets) return;
@@ -484,6 +486,7 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
   using O = Orders3<L, M0, M1>;
   constexpr int N = O::kCount, NX = (N + 1) / 2, NF = N / 2;
   extern __shared__ float4 smem[];
+  after_previous();
   const int T = 1 << tile_shift;
   DepositBatch<B, true> bt(smem, T);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane & 3, g = lane >> 2;
@@ -676,14 +679,16 @@ cudaError_t launch_records3(const Transport3Params &p, const RecordPlan &pl, uns
       pl, layout(scratch, pl), RecordBuffers{buffers(buf_a), buffers(buf_b), fifth(buf_a), fifth(buf_b)}, q, dc.batch,
       p.work, p.n_packets, p.flags,
       [&]() {
-        k_transport3_rec<<<grid, pl.threads, smem, s>>>(q);
-        k_transport3_tail<<<pl.tail_blocks, kTailThreads, smem, s>>>(q);
+        if (q.rec_prev)
+          launch_ahead(k_transport3_rec, grid, pl.threads, smem, s, q);
+        else  // (it follows a memset)
+          k_transport3_rec<<<grid, pl.threads, smem, s>>>(q);
+        launch_ahead(k_transport3_tail, pl.tail_blocks, kTailThreads, smem, s, q);
       },
       [&](const float4 *rec, const float *rec_x, const Scratch &sc) {
         for (int k = 0; k < 2 && dc.pass[k]; ++k)
-          dc.pass[k]<<<sms * dep[k], kDepThreads, dep_smem, s>>>(rec, rec_x, q.rec_hdr, sc.tile_off, sc.dep_unit_off,
-                                                                 pl.n_tiles, pl.tile_shift, (long long)pl.rows, h, p.Cpad,
-                                                                 p.tally, p.flags);
+          launch_ahead(dc.pass[k], sms * dep[k], kDepThreads, dep_smem, s, rec, rec_x, q.rec_hdr, sc.tile_off,
+                       sc.dep_unit_off, pl.n_tiles, pl.tile_shift, (long long)pl.rows, h, p.Cpad, p.tally, p.flags);
       },
       s);
   if (e == cudaSuccess) *closing = q;

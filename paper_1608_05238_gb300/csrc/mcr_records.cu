@@ -36,6 +36,7 @@ constexpr int kFlyMin = 12;
 template <bool BATCH>
 __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __grid_constant__ TransportParams p) {
   extern __shared__ unsigned hist[];  // records per bin of this block
+  after_previous();
   if (*p.flags & kFlagMedium) return;
   // packets that the previous launch left, and whether there are new ones to launch
   const unsigned n_in = p.rec_prev ? p.rec_prev->n_left : 0u;
@@ -317,6 +318,7 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
 // once, one per lane, in the same order of operations.  The pixels ahead are loaded a segment early.
 __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant__ TransportParams p) {
   extern __shared__ unsigned hist[];  // records per bin of this block
+  after_previous();
   if (*p.flags & kFlagMedium) return;
   const unsigned n_in = p.rec_hdr->n_left;
   if (n_in == 0u || n_in > p.tail_max || *p.work + p.work_base < p.total_packets) return;
@@ -515,6 +517,7 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
                   const unsigned *__restrict__ unit_off, int n_tiles, int tile_shift, long long n_rows, int K, int Cpad,
                   unsigned long long *__restrict__ tally, unsigned *flags) {
   extern __shared__ float4 srec[];  // [kDepBatch]
+  after_previous();
   const int T = 1 << tile_shift;
   DepositBatch<kDepBatch, false> bt(srec, T);
   const unsigned short *const idx = bt.idx;
@@ -681,15 +684,16 @@ cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg,
   e = record_chain<false>(
       pl, layout(scratch, pl), RecordBuffers{buf_a, buf_b, nullptr, nullptr}, q, dc.batch, p.work, p.total_packets, p.flags,
       [&]() {
-        if (p.n_problems > 1)
-          k_transport_rec<true><<<grid, pl.threads, smem, s>>>(q);
-        else
-          k_transport_rec<false><<<grid, pl.threads, smem, s>>>(q);
-        k_transport_tail<<<pl.tail_blocks, kTailThreads, smem, s>>>(q);
+        auto *const rec = p.n_problems > 1 ? k_transport_rec<true> : k_transport_rec<false>;
+        if (q.rec_prev)
+          launch_ahead(rec, grid, pl.threads, smem, s, q);
+        else  // (it follows a memset)
+          rec<<<grid, pl.threads, smem, s>>>(q);
+        launch_ahead(k_transport_tail, pl.tail_blocks, kTailThreads, smem, s, q);
       },
       [&](const float4 *rec, const float *, const Scratch &sc) {
-        dc.kernel<<<sms * dep, kDepThreads, dep_smem, s>>>(rec, q.rec_hdr, sc.tile_off, sc.dep_unit_off, pl.n_tiles,
-                                                           pl.tile_shift, (long long)pl.rows, p.K, p.Cpad, tally, p.flags);
+        launch_ahead(dc.kernel, sms * dep, kDepThreads, dep_smem, s, rec, q.rec_hdr, sc.tile_off, sc.dep_unit_off,
+                     pl.n_tiles, pl.tile_shift, (long long)pl.rows, p.K, p.Cpad, tally, p.flags);
       },
       s);
   return e != cudaSuccess ? e : launch_transport(q, TransportLaunch{0, 0, 1, 0}, s);

@@ -5,6 +5,7 @@
 #include <math_constants.h>
 
 #include <mutex>
+#include <utility>
 
 #include "mcr_packet.cuh"
 
@@ -123,6 +124,15 @@ __device__ __forceinline__ void set_axis(float s, float dx, float &o, float &inv
   o = s > 0.f ? dx : 0.f;
 }
 
+// The kernels of a run are launched ahead: the blocks of one take the places that those of the one before
+// free, and wait here for its end.  Nothing of global memory is touched before this.
+// (What a small run spends is mostly the gaps between its 30 to 60 kernels: 1e5 packets into 32^2 pixels
+// 1690 -> 1539 us, 1e5 packets into 12^3 voxels, L = 5, 577 -> 475 us.)
+__device__ __forceinline__ void after_previous() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();  // (the next kernel's blocks wait for this one's end in turn)
+}
+
 // ------------------------------------------------------------------------------------- offsets
 // Inclusive scan of v over the block (1024 threads); warp_tot: 32 words of shared memory.
 __device__ unsigned block_scan(unsigned v, unsigned *warp_tot) {
@@ -175,6 +185,7 @@ __global__ void __launch_bounds__(1024) k_rec_scan(RecordHeader *hdr, unsigned *
                                                    int batch, unsigned *off, unsigned *cur, unsigned *unit_off,
                                                    const unsigned long long *launched, unsigned long long n_packets) {
   __shared__ unsigned warp_tot[32];
+  after_previous();
   if (threadIdx.x == 0) {
     if (*launched < n_packets) hdr->fresh = 1u;
     if (hdr->tail_ran == 1u) {  // what the tail left stands in the other buffer
@@ -216,6 +227,7 @@ __global__ void __launch_bounds__(kSortThreads, 2)
                float *__restrict__ sorted_x, const RecordHeader *hdr, unsigned max_blocks,
                int shift, int n_bins, unsigned *cursor, unsigned capacity, const unsigned *__restrict__ coarse_off, const unsigned *__restrict__ coarse_unit_off,
                int n_coarse, int coarse_shift, unsigned *flags) {
+  after_previous();
   constexpr int kPer = kSortBatch / kSortThreads;
   extern __shared__ float4 srec[];                                  // [kSortBatch]
   unsigned *cnt = reinterpret_cast<unsigned *>(srec + kSortBatch);  // [n_bins] counts, then local starts
@@ -302,6 +314,7 @@ __global__ void __launch_bounds__(kSortThreads) k_rec_count(const float4 *__rest
                                                             int coarse_shift, int tile_shift, unsigned *tile_hist,
                                                             unsigned *flags) {
   __shared__ unsigned cnt[kMaxBins];
+  after_previous();
   const int nb = 1 << coarse_shift;
   const unsigned units = hdr->n_coarse_units;
   for (unsigned u = blockIdx.x; u < units; u += gridDim.x) {
@@ -557,8 +570,8 @@ cudaError_t plan_records(int64_t rows, uint64_t packets, long long capacity, Rec
 
 // The record launches to enqueue, once lanes and tail_blocks are known: those that end on a full buffer, one
 // for each halving of the packets in use down to what the tail takes, one more for a buffer left part full.
-// The five kernels of a launch with nothing left to do take about 8 us (20,000 packets into 12^3 voxels:
-// two runs in 1370 us with eleven launches each, 1212 us with six; all direct 1184 us).
+// The five kernels of a launch with nothing left to do took about 8 us (20,000 packets into 12^3 voxels:
+// two runs in 1370 us with eleven launches each, 1212 us with six; launched ahead 1037 us, all direct 1184 us).
 void set_launches(RecordPlan *pl, uint64_t packets) {
   const uint64_t slots = (uint64_t)pl->blocks * kRecBlock;
   uint64_t n = (packets * kSegmentsPerPacket + slots - 1) / slots;
@@ -574,6 +587,22 @@ struct RecordBuffers {
   float4 *a, *b;
   float *a_x, *b_x;  // X: the fifth words
 };
+
+// Launches a kernel ahead of the end of the kernel before it in the stream (see after_previous()).
+template <typename... P, typename... A>
+void launch_ahead(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A &&...args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)block);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);  // (the caller asks cudaGetLastError)
+}
 
 // The launches of a run: transport() launches the transport and its tail with the fields of q set here,
 // deposit(records, their fifth words, scratch) the deposit of the sorted records.  On return q is set for a
@@ -611,19 +640,18 @@ cudaError_t record_chain(const RecordPlan &pl, const Scratch &sc, const RecordBu
     q.rec_hdr = hdr;
     q.rec_prev = i ? hdr - 1 : nullptr;
     transport();
-    k_rec_scan<<<1, 1024, 0, s>>>(hdr, two ? &hdr->n_coarse_units : &hdr->n_units, sc.hist, pl.n_coarse,
-                                  two ? kSortBatch : dep_batch, sc.off, sc.cur, sc.unit_off, work, to_launch);
-    k_rec_sort<true, X><<<sms * sort1, kSortThreads, smem1, s>>>(buf.a, buf.a_x, buf.b, buf.b_x, hdr, pl.blocks, q.bin_shift,
-                                                                 pl.n_coarse, sc.cur, capacity, nullptr, nullptr, 0, 0,
-                                                                 flags);
+    launch_ahead(k_rec_scan, 1, 1024, 0, s, hdr, two ? &hdr->n_coarse_units : &hdr->n_units, sc.hist, pl.n_coarse,
+                 two ? kSortBatch : dep_batch, sc.off, sc.cur, sc.unit_off, work, to_launch);
+    launch_ahead(k_rec_sort<true, X>, sms * sort1, kSortThreads, smem1, s, buf.a, buf.a_x, buf.b, buf.b_x, hdr,
+                 pl.blocks, q.bin_shift, pl.n_coarse, sc.cur, capacity, nullptr, nullptr, 0, 0, flags);
     if (two) {
-      k_rec_count<<<sms * 4, kSortThreads, 0, s>>>(buf.b, hdr, sc.off, sc.unit_off, pl.n_coarse, pl.coarse_shift,
-                                                   pl.tile_shift, sc.tile_hist, flags);
-      k_rec_scan<<<1, 1024, 0, s>>>(hdr, &hdr->n_units, sc.tile_hist, pl.n_tiles, dep_batch, sc.tile_off, sc.tile_cur,
-                                    sc.dep_unit_off, work, to_launch);
-      k_rec_sort<false, X><<<sms * sort2, kSortThreads, smem2, s>>>(
-          buf.b, buf.b_x, buf.a, buf.a_x, hdr, pl.blocks, pl.tile_shift, 1 << pl.coarse_shift, sc.tile_cur, capacity, sc.off,
-          sc.unit_off, pl.n_coarse, pl.coarse_shift, flags);
+      launch_ahead(k_rec_count, sms * 4, kSortThreads, 0, s, buf.b, hdr, sc.off, sc.unit_off, pl.n_coarse,
+                   pl.coarse_shift, pl.tile_shift, sc.tile_hist, flags);
+      launch_ahead(k_rec_scan, 1, 1024, 0, s, hdr, &hdr->n_units, sc.tile_hist, pl.n_tiles, dep_batch, sc.tile_off,
+                   sc.tile_cur, sc.dep_unit_off, work, to_launch);
+      launch_ahead(k_rec_sort<false, X>, sms * sort2, kSortThreads, smem2, s, buf.b, buf.b_x, buf.a, buf.a_x, hdr,
+                   pl.blocks, pl.tile_shift, 1 << pl.coarse_shift, sc.tile_cur, capacity, sc.off, sc.unit_off,
+                   pl.n_coarse, pl.coarse_shift, flags);
     }
     deposit(two ? buf.a : buf.b, two ? buf.a_x : buf.b_x, sc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
