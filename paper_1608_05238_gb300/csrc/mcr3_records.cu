@@ -492,12 +492,12 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane & 3, g = lane >> 2;
   unsigned char *const my_flush = bt.flush + warp * kFlushBytes;
   const unsigned units = hdr->n_units;
+  if (blockIdx.x < units && warp == 0) bt.find(rec, rec_x, tile_off, unit_off, n_tiles, blockIdx.x);
+  __syncthreads();
   for (unsigned u = blockIdx.x; u < units; u += gridDim.x) {
-    const int tile = block_find(unit_off, n_tiles, u);
-    const unsigned lo = tile_off[tile] + (u - unit_off[tile]) * B;
-    const int n = (int)min((unsigned)B, tile_off[tile + 1] - lo);
-    const int n_items = bt.load(rec, rec_x, lo, n, T);
-    for (int it = warp * 8; it < n_items; it += (kDepThreads / 32) * 8) {
+    const int tile = (int)bt.unit[0];
+    const int n_items = bt.load(rec, rec_x, bt.unit[1], (int)bt.unit[2], T, tile_off, unit_off, n_tiles, u + gridDim.x, units);
+    for (int it = warp * 8; it < n_items; it = bt.next_runs()) {
       const unsigned item = it + g < n_items ? bt.items[it + g] : 0u;
       const int s0 = item & 0xFFFu, len = (item >> 12) & 0x7Fu;
       const long long row = ((long long)tile << tile_shift) + (item >> 19);

@@ -509,6 +509,9 @@ __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant
 }
 
 // ------------------------------------------------------------------------------------- deposit
+// Bound by instruction issue: 27 instructions per order and two records, 68 % of the issue slots with the 12 warps
+// an SM that the sums' registers leave (FMA pipe 45 %, ALU 27 %, XU 33 % of its cycles); at 256^2, K = 32 some
+// 22 ps a record, of which 15 grow with K.
 // Orders n0+1 .. n0+KT per pass, coefficient 0 with the first; TWO: two passes, the second starting from
 // the powers that the first left in shared memory.
 template <int KT, int MINB, int kDepBatch, bool TWO>
@@ -526,13 +529,13 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
   unsigned char *const my_flush = bt.flush + warp * kFlushBytes;
   const int C = 2 * K + 1;
   const unsigned units = hdr->n_units;
+  if (blockIdx.x < units && warp == 0) bt.find(rec, nullptr, tile_off, unit_off, n_tiles, blockIdx.x);
+  __syncthreads();
   for (unsigned u = blockIdx.x; u < units; u += gridDim.x) {
-    const int tile = block_find(unit_off, n_tiles, u);
-    const unsigned lo = tile_off[tile] + (u - unit_off[tile]) * kDepBatch;
-    const int n = (int)min((unsigned)kDepBatch, tile_off[tile + 1] - lo);
-    const int n_items = bt.load(rec, nullptr, lo, n, T);
+    const int tile = (int)bt.unit[0];
+    const int n_items = bt.load(rec, nullptr, bt.unit[1], (int)bt.unit[2], T, tile_off, unit_off, n_tiles, u + gridDim.x, units);
     // ------------------------------------------------------------- eight runs a warp, four lanes each
-    for (int it = warp * 8; it < n_items; it += (kDepThreads / 32) * 8) {
+    for (int it = warp * 8; it < n_items; it = bt.next_runs()) {
       const unsigned item = it + g < n_items ? bt.items[it + g] : 0u;
       const int s0 = item & 0xFFFu, len = (item >> 12) & 0x7Fu;
       const long long row = ((long long)tile << tile_shift) + (item >> 19);
@@ -631,14 +634,16 @@ DepositChoice deposit_choice() {
             return DepositBatch<B, false>::bytes(T) + (TWO ? (size_t)(kDepThreads / 32) * (kItem / 8) * 32 * 16 : 0);
           }};
 }
-// (orders a pass, blocks per SM that its sums' registers allow, and the largest batch that fits beside them)
+// Orders a pass, blocks per SM that its sums' registers allow, and the batch: as many records as measured best
+// (K = 32: 2304 47.4, 2560 46.5, 2816 44.9, 3072 45.1, 3328 48.4, 3840 51.9 ps a segment of the whole run; K = 16:
+// 2304 38.8, 2560 38.1, 2816 36.9; two passes of 16 orders at K = 32: 51.6, four of 8: 52.7).
 DepositChoice deposit_kernel(int K) {
   if (K <= 4) return deposit_choice<4, 5, 2048, false>();
   if (K <= 8) return deposit_choice<8, 5, 2048, false>();
   if (K <= 12) return deposit_choice<12, 5, 2048, false>();
-  if (K <= 16) return deposit_choice<16, 4, 2560, false>();
-  if (K <= 24) return deposit_choice<24, 3, 3072, false>();
-  if (K <= 32) return deposit_choice<32, 3, 3072, false>();
+  if (K <= 16) return deposit_choice<16, 4, 2816, false>();
+  if (K <= 24) return deposit_choice<24, 3, 2816, false>();
+  if (K <= 32) return deposit_choice<32, 3, 2816, false>();
   if (K <= 48) return deposit_choice<24, 3, 2304, true>();
   return deposit_choice<32, 3, 2304, true>();
 }

@@ -376,23 +376,47 @@ struct SumF {
 constexpr int kFlushStride = 32 * 8 + 16;  // bytes per coefficient of a warp's flush buffer
 constexpr int kFlushBytes = 8 * kFlushStride;
 
+// The last i < n with off[i] <= u (off nondecreasing, off[0] = 0), found by one warp.
+__device__ __forceinline__ int warp_find(const unsigned *__restrict__ off, int n, unsigned u) {
+  const int lane = threadIdx.x & 31;
+  int a = 0;
+  while (n > 1) {
+    const int step = (n + 31) / 32;
+    const bool le = lane * step < n && __ldg(off + a + lane * step) <= u;
+    const int k = (__popc(__ballot_sync(kFull, le)) - 1) * step;
+    a += k;
+    n = min(step, n - k);
+  }
+  return a;
+}
+
 // One unit of a deposit: a batch of at most B records of one tile of T rows, in shared memory, its records'
 // indices sorted by row and cut into runs of at most kItem records of one row.  The runs are listed longest
-// first, so that the eight runs a warp takes at a time have about equal lengths.
+// first and taken by eight, one warp after the other, so that the eight have about equal lengths and the
+// warps end at about the same time.
+// (Of a unit's 60,000 cycles at K = 32 and 31,000 at K = 16, 11,000 went into its preparation, where a warp
+// waited for one answer after the other, and 13 % of the rest were spent waiting for the slowest warp.  So a
+// thread's rows and ranks stay in registers, the unit to come is found and fetched into L2 beside the scan,
+// the runs are listed beside the index and taken as warps get to them: 256^2, K = 32, 47.3 -> 44.9 ps a
+// segment in all, K = 16 37.1 -> 36.8, 1024^2, K = 64, 92.5 -> 84.7 with tiles of 64 rows.)
 // (Small loops: the blocks of an SM are in different phases of the deposit and share its instruction cache.)
 template <int B, bool X>
 struct DepositBatch {
+  static constexpr int kPer = B / kDepThreads;
+  static_assert(B % kDepThreads == 0 && B <= 4096, "a run's first index has 12 bits");
+  static_assert(B % (4 * kItem) == 0, "what lies behind the runs is aligned to 16 bytes");
   float4 *rec;             // [B]
   float *rec_x;            // X: [B]
   unsigned char *flush;    // [warps][kFlushBytes]
   unsigned *cnt, *start;   // [T] records per row, first index of the row
   unsigned *items;         // runs: start | length << 12 | row << 19
-  unsigned *bucket;        // [16] runs by their number of steps, then places
-  unsigned short *idx, *rank;  // [B] record indices by row; place within the row
+  unsigned *bucket;        // [16] runs by their number of steps, then places; [16] runs taken
+  unsigned *unit;          // the unit to come: tile, first record, records
+  unsigned short *idx;     // [B] record indices by row
   void *rest;
   static size_t bytes(int T) {
-    return (size_t)B * (X ? 20 : 16) + (kDepThreads / 32) * kFlushBytes + (size_t)T * 8 + (size_t)(B / kItem + T) * 4 + 64 +
-           B * 4;
+    return (size_t)B * (X ? 20 : 16) + (kDepThreads / 32) * kFlushBytes + (size_t)T * 8 + (size_t)(B / kItem + T) * 4 + 80 +
+           B * 2;
   }
   __device__ __forceinline__ DepositBatch(float4 *smem, int T) {
     rec = smem;
@@ -402,14 +426,31 @@ struct DepositBatch {
     start = cnt + T;
     items = start + T;
     bucket = items + B / kItem + T;
-    idx = reinterpret_cast<unsigned short *>(bucket + 16);
-    rank = idx + B;
-    rest = rank + B;
+    unit = bucket + 17;
+    idx = reinterpret_cast<unsigned short *>(bucket + 20);
+    rest = idx + B;
   }
-  // Loads and sorts records [lo, lo + n); returns the number of runs.
-  __device__ __forceinline__ int load(const float4 *__restrict__ src, const float *__restrict__ src_x, unsigned lo, int n,
-                                      int T) {
-    const int lane = threadIdx.x & 31;
+  // Unit u, found by one warp and fetched into L2.
+  __device__ __forceinline__ void find(const float4 *src, const float *src_x, const unsigned *__restrict__ tile_off,
+                                       const unsigned *__restrict__ unit_off, int n_tiles, unsigned u) {
+    const int t = warp_find(unit_off, n_tiles, u);
+    if ((threadIdx.x & 31) != 0) return;
+    const unsigned lo = tile_off[t] + (u - unit_off[t]) * B, n = min((unsigned)B, tile_off[t + 1] - lo);
+    unit[0] = (unsigned)t;
+    unit[1] = lo;
+    unit[2] = n;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src + lo), "r"(n * 16u) : "memory");
+    if (X) {  // (whole 16 bytes: the buffer is a multiple of them)
+      const unsigned a = lo & ~3u, e = (lo + n + 3u) & ~3u;
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src_x + a), "r"((e - a) * 4u) : "memory");
+    }
+  }
+  // Loads and sorts the n records from lo on; returns the number of runs.  u_next: the unit to come, if below
+  // `units`.
+  __device__ __forceinline__ int load(const float4 *src, const float *src_x, unsigned lo, int n, int T,
+                                      const unsigned *__restrict__ tile_off, const unsigned *__restrict__ unit_off,
+                                      int n_tiles, unsigned u_next, unsigned units) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll 4
     for (int i = threadIdx.x; i < n; i += kDepThreads) {
       const unsigned dst = (unsigned)__cvta_generic_to_shared(rec + i);
@@ -423,14 +464,20 @@ struct DepositBatch {
 #pragma unroll 1
     for (int i = threadIdx.x; i < T; i += kDepThreads) cnt[i] = 0u;
     if (threadIdx.x < 16) bucket[threadIdx.x] = 0u;
+    if (threadIdx.x == 16) bucket[16] = (kDepThreads / 32) * 8;
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-#pragma unroll 4
-    for (int i = threadIdx.x; i < n; i += kDepThreads)
-      rank[i] = (unsigned short)atomicAdd(&cnt[__float_as_uint(rec[i].x) & (T - 1)], 1u);
+    unsigned key[kPer];  // row | rank << 16
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int i = k * kDepThreads + (int)threadIdx.x;
+      key[k] = i < n ? __float_as_uint(rec[i].x) & (T - 1) : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+      if (k * kDepThreads + (int)threadIdx.x < n) key[k] |= atomicAdd(&cnt[key[k]], 1u) << 16;
     __syncthreads();
-    // starts of the rows, and how many runs of how many steps (8 records a step) they make
-    if (threadIdx.x < 32) {
+    if (warp == 0) {  // starts of the rows
       unsigned carry = 0;
 #pragma unroll 1
       for (int b = 0; b < T; b += 32) {
@@ -444,13 +491,17 @@ struct DepositBatch {
         }
         if (row < T) start[row] = carry + v - c;
         carry += __shfl_sync(kFull, v, 31);
-        if (c) {
-          const unsigned k = (c + kItem - 1) / kItem, len = (c + k - 1) / k;
-          atomicAdd(&bucket[(len + 7) / 8], k);
-        }
+      }
+    } else if (warp == 1) {  // how many runs of how many steps (8 records a step) they make
+#pragma unroll 1
+      for (int row = lane; row < T; row += 32) {
+        const unsigned c = cnt[row];
+        if (!c) continue;
+        const unsigned k = (c + kItem - 1) / kItem, len = (c + k - 1) / k;
+        atomicAdd(&bucket[(len + 7) / 8], k);
       }
       __syncwarp();
-      unsigned v = lane < 16 ? bucket[lane] : 0u;  // longest runs first
+      const unsigned v = lane < 16 ? bucket[lane] : 0u;  // longest runs first
       unsigned sum = v;
 #pragma unroll
       for (int o = 1; o < 16; o <<= 1) {
@@ -459,27 +510,39 @@ struct DepositBatch {
       }
       if (lane < 16) bucket[lane] = sum - v;
       if (lane == 0) bucket[15] = sum;  // (no run has 15 steps) their total
+    } else if (warp == 2 && u_next < units) {
+      find(src, src_x, tile_off, unit_off, n_tiles, u_next);
     }
     __syncthreads();
-#pragma unroll 4
-    for (int i = threadIdx.x; i < n; i += kDepThreads)
-      idx[start[__float_as_uint(rec[i].x) & (T - 1)] + rank[i]] = (unsigned short)i;
+    if (warp == 3) {
+#pragma unroll 1
+      for (int row = lane; row < T; row += 32) {
+        const unsigned c = cnt[row];
+        if (!c) continue;
+        const unsigned k = (c + kItem - 1) / kItem, len = (c + k - 1) / k;
+        const unsigned at = atomicAdd(&bucket[(len + 7) / 8], k);
+#pragma unroll 1
+        for (unsigned q = 0; q < k; ++q)
+          items[at + q] = (start[row] + q * len) | (min(len, c - q * len) << 12) | ((unsigned)row << 19);
+      }
+    }
     const int n_items = (int)bucket[15];
-    __syncthreads();
-#pragma unroll 1
-    for (int row = threadIdx.x; row < T; row += kDepThreads) {
-      const unsigned c = cnt[row];
-      if (!c) continue;
-      const unsigned k = (c + kItem - 1) / kItem, len = (c + k - 1) / k;
-      const unsigned at = atomicAdd(&bucket[(len + 7) / 8], k);
-#pragma unroll 1
-      for (unsigned q = 0; q < k; ++q)
-        items[at + q] = (start[row] + q * len) | (min(len, c - q * len) << 12) | ((unsigned)row << 19);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int i = k * kDepThreads + (int)threadIdx.x;
+      if (i < n) idx[start[key[k] & 0xFFFFu] + (key[k] >> 16)] = (unsigned short)i;
     }
     __syncthreads();
     return n_items;
   }
+  // The next eight runs for this warp.
+  __device__ __forceinline__ int next_runs() const {
+    int it = 0;
+    if ((threadIdx.x & 31) == 0) it = (int)atomicAdd(&bucket[16], 8u);
+    return __shfl_sync(kFull, it, 0);
+  }
 };
+static_assert(kDepThreads == 128, "four warps share the steps of DepositBatch::load");
 
 // ------------------------------------------------------------------------------------- host side
 std::mutex g_rec_mu;
@@ -549,9 +612,10 @@ unsigned tail_packets(const RecordPlan &pl) { return (unsigned)pl.tail_blocks * 
 cudaError_t plan_records(int64_t rows, uint64_t packets, long long capacity, RecordPlan *out) {
   RecordPlan pl{};
   pl.rows = rows;
-  // Tiles of 32 rows (more where they would be over kMaxTiles); over kMaxBins of them are sorted in two
-  // passes of about equal width.
-  pl.tile_shift = 5;
+  // Tiles of 32 rows, 64 where one pass of the sort does not hold so many (half the bins, runs of twice the
+  // length: 1024^2, K = 64, 110 -> 100 ps a segment; 256^2, K = 32, 49.9 -> 53), more where they would be over
+  // kMaxTiles; over kMaxBins of them are sorted in two passes of about equal width.
+  pl.tile_shift = rows > ((int64_t)kMaxBins << 5) ? 6 : 5;
   while (((rows + (1ll << pl.tile_shift) - 1) >> pl.tile_shift) > kMaxTiles) ++pl.tile_shift;
   if (pl.tile_shift > 12) return cudaErrorInvalidValue;  // (a run's row field has 13 bits)
   pl.n_tiles = (int)((rows + (1ll << pl.tile_shift) - 1) >> pl.tile_shift);
