@@ -33,25 +33,27 @@ if ROOT not in sys.path:
 
 METRIC = "photons/s fwd+adjoint harmonic MC; grad evals/s vs plain MC at stated error"
 UNIT = "photons/s"
-# kernels of libmcr per step: forward (pack, transport, finalize, H) | eps (residual, reduction) |
-# backward (adjoint source | pack, 4 CDF, transport, finalize | gradient)
+# kernels of libmcr per step beside the record launches: forward (pack, closing transport, finalize, H) | eps
+# (residual, reduction) | backward (adjoint source | pack, 4 CDF, closing transport, finalize | gradient)
 KERNELS_PER_STEP = 15
-# The L2's peak rate for reduction sectors on GB300 from ncu (lts__t_sectors_op_red.sum.peak_sustained
-# = 188 sectors per cycle, lts__cycles_elapsed.avg.per_second = 2.017 GHz under load), times 32 B per
-# sector: the ceiling of the transport's 64-bit tally reductions (profiles/k_transport_grad256_l2_reduction.md).
-L2_RED_SECTORS_PER_CYCLE = 188
-L2_CLOCK_HZ = 2.017e9
-L2_RED_PEAK_GBS = L2_RED_SECTORS_PER_CYCLE * L2_CLOCK_HZ * 32 / 1e9
-# DRAM bytes (read + write) per K = 32 transport launch of the grad256 gradient evaluation, from
-# one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the benchmark's forward
-# (40.36 MB) and adjoint (41.68 MB) launches at full size: the tally footprint, read once.
-TRANSPORT_DRAM_BYTES = {"grad256": 41_017_344}
-# DRAM bytes per pixel segment of the sorted-record deposit (transport in record mode, counting
-# sort, deposit), from one ncu capture at 1024^2, K = 64 (1e6 packets, 1.327e9 segments: 126.3 GB;
-# profiles/k_transport_large1024_records_dram.md), scaled to a launch by its segments.  Its
-# algorithmic DRAM bytes: a 16-byte record written, read and rewritten by the sort, read by the deposit.
-RECORD_DRAM_BYTES_PER_SEGMENT = 95.2
-RECORD_ALG_BYTES_PER_SEGMENT = 64
+# Algorithmic DRAM bytes per pixel segment of the record deposit: a 16-byte record written, read and rewritten
+# by the sort, read by the deposit; a second sorting pass (over 131,072 tally rows) counts, reads and rewrites
+# it once more.
+RECORD_BYTES_PER_SEGMENT = (64, 112)
+RECORD_ONE_PASS_ROWS = 131_072
+
+
+def record_kernels(packets, rows, deposits=1):
+    """Kernels that the record launches of one run enqueue (152 SMs): a launch per full buffer (4,096 segments a
+    packet), one per halving of the packets in use down to what the tail takes, one for a part-full buffer."""
+    buffer = min(max(packets * 1024, 1 << 22), 1 << 28)
+    n = max(4, -(-packets * 4096 // buffer)) + 1
+    in_use = min(packets, 152 * 4 * 256)
+    while in_use > 152 * 2 * 8 * 4:
+        in_use //= 2
+        n += 1
+    # transport, tail, scan, sort, deposit; a second sorting pass: count, scan, sort
+    return min(n, 1024) * (4 + deposits + (3 if rows > RECORD_ONE_PASS_ROWS else 0))
 
 
 def _args():
@@ -431,52 +433,32 @@ def _gpu(args):
         grad_err = {"d_eps_d_mua": ea, "d_eps_d_mus": es,
                     "how": "relative L2 error vs a 10x-packet evaluation, corrected for its noise"}
 
-    # roofline of the dominant kernel (the transport): algorithmic bytes = (2K+1) fixed-point
-    # read-modify-writes of 8 B per pixel segment; achieved = bytes / event-timed kernel duration
+    # roofline of a run's record launches (transport, sort, deposit): algorithmic DRAM bytes of the records
+    # over the event-timed launches.  The largest of the kernels, the deposit, is bound by instruction issue.
     C = 2 * w.K + 1
     launches = len(tr_ms)
     avg_ms = float(np.mean(tr_ms))
     avg_segs = float(np.mean(segs))
-    achieved_gbs = C * 8 * avg_segs / (avg_ms * 1e-3) / 1e9
     peaks = {}
     try:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
     except Exception:
         pass
     hbm = float(peaks.get("hbm_gbs", 6800.0))
-    # the tally reductions go to L2 (the grad256 tally is L2-resident): the bound is the L2's
-    # reduction-sector rate; the HBM ratio is kept as a secondary figure
-    row_words = (C + 15) // 16 * 16 if C > 32 else (C + 3) // 4 * 4
-    # tallies beyond 256 MB take the sorted-record deposit: its roofline is HBM for the records
-    in_hbm = w.nx * w.nz * row_words * 8 > 256 << 20
-    if in_hbm:
-        bound, peak = "hbm", hbm
-        achieved_gbs = RECORD_ALG_BYTES_PER_SEGMENT * avg_segs / (avg_ms * 1e-3) / 1e9
-    else:
-        bound, peak = "l2_reduction", L2_RED_PEAK_GBS
-    roofline = {"bound": bound, "achieved": achieved_gbs, "peak": peak, "unit": "GB/s",
-                "frac": achieved_gbs / peak,
-                "traffic": (RECORD_DRAM_BYTES_PER_SEGMENT * avg_segs if in_hbm else TRANSPORT_DRAM_BYTES.get(w.name)),
-                "kernel": "k_transport", "launch_ms": avg_ms, "launches_timed": launches,
-                "segments_per_launch": avg_segs,
-                "bytes_per_segment": RECORD_ALG_BYTES_PER_SEGMENT if in_hbm else C * 8,
-                "peak_source": ("MEASURED_PEAKS.json hbm_gbs (of measured): the tally lives in HBM" if in_hbm else
-                                "ncu lts__t_sectors_op_red.sum.peak_sustained (188 sectors/cycle) x L2 clock "
-                                "2.017 GHz x 32 B (of measured peak rate; profiles/k_transport_grad256_l2_reduction.md)"),
-                "achieved_is": ("sorted-record deposit (transport + sort + deposit, event-timed): algorithmic DRAM "
-                                "bytes 64 per segment (a 16-byte record written, read and rewritten by the sort, read "
-                                "by the deposit); traffic = the measured 95.2 B per segment x segments.  The pipeline "
-                                "is bound by its deposit kernel's instruction issue, far below HBM"
-                                if in_hbm else
-                                "algorithmic reduction payload 8 (2K+1) B per segment / event-timed launch")}
-    if not in_hbm:
-        roofline["hbm"] = {"peak": hbm, "frac": achieved_gbs / hbm,
-                           "note": "payload rate over the measured HBM copy rate (MEASURED_PEAKS.json hbm_gbs); the "
-                                   "payload goes to L2, DRAM sees `traffic` per launch"}
+    rec_bytes = RECORD_BYTES_PER_SEGMENT[w.nx * w.nz > RECORD_ONE_PASS_ROWS]
+    achieved_gbs = rec_bytes * avg_segs / (avg_ms * 1e-3) / 1e9
+    roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm, "unit": "GB/s", "frac": achieved_gbs / hbm,
+                "traffic": None, "kernel": "k_transport_rec + k_rec_sort + k_rec_deposit", "launch_ms": avg_ms,
+                "launches_timed": launches, "segments_per_launch": avg_segs, "bytes_per_segment": rec_bytes,
+                "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks else "fallback 6.8 TB/s",
+                "achieved_is": "algorithmic DRAM bytes of the records (written, read and rewritten by each sorting "
+                               "pass, read by the deposit) / event-timed run; the deposit's instruction issue, not "
+                               "HBM, is the bound",
+                "reductions_saved": {"direct_payload_gbs": C * 8 * avg_segs / (avg_ms * 1e-3) / 1e9,
+                                     "note": "what 8 (2K+1) bytes of reductions per segment would be at this rate"}}
     if not args.no_red_probe:
-        red = l2_reduction_peak(w.nx * w.nz, C)
-        roofline["reduction_probe"] = dict(red, frac=achieved_gbs / red["value"],
-                                           note="a measured rate of random-row reductions alone, not a ceiling")
+        roofline["reduction_probe"] = dict(l2_reduction_peak(w.nx * w.nz, C),
+                                           note="a measured rate of random-row reductions alone")
 
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
@@ -502,8 +484,9 @@ def _gpu(args):
                "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
                # sharded runs add one raw export per run and, for the adjoint, the source strength
                # (4 CDF kernels) in the finalisation
-               "gpu_launches": (KERNELS_PER_STEP + 3 * (len(srcs) - 1) + (len(srcs) + 5 if sharded else 0))
-               * args.steps, "roofline": roofline,
+               "gpu_launches": (KERNELS_PER_STEP + 3 * (len(srcs) - 1) + (len(srcs) + 5 if sharded else 0)
+                                + len(srcs) * record_kernels(per_src, w.nx * w.nz)
+                                + record_kernels(n, w.nx * w.nz)) * args.steps, "roofline": roofline,
                "cpu_baseline": cpu}
         print(json.dumps(out), flush=True)
     if world > 1:
@@ -1249,22 +1232,23 @@ def _grad3d(args):
     C = (L + 1) ** 2
     ms = float(np.mean([t for t, _ in tr]))
     seg = float(np.mean([s for _, s in tr]))
-    achieved = C * 8 * seg / (ms * 1e-3) / 1e9
+    rec_bytes = RECORD_BYTES_PER_SEGMENT[n ** 3 > RECORD_ONE_PASS_ROWS] // 16 * 20
+    achieved = rec_bytes * seg / (ms * 1e-3) / 1e9
     peaks = {}
     try:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
     except Exception:
         pass
     hbm = float(peaks.get("hbm_gbs", 6800.0))
-    # DRAM bytes per forward launch: 21.05 GB at 1e6 packets (ncu, 96^3, L = 4), scaled by packets
-    traffic = 21.05e9 * N / 1e6 if (n, L) == (96, 4) else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-                "traffic": traffic, "kernel": "k_transport3", "launch_ms": ms, "segments_per_launch": seg,
-                "bytes_per_segment": C * 8,
+                "traffic": None, "kernel": "k_transport3_rec + k_rec_sort + k_rec_deposit3", "launch_ms": ms,
+                "segments_per_launch": seg, "bytes_per_segment": rec_bytes,
+                "achieved_is": "algorithmic DRAM bytes of the 20-byte records (written, read and rewritten by each "
+                               "sorting pass, read by the deposit) / event-timed run; the bound is instruction issue",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks else "fallback 6.8 TB/s"}
     if not args.no_red_probe:
         red = l2_reduction_peak(n ** 3, C, row_words=(C + 15) // 16 * 16 if C > 16 else (C + 3) // 4 * 4)
-        roofline["l2_reduction_peak"] = dict(red, frac=achieved / red["value"])
+        roofline["l2_reduction_peak"] = dict(red, note="a measured rate of random-row reductions alone")
     value = 2 * N * args.steps / T
     cpu = None
     if not args.no_cpu_baseline:
@@ -1280,7 +1264,9 @@ def _grad3d(args):
            "config": {"workload": f"grad3d: {n}^3 voxels of {dx} mm, L={L} ({C} channels), g={g}, pencil beam, "
                                   f"{N:.0e} forward + {N:.0e} adjoint packets per step",
                       "segments_per_photon": float(np.mean(segs)) / N, "l2": "flushed between timed steps (256 MB write)"},
-           "clocks": clocks, "gpu_launches": 14 * args.steps, "roofline": roofline, "cpu_baseline": cpu}
+           "clocks": clocks,
+           "gpu_launches": (14 + 2 * record_kernels(N, n ** 3, 2 if L > 6 else 1)) * args.steps, "roofline": roofline,
+           "cpu_baseline": cpu}
     print(json.dumps(out), flush=True)
     return 0
 

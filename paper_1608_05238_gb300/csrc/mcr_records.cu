@@ -13,14 +13,18 @@
 //      a batch in shared memory and writes each bin's run to its place in one go.
 //   4. k_rec_deposit takes a batch of one tile's records, sorts their indices by row in shared memory,
 //      and gives each group of four lanes a run of one row's records: every lane rebuilds the harmonic
-//      row of two records at a time (the same complex products as harmonic_row, as packed FP32 pairs)
-//      and sums the rounded products in registers; one reduction per coefficient and run follows.
+//      row of two records at a time (the same complex products as harmonic_row) and sums the rounded
+//      products in registers; one reduction per coefficient and run follows.
 // Every product is rounded exactly as in the direct deposit and integer addition is exact, so the
 // tally is bit-identical to it.
 //
 // Nothing is read back: a call enqueues more record launches than it is likely to need (one that finds
 // nothing to do ends at once) and then one direct transport launch that adopts whatever packets are
 // left, so the call stays asynchronous and can be captured into a graph.
+//
+// 1e7 + 1e7 packets at 256 x 256, K = 32: 871 ms by the direct deposit, 475 to 514 so (a record: transport 10 to
+// 14 ps, sort 9 to 10, deposit 22 to 23, the waits of kernels launched ahead included); 1e6 packets at
+// 1024 x 1024, K = 64: 211 -> 111 ms.
 #include "mcr_records.cuh"
 
 namespace mcr {

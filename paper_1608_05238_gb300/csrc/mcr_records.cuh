@@ -19,7 +19,7 @@ constexpr int kTailThreads = 256;
 // The tail takes over at this many packets to one of its warps (256 x 256, K = 16, 1e5 packets, transport:
 // 3.9 ms at 1, 3.8 at 2, 3.5 at 4, 4.1 at 8; the 128 registers of two blocks per SM beat three blocks by 0.3 ms).
 constexpr unsigned kTailPackets = 4;
-constexpr int kSortBatch = 3072;    // records a block sorts at a time (2048: 8 % slower, 4096: 10 %, its registers spill)
+constexpr int kSortBatch = 3072;    // records a block sorts at a time (2048: 8 % slower; 4096: 10 %, it spills)
 static_assert(kMaxBins % kSortThreads == 0 && kSortBatch % kSortThreads == 0, "every bin and record has a thread");
 constexpr int kDepThreads = 128;
 constexpr int kItem = 64;           // most records of one run (a group of four lanes, two records each)
@@ -220,13 +220,16 @@ __device__ int block_find(const unsigned *__restrict__ off, int n, unsigned u) {
 // bins of 2^shift rows.  Otherwise: one coarse bin's records into its tiles.
 // The batch is sorted in shared memory first, so that a bin's records leave as one contiguous run and
 // take one cursor update per batch and bin instead of one per record.
+// 9 to 10 ps a record and pass (the copy rate would allow 4.7): the shared-memory and cursor wavefronts take
+// 58 to 68 % of the load-store slots, and a block's phases wait at its barriers (two blocks an SM; writing each
+// record straight to its place took 21 ps, its 16 bytes being half a sector).
 // X: records of five words, the fifth in arrays of its own (in_x, sorted_x).
 template <bool FIRST, bool X = false>
 __global__ void __launch_bounds__(kSortThreads, 2)
     k_rec_sort(const float4 *__restrict__ in, const float *__restrict__ in_x, float4 *__restrict__ sorted,
-               float *__restrict__ sorted_x, const RecordHeader *hdr, unsigned max_blocks,
-               int shift, int n_bins, unsigned *cursor, unsigned capacity, const unsigned *__restrict__ coarse_off, const unsigned *__restrict__ coarse_unit_off,
-               int n_coarse, int coarse_shift, unsigned *flags) {
+               float *__restrict__ sorted_x, const RecordHeader *hdr, unsigned max_blocks, int shift, int n_bins,
+               unsigned *cursor, unsigned capacity, const unsigned *__restrict__ coarse_off,
+               const unsigned *__restrict__ coarse_unit_off, int n_coarse, int coarse_shift, unsigned *flags) {
   after_previous();
   constexpr int kPer = kSortBatch / kSortThreads;
   extern __shared__ float4 srec[];                                  // [kSortBatch]
