@@ -2,7 +2,6 @@
 // up-sampling with their backward passes (ReLU masks and skip gradients fused), bias
 // gradients, the residual MSE loss and the Adam update that also writes the BF16 weight copies.
 // Tensors are NHWC bf16 slices described by (pointer, channel stride, channel offset).
-#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "dn_internal.h"
@@ -486,33 +485,12 @@ __global__ void __launch_bounds__(256) k_pack_input_v8(const float *__restrict__
 }
 
 // per-sample input scale 1 / mean(channel 0) of channel-major fp32 maps [B][C][HW] (the fluence
-// a_0 of a harmonic map), FP64 sum in a fixed order.  A cluster of eight blocks per sample: the sum is bound
-// by the FP64 pipe (two additions a cycle and SM), so one SM alone took 40 us for 256^2 pixels
-// (denoising one 256^2 map 344 -> 313 us, a training step on eight 1921 -> 1886).
-constexpr int kScaleBlocks = 8;
-template <bool VEC>  // HW and every sample's first pixel are multiples of four floats
-__global__ void __cluster_dims__(kScaleBlocks, 1, 1) k_sample_scale(const float *__restrict__ src, int C, long long HW,
-                                                                    float *__restrict__ scale) {
+// a_0 of a harmonic map), one block per sample, FP64 sum in a fixed order
+__global__ void k_sample_scale(const float *__restrict__ src, int C, long long HW, float *__restrict__ scale) {
   __shared__ double red[kT / 32];
-  __shared__ double part;
-  const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
-  const float *x = src + (size_t)blockIdx.y * C * HW;
-  const long long chunk = (HW + 4 * kScaleBlocks - 1) / (4 * kScaleBlocks) * 4, lo = blockIdx.x * chunk;
-  const long long hi = lo + chunk < HW ? lo + chunk : HW;
-  double acc = 0.0;  // signed (adjoint) maps: mean |a_0|
-  if (VEC) {
-#pragma unroll 4
-    for (long long i = lo + 4 * threadIdx.x; i < hi; i += 4 * kT) {
-      const float4 v = __ldg(reinterpret_cast<const float4 *>(x + i));
-      acc += fabsf(v.x);
-      acc += fabsf(v.y);
-      acc += fabsf(v.z);
-      acc += fabsf(v.w);
-    }
-  } else {
-#pragma unroll 4
-    for (long long i = lo + threadIdx.x; i < hi; i += kT) acc += fabsf(__ldg(x + i));
-  }
+  const float *x = src + (size_t)blockIdx.x * C * HW;
+  double acc = 0.0;
+  for (long long i = threadIdx.x; i < HW; i += kT) acc += fabsf(x[i]);  // signed (adjoint) maps: mean |a_0|
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -520,16 +498,9 @@ __global__ void __cluster_dims__(kScaleBlocks, 1, 1) k_sample_scale(const float 
   if (threadIdx.x == 0) {
     double s = 0.0;
     for (int k = 0; k < kT / 32; ++k) s += red[k];
-    part = s;
-  }
-  cluster.sync();
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < kScaleBlocks; ++k) s += *cluster.map_shared_rank(&part, k);
     const double m = s / (double)HW;
-    scale[blockIdx.y] = (float)(1.0 / (m > 1e-30 ? m : 1e-30));
+    scale[blockIdx.x] = (float)(1.0 / (m > 1e-30 ? m : 1e-30));
   }
-  cluster.sync();  // the other blocks' shared memory is read until here
 }
 
 // channel-major fp32 [B][C][HW] * scale[b] -> NHWC fp32 [B][HW][C]   (training targets)
@@ -735,15 +706,7 @@ cudaError_t pack_input(const float *src, const float *scale, int B, long long HW
   return cudaGetLastError();
 }
 cudaError_t sample_scale(const float *src, int B, long long HW, int C, float *scale, cudaStream_t s) {
-  const bool vec = HW % 4 == 0 && (uintptr_t)src % 16 == 0;
-  for (int b = 0; b < B; b += 65535) {  // (a grid's second dimension)
-    const dim3 grid(kScaleBlocks, B - b < 65535 ? B - b : 65535);
-    const float *from = src + (size_t)b * C * HW;
-    if (vec)
-      k_sample_scale<true><<<grid, kT, 0, s>>>(from, C, HW, scale + b);
-    else
-      k_sample_scale<false><<<grid, kT, 0, s>>>(from, C, HW, scale + b);
-  }
+  k_sample_scale<<<B, kT, 0, s>>>(src, C, HW, scale);
   return cudaGetLastError();
 }
 cudaError_t pack_target(const float *src, const float *scale, int B, long long HW, int C, float *dst, cudaStream_t s) {
