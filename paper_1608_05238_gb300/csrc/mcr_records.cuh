@@ -511,8 +511,8 @@ struct DepositBatch {
         const unsigned t = __shfl_down_sync(kFull, sum, o);
         if (lane + o < 16) sum += t;
       }
-      if (lane < 16) bucket[lane] = sum - v;
-      if (lane == 0) bucket[15] = sum;  // (no run has 15 steps) their total
+      const unsigned total = __shfl_sync(kFull, sum, 0);
+      if (lane < 16) bucket[lane] = lane == 15 ? total : sum - v;  // (no run has 15 steps: there stands the total)
     } else if (warp == 2 && u_next < units) {
       find(src, src_x, tile_off, unit_off, n_tiles, u_next);
     }

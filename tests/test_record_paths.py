@@ -1,0 +1,46 @@
+"""Paths of the record deposit that short runs do not reach: many work units of one tally row, two sorting
+passes, small launch shapes, full buffers -- each against the direct deposit, bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1608_05238_gb300 import _build, mcr
+from parity_util import f32
+
+pytestmark = pytest.mark.gpu
+
+DIRECT, RECORDS = (0, 0, 1, 0, 1, 1, 0), (0, 0, 0, 0, 0, 2, 0)
+COUNTERS = ("launched", "flights", "collisions", "segments", "escapes", "rr_kill", "rr_survive", "scatter_limit",
+            "event_limit")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    _build.build()
+    mcr.load()
+
+
+def _medium(nz, nx, dx, seed):
+    r = np.random.default_rng(seed)
+    mua = torch.from_numpy((0.01 + 0.1 * r.random((nz, nx))).astype(np.float32)).cuda()
+    mus = torch.from_numpy((5.0 + 10.0 * r.random((nz, nx))).astype(np.float32)).cuda()
+    return mcr.Medium(mua, mus, f32(dx), f32(0.9))
+
+
+def _same(problems, common, records=RECORDS):
+    ref, st_ref = mcr.run_batch(problems, common, launch=DIRECT, stats=True)
+    ref = [x.clone() for x in ref]
+    got, st = mcr.run_batch(problems, common, launch=records, stats=True)
+    assert all(torch.equal(a, b) for a, b in zip(ref, got))
+    assert [st[k] for k in COUNTERS] == [st_ref[k] for k in COUNTERS]
+    mcr.check()
+
+
+@pytest.mark.parametrize("nz,nx", [(1, 1), (1, 2), (2, 33)])
+@pytest.mark.parametrize("K", [4, 64])
+def test_many_units_of_few_rows(nz, nx, K):
+    """Every unit of the deposit holds records of one or a few rows: runs of the greatest length only, as
+    many units as the run has batches, each of which lists its runs anew."""
+    med = _medium(nz, nx, 2.0, K)
+    _same([mcr.Problem(med, 100_000, seed=K, source=mcr.Source(mcr.ISO_POINT, x0=1.0, z0=1.0))],
+          mcr.Run(K=K, n_packets=0))
