@@ -310,8 +310,10 @@ __global__ void __launch_bounds__(kSortThreads, 2)
   }
 }
 
-// Counts per tile of the coarse-sorted records, before the second pass.
-__global__ void __launch_bounds__(kSortThreads) k_rec_count(const float4 *__restrict__ rec, const RecordHeader *hdr,
+// Counts per tile of the coarse-sorted records, before the second pass.  (The kernel just ahead writes rec
+// while this one's blocks may already be resident, so it is read by L2 loads and not by the read-only path,
+// which wants data that is constant for as long as the kernel lives.)
+__global__ void __launch_bounds__(kSortThreads) k_rec_count(const float4 *rec, const RecordHeader *hdr,
                                                             const unsigned *__restrict__ coarse_off,
                                                             const unsigned *__restrict__ coarse_unit_off, int n_coarse,
                                                             int coarse_shift, int tile_shift, unsigned *tile_hist,
@@ -329,7 +331,7 @@ __global__ void __launch_bounds__(kSortThreads) k_rec_count(const float4 *__rest
     for (int k = 0; k < kSortBatch / kSortThreads; ++k) {
       const unsigned i = lo + k * kSortThreads + threadIdx.x;
       if (i >= hi) continue;
-      const unsigned b = (__float_as_uint(__ldg(&rec[i].x)) >> tile_shift) - bin0;
+      const unsigned b = (__float_as_uint(__ldcg(&rec[i].x)) >> tile_shift) - bin0;
       if (MCR_GUARD(flags, b < (unsigned)nb)) atomicAdd(&cnt[b], 1u);
     }
     __syncthreads();

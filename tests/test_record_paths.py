@@ -44,3 +44,11 @@ def test_many_units_of_few_rows(nz, nx, K):
     med = _medium(nz, nx, 2.0, K)
     _same([mcr.Problem(med, 100_000, seed=K, source=mcr.Source(mcr.ISO_POINT, x0=1.0, z0=1.0))],
           mcr.Run(K=K, n_packets=0))
+
+
+@pytest.mark.parametrize("nz,nx", [(256, 512), (1, 131_073), (363, 362), (700, 601)])
+def test_both_sides_of_the_second_sorting_pass(nz, nx):
+    """131,072 rows are 2,048 tiles of 64, one pass; one row more takes the second pass (and its count)."""
+    med = _medium(nz, nx, 0.05, nx)
+    src = mcr.Source(mcr.LINE, x0=0.0, z0=0.0, x1=f32(nx * 0.05), z1=0.0, dir_x=0.2, dir_z=1.0)
+    _same([mcr.Problem(med, 40_000, seed=2, source=src)], mcr.Run(K=7, n_packets=0))
