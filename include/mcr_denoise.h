@@ -87,8 +87,11 @@ int dn_conv_head(const dn_conv_desc *d, const dn_head_desc *h, void *stream);
  *   dw[n][tap][c] += sum_{b, pixel} dz[b, pixel][n] x[b, pixel + tap][c]     (FP32 accumulate)
  * with the operands in pixel-contiguous ("transposed") layouts made by dn_to_ct: dzT
  * [cout][B][H*W] and xT = three x-shifted copies [3][cin][B][H*W].  dw is fp32
- * [cout][taps][cin] and is ADDED to (zero it first); partial sums of split reductions are added
- * with atomics, so the last bits depend on scheduling.  Requires W >= 16 a power of two and
+ * [cout][taps][cin] and is ADDED to (zero it first); the partial sums of a split reduction are added
+ * in a fixed order, so that a call's result depends on its inputs alone (the same holds for the bias
+ * gradients).  They take up to some 30 MB from a memory pool of the device, in the stream's order (the
+ * pool keeps up to 64 MB until mc_release_workspace); without that memory one block per tile sums
+ * all pixels.  Requires W >= 16 a power of two and
  * H*W a multiple of 64; cout, cin <= 512.
  */
 int dn_wgrad(int32_t B, int32_t H, int32_t W, int32_t taps, int32_t cout, int32_t cin, const void *dzT,

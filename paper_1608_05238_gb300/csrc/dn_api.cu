@@ -72,6 +72,73 @@ double *partials_buffer() {
   return g_partials[dev];
 }
 
+// Scratch of one call, from a memory pool of the device in the stream's order: calls on several streams (or
+// threads) have their own, and it can be captured.  The pool keeps up to kPoolKeeps bytes between calls
+// (a weight gradient's partial tiles take at most some 30 MB); release_scratch gives them back.
+constexpr uint64_t kPoolKeeps = 64ull << 20;
+cudaMemPool_t g_pool[64];
+
+cudaMemPool_t scratch_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t keep = kPoolKeeps;
+    cudaMemPool_t pool = nullptr;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      cudaMemPoolDestroy(pool);
+      return nullptr;
+    }
+    g_pool[dev] = pool;
+  }
+  return g_pool[dev];
+}
+
+void release_scratch(int dev) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (dev >= 0 && dev < 64 && g_pool[dev]) cudaMemPoolTrimTo(g_pool[dev], 0);
+}
+
+struct Scratch {
+  void *p = nullptr;
+  cudaStream_t s;
+  Scratch(size_t bytes, cudaStream_t stream) : s(stream) {
+    cudaMemPool_t pool = bytes ? scratch_pool() : nullptr;
+    if (!pool || cudaMallocFromPoolAsync(&p, bytes, pool, s) != cudaSuccess) {
+      if (pool) cudaGetLastError();
+      p = nullptr;
+    }
+  }
+  Scratch(const Scratch &) = delete;
+  Scratch &operator=(const Scratch &) = delete;
+  ~Scratch() {
+    if (p) cudaFreeAsync(p, s);
+  }
+};
+
+// db[c] += sums of dz over pixels, in a fixed order
+cudaError_t bias_sums(const dn_slice &dz, long long P, int C, float *db, cudaStream_t s) {
+  const __nv_bfloat16 *z = static_cast<const __nv_bfloat16 *>(dz.data);
+  const int rows = bias_rows(z, P, dz.stride, dz.off, C);
+  Scratch sc(rows > 1 ? (size_t)rows * C * sizeof(float) : 0, s);
+  if (!sc.p) return bias_grad(z, P, dz.stride, dz.off, C, 1, true, db, false, s);
+  cudaError_t e = bias_grad(z, P, dz.stride, dz.off, C, rows, false, static_cast<float *>(sc.p), false, s);
+  if (e != cudaSuccess) return e;
+  WgradArgs a{};
+  a.cout = C;
+  a.db = db;
+  return launch_wgrad_sum(a, false, static_cast<float *>(sc.p), rows, s);
+}
+
 bool conv_shape_ok(int B, int H, int W) {
   if (B <= 0 || H <= 0 || W < 16 || (W & (W - 1))) return false;
   if (((long long)H * W) % 128) return false;
@@ -255,7 +322,6 @@ int dn_wgrad(int32_t B, int32_t H, int32_t W, int32_t taps, int32_t cout, int32_
   a.taps = taps;
   a.cout = cout;
   a.cin = cin;
-  a.cin_pad = cin;
   a.N = N;
   a.m_tiles = (cout + 127) / 128;
   a.n_tiles = (cin + N - 1) / N;
@@ -269,7 +335,12 @@ int dn_wgrad(int32_t B, int32_t H, int32_t W, int32_t taps, int32_t cout, int32_
   a.tmem_cols = cols;
   a.dw = dw;
   a.err = err;
-  if (launch_wgrad_tc(tmA, tmB, a, (cudaStream_t)stream) != cudaSuccess) return MCR_ERR_CUDA;
+  cudaStream_t s = (cudaStream_t)stream;
+  Scratch sc(a.splits > 1 ? wgrad_part_bytes(a, false) : 0, s);
+  a.part = static_cast<float4 *>(sc.p);
+  if (!a.part) a.splits = 1;
+  if (launch_wgrad_tc(tmA, tmB, a, s) != cudaSuccess) return MCR_ERR_CUDA;
+  if (a.part && launch_wgrad_sum(a, false, nullptr, 0, s) != cudaSuccess) return MCR_ERR_CUDA;
   return MCR_OK;
 }
 
@@ -291,6 +362,7 @@ int dn_wgrad_bias_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W,
   if (dz.off % 8 || dz.stride % 8 || x.off % 8 || x.stride % 8) return MCR_ERR_ARG;
   unsigned *err = error_word();
   if (!err) return MCR_ERR_CUDA;
+  cudaStream_t s = (cudaStream_t)stream;
   const uint64_t HW = (uint64_t)H * W;
   CUtensorMap tmA, tmB;
   {
@@ -319,7 +391,6 @@ int dn_wgrad_bias_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W,
   a.taps = taps;
   a.cout = cout;
   a.cin = cin;
-  a.cin_pad = cin;
   a.dw = dw;
   a.err = err;
   if (wgrad_halo_applies(taps, cout, W)) {  // few output channels: all nine taps from one haloed box
@@ -340,7 +411,11 @@ int dn_wgrad_bias_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W,
     if (splits > segs) splits = segs;
     if (splits < 1) splits = 1;
     a.splits = (int)splits;
-    if (launch_wgrad_halo(tmA, tmH, a, (cudaStream_t)stream) != cudaSuccess) return MCR_ERR_CUDA;
+    Scratch sc(a.splits > 1 ? wgrad_part_bytes(a, true) : 0, s);
+    a.part = static_cast<float4 *>(sc.p);
+    if (!a.part) a.splits = 1;
+    if (launch_wgrad_halo(tmA, tmH, a, s) != cudaSuccess) return MCR_ERR_CUDA;
+    if (a.part && launch_wgrad_sum(a, true, nullptr, 0, s) != cudaSuccess) return MCR_ERR_CUDA;
     return MCR_OK;
   }
   a.N = cin > 128 ? 128 : ((cin + 15) / 16) * 16;  // MMA N; B arrives in whole 64-channel boxes
@@ -348,16 +423,26 @@ int dn_wgrad_bias_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W,
   a.n_tiles = (cin + a.N - 1) / a.N;
   const long long kblocks = (long long)B * HW / 64;
   long long splits = (2 * 152) / (taps * a.m_tiles * a.n_tiles);  // one wave of two blocks per SM
-  if (splits > kblocks / 16) splits = kblocks / 16;  // >= 16 K blocks per CTA: its atomic epilogue stays small
+  if (splits > kblocks / 16) splits = kblocks / 16;  // >= 16 K blocks per CTA: its epilogue stays small
   if (splits < 1) splits = 1;
   a.splits = (int)splits;
   uint32_t cols = 32;
   while (cols < (uint32_t)a.N) cols <<= 1;
   a.tmem_cols = cols;
-  if (launch_wgrad_mn(tmA, tmB, a, (cudaStream_t)stream) != cudaSuccess) return MCR_ERR_CUDA;
-  if (db && bias_grad(static_cast<const __nv_bfloat16 *>(dz.data), (long long)B * HW, dz.stride, dz.off, cout, db,
-                      (cudaStream_t)stream) != cudaSuccess)
+  // one scratch, and one sum, for the weight gradient's partial tiles and the bias gradient's partial sums
+  const __nv_bfloat16 *z = static_cast<const __nv_bfloat16 *>(dz.data);
+  const size_t tiles = a.splits > 1 ? wgrad_part_bytes(a, false) : 0;
+  const int rows = db ? bias_rows(z, (long long)B * HW, dz.stride, dz.off, cout) : 0;
+  Scratch sc(tiles + (size_t)rows * cout * sizeof(float), s);
+  a.part = tiles ? static_cast<float4 *>(sc.p) : nullptr;
+  if (!a.part) a.splits = 1;
+  a.db = db;
+  if (launch_wgrad_mn(tmA, tmB, a, s) != cudaSuccess) return MCR_ERR_CUDA;
+  float *bias = sc.p ? reinterpret_cast<float *>(static_cast<char *>(sc.p) + tiles) : nullptr;
+  if (db && bias_grad(z, (long long)B * HW, dz.stride, dz.off, cout, bias ? rows : 1, !bias, bias ? bias : db, true,
+                      s) != cudaSuccess)
     return MCR_ERR_CUDA;
+  if (sc.p && launch_wgrad_sum(a, false, db ? bias : nullptr, rows, s) != cudaSuccess) return MCR_ERR_CUDA;
   return MCR_OK;
 }
 
@@ -398,8 +483,7 @@ int dn_up2_bwd(dn_slice du, dn_slice act, int32_t B, int32_t H, int32_t W, int32
 
 int dn_bias_grad(dn_slice dz, int64_t pixels, int32_t C, float *db, void *stream) {
   if (!slice_ok(dz, C) || !db || pixels <= 0) return MCR_ERR_ARG;
-  DN_TRY(bias_grad(static_cast<const __nv_bfloat16 *>(dz.data), pixels, dz.stride, dz.off, C, db,
-                   (cudaStream_t)stream));
+  DN_TRY(bias_sums(dz, pixels, C, db, (cudaStream_t)stream));
 }
 
 int dn_mse(const float *out, int32_t ostride, const void *x, int32_t xstride, const float *t, int64_t P, int32_t C,

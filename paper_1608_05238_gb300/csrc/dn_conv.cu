@@ -16,6 +16,8 @@
 //     offset/stride, so concatenations are free).
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "dn_internal.h"
 #include "dn_sm100.cuh"
 
@@ -608,16 +610,108 @@ __global__ void __launch_bounds__(kWsThreads, 1)
   if (warp == 0) tmem_dealloc(tmem, 2 * acc_cols);
 }
 
+// Weight gradients are sums over pixels that many CTAs share (`splits` to an accumulator tile).  Each writes
+// its partial tile to scratch, and k_wgrad_sum adds a tile's partials in the order of their splits: added to dW
+// by atomics instead, the sums' last bits depended on the blocks' timing, and Adam, which divides a gradient
+// by its own size, made steps of it that differed between two runs of the same training.
+// part: float4 [tile][split][columns / 4][128 rows], so that the lanes of a warp (rows) write whole lines.
+__device__ __forceinline__ void put_part(float4 *part, int tile, int split, int splits, int columns, int row, int c0,
+                                         const uint32_t v[16], bool have) {
+  float4 *o = part + ((size_t)(tile * splits + split) * (columns / 4) + c0 / 4) * kBlockM + row;
+#pragma unroll
+  for (int j = 0; j < 16; j += 4)
+    o[(j / 4) * kBlockM] = have ? make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]),
+                                              __uint_as_float(v[j + 3]))
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// dW (and db) += the partial tiles, and db += the rows of k_bias_grad's partial sums (blocks from sum_blocks on).
+// A warp takes 32 rows of four columns; G warps share a tile's splits (ranges of them, added in order).  Bound by
+// the latency of its loads from L2 (the partials, 5 to 25 MB, have just been written): 5 to 9 us a layer under ncu,
+// of which the launch ahead hides a part; the training step at 8 x 256^2 takes what it took with atomics (1920 us).
+// HALO: rows (tap, input channel), columns output channels (k_wgrad_halo); else rows output channels,
+// columns input channels.
+template <bool HALO, int G>
+__global__ void __launch_bounds__(G > 8 ? 32 * G : 256) k_wgrad_sum(const WgradArgs a, int columns, int units, int sum_blocks,
+                                                   const float *bias_part, int bias_rows) {
+  constexpr int kWarps = G > 8 ? G : 8;
+  __shared__ float4 red[kWarps][32];
+  cudaGridDependencySynchronize();  // launched ahead: the kernels that write the partials have ended from here on
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if ((int)blockIdx.x >= sum_blocks) {
+    const int c = ((int)blockIdx.x - sum_blocks) * 32 + lane;
+    float s = 0.f;
+    if (c < a.cout) {
+#pragma unroll 8
+      for (int k = bias_rows * warp / kWarps; k < bias_rows * (warp + 1) / kWarps; ++k) s += __ldcs(bias_part + (size_t)k * a.cout + c);
+    }
+    red[warp][lane].x = s;
+    __syncthreads();
+    if (warp == 0 && c < a.cout) {
+      for (int w = 1; w < kWarps; ++w) s += red[w][lane].x;
+      a.db[c] += s;
+    }
+    return;
+  }
+  const int unit = (int)blockIdx.x * (kWarps / G) + warp / G, g = warp % G;
+  const int n4 = columns / 4, tile = unit / (4 * n4), col = (unit >> 2) % n4, row = (unit & 3) * 32 + lane;
+  const int tap = HALO ? 2 * (tile % 5) + (row >> 6) : tile % a.taps;
+  const int m = HALO ? (tile / 5) * 64 + (row & 63) : (tile / a.taps % a.m_tiles) * kBlockM + row;
+  const bool ones_row = HALO && tap == 9 && row == 64 && tile / 5 == 0 && a.db;
+  const bool mine = unit < units && (HALO ? ones_row || (tap < 9 && m < a.cin) : m < a.cout);
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [&](const float4 &v) {
+    s.x += v.x;
+    s.y += v.y;
+    s.z += v.z;
+    s.w += v.w;
+  };
+  if (mine) {
+    const float4 *p = a.part + ((size_t)tile * a.splits * n4 + col) * kBlockM + row;
+#pragma unroll 8
+    for (int k = a.splits * g / G; k < a.splits * (g + 1) / G; ++k) add(__ldcs(p + (size_t)k * n4 * kBlockM));
+  }
+  if (G > 1) {
+    red[warp][lane] = s;
+    __syncthreads();
+    if (g != 0) return;
+#pragma unroll
+    for (int w = 1; w < G; ++w) add(red[warp + w][lane]);
+  }
+  if (!mine) return;
+  const float t[4] = {s.x, s.y, s.z, s.w};
+  if (HALO) {
+    float *o = ones_row ? a.db : a.dw + (size_t)tap * a.cin + m;
+    const size_t step = ones_row ? 1 : (size_t)9 * a.cin;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (4 * col + j < a.cout) o[(4 * col + j) * step] += t[j];
+  } else {
+    const int c = tile / a.taps / a.m_tiles * a.N + 4 * col;
+    float *o = a.dw + ((size_t)m * a.taps + tap) * a.cin + c;
+    if (c + 4 <= a.cin && (reinterpret_cast<uintptr_t>(o) & 15) == 0) {
+      float4 d = *reinterpret_cast<float4 *>(o);
+      add(d);
+      *reinterpret_cast<float4 *>(o) = s;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (c + j < a.cin) o[j] += t[j];
+    }
+  }
+}
+
 // k_wgrad_tc: weight gradient dW[n][tap][c] += sum_p dZ[p][n] X[p + tap][c] as a GEMM over pixels
 // with M = 128 output channels, N = `N` input channels, K = 64-pixel blocks.  Operands are
 // K-major (pixels contiguous): dZ^T [cout][B][HW] and three x-shifted copies
 // X^T_kx [cin][B][HW] (X^T_kx[c][b][y W + x] = X[b][y][x + kx - 1][c], zero outside the row).
 // The y shift of a tap is a TMA coordinate offset of (ky - 1) W pixels inside one image (zero
 // filled outside it), which keeps every box start 16-byte aligned.  Each CTA sums a contiguous
-// range of K blocks for one tap and one (M, N) tile and adds its partial tile to dW (FP32).
+// range of K blocks for one tap and one (M, N) tile and writes its partial tile (FP32; put_part).
 __global__ void __launch_bounds__(128, 1)
     k_wgrad_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2, const WgradArgs a) {
+  cudaTriggerProgrammaticLaunchCompletion();  // (what follows waits for this kernel's end: k_wgrad_sum)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t bTileBytes = (uint32_t)a.N * kBlockK * 2;
@@ -701,18 +795,15 @@ __global__ void __launch_bounds__(128, 1)
     uint32_t v[16];
     tmem_ld16(trow + (uint32_t)c0, v);
     tmem_ld_wait();
-    if (!have || m >= a.cout) continue;
-    float *o = a.dw + ((size_t)m * a.taps + tap) * a.cin_pad + n_tile * a.N + c0;
-    const int cb = n_tile * a.N + c0;
-    if (a.cin_pad % 4 == 0 && cb + 16 <= a.cin) {  // 16-byte aligned: four 4-wide reductions
-#pragma unroll
-      for (int j = 0; j < 16; j += 4)
-        red_add_v4(o + j, __uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]),
-                   __uint_as_float(v[j + 3]));
-    } else {
+    if (m >= a.cout) continue;
+    if (a.part) {
+      put_part(a.part, (int)blockIdx.z * a.taps + tap, split, a.splits, a.N, warp * 32 + lane, c0, v, have);
+    } else if (have) {
+      float *o = a.dw + ((size_t)m * a.taps + tap) * a.cin + n_tile * a.N + c0;
+      const int cb = n_tile * a.N + c0;
 #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (cb + j < a.cin) atomicAdd(o + j, __uint_as_float(v[j]));
+        if (cb + j < a.cin) o[j] += __uint_as_float(v[j]);
     }
   }
   tc_fence_before();
@@ -735,6 +826,7 @@ static int wgrad_mn_stages(int N) { return N <= 64 ? 4 : 3; }
 __global__ void __launch_bounds__(128, 1)
     k_wgrad_mn(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const WgradArgs a,
                int stages) {
+  cudaTriggerProgrammaticLaunchCompletion();  // (what follows waits for this kernel's end: k_wgrad_sum)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int nb = (a.N + 63) / 64;  // 64-channel B boxes per stage (the MMA uses the first N)
@@ -822,18 +914,15 @@ __global__ void __launch_bounds__(128, 1)
     uint32_t v[16];
     tmem_ld16(trow + (uint32_t)c0, v);
     tmem_ld_wait();
-    if (!have || m >= a.cout) continue;
-    float *o = a.dw + ((size_t)m * a.taps + tap) * a.cin_pad + n_tile * a.N + c0;
-    const int cb = n_tile * a.N + c0;
-    if (a.cin_pad % 4 == 0 && cb + 16 <= a.cin) {  // 16-byte aligned: four 4-wide reductions
-#pragma unroll
-      for (int j = 0; j < 16; j += 4)
-        red_add_v4(o + j, __uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]),
-                   __uint_as_float(v[j + 3]));
-    } else {
+    if (m >= a.cout) continue;
+    if (a.part) {
+      put_part(a.part, (int)blockIdx.z * a.taps + tap, split, a.splits, a.N, warp * 32 + lane, c0, v, have);
+    } else if (have) {
+      float *o = a.dw + ((size_t)m * a.taps + tap) * a.cin + n_tile * a.N + c0;
+      const int cb = n_tile * a.N + c0;
 #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (cb + j < a.cin) atomicAdd(o + j, __uint_as_float(v[j]));
+        if (cb + j < a.cin) o[j] += __uint_as_float(v[j]);
     }
   }
   tc_fence_before();
@@ -852,9 +941,8 @@ __global__ void __launch_bounds__(128, 1)
 // the distance of the two windows).  Tap 8's partner is a 16-row block of ones in shared memory,
 // so those 64 accumulator rows hold sum_p dZ[p][o]: the bias gradient comes free with the
 // weight gradient.  Five accumulators of 64 columns (taps 0-1, 2-3, 4-5, 6-7, 8 + ones) stay in
-// TMEM for the CTA's contiguous range of segments; the epilogue adds them into dw with one atomic
-// per element (consecutive lanes = consecutive input channels) and, on channel block 0, the
-// ones row into db.  Per segment the CTA reads 25 KB of
+// TMEM for the CTA's contiguous range of segments; the epilogue writes them out as partial sums
+// (with the ones row on channel block 0).  Per segment the CTA reads 25 KB of
 // X and 8 KB of dZ instead of 9 x (8 + 8) KB for nine separate shifted GEMMs.
 constexpr uint32_t kWhBytes = 3 * 66 * 128;                          // 25,344 B written by the box
 constexpr uint32_t kWhStride = (kWhBytes + 1023) & ~1023u;           // 25,600 B
@@ -864,6 +952,7 @@ constexpr uint32_t kWhOnes = 2048;  // 16 rows x 64 bf16 ones (tap 8's partner M
 
 __global__ void __launch_bounds__(128, 1)
     k_wgrad_halo(const __grid_constant__ CUtensorMap tmZ, const __grid_constant__ CUtensorMap tmH, const WgradArgs a) {
+  cudaTriggerProgrammaticLaunchCompletion();  // (what follows waits for this kernel's end: k_wgrad_sum)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *ones = smem + kWhStages * kWhStage;
@@ -959,16 +1048,17 @@ __global__ void __launch_bounds__(128, 1)
       uint32_t v[16];
       tmem_ld16(trow + (uint32_t)c0, v);
       tmem_ld_wait();
-      if (have && tap == 9 && mrow == 64 && cb == 0 && a.db) {  // the ones row: sum_p dZ[p][o]
+      const bool ones_row = tap == 9 && mrow == 64 && cb == 0 && a.db;  // sum_p dZ[p][o]
+      if (!ones_row && (tap > 8 || c >= a.cin)) continue;
+      if (a.part) {
+        put_part(a.part, cb * 5 + mt, split, a.splits, (a.cout + 15) / 16 * 16, mrow, c0, v, have);
+      } else if (have) {
+        float *o = ones_row ? a.db : a.dw + (size_t)tap * a.cin + c;
+        const size_t step = ones_row ? 1 : (size_t)9 * a.cin;
 #pragma unroll
         for (int j = 0; j < 16; ++j)
-          if (c0 + j < a.cout) atomicAdd(a.db + c0 + j, __uint_as_float(v[j]));
+          if (c0 + j < a.cout) o[(c0 + j) * step] += __uint_as_float(v[j]);
       }
-      if (!have || tap > 8 || c >= a.cin) continue;
-      float *o = a.dw + (size_t)tap * a.cin_pad + c;
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (c0 + j < a.cout) atomicAdd(o + (size_t)(c0 + j) * 9 * a.cin_pad, __uint_as_float(v[j]));
     }
   }
   tc_fence_before();
@@ -977,6 +1067,9 @@ __global__ void __launch_bounds__(128, 1)
 }
 
 }  // namespace
+
+// accumulator columns of a tile that are written out
+static int wgrad_columns(const WgradArgs &a, bool halo) { return halo ? (a.cout + 15) / 16 * 16 : a.N; }
 
 cudaError_t launch_wgrad_tc(const CUtensorMap &tmA, const CUtensorMap tmB[3], const WgradArgs &a, cudaStream_t s) {
   const size_t smem = 1024 + kStages * (kATileBytes + (size_t)a.N * kBlockK * 2) + 256;
@@ -1107,6 +1200,32 @@ cudaError_t launch_wgrad_halo(const CUtensorMap &tmZ, const CUtensorMap &tmH, co
   const int cblocks = (a.cin + 63) / 64;
   k_wgrad_halo<<<dim3((unsigned)a.splits, (unsigned)cblocks), 128, smem, s>>>(tmZ, tmH, a);
   return cudaGetLastError();
+}
+
+size_t wgrad_part_bytes(const WgradArgs &a, bool halo) {
+  const size_t tiles = halo ? (size_t)(a.cin + 63) / 64 * 5 : (size_t)a.taps * a.m_tiles * a.n_tiles;
+  return tiles * a.splits * wgrad_columns(a, halo) * kBlockM * sizeof(float);
+}
+
+cudaError_t launch_wgrad_sum(const WgradArgs &a, bool halo, const float *bias_part, int bias_rows, cudaStream_t s) {
+  const int columns = wgrad_columns(a, halo);
+  const int tiles = !a.part ? 0 : halo ? (a.cin + 63) / 64 * 5 : a.taps * a.m_tiles * a.n_tiles;
+  const int units = tiles * columns;  // (columns / 4 x 4 blocks of 32 rows)
+  // a warp adds up to 16 splits alone; of more, several warps a range each: eight, or for many splits as many as
+  // leave the chip's warp slots some room (1x1 head, 304 splits, 32 units: 16.4 us with 8 warps, 8.2 with 32;
+  // 32 -> 64 channels at 8 x 128^2, 152 splits, 320 units: 9.1 with 8, 9.4 with 16, 14 with 32)
+  int G = a.splits > 16 ? 8 : 1;
+  while (a.splits > 64 && G < 32 && units * 2 * G <= 152 * 40) G *= 2;
+  const int warps = G > 8 ? G : 8;
+  const int sum_blocks = (units * G + warps - 1) / warps;
+  const int blocks = sum_blocks + (bias_part ? (a.cout + 31) / 32 : 0);
+  auto pick = [&](auto h) {
+    constexpr bool H = decltype(h)::value;
+    return G == 32 ? k_wgrad_sum<H, 32> : G == 16 ? k_wgrad_sum<H, 16> : G == 8 ? k_wgrad_sum<H, 8> : k_wgrad_sum<H, 1>;
+  };
+  auto *k = halo ? pick(std::true_type{}) : pick(std::false_type{});
+  if (!blocks) return cudaSuccess;
+  return launch(k, dim3((unsigned)blocks), dim3(32u * warps), true, s, a, columns, units, sum_blocks, bias_part, bias_rows);
 }
 
 // ---------------------------------------------------------------- bounded-wait test hook

@@ -54,13 +54,13 @@ struct WgradArgs {
   int B, HW, W;      // images, pixels per image, row length (for the y shift)
   int taps;          // 9 or 1
   int cout, cin;     // real channel counts
-  int cin_pad;       // dW row length per tap
   int N;             // input channels per CTA tile (multiple of 16, <= 256)
   int m_tiles, n_tiles, splits;
   uint32_t tmem_cols;
-  float *dw;         // fp32 [n_pad][taps][cin_pad], accumulated with atomics
+  float *dw;         // fp32 [cout][taps][cin], added to
   unsigned *err;
-  float *db;         // k_wgrad_halo: if set, db[o] += sum_p dZ[p][o] (the bias gradient), else unused
+  float *db;         // if set, db[o] += sum_p dZ[p][o] (the bias gradient)
+  float4 *part;      // the CTAs' partial tiles (wgrad_part_bytes), or null: one split, added to dw (and db) directly
 };
 cudaError_t launch_wgrad_tc(const CUtensorMap &tmA, const CUtensorMap tmB[3], const WgradArgs &a, cudaStream_t s);
 cudaError_t launch_wgrad_mn(const CUtensorMap &tmA, const CUtensorMap &tmB, const WgradArgs &a, cudaStream_t s);
@@ -68,6 +68,27 @@ cudaError_t launch_wgrad_mn(const CUtensorMap &tmA, const CUtensorMap &tmB, cons
 // per segment serves all nine taps (grid: splits x 64-channel blocks of cin; one block per SM)
 bool wgrad_halo_applies(int taps, int cout, int W);
 cudaError_t launch_wgrad_halo(const CUtensorMap &tmZ, const CUtensorMap &tmH, const WgradArgs &a, cudaStream_t s);
+
+// Launches a kernel; ahead: before the end of the kernel before it in the stream, which it then waits for itself
+// (cudaGridDependencySynchronize).
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, bool ahead, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = ahead ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
+// Scratch for the partial tiles of `a` (its splits and tiles set), and the sum of them into a.dw (and, k_wgrad_halo's,
+// a.db) in a fixed order; bias_part: rows [bias_rows][cout] of bias_grad's partial sums to add to a.db.
+size_t wgrad_part_bytes(const WgradArgs &a, bool halo);
+cudaError_t launch_wgrad_sum(const WgradArgs &a, bool halo, const float *bias_part, int bias_rows, cudaStream_t s);
 
 // Test hook (dn_conv.cu): one warp waits, with the kernels' own bounded mbarrier wait limited to
 // `spins` polls, on an mbarrier that nothing arrives at; on the timeout it latches the kernels'
@@ -86,7 +107,11 @@ cudaError_t up2(const __nv_bfloat16 *src, int B, int H, int W, int sstride, int 
                 int dstride, int doff, cudaStream_t s);
 cudaError_t up2_bwd(const __nv_bfloat16 *du, int ustride, int uoff, const __nv_bfloat16 *act, int astride, int aoff,
                     int B, int H, int W, int C, __nv_bfloat16 *dz, int zstride, int zoff, cudaStream_t s);
-cudaError_t bias_grad(const __nv_bfloat16 *dz, long long P, int stride, int off, int C, float *db, cudaStream_t s);
+// Sums of dz over pixels, per channel: `rows` blocks' partial sums to out[row][C], or, with rows = 1 and add, onto
+// out[C].  bias_rows: how many rows are best.  ahead: the kernel before it in the stream writes neither dz nor out.
+int bias_rows(const __nv_bfloat16 *dz, long long P, int stride, int off, int C);
+cudaError_t bias_grad(const __nv_bfloat16 *dz, long long P, int stride, int off, int C, int rows, bool add, float *out,
+                      bool ahead, cudaStream_t s);
 // One layer of a multi-tensor Adam step (k_adam_multi): tile0 = its first block.
 struct AdamLayer {
   float *w, *m, *v, *g;
@@ -121,6 +146,9 @@ cudaError_t predict_output(const float *out, int ostride, const __nv_bfloat16 *x
                            int B, long long HW, int C, float *dst, cudaStream_t s);
 cudaError_t unpack_output(const float *src, const float *scale, int B, long long HW, int C, float *dst,
                           cudaStream_t s);
+
+// Gives the device's pooled scratch back to the driver (what is in use stays).
+void release_scratch(int dev);
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link needed).
 CUresult encode_tiled(CUtensorMap *map, CUtensorMapDataType dtype, uint32_t rank, void *base, const uint64_t *dims,

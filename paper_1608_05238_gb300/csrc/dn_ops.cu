@@ -198,9 +198,12 @@ __global__ void k_up2_bwd_v8(const __nv_bfloat16 *__restrict__ du, int ustride, 
   st8(dz + pix * zstride + zoff + 8 * g, o.u);
 }
 
-// db[c] += sum over pixels of dz[p][c]
-__global__ void k_bias_grad(const __nv_bfloat16 *__restrict__ dz, long long P, int stride, int off, int C,
-                            float *__restrict__ db) {
+// out[block][c] = the block's sum over pixels of dz[p][c] (add: onto out[c], for one block).  May be launched
+// ahead of the end of a kernel that writes neither dz nor out (the weight gradient); it ends after that kernel,
+// so that what follows needs to wait for this one alone.
+__global__ void k_bias_grad(const __nv_bfloat16 *__restrict__ dz, long long P, int stride, int off, int C, bool add,
+                            float *__restrict__ out) {
+  cudaTriggerProgrammaticLaunchCompletion();
   const int c = blockIdx.y * 32 + threadIdx.x;
   float acc = 0.f;
   if (c < C)
@@ -212,16 +215,19 @@ __global__ void k_bias_grad(const __nv_bfloat16 *__restrict__ dz, long long P, i
   if (threadIdx.y == 0 && c < C) {
     float s = 0.f;
     for (int k = 0; k < (int)blockDim.y; ++k) s += red[k][threadIdx.x];
-    atomicAdd(db + c, s);
+    float *o = out + (size_t)blockIdx.x * C + c;
+    *o = add ? *o + s : s;
   }
+  cudaGridDependencySynchronize();
 }
 
-// db[c] += sum over pixels of dz[p][off + c] (c < C) with 16-byte loads: G = ceil(C / 8) threads
+// The same with 16-byte loads: G = ceil(C / 8) threads
 // cover one pixel row (8 channels each; the row holds at least 8 G channels from off, those past
 // C are read and dropped), 256 / G rows per pass of the block; per-thread FP32 sums, a
-// fixed-order sum over the block's rows in shared memory, one atomic add per channel and block.
+// fixed-order sum over the block's rows in shared memory, one value per channel and block.
 __global__ void __launch_bounds__(256) k_bias_grad_v8(const __nv_bfloat16 *__restrict__ dz, long long P, int stride,
-                                                      int off, int G, int C, float *__restrict__ db) {
+                                                      int off, int G, int C, bool add, float *__restrict__ out) {
+  cudaTriggerProgrammaticLaunchCompletion();
   __shared__ float red[256 * 8];
   const int R = 256 / G, t = threadIdx.x, g = t % G, r = t / G, CG = 8 * G;
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -244,8 +250,10 @@ __global__ void __launch_bounds__(256) k_bias_grad_v8(const __nv_bfloat16 *__res
   for (int c = t; c < C; c += 256) {
     float sum = 0.f;
     for (int k = 0; k < R; ++k) sum += red[k * CG + c];
-    atomicAdd(db + c, sum);
+    float *o = out + (size_t)blockIdx.x * C + c;
+    *o = add ? *o + sum : sum;
   }
+  cudaGridDependencySynchronize();
 }
 
 // residual MSE: y = x + out over C channels; loss partials (FP64) and dout = 2 (y - t) / count
@@ -628,20 +636,24 @@ cudaError_t up2_bwd(const __nv_bfloat16 *du, int ustride, int uoff, const __nv_b
                                                            zoff);
   return cudaGetLastError();
 }
-cudaError_t bias_grad(const __nv_bfloat16 *dz, long long P, int stride, int off, int C, float *db, cudaStream_t s) {
+static bool bias_v8(const __nv_bfloat16 *dz, int stride, int off, int C) {
   const int G = (C + 7) / 8;
-  if (al8(stride, off, 0, 0) && G <= 256 && off + 8 * G <= stride && (reinterpret_cast<uintptr_t>(dz) & 15) == 0) {
-    const int R = 256 / G;
-    long long gx = (P + 4LL * R - 1) / (4LL * R);  // at least ~4 rows per thread
-    if (gx > 152 * 8) gx = 152 * 8;
-    k_bias_grad_v8<<<(unsigned)gx, 256, 0, s>>>(dz, P, stride, off, G, C, db);
-    return cudaGetLastError();
+  return al8(stride, off, 0, 0) && G <= 256 && off + 8 * G <= stride && (reinterpret_cast<uintptr_t>(dz) & 15) == 0;
+}
+int bias_rows(const __nv_bfloat16 *dz, long long P, int stride, int off, int C) {
+  if (bias_v8(dz, stride, off, C)) {
+    const int R = 256 / ((C + 7) / 8);
+    const long long gx = (P + 4LL * R - 1) / (4LL * R);  // at least ~4 rows per thread
+    return (int)(gx > 152 * 2 ? 152 * 2 : gx);
   }
-  long long gx = (P + 8 * 64 - 1) / (8 * 64);
-  if (gx > 256) gx = 256;
-  const dim3 grid((unsigned)gx, (C + 31) / 32), block(32, 8);
-  k_bias_grad<<<grid, block, 0, s>>>(dz, P, stride, off, C, db);
-  return cudaGetLastError();
+  const long long gx = (P + 8 * 64 - 1) / (8 * 64);
+  return (int)(gx > 256 ? 256 : gx);
+}
+cudaError_t bias_grad(const __nv_bfloat16 *dz, long long P, int stride, int off, int C, int rows, bool add, float *out,
+                      bool ahead, cudaStream_t s) {
+  if (bias_v8(dz, stride, off, C))
+    return launch(k_bias_grad_v8, dim3((unsigned)rows), dim3(256), ahead, s, dz, P, stride, off, (C + 7) / 8, C, add, out);
+  return launch(k_bias_grad, dim3((unsigned)rows, (C + 31) / 32), dim3(32, 8), ahead, s, dz, P, stride, off, C, add, out);
 }
 cudaError_t mse(const float *out, int ostride, const __nv_bfloat16 *x, int xstride, const float *t, long long P, int C,
                 __nv_bfloat16 *dout, int dstride, double *partials, int partials_cap, double *loss, cudaStream_t s) {

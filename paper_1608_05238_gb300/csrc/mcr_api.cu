@@ -9,6 +9,10 @@
 
 #include "mcr_internal.h"
 
+namespace dn {
+void release_scratch(int dev);  // dn_api.cu
+}
+
 using namespace mcr;
 
 namespace {
@@ -558,6 +562,9 @@ int mc_release_workspace(void) {
     if (w.ev_stop[k]) cudaEventDestroy(w.ev_stop[k]);
   }
   w = Workspace{};
+#ifndef MCR_CHECKED  // (the checked library has no denoiser)
+  dn::release_scratch(dev);
+#endif
   return release_workspace3(dev);
 }
 
