@@ -21,7 +21,9 @@
  * The library keeps one grow-only workspace per device (fixed-point tallies, packed medium,
  * source CDF, counters, and two record buffers of up to 4 GB each, see mcr_launch.deposit), allocated with cudaMalloc on first use and freed by
  * mc_release_workspace().  Calls that share a device share that workspace: calls on different
- * streams of one device must not overlap in time.
+ * streams of one device must not overlap in time.  A graph captured from a call holds the addresses of the
+ * workspace of that time: those buffers are kept when later calls grow past them, so that it can be replayed
+ * until mc_release_workspace(), after which it must not be.
  */
 #ifndef MCR_H
 #define MCR_H

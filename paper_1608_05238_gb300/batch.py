@@ -9,6 +9,8 @@ adds:
   graph captured once (the packing, CDF, transport and finalize launches of the whole batch
   become one graph launch).  A graph replays the same packets (its seeds are baked in); build a
   new runner, or call ``recapture(seed)``, for a fresh ensemble.
+  Other calls may run between replays, larger ones too (the library keeps the buffers that a graph
+  uses); after ``mcr.release_workspace()`` a graph must be captured again.
 * ``autotune`` -- times the candidate launch shapes (threads per block, resident blocks per SM,
   collision merge default/off/on, shared-memory tally for a small single problem) on the actual batch with CUDA events and keeps the fastest,
   cached per device, K and batch size.  Results do not depend on the shape (fixed-point

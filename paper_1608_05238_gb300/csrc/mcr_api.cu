@@ -4,7 +4,9 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "mcr_internal.h"
@@ -27,11 +29,11 @@ std::mutex g_mu;
     if (e_ != cudaSuccess) return MCR_ERR_CUDA; \
   } while (0)
 
-int grow(void **ptr, size_t *cap, size_t need) {
+int grow(Workspace &w, void **ptr, size_t *cap, size_t need) {
   if (need == 0) need = 256;
   if (*cap >= need && *ptr) return MCR_OK;
   if (*ptr) {
-    cudaFree(*ptr);
+    if (std::find(w.captured.begin(), w.captured.end(), *ptr) == w.captured.end()) cudaFree(*ptr);
     *ptr = nullptr;
     *cap = 0;
   }
@@ -50,8 +52,8 @@ struct Need {
   size_t records = 0, rec_scratch = 0;  // record deposit (records: each of the two buffers)
 };
 
-// Workspace of the current device, grown to `need`.
-int workspace(const Need &need, Workspace **out) {
+// Workspace of the current device, grown to `need`, for a call on stream s.
+int workspace(const Need &need, cudaStream_t s, Workspace **out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MCR_ERR_CUDA;
   Workspace &w = g_ws[dev];
@@ -67,18 +69,35 @@ int workspace(const Need &need, Workspace **out) {
       if (cudaEventCreate(&w.ev_start[k]) != cudaSuccess || cudaEventCreate(&w.ev_stop[k]) != cudaSuccess)
         return MCR_ERR_CUDA;
   }
-  if ((rc = grow((void **)&w.partials, &w.partials_bytes, (size_t)4096 * sizeof(double)))) return rc;
-  if (need.tally && (rc = grow((void **)&w.tally, &w.tally_bytes, need.tally))) return rc;
-  if (need.mu && (rc = grow((void **)&w.mu, &w.mu_bytes, need.mu))) return rc;
-  if (need.acc && (rc = grow((void **)&w.acc, &w.acc_bytes, need.acc))) return rc;
-  if (need.cdf && (rc = grow((void **)&w.cdf, &w.cdf_bytes, need.cdf))) return rc;
-  if (need.block_sums && (rc = grow((void **)&w.block_sums, &w.block_sums_bytes, need.block_sums))) return rc;
-  if (need.order && (rc = grow((void **)&w.order, &w.order_bytes, need.order))) return rc;
-  if (need.order_hist && (rc = grow((void **)&w.order_hist, &w.order_hist_bytes, need.order_hist))) return rc;
+  if ((rc = grow(w, (void **)&w.partials, &w.partials_bytes, (size_t)4096 * sizeof(double)))) return rc;
+  if (need.tally && (rc = grow(w, (void **)&w.tally, &w.tally_bytes, need.tally))) return rc;
+  if (need.mu && (rc = grow(w, (void **)&w.mu, &w.mu_bytes, need.mu))) return rc;
+  if (need.acc && (rc = grow(w, (void **)&w.acc, &w.acc_bytes, need.acc))) return rc;
+  if (need.cdf && (rc = grow(w, (void **)&w.cdf, &w.cdf_bytes, need.cdf))) return rc;
+  if (need.block_sums && (rc = grow(w, (void **)&w.block_sums, &w.block_sums_bytes, need.block_sums))) return rc;
+  if (need.order && (rc = grow(w, (void **)&w.order, &w.order_bytes, need.order))) return rc;
+  if (need.order_hist && (rc = grow(w, (void **)&w.order_hist, &w.order_hist_bytes, need.order_hist))) return rc;
   if (need.records) {
-    if ((rc = grow((void **)&w.records, &w.records_bytes, need.records))) return rc;
-    if ((rc = grow((void **)&w.sorted, &w.sorted_bytes, need.records))) return rc;
-    if ((rc = grow((void **)&w.rec_scratch, &w.rec_scratch_bytes, need.rec_scratch))) return rc;
+    if ((rc = grow(w, (void **)&w.records, &w.records_bytes, need.records))) return rc;
+    if ((rc = grow(w, (void **)&w.sorted, &w.sorted_bytes, need.records))) return rc;
+    if ((rc = grow(w, (void **)&w.rec_scratch, &w.rec_scratch_bytes, need.rec_scratch))) return rc;
+  }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  MCR_TRY_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) {  // the graph will use what this call uses
+    const std::pair<size_t, void *> uses[] = {{need.tally, w.tally},     {need.acc, w.acc},
+                                              {need.mu, w.mu},           {need.cdf, w.cdf},
+                                              {need.block_sums, w.block_sums}, {need.order, w.order},
+                                              {need.order_hist, w.order_hist}, {need.records, w.records},
+                                              {need.records, w.sorted},  {need.rec_scratch, w.rec_scratch}};
+    for (const auto &u : uses) {
+      if (!u.first || std::find(w.captured.begin(), w.captured.end(), u.second) != w.captured.end()) continue;
+      try {
+        w.captured.push_back(u.second);
+      } catch (...) {
+        return MCR_ERR_NOMEM;
+      }
+    }
   }
   *out = &w;
   return MCR_OK;
@@ -207,11 +226,11 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
   Workspace *w = nullptr;
   if (rec_mode && !timed && !holds_records(need)) rec_mode = false;
   if (!rec_mode) need.records = need.rec_scratch = 0;
-  int rc = workspace(need, &w);
+  int rc = workspace(need, s, &w);
   if (rc == MCR_ERR_NOMEM && rec_mode) {  // no room for the record buffers: deposit directly
     rec_mode = false;
     need.records = need.rec_scratch = 0;
-    rc = workspace(need, &w);
+    rc = workspace(need, s, &w);
   }
   if (rc) return rc;
 
@@ -403,7 +422,7 @@ int mc_finalize(const mcr_medium *med, const mcr_source *src, const float *qstar
     need.block_sums = (size_t)((npix + 255) / 256) * 8;
   }
   Workspace *w = nullptr;
-  if ((rc = workspace(need, &w))) return rc;
+  if ((rc = workspace(need, s, &w))) return rc;
   if (qstar) {  // the source strength S of the adjoint run, from q* as mc_adjoint computes it
     MCR_TRY_CUDA(launch_source_cdf(qstar, npix, w->cdf, w->block_sums, (size_t)((npix + 255) / 256),
                                    w->qmax_bits(0), s));
@@ -457,7 +476,7 @@ int mc_h_eps(const mcr_medium *med, const float *coeff, const float *Hmeas, floa
   const int64_t npix = (int64_t)med->nx * med->nz;
   std::lock_guard<std::mutex> lock(g_mu);
   Workspace *w = nullptr;
-  if ((rc = workspace(Need{}, &w))) return rc;
+  if ((rc = workspace(Need{}, (cudaStream_t)stream, &w))) return rc;
   MCR_TRY_CUDA(launch_h_eps(med->mua, coeff, Hmeas, npix, (double)med->dx * (double)med->dx, H, dL_dH, w->partials,
                             w->partials_bytes / sizeof(double), eps, (cudaStream_t)stream));
   return MCR_OK;
@@ -469,7 +488,7 @@ int mc_eps(int64_t npix, double pixel_area, const float *H, const float *Hmeas, 
   std::lock_guard<std::mutex> lock(g_mu);
   Workspace *w = nullptr;
   int rc;
-  if ((rc = workspace(Need{}, &w))) return rc;
+  if ((rc = workspace(Need{}, (cudaStream_t)stream, &w))) return rc;
   MCR_TRY_CUDA(launch_h_eps(nullptr, H, Hmeas, npix, pixel_area, nullptr, dL_dH, w->partials,
                             w->partials_bytes / sizeof(double), eps, (cudaStream_t)stream));
   return MCR_OK;
@@ -480,7 +499,7 @@ int mc_dot(int64_t n, const float *a, const float *b, double *out, void *stream)
   std::lock_guard<std::mutex> lock(g_mu);
   Workspace *w = nullptr;
   int rc;
-  if ((rc = workspace(Need{}, &w))) return rc;
+  if ((rc = workspace(Need{}, (cudaStream_t)stream, &w))) return rc;
   MCR_TRY_CUDA(launch_dot(a, b, n, w->partials, w->partials_bytes / sizeof(double), out, (cudaStream_t)stream));
   return MCR_OK;
 }
@@ -556,7 +575,8 @@ int mc_release_workspace(void) {
   void *ptrs[] = {w.tally, w.acc, w.mu, w.cdf, w.block_sums, w.partials, w.small, w.order, w.order_hist,
                   w.records, w.sorted, w.rec_scratch};
   for (void *p : ptrs)
-    if (p) cudaFree(p);
+    if (p && std::find(w.captured.begin(), w.captured.end(), p) == w.captured.end()) cudaFree(p);
+  for (void *p : w.captured) cudaFree(p);
   for (int k = 0; k < 3; ++k) {
     if (w.ev_start[k]) cudaEventDestroy(w.ev_start[k]);
     if (w.ev_stop[k]) cudaEventDestroy(w.ev_stop[k]);

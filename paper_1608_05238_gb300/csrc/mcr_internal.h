@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/mcr.h"
 
 namespace mcr {
@@ -171,6 +173,9 @@ cudaError_t launch_order(const TransportParams &p, unsigned total_bins, unsigned
 // Workspace of one device (grow-only).
 struct Workspace {
   int device = -1;
+  // Buffers that a call under stream capture used: the graph holds their addresses, so they are kept until
+  // mc_release_workspace() also when a later call grows past them.
+  std::vector<void *> captured;
   unsigned long long *tally = nullptr;
   size_t tally_bytes = 0;
   double *acc = nullptr;  // FP64 chunk accumulator [C][npix]

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1608_05238_gb300 import _build, mcr
+from paper_1608_05238_gb300 import _build, batch, mcr
 from parity_util import f32
 
 pytestmark = pytest.mark.gpu
@@ -52,3 +52,29 @@ def test_both_sides_of_the_second_sorting_pass(nz, nx):
     med = _medium(nz, nx, 0.05, nx)
     src = mcr.Source(mcr.LINE, x0=0.0, z0=0.0, x1=f32(nx * 0.05), z1=0.0, dir_x=0.2, dir_z=1.0)
     _same([mcr.Problem(med, 40_000, seed=2, source=src)], mcr.Run(K=7, n_packets=0))
+
+
+@pytest.mark.parametrize("launch", [None, DIRECT])
+def test_a_graph_outlives_larger_calls(launch):
+    """Later calls with more packets, and then with a larger grid and order, grow every buffer of the workspace;
+    the graph goes on with its own."""
+    mcr.release_workspace()
+    problems = [mcr.Problem(_medium(64, 64, 0.1, i), 10_000, seed=i, stream_id=i,
+                            source=mcr.Source(mcr.ISO_POINT, x0=3.0, z0=3.0)) for i in range(3)]
+    q = torch.from_numpy(np.random.default_rng(4).normal(size=(64, 64)).astype(np.float32)).cuda()
+    problems.append(mcr.Problem(_medium(64, 64, 0.1, 9), 10_000, seed=9, stream_id=1, qstar=q))
+    common = mcr.Run(K=16, n_packets=0)
+    ref = [x.clone() for x in mcr.run_batch(problems, common, launch=DIRECT)]
+    runner = batch.BatchRunner(problems, common, launch=launch)
+    runner.capture()
+    for n, K, packets in ((64, 16, 1_000_000), (300, 33, 2_000_000), (64, 16, 1_000)):
+        med = _medium(n, n, 0.05, n)
+        big = torch.ones(n, n, device="cuda")
+        a = mcr.adjoint(med, big, mcr.Run(K=K, n_packets=packets, seed=2))
+        for p in problems:
+            p.out.zero_()
+        assert all(torch.equal(x, y) for x, y in zip(ref, runner.replay()))
+        assert torch.equal(a, mcr.adjoint(med, big, mcr.Run(K=K, n_packets=packets, seed=2)))
+    mcr.check()
+    torch.cuda.synchronize()
+    mcr.release_workspace()
