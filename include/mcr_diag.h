@@ -1,8 +1,8 @@
 /*
  * mcr_diag.h -- measurement and test entry points of libmcr.  They are not part of the method's
  * interface (include/mcr.h): one measures a hardware ceiling that the transport is compared
- * with, the other exposes the random-number function that the transport kernels use, so that
- * tests can hold it to the generator's published known answers.
+ * with, the others expose what the transport kernels use or did, so that tests can hold them to it
+ * (the random-number generator's published known answers; who finished a run's packets).
  */
 #ifndef MCR_DIAG_H
 #define MCR_DIAG_H
@@ -38,6 +38,14 @@ int mc_reduction_probe(void *tally, int64_t rows, int32_t row_words, int32_t C, 
  * 1 <= n <= 2^20, else MCR_ERR_ARG.
  */
 int mc_philox_blocks(const uint32_t *ctr, const uint32_t *key, int32_t n, uint32_t *out);
+
+/*
+ * mc_record_info -- what the last 2D (dim 2) or 3D (dim 3) run on the current device enqueued by its record
+ * deposit: *kernels kernels of its record launches (0 for a direct run), and *closing packets that they left to
+ * the closing direct launch (of the last 2^26 packets of a longer run; -1 for a direct run).  Both host.
+ * Synchronises the device after a run by records.  MCR_ERR_ARG for another dim or a null pointer.
+ */
+int mc_record_info(int32_t dim, int64_t *kernels, int64_t *closing);
 
 /*
  * dn_wait_probe -- test hook (the paper has no counterpart): the denoiser kernels' bounded

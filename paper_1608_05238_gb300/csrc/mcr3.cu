@@ -438,6 +438,7 @@ struct Work3 {
   size_t mu_bytes = 0;
   unsigned char *rec_a = nullptr, *rec_b = nullptr, *rec_scratch = nullptr;  // record deposit
   size_t rec_a_bytes = 0, rec_b_bytes = 0, rec_scratch_bytes = 0;
+  RecordInfo rec_info;
   unsigned char *small = nullptr;  // [0,8) counter, [64,192) stats, [448] flags, [512] qmax bits
   double *partials = nullptr;
 };
@@ -579,11 +580,12 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   MCR3_TRY(cudaStreamIsCapturing(s, &cap));
   RecordPlan plan{};
+  w->rec_info = RecordInfo{};
   if (run->n_packets && cap == cudaStreamCaptureStatusNone && rec_plan3(p, nvox, &plan) == cudaSuccess) {
     const size_t bytes = rec_buffer_bytes3(plan);
     if (grow3((void **)&w->rec_a, &w->rec_a_bytes, bytes) == MCR_OK && grow3((void **)&w->rec_b, &w->rec_b_bytes, bytes) == MCR_OK &&
         grow3((void **)&w->rec_scratch, &w->rec_scratch_bytes, rec_scratch_bytes(plan)) == MCR_OK) {
-      MCR3_TRY(launch_records3(p, plan, w->rec_a, w->rec_b, w->rec_scratch, &p, s));
+      MCR3_TRY(launch_records3(p, plan, w->rec_a, w->rec_b, w->rec_scratch, &p, &w->rec_info, s));
     } else {
       cudaGetLastError();
     }
@@ -645,6 +647,13 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
 }
 
 }  // namespace
+
+int record_info3(int dev, int64_t *kernels, int64_t *closing) {
+  if (dev < 0 || dev >= 64) return MCR_ERR_CUDA;
+  std::lock_guard<std::mutex> lock(g_mu3);
+  *kernels = g_w3[dev].rec_info.kernels;
+  return closing_packets(g_w3[dev].rec_info, closing);
+}
 
 // Frees this device's 3D workspace (called by mc_release_workspace).
 int release_workspace3(int dev) {

@@ -200,6 +200,6 @@ size_t rec_buffer_bytes3(const RecordPlan &pl);  // of each of the two record bu
 // As launch_records: record launches; on return `closing` is set for the direct transport that adopts the
 // packets left.
 cudaError_t launch_records3(const Transport3Params &p, const RecordPlan &pl, unsigned char *buf_a, unsigned char *buf_b,
-                            unsigned char *scratch, Transport3Params *closing, cudaStream_t s);
+                            unsigned char *scratch, Transport3Params *closing, RecordInfo *info, cudaStream_t s);
 
 }  // namespace mcr

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
   };
 
   RecordWriter w;
-  w.stop = in_use <= enough;  // nothing for this kernel to do but launch the first packets
+  w.stop = in_use <= enough && !(fresh && p.n_packets > lanes);  // as in 2D
   bool first = p.rec_prev == nullptr;
   for (;;) {
     w.room(p, lane);
@@ -663,7 +663,7 @@ cudaError_t rec_plan3(const Transport3Params &p, int64_t rows, RecordPlan *out) 
 size_t rec_buffer_bytes3(const RecordPlan &pl) { return record_slots(pl) * 20; }
 
 cudaError_t launch_records3(const Transport3Params &p, const RecordPlan &pl, unsigned char *buf_a, unsigned char *buf_b,
-                            unsigned char *scratch, Transport3Params *closing, cudaStream_t s) {
+                            unsigned char *scratch, Transport3Params *closing, RecordInfo *info, cudaStream_t s) {
   const DepositChoice3 dc = deposit_kernel3(p.L);
   const size_t dep_smem = dc.bytes(1 << pl.tile_shift);
   int sms = 0, dep[2] = {0, 0};
@@ -690,11 +690,13 @@ cudaError_t launch_records3(const Transport3Params &p, const RecordPlan &pl, uns
         launch_ahead(k_transport3_tail, pl.tail_blocks, kTailThreads, smem, s, q);
       },
       [&](const float4 *rec, const float *rec_x, const Scratch &sc) {
-        for (int k = 0; k < 2 && dc.pass[k]; ++k)
+        int k = 0;
+        for (; k < 2 && dc.pass[k]; ++k)
           launch_ahead(dc.pass[k], sms * dep[k], kDepThreads, dep_smem, s, rec, rec_x, q.rec_hdr, sc.tile_off,
                        sc.dep_unit_off, pl.n_tiles, pl.tile_shift, (long long)pl.rows, h, p.Cpad, p.tally, p.flags);
+        return k;
       },
-      s);
+      info, s);
   if (e == cudaSuccess) *closing = q;
   return e;
 }

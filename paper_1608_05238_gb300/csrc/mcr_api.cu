@@ -9,6 +9,7 @@
 #include <utility>
 #include <vector>
 
+#include "../../include/mcr_diag.h"
 #include "mcr_internal.h"
 
 namespace dn {
@@ -234,6 +235,7 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
   }
   if (rc) return rc;
 
+  w->rec_info = RecordInfo{};
   MCR_TRY_CUDA(cudaMemsetAsync(w->stats(slot), 0, sizeof(DevStats), s));
   p.K = common->K;
   p.C = C;
@@ -305,7 +307,8 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
     if (!count) return MCR_OK;
     MCR_TRY_CUDA(cudaMemsetAsync(w->work(), 0, 8, s));
     if (rec_mode) {
-      MCR_TRY_CUDA(launch_records(p, cfg, plan, w->records, w->sorted, w->rec_scratch, w->tally + roff, s));
+      MCR_TRY_CUDA(launch_records(p, cfg, plan, w->records, w->sorted, w->rec_scratch, w->tally + roff,
+                                  &w->rec_info, s));
       return MCR_OK;
     }
     if (ordered) MCR_TRY_CUDA(launch_order(p, total_bins, w->order_hist, w->order, s));
@@ -566,6 +569,16 @@ int mc_last_run_info(int32_t which, mcr_stats *stats, float *transport_ms) {
   return MCR_OK;
 }
 
+int mc_record_info(int32_t dim, int64_t *kernels, int64_t *closing) {
+  int dev = 0;
+  if ((dim != 2 && dim != 3) || !kernels || !closing) return MCR_ERR_ARG;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MCR_ERR_CUDA;
+  if (dim == 3) return record_info3(dev, kernels, closing);
+  std::lock_guard<std::mutex> lock(g_mu);
+  *kernels = g_ws[dev].rec_info.kernels;
+  return closing_packets(g_ws[dev].rec_info, closing);
+}
+
 int mc_release_workspace(void) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MCR_ERR_CUDA;
@@ -612,6 +625,16 @@ const char *mc_version(void) { return "mcr 1.1 sm_103a"; }
 }  // extern "C"
 
 namespace mcr {
+
+int closing_packets(const RecordInfo &info, int64_t *closing) {
+  *closing = -1;
+  if (!info.last) return MCR_OK;
+  RecordHeader h;
+  MCR_TRY_CUDA(cudaDeviceSynchronize());
+  MCR_TRY_CUDA(cudaMemcpy(&h, info.last, sizeof(h), cudaMemcpyDeviceToHost));
+  *closing = (int64_t)h.unlaunched + h.n_left;
+  return MCR_OK;
+}
 
 int check_medium(const mcr_medium *m) {
   if (!m || !m->mua || !m->mus) return MCR_ERR_ARG;

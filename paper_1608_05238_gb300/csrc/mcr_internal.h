@@ -132,6 +132,12 @@ struct RecordHeader {                           // one per record launch of a ca
   unsigned fresh;                               // 1: packets were still to be launched at its end
   unsigned tail_ran, n_tail_left, tail_next;    // the tail took them over; packets it left; the next to take
   unsigned n_units, n_coarse_units;             // work units of the deposit and of the second sorting pass
+  unsigned long long unlaunched;                // packets still to be launched at its end (fresh)
+};
+// What the last run by records was (mc_record_info).
+struct RecordInfo {
+  int64_t kernels = 0;                 // enqueued by its record launches
+  const RecordHeader *last = nullptr;  // of its last record launch (null: a direct run)
 };
 // How a call's records are laid out and sorted (rec_plan).
 struct RecordPlan {
@@ -155,7 +161,8 @@ size_t rec_scratch_bytes(const RecordPlan &pl);  // headers, counts, cursors, sa
 // launches and a closing direct transport launch that takes over whatever packets they leave.
 // Asynchronous on s: nothing is read back.
 cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg, const RecordPlan &pl, float4 *buf_a,
-                           float4 *buf_b, unsigned char *scratch, unsigned long long *tally, cudaStream_t s);
+                           float4 *buf_b, unsigned char *scratch, unsigned long long *tally, RecordInfo *info,
+                           cudaStream_t s);
 
 // Launch order: packets processed in the order of their launch position (line sources: bins of
 // 1/4096 of the line; volumetric sources: 32 x 32-pixel tiles of the launch pixel; other kinds
@@ -197,6 +204,7 @@ struct Workspace {
   size_t sorted_bytes = 0;
   unsigned char *rec_scratch = nullptr;
   size_t rec_scratch_bytes = 0;
+  RecordInfo rec_info;
   double *partials = nullptr;
   size_t partials_bytes = 0;
   // small block: packet counter, run counters per call kind (0 forward, 1 adjoint, 2 batch),
@@ -297,5 +305,8 @@ int noalloc_take_flags(cudaStream_t s);
 
 // Frees the 3D transport's workspace on device dev (mcr3.cu).
 int release_workspace3(int dev);
+// The 3D part of mc_record_info, and the packets that `info`'s record launches left.
+int record_info3(int dev, int64_t *kernels, int64_t *closing);
+int closing_packets(const RecordInfo &info, int64_t *closing);
 
 }  // namespace mcr

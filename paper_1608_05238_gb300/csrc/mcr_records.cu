@@ -213,7 +213,8 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
   };
 
   RecordWriter w;
-  w.stop = in_use <= enough;  // nothing for this kernel to do but launch the first packets
+  // nothing for this kernel to do but launch the first packets, all there are
+  w.stop = in_use <= enough && !(fresh && p.total_packets > lanes);
   bool first = p.rec_prev == nullptr;
   for (;;) {
     w.room(p, lane);
@@ -679,7 +680,8 @@ size_t rec_buffer_bytes(const RecordPlan &pl) { return record_slots(pl) * sizeof
 size_t rec_scratch_bytes(const RecordPlan &pl) { return layout(nullptr, pl).total; }
 
 cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg, const RecordPlan &pl, float4 *buf_a,
-                           float4 *buf_b, unsigned char *scratch, unsigned long long *tally, cudaStream_t s) {
+                           float4 *buf_b, unsigned char *scratch, unsigned long long *tally, RecordInfo *info,
+                           cudaStream_t s) {
   const DepositChoice dc = deposit_kernel(p.K);
   const size_t dep_smem = dc.bytes(1 << pl.tile_shift);
   int sms = 0, dep = 0;
@@ -703,8 +705,9 @@ cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg,
       [&](const float4 *rec, const float *, const Scratch &sc) {
         launch_ahead(dc.kernel, sms * dep, kDepThreads, dep_smem, s, rec, q.rec_hdr, sc.tile_off, sc.dep_unit_off,
                      pl.n_tiles, pl.tile_shift, (long long)pl.rows, p.K, p.Cpad, tally, p.flags);
+        return 1;
       },
-      s);
+      info, s);
   return e != cudaSuccess ? e : launch_transport(q, TransportLaunch{0, 0, 1, 0}, s);
 }
 

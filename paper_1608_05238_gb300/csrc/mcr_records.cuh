@@ -187,7 +187,10 @@ __global__ void __launch_bounds__(1024) k_rec_scan(RecordHeader *hdr, unsigned *
   __shared__ unsigned warp_tot[32];
   after_previous();
   if (threadIdx.x == 0) {
-    if (*launched < n_packets) hdr->fresh = 1u;
+    if (*launched < n_packets) {
+      hdr->fresh = 1u;
+      hdr->unlaunched = n_packets - *launched;
+    }
     if (hdr->tail_ran == 1u) {  // what the tail left stands in the other buffer
       hdr->n_left = hdr->n_tail_left;
       hdr->buf = 1u - hdr->buf;
@@ -674,12 +677,12 @@ void launch_ahead(void (*kernel)(P...), int grid, int block, size_t smem, cudaSt
 }
 
 // The launches of a run: transport() launches the transport and its tail with the fields of q set here,
-// deposit(records, their fifth words, scratch) the deposit of the sorted records.  On return q is set for a
-// direct transport that adopts the packets left.
+// deposit(records, their fifth words, scratch) the deposit of the sorted records, and returns its number of
+// kernels.  On return q is set for a direct transport that adopts the packets left.
 template <bool X, typename Transport, typename Deposit>
 cudaError_t record_chain(const RecordPlan &pl, const Scratch &sc, const RecordBuffers &buf, RecordParams &q, int dep_batch,
                          const unsigned long long *work, unsigned long long total_packets, unsigned *flags,
-                         Transport transport, Deposit deposit, cudaStream_t s) {
+                         Transport transport, Deposit deposit, RecordInfo *info, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(sc.hdr, 0, sc.zeroed, s);
   if (e != cudaSuccess) return e;
   int sms = 0, sort1 = 0, sort2 = 0;
@@ -722,10 +725,11 @@ cudaError_t record_chain(const RecordPlan &pl, const Scratch &sc, const RecordBu
                    pl.blocks, pl.tile_shift, 1 << pl.coarse_shift, sc.tile_cur, capacity, sc.off, sc.unit_off,
                    pl.n_coarse, pl.coarse_shift, flags);
     }
-    deposit(two ? buf.a : buf.b, two ? buf.a_x : buf.b_x, sc);
+    info->kernels += 4 + (two ? 3 : 0) + deposit(two ? buf.a : buf.b, two ? buf.a_x : buf.b_x, sc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   q.rec_prev = sc.hdr + pl.launches - 1;
+  info->last = q.rec_prev;
   return cudaSuccess;
 }
 

@@ -31,7 +31,7 @@ EXPORTS = ("mc_forward", "mc_forward_noalloc", "mc_adjoint", "mc_forward_raw", "
            "mc_adjoint_source", "mc_gradient", "mc_gradient_f32", "mc_check", "mc_last_run_info",
            "mc_release_workspace", "mc_status_string", "mc_version")
 # measurement and test entry points (include/mcr_diag.h), not part of the method's interface
-DIAG_EXPORTS = ("mc_reduction_probe", "mc_philox_blocks", "dn_wait_probe")
+DIAG_EXPORTS = ("mc_reduction_probe", "mc_philox_blocks", "mc_record_info", "dn_wait_probe")
 MAX_BATCH = 64
 ERR_SCRATCH = -7
 
@@ -140,6 +140,8 @@ def _declare(lib: C.CDLL) -> C.CDLL:
     lib.mc_philox_blocks.argtypes = [C.POINTER(C.c_uint32), C.POINTER(C.c_uint32), C.c_int32,
                                      C.POINTER(C.c_uint32)]
     lib.mc_philox_blocks.restype = C.c_int
+    lib.mc_record_info.argtypes = [C.c_int32, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]
+    lib.mc_record_info.restype = C.c_int
     lib.mc_last_run_info.argtypes = [C.c_int32, C.POINTER(_Stats), C.POINTER(C.c_float)]
     lib.mc_release_workspace.argtypes = []
     lib.mc_status_string.argtypes = [C.c_int]
@@ -503,6 +505,14 @@ def last_run_info(which: str = "forward"):
     code = {"forward": 0, "adjoint": 1, "batch": 2}[which]
     _check(load().mc_last_run_info(code, C.byref(st), C.byref(ms)), "mc_last_run_info")
     return _stats_dict(st), float(ms.value)
+
+
+def record_info(dim: int = 2):
+    """(kernels that the record launches of the last 2D or 3D run enqueued, packets that they left to the closing
+    direct launch); (0, -1) after a direct run (``mc_record_info``)."""
+    k, c = C.c_int64(0), C.c_int64(0)
+    _check(load().mc_record_info(dim, C.byref(k), C.byref(c)), "mc_record_info")
+    return k.value, c.value
 
 
 def release_workspace():

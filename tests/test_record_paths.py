@@ -78,3 +78,16 @@ def test_a_graph_outlives_larger_calls(launch):
     mcr.check()
     torch.cuda.synchronize()
     mcr.release_workspace()
+
+
+@pytest.mark.parametrize("threads,blocks", [(32, 1), (64, 1), (32, 2), (96, 1), (256, 1)])
+def test_small_launch_shapes_run_by_records(threads, blocks):
+    """Shapes with fewer lanes than the tail takes packets: the record launches go through the packets all the
+    same, a few at a time, and leave none to the closing launch."""
+    med = _medium(64, 80, 0.1, threads)
+    src = mcr.Source(mcr.LINE, x0=0.0, z0=0.0, x1=8.0, z1=0.0, dir_x=0.1, dir_z=1.0)
+    _same([mcr.Problem(med, 60_000, seed=3, source=src)], mcr.Run(K=8, n_packets=0), (threads, blocks, 0, 0, 0, 2, 0))
+    kernels, closing = mcr.record_info()
+    assert kernels > 0 and closing == 0
+    mcr.run_batch([mcr.Problem(med, 100, seed=3, source=src)], mcr.Run(K=8, n_packets=0), DIRECT)
+    assert mcr.record_info() == (0, -1)
