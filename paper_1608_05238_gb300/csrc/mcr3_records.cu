@@ -92,6 +92,8 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
   Packet3 a;
   float4 m = make_float4(0.f, 0.f, CUDART_INF_F, CUDART_INF_F);  // (mu_a, mu_s, 1/mu_a, 1/mu_s) of the voxel
   unsigned cu1 = 0, cu2 = 0, cu3 = 0;
+  __shared__ double w_esc[256], w_rr[256], w_kill[256];  // weights of the lane's packets that escaped, ...
+  w_esc[threadIdx.x] = w_rr[threadIdx.x] = w_kill[threadIdx.x] = 0.0;
   PacketCounts n;
   auto load_mu = [&]() { m = __ldg(p.mu + a.voxel(p)); };
   auto draw_uniforms = [&](unsigned f) {
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
   auto begin_flight = [&]() {
     if (a.flight >= p.max_events) {
       ++n.evl;
-      n.w_kill.add(a.W);
+      w_kill[threadIdx.x] += a.W;
       alive = false;
       return;
     }
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
     ++n.coll;
     if (a.nscat >= p.max_scatter) {
       ++n.scl;
-      n.w_kill.add(a.W);
+      w_kill[threadIdx.x] += a.W;
       alive = false;
       return;
     }
@@ -139,12 +141,11 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
     if (fabsf(a.W) < p.w_threshold) {  // |W0| = 1
       if (u01(u2) < p.rr_p) {
         const float Wn = a.W * p.rr_inv_p;
-        n.w_rr.add(Wn);
-        n.w_rr.add(-a.W);
+        w_rr[threadIdx.x] += (double)Wn - (double)a.W;
         a.W = Wn;
         ++n.rrs;
       } else {
-        n.w_rr.add(-a.W);
+        w_rr[threadIdx.x] -= a.W;
         ++n.rrk;
         alive = false;
         return;
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
               load_mu();
             } else {
               ++n.esc;
-              n.w_esc.add(a.W);
+              w_esc[threadIdx.x] += a.W;
             }
           }
         }
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
           load_mu();
         } else {
           ++n.esc;
-          n.w_esc.add(a.W);
+          w_esc[threadIdx.x] += a.W;
           alive = false;
         }
       }
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(256, 4) k_transport3_rec(const __grid_constant
     at = __shfl_sync(kFull, at, 0) + __popc(left & ((1u << lane) - 1u));
     if (alive && MCR_GUARD(p.flags, at < p.n_saved)) a.save(p.saved + (size_t)(1u - in_buf) * 4 * p.n_saved, p.n_saved, at);
   }
-  n.add_to(p.stats, p.flags, lane);
+  n.add_to(p.stats, p.flags, lane, w_esc[threadIdx.x], w_rr[threadIdx.x], w_kill[threadIdx.x]);
   __syncthreads();
   for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x)
     if (hist[i]) atomicAdd(p.rec_hist + i, hist[i]);
@@ -273,6 +274,8 @@ __global__ void __launch_bounds__(kTailThreads, 2) k_transport3_tail(const __gri
   const unsigned n_warps = gridDim.x * (blockDim.x >> 5), in_buf = p.rec_hdr->buf;
   const float dx = p.dx;
   const int stride_y = p.nx, stride_z = p.nx * p.ny;
+  __shared__ double w_esc[256], w_rr[256], w_kill[256];  // weights of the lane's packets that escaped, ...
+  w_esc[threadIdx.x] = w_rr[threadIdx.x] = w_kill[threadIdx.x] = 0.0;
   PacketCounts n;
   RecordWriter w;
   unsigned i = warp_place(p.n_sm);  // the warp's packet; then the next one not yet taken
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(kTailThreads, 2) k_transport3_tail(const __gri
           flush();
           if (lane == 0) {
             ++n.esc;
-            n.w_esc.add(a.W);
+            w_esc[threadIdx.x] += a.W;
           }
           ended = true;
           continue;
@@ -370,7 +373,7 @@ __global__ void __launch_bounds__(kTailThreads, 2) k_transport3_tail(const __gri
           flush();
           if (lane == 0) {
             ++n.scl;
-            n.w_kill.add(a.W);
+            w_kill[threadIdx.x] += a.W;
           }
           ended = true;
           continue;
@@ -386,14 +389,13 @@ __global__ void __launch_bounds__(kTailThreads, 2) k_transport3_tail(const __gri
             if (__shfl_sync(kFull, n_u, k) < p.rr_p) {
               const float Wn = a.W * p.rr_inv_p;
               if (lane == 0) {
-                n.w_rr.add(Wn);
-                n.w_rr.add(-a.W);
+                w_rr[threadIdx.x] += (double)Wn - (double)a.W;
                 ++n.rrs;
               }
               a.W = Wn;
             } else {
               if (lane == 0) {
-                n.w_rr.add(-a.W);
+                w_rr[threadIdx.x] -= a.W;
                 ++n.rrk;
               }
               ended = true;
@@ -405,7 +407,7 @@ __global__ void __launch_bounds__(kTailThreads, 2) k_transport3_tail(const __gri
           flush();
           if (lane == 0) {
             ++n.evl;
-            n.w_kill.add(a.W);
+            w_kill[threadIdx.x] += a.W;
           }
           ended = true;
           continue;
@@ -429,7 +431,7 @@ __global__ void __launch_bounds__(kTailThreads, 2) k_transport3_tail(const __gri
     i = __shfl_sync(kFull, i, 0);
   }
   if (w.fill < kRecBlock) w.pad(lane);
-  n.add_to(p.stats, p.flags, lane);
+  n.add_to(p.stats, p.flags, lane, w_esc[threadIdx.x], w_rr[threadIdx.x], w_kill[threadIdx.x]);
   __syncthreads();
   if (threadIdx.x == 0) p.rec_hdr->tail_ran = 1u;
   for (int k = threadIdx.x; k < p.n_bins; k += blockDim.x)

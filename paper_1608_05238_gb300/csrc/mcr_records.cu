@@ -95,6 +95,8 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
   int ix = 0, iz = 0;
   float4 m = make_float4(0.f, 0.f, CUDART_INF_F, CUDART_INF_F);
   unsigned flight = 0, nscat = 0, cu1 = 0, cu2 = 0;
+  __shared__ double w_esc[256], w_rr[256], w_kill[256];  // weights of the lane's packets that escaped, ...
+  w_esc[threadIdx.x] = w_rr[threadIdx.x] = w_kill[threadIdx.x] = 0.0;
   PacketCounts n;
 
   auto load_mu = [&]() {
@@ -143,7 +145,7 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
       fz = cx ? fz : DX() - oz;
       if ((unsigned)ix >= (unsigned)NX() || (unsigned)iz >= (unsigned)NZ()) {
         ++n.esc;
-        n.w_esc.add(W);
+        w_esc[threadIdx.x] += W;
         alive = false;
       } else {
         m = __ldg(MU() + iz * NX() + ix);
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
     ++n.coll;
     if (nscat >= p.max_scatter) {
       ++n.scl;
-      n.w_kill.add(W);
+      w_kill[threadIdx.x] += W;
       alive = false;
       return;
     }
@@ -177,12 +179,11 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
     if (fabsf(W) < p.w_threshold) {  // |W0| = 1
       if (u01(u2) < p.rr_p) {
         const float Wn = W * p.rr_inv_p;
-        n.w_rr.add(Wn);
-        n.w_rr.add(-W);
+        w_rr[threadIdx.x] += (double)Wn - (double)W;
         W = Wn;
         ++n.rrs;
       } else {
-        n.w_rr.add(-W);
+        w_rr[threadIdx.x] -= W;
         ++n.rrk;
         alive = false;
         return;
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
     }
     if (flight >= p.max_events) {
       ++n.evl;
-      n.w_kill.add(W);
+      w_kill[threadIdx.x] += W;
       alive = false;
       return;
     }
@@ -260,10 +261,10 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
             flight = 0;
             if (!inside) {
               ++n.esc;
-              n.w_esc.add(W);
+              w_esc[threadIdx.x] += W;
             } else if (p.max_events == 0u) {
               ++n.evl;
-              n.w_kill.add(W);
+              w_kill[threadIdx.x] += W;
             } else {
               flight = 1;
               ++n.flight;
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(256, BATCH ? 3 : 4) k_transport_rec(const __gr
       save_packet(p.saved + (size_t)(1u - in_buf) * 4 * p.n_saved, p.n_saved, at, s);
     }
   }
-  n.add_to(p.stats, p.flags, lane);
+  n.add_to(p.stats, p.flags, lane, w_esc[threadIdx.x], w_rr[threadIdx.x], w_kill[threadIdx.x]);
   __syncthreads();
   for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x)
     if (hist[i]) atomicAdd(p.rec_hist + i, hist[i]);
@@ -331,6 +332,8 @@ __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const unsigned n_warps = gridDim.x * (blockDim.x >> 5), in_buf = p.rec_hdr->buf;
+  __shared__ double w_esc[256], w_rr[256], w_kill[256];  // weights of the lane's packets that escaped, ...
+  w_esc[threadIdx.x] = w_rr[threadIdx.x] = w_kill[threadIdx.x] = 0.0;
   PacketCounts n;
   RecordWriter w;
   unsigned i = warp_place(p.n_sm);  // the warp's packet; then the next one not yet taken
@@ -433,7 +436,7 @@ __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant
           flush();
           if (lane == 0) {
             ++n.esc;
-            n.w_esc.add(W);
+            w_esc[threadIdx.x] += W;
           }
           ended = true;
           continue;
@@ -443,7 +446,7 @@ __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant
           flush();
           if (lane == 0) {
             ++n.scl;
-            n.w_kill.add(W);
+            w_kill[threadIdx.x] += W;
           }
           ended = true;
           continue;
@@ -459,14 +462,13 @@ __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant
             if (__shfl_sync(kFull, n_u, k) < p.rr_p) {
               const float Wn = W * p.rr_inv_p;
               if (lane == 0) {
-                n.w_rr.add(Wn);
-                n.w_rr.add(-W);
+                w_rr[threadIdx.x] += (double)Wn - (double)W;
                 ++n.rrs;
               }
               W = Wn;
             } else {
               if (lane == 0) {
-                n.w_rr.add(-W);
+                w_rr[threadIdx.x] -= W;
                 ++n.rrk;
               }
               ended = true;
@@ -478,7 +480,7 @@ __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant
           flush();
           if (lane == 0) {
             ++n.evl;
-            n.w_kill.add(W);
+            w_kill[threadIdx.x] += W;
           }
           ended = true;
           continue;
@@ -506,7 +508,7 @@ __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant
     i = __shfl_sync(kFull, i, 0);
   }
   if (w.fill < kRecBlock) w.pad(lane);
-  n.add_to(p.stats, p.flags, lane);
+  n.add_to(p.stats, p.flags, lane, w_esc[threadIdx.x], w_rr[threadIdx.x], w_kill[threadIdx.x]);
   __syncthreads();
   if (threadIdx.x == 0) p.rec_hdr->tail_ran = 1u;
   for (int i = threadIdx.x; i < p.n_bins; i += blockDim.x)

@@ -27,18 +27,6 @@ constexpr int kCurStride = 8;       // words between cursors: one 32-byte sector
 constexpr unsigned kMaxLaunches = 1024;
 constexpr unsigned kSegmentsPerPacket = 4096;  // record launches are enqueued for this many per packet
 
-// A sum of FP32 weights and, apart, of its rounding errors (Knuth's two-sum): FP64's accuracy for a
-// lane's few thousand terms without the FP64 pipe, which is narrow on this part.
-struct WeightSum {
-  float s = 0.f, e = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = s + v, b = t - s;
-    e += (s - (t - b)) + (v - b);
-    s = t;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
-};
-
 // The warp's record slots: a block of kRecBlock at a time from the launch's buffer.
 struct RecordWriter {
   float4 *out = nullptr;
@@ -81,8 +69,7 @@ struct RecordWriter {
 struct PacketCounts {
   unsigned launch = 0, flight = 0, coll = 0, seg = 0, esc = 0, rrk = 0, rrs = 0, scl = 0, evl = 0;
   int w_launch = 0;  // |W0| = 1
-  WeightSum w_esc, w_rr, w_kill;
-  __device__ void add_to(DevStats *st, unsigned *flags, int lane) const {
+  __device__ void add_to(DevStats *st, unsigned *flags, int lane, double w_esc, double w_rr, double w_kill) const {
     auto add = [&](unsigned long long *dst, unsigned v) {
       const unsigned t = __reduce_add_sync(kFull, v);
       if (lane == 0 && t) atomicAdd(dst, (unsigned long long)t);
@@ -102,9 +89,9 @@ struct PacketCounts {
     add(&st->scatter_limit, scl);
     if (add(&st->event_limit, evl) && lane == 0) atomicOr(flags, kFlagEventLimit);
     addw(&st->launched_w, (double)w_launch);
-    addw(&st->escaped_w, w_esc.value());
-    addw(&st->rr_net_w, w_rr.value());
-    addw(&st->killed_w, w_kill.value());
+    addw(&st->escaped_w, w_esc);
+    addw(&st->rr_net_w, w_rr);
+    addw(&st->killed_w, w_kill);
   }
 };
 

@@ -91,3 +91,20 @@ def test_small_launch_shapes_run_by_records(threads, blocks):
     assert kernels > 0 and closing == 0
     mcr.run_batch([mcr.Problem(med, 100, seed=3, source=src)], mcr.Run(K=8, n_packets=0), DIRECT)
     assert mcr.record_info() == (0, -1)
+
+
+@pytest.mark.parametrize("mua", [0.2, 0.22, 0.41])
+def test_weight_counters_are_summed_in_64_bits(mua):
+    """2^26 packets of equal weight through one absorbing pixel, few lanes: some 13,800 additions to a lane's sum.
+    FP64 sums of them err by at most 2^-53 of the whole per addition of the longest chain: a lane's additions (at
+    most four times the mean), the warps' sums and their 152 atomic additions in each of two launches."""
+    n, lanes = 1 << 26, 152 * 32
+    med = mcr.Medium(torch.full((1, 1), mua, device="cuda"), torch.zeros(1, 1, device="cuda"), 1.5, 0.0)
+    src = mcr.Source(mcr.PENCIL, x0=0.7, z0=0.0, dir_x=0.0, dir_z=1.0)
+    run = mcr.Run(K=0, n_packets=0)
+    _, one = mcr.run_batch([mcr.Problem(med, 1, seed=1, source=src)], run, launch=RECORDS, stats=True)
+    w = one["escaped_w"]  # FP32: a product of 2^26 and it is exact
+    assert w == float(np.float32(w)) and 0.5 < w < 1.0
+    _, st = mcr.run_batch([mcr.Problem(med, n, seed=1, source=src)], run, launch=(32, 1, 0, 0, 0, 2, 0), stats=True)
+    assert mcr.record_info()[1] == 0 and st["escapes"] == n
+    assert abs(st["escaped_w"] - n * w) <= (4 * n / lanes + 5 + 2 * 152) * 2.0 ** -53 * n * w
