@@ -185,7 +185,7 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
     if (chunked) need.acc = (size_t)npix * C * sizeof(double);
   }
   need.tally = (size_t)rows * Cpad * 8;
-  // launch order: by default once the tallies no longer fit in L2, for the kinds it orders
+  // launch order (of a direct run): by default once the tallies no longer fit in L2, for the kinds it orders
   bool ordered = false;
   unsigned total_bins = 0;
   {
@@ -200,10 +200,6 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
     }
     ordered = orderable && launch_packets > 0 && launch_packets <= 0xFFFFFFFFull && !common->sectors && !common->time_bins &&
               (cfg.launch_order == 2 || (cfg.launch_order == 0 && (double)need.tally > kOrderTallyBytes));
-    if (ordered) {
-      need.order = (size_t)launch_packets * sizeof(unsigned);
-      need.order_hist = (size_t)total_bins * sizeof(unsigned);
-    }
   }
   TransportParams p;
   memset(&p, 0, sizeof(p));
@@ -226,11 +222,17 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
   }
   Workspace *w = nullptr;
   if (rec_mode && !timed && !holds_records(need)) rec_mode = false;
-  if (!rec_mode) need.records = need.rec_scratch = 0;
+  auto direct_need = [&]() {
+    need.records = need.rec_scratch = 0;
+    if (!ordered) return;
+    need.order = (size_t)launch_packets * sizeof(unsigned);
+    need.order_hist = (size_t)total_bins * sizeof(unsigned);
+  };
+  if (!rec_mode) direct_need();
   int rc = workspace(need, s, &w);
   if (rc == MCR_ERR_NOMEM && rec_mode) {  // no room for the record buffers: deposit directly
     rec_mode = false;
-    need.records = need.rec_scratch = 0;
+    direct_need();
     rc = workspace(need, s, &w);
   }
   if (rc) return rc;
@@ -297,7 +299,7 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
     d.row_base = (unsigned)(tally_off[i] / Cpad);
     bin_base += order_bins(d);
   }
-  p.order = ordered ? w->order : nullptr;
+  p.order = ordered && !rec_mode ? w->order : nullptr;
   MCR_TRY_CUDA(cudaMemsetAsync(w->tally, 0, need.tally, s));
   if (chunked) MCR_TRY_CUDA(cudaMemsetAsync(w->acc, 0, need.acc, s));
   if (timed) MCR_TRY_CUDA(cudaEventRecord(w->ev_start[slot], s));

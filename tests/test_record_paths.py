@@ -108,3 +108,24 @@ def test_weight_counters_are_summed_in_64_bits(mua):
     _, st = mcr.run_batch([mcr.Problem(med, n, seed=1, source=src)], run, launch=(32, 1, 0, 0, 0, 2, 0), stats=True)
     assert mcr.record_info()[1] == 0 and st["escapes"] == n
     assert abs(st["escaped_w"] - n * w) <= (4 * n / lanes + 5 + 2 * 152) * 2.0 ** -53 * n * w
+
+
+def test_runs_by_records_hold_no_launch_order():
+    """The launch order is the direct deposit's: a line source (whose packets it would order once the tally is
+    over 96 MB) takes no more memory by records than a pencil beam (whose packets it never orders)."""
+    n = 1 << 24  # 64 MB of order; the packets leave the grid at once
+    mua = torch.full((512, 512), 0.1, device="cuda")
+    med = mcr.Medium(mua, mua, 0.1, 0.0)
+    up = dict(x0=10.0, z0=0.0, dir_x=0.0, dir_z=-1.0)
+    line, pencil = mcr.Source(mcr.LINE, x1=40.0, z1=0.0, **up), mcr.Source(mcr.PENCIL, **up)
+    held = []
+    mcr.forward(med, line, mcr.Run(K=32, n_packets=n))
+    for src in (pencil, line):
+        torch.cuda.synchronize()
+        mcr.release_workspace()
+        free = torch.cuda.mem_get_info()[0]
+        mcr.forward(med, src, mcr.Run(K=32, n_packets=n))
+        torch.cuda.synchronize()
+        assert mcr.record_info()[0] > 0
+        held.append(free - torch.cuda.mem_get_info()[0])
+    assert held[1] - held[0] < n
