@@ -255,8 +255,10 @@ typedef struct {
                                 captured into a graph; during a capture records are used if the workspace
                                 already holds buffers of the needed size (after one call outside capture) */
   int64_t record_capacity;   /* records per launch of the record deposit (0: 1024 per packet, at least 2^22 and
-                                at most 2^28: two buffers of 64 MB to 4 GB; if they cannot be allocated the
-                                run deposits directly).  A launch whose buffer is full pauses and the next one
+                                at most 2^28: two buffers of 64 MB to 4 GB, which take no more than a quarter
+                                of the memory free; where there is no room for that the buffers are smaller
+                                and the launches more, and without 2 x 64 MB the run deposits directly; a
+                                size that was not to be had is not tried again before mc_release_workspace()).  A launch whose buffer is full pauses and the next one
                                 goes on with its packets; packets left after all launches (some 4096 records per
                                 packet, at most 1024 launches) are finished by the direct deposit */
 } mcr_launch;

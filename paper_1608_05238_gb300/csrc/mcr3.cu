@@ -436,8 +436,9 @@ struct Work3 {
   size_t cdf_bytes = 0, bs_bytes = 0;
   float4 *mu = nullptr;
   size_t mu_bytes = 0;
-  unsigned char *rec_a = nullptr, *rec_b = nullptr, *rec_scratch = nullptr;  // record deposit
-  size_t rec_a_bytes = 0, rec_b_bytes = 0, rec_scratch_bytes = 0;
+  RecordStore rec;  // record deposit
+  unsigned char *rec_scratch = nullptr;
+  size_t rec_scratch_bytes = 0;
   RecordInfo rec_info;
   unsigned char *small = nullptr;  // [0,8) counter, [64,192) stats, [448] flags, [512] qmax bits
   double *partials = nullptr;
@@ -582,10 +583,9 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
   RecordPlan plan{};
   w->rec_info = RecordInfo{};
   if (run->n_packets && cap == cudaStreamCaptureStatusNone && rec_plan3(p, nvox, &plan) == cudaSuccess) {
-    const size_t bytes = rec_buffer_bytes3(plan);
-    if (grow3((void **)&w->rec_a, &w->rec_a_bytes, bytes) == MCR_OK && grow3((void **)&w->rec_b, &w->rec_b_bytes, bytes) == MCR_OK &&
+    if (rec_store(w->rec, 20, run->n_packets, &plan, [](void *) { return false; }) &&
         grow3((void **)&w->rec_scratch, &w->rec_scratch_bytes, rec_scratch_bytes(plan)) == MCR_OK) {
-      MCR3_TRY(launch_records3(p, plan, w->rec_a, w->rec_b, w->rec_scratch, &p, &w->rec_info, s));
+      MCR3_TRY(launch_records3(p, plan, w->rec.a, w->rec.b, w->rec_scratch, &p, &w->rec_info, s));
     } else {
       cudaGetLastError();
     }
@@ -660,7 +660,7 @@ int release_workspace3(int dev) {
   if (dev < 0 || dev >= 64) return MCR_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mu3);
   Work3 &w = g_w3[dev];
-  void *ptrs[] = {w.tally, w.cdf, w.block_sums, w.mu, w.small, w.partials, w.rec_a, w.rec_b, w.rec_scratch};
+  void *ptrs[] = {w.tally, w.cdf, w.block_sums, w.mu, w.small, w.partials, w.rec.a, w.rec.b, w.rec_scratch};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   w = Work3{};

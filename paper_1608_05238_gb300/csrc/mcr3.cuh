@@ -196,7 +196,6 @@ __device__ __forceinline__ SavedPacket3 load_packet3(const uint4 *saved, size_t 
 
 // ---- the record deposit (mcr3_records.cu)
 cudaError_t rec_plan3(const Transport3Params &p, int64_t rows, RecordPlan *out);
-size_t rec_buffer_bytes3(const RecordPlan &pl);  // of each of the two record buffers
 // As launch_records: record launches; on return `closing` is set for the direct transport that adopts the
 // packets left.
 cudaError_t launch_records3(const Transport3Params &p, const RecordPlan &pl, unsigned char *buf_a, unsigned char *buf_b,

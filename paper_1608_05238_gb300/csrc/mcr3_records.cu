@@ -662,8 +662,6 @@ cudaError_t rec_plan3(const Transport3Params &p, int64_t rows, RecordPlan *out) 
   return cudaSuccess;
 }
 
-size_t rec_buffer_bytes3(const RecordPlan &pl) { return record_slots(pl) * 20; }
-
 cudaError_t launch_records3(const Transport3Params &p, const RecordPlan &pl, unsigned char *buf_a, unsigned char *buf_b,
                             unsigned char *scratch, Transport3Params *closing, RecordInfo *info, cudaStream_t s) {
   const DepositChoice3 dc = deposit_kernel3(p.L);

@@ -50,7 +50,8 @@ int grow(Workspace &w, void **ptr, size_t *cap, size_t need) {
 // Sizes the workspace of one launch needs (all problems together).
 struct Need {
   size_t tally = 0, acc = 0, mu = 0, cdf = 0, block_sums = 0, order = 0, order_hist = 0;
-  size_t records = 0, rec_scratch = 0;  // record deposit (records: each of the two buffers)
+  RecordPlan *records = nullptr;  // record deposit: its plan (fitted to the buffers there are) ...
+  uint64_t packets = 0;           // ... and the launch's packets
 };
 
 // Workspace of the current device, grown to `need`, for a call on stream s.
@@ -78,19 +79,20 @@ int workspace(const Need &need, cudaStream_t s, Workspace **out) {
   if (need.block_sums && (rc = grow(w, (void **)&w.block_sums, &w.block_sums_bytes, need.block_sums))) return rc;
   if (need.order && (rc = grow(w, (void **)&w.order, &w.order_bytes, need.order))) return rc;
   if (need.order_hist && (rc = grow(w, (void **)&w.order_hist, &w.order_hist_bytes, need.order_hist))) return rc;
-  if (need.records) {
-    if ((rc = grow(w, (void **)&w.records, &w.records_bytes, need.records))) return rc;
-    if ((rc = grow(w, (void **)&w.sorted, &w.sorted_bytes, need.records))) return rc;
-    if ((rc = grow(w, (void **)&w.rec_scratch, &w.rec_scratch_bytes, need.rec_scratch))) return rc;
-  }
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   MCR_TRY_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (need.records) {
+    auto keep = [&](void *p) { return std::find(w.captured.begin(), w.captured.end(), p) != w.captured.end(); };
+    if (!rec_store(w.rec, sizeof(float4), need.packets, need.records, keep)) return MCR_ERR_NOMEM;
+    if ((rc = grow(w, (void **)&w.rec_scratch, &w.rec_scratch_bytes, rec_scratch_bytes(*need.records)))) return rc;
+  }
   if (cap != cudaStreamCaptureStatusNone) {  // the graph will use what this call uses
     const std::pair<size_t, void *> uses[] = {{need.tally, w.tally},     {need.acc, w.acc},
                                               {need.mu, w.mu},           {need.cdf, w.cdf},
                                               {need.block_sums, w.block_sums}, {need.order, w.order},
-                                              {need.order_hist, w.order_hist}, {need.records, w.records},
-                                              {need.records, w.sorted},  {need.rec_scratch, w.rec_scratch}};
+                                              {need.order_hist, w.order_hist}, {need.records != nullptr, w.rec.a},
+                                              {need.records != nullptr, w.rec.b},
+                                              {need.records != nullptr, w.rec_scratch}};
     for (const auto &u : uses) {
       if (!u.first || std::find(w.captured.begin(), w.captured.end(), u.second) != w.captured.end()) continue;
       try {
@@ -104,12 +106,12 @@ int workspace(const Need &need, cudaStream_t s, Workspace **out) {
   return MCR_OK;
 }
 
-// Whether the current device's workspace already has room for `need`'s record buffers.
-bool holds_records(const Need &need) {
+// Whether the current device's workspace already holds what a run by records of plan `pl` would get.
+bool holds_records(RecordPlan pl, uint64_t packets) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
   const Workspace &w = g_ws[dev];
-  return w.records_bytes >= need.records && w.sorted_bytes >= need.records && w.rec_scratch_bytes >= need.rec_scratch;
+  return rec_held(w.rec, packets, &pl) && w.rec_scratch_bytes >= rec_scratch_bytes(pl);
 }
 
 void fill_stats(const DevStats &d, mcr_stats *s) {
@@ -216,14 +218,12 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
                   (cfg.deposit == 2 ||
                    (cfg.deposit == 0 && cfg.merge != 2 && cfg.shared_tally != 2 && cfg.launch_order != 2));
   if (rec_mode) rec_mode = rec_plan(p, cfg, rows, launch_packets, &plan) == cudaSuccess;
-  if (rec_mode) {
-    need.records = rec_buffer_bytes(plan);
-    need.rec_scratch = rec_scratch_bytes(plan);
-  }
+  need.records = &plan;
+  need.packets = launch_packets;
   Workspace *w = nullptr;
-  if (rec_mode && !timed && !holds_records(need)) rec_mode = false;
+  if (rec_mode && !timed && !holds_records(plan, launch_packets)) rec_mode = false;
   auto direct_need = [&]() {
-    need.records = need.rec_scratch = 0;
+    need.records = nullptr;
     if (!ordered) return;
     need.order = (size_t)launch_packets * sizeof(unsigned);
     need.order_hist = (size_t)total_bins * sizeof(unsigned);
@@ -309,7 +309,7 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
     if (!count) return MCR_OK;
     MCR_TRY_CUDA(cudaMemsetAsync(w->work(), 0, 8, s));
     if (rec_mode) {
-      MCR_TRY_CUDA(launch_records(p, cfg, plan, w->records, w->sorted, w->rec_scratch, w->tally + roff,
+      MCR_TRY_CUDA(launch_records(p, cfg, plan, w->rec.a, w->rec.b, w->rec_scratch, w->tally + roff,
                                   &w->rec_info, s));
       return MCR_OK;
     }
@@ -588,7 +588,7 @@ int mc_release_workspace(void) {
   MCR_TRY_CUDA(cudaDeviceSynchronize());
   Workspace &w = g_ws[dev];
   void *ptrs[] = {w.tally, w.acc, w.mu, w.cdf, w.block_sums, w.partials, w.small, w.order, w.order_hist,
-                  w.records, w.sorted, w.rec_scratch};
+                  w.rec.a, w.rec.b, w.rec_scratch};
   for (void *p : ptrs)
     if (p && std::find(w.captured.begin(), w.captured.end(), p) == w.captured.end()) cudaFree(p);
   for (void *p : w.captured) cudaFree(p);

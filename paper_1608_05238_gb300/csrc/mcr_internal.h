@@ -155,14 +155,53 @@ struct RecordPlan {
 // capacity_records: 0 for the default.  Device limits are read from the current device.
 cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64_t rows, uint64_t packets,
                      RecordPlan *out);
-size_t rec_buffer_bytes(const RecordPlan &pl);   // of each of the two record buffers
 size_t rec_scratch_bytes(const RecordPlan &pl);  // headers, counts, cursors, saved packets
+// The two record buffers of a device, of slot_bytes a record.
+struct RecordStore {
+  unsigned char *a = nullptr, *b = nullptr;
+  unsigned blocks = 0;  // of kRecBlock records in each
+  unsigned denied = 0;  // blocks that were asked for and not to be had
+};
+// Grows st to pl->blocks, or as far as there is room: the pair takes at most a quarter of the free memory, at
+// least 2^22 records each where the plan wants as many.  What is held is given up only for larger buffers, and a
+// size that was not to be had is not tried again.  pl->blocks becomes what there is (and pl->launches what that
+// takes); false: there are no buffers of a useful size.  keep(p): p is not to be freed.
+template <typename Keep>
+bool rec_store(RecordStore &st, size_t slot_bytes, uint64_t packets, RecordPlan *pl, Keep keep);
+// Whether it would do that without an allocation (and as rec_store, pl->blocks).
+bool rec_held(const RecordStore &st, uint64_t packets, RecordPlan *pl);
+void rec_set_blocks(RecordPlan *pl, uint64_t packets, unsigned blocks);
 // Runs p's packets (p.prob[].row_base set, all tallies one array of rows from `tally`) through record
 // launches and a closing direct transport launch that takes over whatever packets they leave.
 // Asynchronous on s: nothing is read back.
-cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg, const RecordPlan &pl, float4 *buf_a,
-                           float4 *buf_b, unsigned char *scratch, unsigned long long *tally, RecordInfo *info,
+cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg, const RecordPlan &pl,
+                           unsigned char *buf_a, unsigned char *buf_b, unsigned char *scratch, unsigned long long *tally, RecordInfo *info,
                            cudaStream_t s);
+
+constexpr unsigned kRecLeastBlocks = (1u << 22) / kRecBlock;
+template <typename Keep>
+bool rec_store(RecordStore &st, size_t slot_bytes, uint64_t packets, RecordPlan *pl, Keep keep) {
+  if (rec_held(st, packets, pl)) return true;
+  const unsigned want = pl->blocks, least = want < kRecLeastBlocks ? want : kRecLeastBlocks;
+  if (st.denied && want >= st.denied) return false;  // (and what is held is of no use)
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) cudaGetLastError();
+  for (unsigned n = want; n > st.blocks && n >= least; n = n > least && n / 2 < least ? least : n / 2) {
+    const size_t bytes = (size_t)n * kRecBlock * slot_bytes;
+    unsigned char *a = nullptr, *b = nullptr;
+    if ((n == least || 2 * bytes <= free_bytes / 4) && cudaMalloc(&a, bytes) == cudaSuccess &&
+        cudaMalloc(&b, bytes) == cudaSuccess) {
+      for (unsigned char *p : {st.a, st.b})
+        if (p && !keep(p)) cudaFree(p);
+      st.a = a, st.b = b, st.blocks = n;
+      break;
+    }
+    cudaGetLastError();
+    if (a) cudaFree(a);
+    st.denied = n;
+  }
+  return rec_held(st, packets, pl);
+}
 
 // Launch order: packets processed in the order of their launch position (line sources: bins of
 // 1/4096 of the line; volumetric sources: 32 x 32-pixel tiles of the launch pixel; other kinds
@@ -197,11 +236,8 @@ struct Workspace {
   size_t order_bytes = 0;
   unsigned *order_hist = nullptr;
   size_t order_hist_bytes = 0;
-  // record deposit: two record buffers, and headers, counts, cursors and saved packets
-  float4 *records = nullptr;
-  size_t records_bytes = 0;
-  float4 *sorted = nullptr;
-  size_t sorted_bytes = 0;
+  // record deposit: the record buffers, and headers, counts, cursors and saved packets
+  RecordStore rec;
   unsigned char *rec_scratch = nullptr;
   size_t rec_scratch_bytes = 0;
   RecordInfo rec_info;

@@ -678,11 +678,22 @@ cudaError_t rec_plan(const TransportParams &p, const TransportLaunch &cfg, int64
   return cudaSuccess;
 }
 
-size_t rec_buffer_bytes(const RecordPlan &pl) { return record_slots(pl) * sizeof(float4); }
+void rec_set_blocks(RecordPlan *pl, uint64_t packets, unsigned blocks) {
+  pl->blocks = blocks;
+  set_launches(pl, packets);
+}
+bool rec_held(const RecordStore &st, uint64_t packets, RecordPlan *pl) {
+  if (st.blocks >= pl->blocks) return true;
+  // smaller buffers will do where the size wanted was not to be had
+  const unsigned least = pl->blocks < kRecLeastBlocks ? pl->blocks : kRecLeastBlocks;
+  if (!st.denied || pl->blocks < st.denied || st.blocks < least) return false;
+  rec_set_blocks(pl, packets, st.blocks);
+  return true;
+}
 size_t rec_scratch_bytes(const RecordPlan &pl) { return layout(nullptr, pl).total; }
 
-cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg, const RecordPlan &pl, float4 *buf_a,
-                           float4 *buf_b, unsigned char *scratch, unsigned long long *tally, RecordInfo *info,
+cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg, const RecordPlan &pl,
+                           unsigned char *buf_a, unsigned char *buf_b, unsigned char *scratch, unsigned long long *tally, RecordInfo *info,
                            cudaStream_t s) {
   const DepositChoice dc = deposit_kernel(p.K);
   const size_t dep_smem = dc.bytes(1 << pl.tile_shift);
@@ -695,7 +706,7 @@ cudaError_t launch_records(const TransportParams &p, const TransportLaunch &cfg,
   const unsigned grid = pl.lanes / pl.threads;
   const size_t smem = (size_t)pl.n_coarse * 4;
   e = record_chain<false>(
-      pl, layout(scratch, pl), RecordBuffers{buf_a, buf_b, nullptr, nullptr}, q, dc.batch, p.work, p.total_packets, p.flags,
+      pl, layout(scratch, pl), RecordBuffers{reinterpret_cast<float4 *>(buf_a), reinterpret_cast<float4 *>(buf_b), nullptr, nullptr}, q, dc.batch, p.work, p.total_packets, p.flags,
       [&]() {
         auto *const rec = p.n_problems > 1 ? k_transport_rec<true> : k_transport_rec<false>;
         if (q.rec_prev)

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1608_05238_gb300 import _build, batch, mcr
+from paper_1608_05238_gb300 import _build, batch, mcr, mcr3
 from parity_util import f32
 
 pytestmark = pytest.mark.gpu
@@ -129,3 +129,49 @@ def test_runs_by_records_hold_no_launch_order():
         assert mcr.record_info()[0] > 0
         held.append(free - torch.cuda.mem_get_info()[0])
     assert held[1] - held[0] < n
+
+
+@pytest.fixture
+def little_memory():
+    """Leaves `room` bytes of the GPU's memory free (asked for by calling it)."""
+    held = []
+
+    def leave(room):
+        mcr.release_workspace()
+        torch.cuda.empty_cache()
+        torch.cuda.synchronize()
+        while (take := min(torch.cuda.mem_get_info()[0] - room, 16 << 30)) > 1 << 26:
+            held.append(torch.empty(take, dtype=torch.uint8, device="cuda"))
+
+    yield leave
+    held.clear()
+    torch.cuda.empty_cache()
+    mcr.release_workspace()
+
+
+@pytest.mark.parametrize("room", [600 << 20, 6 << 30])
+def test_little_memory_means_smaller_record_buffers(little_memory, room):
+    """Where two buffers of 4 GB (3D: 5.4 GB) do not fit, smaller ones take more launches: the same sums, by
+    records, in at most a quarter of what was free (or the least size); buffers of a smaller run are kept."""
+    med = _medium(64, 64, 0.1, 5)
+    src = mcr.Source(mcr.ISO_POINT, x0=3.0, z0=3.0)
+    med3 = mcr3.Medium3(torch.full((24, 24, 24), 0.02, device="cuda"), torch.full((24, 24, 24), 8.0, device="cuda"),
+                        f32(0.2), f32(0.9))
+    src3 = mcr3.Source3(mcr.ISO_POINT, x0=2.1, y0=2.2, z0=2.3)
+    run = mcr.Run(K=12, n_packets=400_000, seed=3)
+    run3 = mcr.Run(K=3, n_packets=400_000, seed=3)
+    ref, ref3 = mcr.forward(med, src, run), mcr3.forward(med3, src3, run3)
+    small = mcr.forward(med, src, mcr.Run(K=12, n_packets=2_000, seed=3))
+    torch.cuda.synchronize()
+    little_memory(room)
+    assert torch.equal(small, mcr.forward(med, src, mcr.Run(K=12, n_packets=2_000, seed=3)))
+    free = torch.cuda.mem_get_info()[0]
+    for _ in range(2):
+        assert torch.equal(ref, mcr.forward(med, src, run))
+        kernels, closing = mcr.record_info(2)
+        assert kernels > 0 and closing == 0
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] <= max(room // 4, 0) + (40 << 20)
+    assert torch.equal(ref3, mcr3.forward(med3, src3, run3))
+    assert mcr.record_info(3)[0] > 0 and mcr.record_info(3)[1] == 0
+    mcr.check()
