@@ -36,36 +36,39 @@ struct Transport3Params : RecordParams {
 // Real orthonormal spherical harmonics of the unit direction u into row[c], c = l^2 + l + m:
 // Y_lm = N_lm Q_l^|m|(u_z) Re/Im[(u_x + i u_y)^|m|], with P_l^m = (1 - u_z^2)^{m/2} Q_l^m and
 // Q_m^m = (2m-1)!!, Q_{m+1}^m = (2m+1) u_z Q_m^m, (l - m) Q_l^m = (2l-1) u_z Q_{l-1}^m - (l+m-1) Q_{l-2}^m.
+// Every rounding is spelled out (sh_q, sh_power): the record deposit rebuilds the same bits from the same steps.
+__device__ __forceinline__ float sh_q(int l, int m, float uz, float qmm, float q1, float q2, float rinv) {
+  if (l == m) return qmm;
+  if (l == m + 1) return __fmul_rn(__fmul_rn(2.f * m + 1.f, uz), qmm);
+  return __fmul_rn(fmaf(__fmul_rn(2.f * l - 1.f, uz), q1, -__fmul_rn(l + m - 1.f, q2)), rinv);
+}
+__device__ __forceinline__ void sh_power(float &cr, float &ci, float ux, float uy) {  // (cr + i ci) (u_x + i u_y)
+  const float nr = fmaf(cr, ux, -__fmul_rn(ci, uy)), ni = fmaf(ci, ux, __fmul_rn(cr, uy));
+  cr = nr;
+  ci = ni;
+}
 __device__ __forceinline__ void sh_row(const Transport3Params &p, float ux, float uy, float uz, float *row) {
   float cr = 1.f, ci = 0.f;  // (u_x + i u_y)^m
   float qmm = 1.f;           // Q_m^m
   for (int m = 0; m <= p.L; ++m) {
     float q2 = 0.f, q1 = qmm;
     for (int l = m; l <= p.L; ++l) {
-      float ql;
-      if (l == m)
-        ql = qmm;
-      else if (l == m + 1)
-        ql = (2.f * m + 1.f) * uz * qmm;
-      else
-        ql = ((2.f * l - 1.f) * uz * q1 - (l + m - 1.f) * q2) * p.rinv[l - m];
+      const float ql = sh_q(l, m, uz, qmm, q1, q2, p.rinv[l - m]);
       if (l > m) {
         q2 = q1;
         q1 = ql;
       }
       const int c0 = l * l + l;
-      const float a = p.nlm[c0 + m] * ql;
+      const float a = __fmul_rn(p.nlm[c0 + m], ql);
       if (m == 0) {
         row[c0] = a;
       } else {
-        row[c0 + m] = a * cr;
-        row[c0 - m] = a * ci;
+        row[c0 + m] = __fmul_rn(a, cr);
+        row[c0 - m] = __fmul_rn(a, ci);
       }
     }
-    const float nr = cr * ux - ci * uy, ni = cr * uy + ci * ux;
-    cr = nr;
-    ci = ni;
-    qmm *= 2.f * m + 1.f;
+    sh_power(cr, ci, ux, uy);
+    qmm = __fmul_rn(qmm, 2.f * m + 1.f);
   }
 }
 

@@ -535,11 +535,6 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
         };
         // as sh_row: (u_x + i u_y)^m and Q_l^m by the recurrence in l, for both records
         float ca = 1.f, ia_ = 0.f, cb = 1.f, ib_ = 0.f;
-        auto power = [](float &cr, float &ci, float x, float y) {
-          const float nr = fmaf(cr, x, -(ci * y)), ni = fmaf(ci, x, cr * y);
-          cr = nr;
-          ci = ni;
-        };
         unroll<0, M1>([&](auto m_) {
           constexpr int m = decltype(m_)::value;
           if constexpr (m >= M0) {
@@ -552,13 +547,7 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
             unroll<m, L + 1>([&](auto l_) {
               constexpr int l = decltype(l_)::value;
               auto next = [&](float &q2, float &q1, float uz) -> float {
-                float ql;
-                if constexpr (l == m)
-                  ql = qmm;
-                else if constexpr (l == m + 1)
-                  ql = __fmul_rn(__fmul_rn(2.f * m + 1.f, uz), qmm);
-                else
-                  ql = __fmul_rn(fmaf(__fmul_rn(2.f * l - 1.f, uz), q1, -__fmul_rn(l + m - 1.f, q2)), h.rinv[l - m]);
+                const float ql = sh_q(l, m, uz, qmm, q1, q2, h.rinv[l - m]);
                 if constexpr (l > m) {
                   q2 = q1;
                   q1 = ql;
@@ -575,8 +564,8 @@ __global__ void __launch_bounds__(kDepThreads, MINB)
               }
             });
           }
-          power(ca, ia_, ax, ay);
-          power(cb, ib_, bx, by);
+          sh_power(ca, ia_, ax, ay);
+          sh_power(cb, ib_, bx, by);
         });
       }
       // sums of the four lanes, 8 channels a round

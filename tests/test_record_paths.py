@@ -143,6 +143,7 @@ def little_memory():
         while (take := min(torch.cuda.mem_get_info()[0] - room, 16 << 30)) > 1 << 26:
             held.append(torch.empty(take, dtype=torch.uint8, device="cuda"))
 
+    leave.drop = held.clear
     yield leave
     held.clear()
     torch.cuda.empty_cache()
@@ -175,3 +176,49 @@ def test_little_memory_means_smaller_record_buffers(little_memory, room):
     assert torch.equal(ref3, mcr3.forward(med3, src3, run3))
     assert mcr.record_info(3)[0] > 0 and mcr.record_info(3)[1] == 0
     mcr.check()
+
+
+@pytest.fixture
+def direct3(little_memory):
+    """3D runs deposit directly: there was no room for record buffers when they were first asked for, and what
+    was not to be had is not asked for again."""
+    one = torch.ones(1, 1, 1, device="cuda")
+    little_memory(100 << 20)
+    mcr3.forward(mcr3.Medium3(one, one, 1.0, 0.0), mcr3.Source3(mcr.ISO_POINT, x0=0.5, y0=0.5, z0=0.5),
+                 mcr.Run(K=0, n_packets=10))
+    assert mcr.record_info(3) == (0, -1)
+    little_memory.drop()
+    torch.cuda.empty_cache()
+
+
+COUNTERS3 = ("launched", "flights", "collisions", "segments", "escapes", "rr_kill", "rr_survive")
+# a few tiles; and 132,192 voxels: 64-row tiles over two sorting passes
+GRIDS3 = [((9, 14, 11), 0.25, 40_000), ((51, 54, 48), 0.08, 30_000)]
+
+
+def _runs3(shape, dx, n, L, seed=5):
+    r = np.random.default_rng(L)
+    med = mcr3.Medium3(torch.from_numpy((0.01 + 0.1 * r.random(shape)).astype(np.float32)).cuda(),
+                       torch.from_numpy((5 + 10 * r.random(shape)).astype(np.float32)).cuda(), f32(dx), f32(0.9))
+    run = mcr.Run(K=L, n_packets=n, seed=seed, w_threshold=0.02, roulette_p=0.25)
+    src = mcr3.Source3(mcr.PENCIL, x0=f32(0.4 * shape[2] * dx), y0=f32(0.6 * shape[1] * dx), z0=0.0, dir_x=0.2,
+                       dir_y=-0.1, dir_z=1.0)
+    q = torch.from_numpy(r.normal(size=shape).astype(np.float32)).cuda()
+    out, st = mcr3.forward(med, src, run, stats=True)
+    info = mcr.record_info(3)
+    return out.cpu(), mcr3.adjoint(med, q, run).cpu(), [st[k] for k in COUNTERS3], info
+
+
+@pytest.fixture(scope="module")
+def by_records3():
+    return {(g, L): _runs3(*GRIDS3[g], L) for g in range(2) for L in range(9)}
+
+
+def test_records_equal_the_direct_deposit_in_3d(by_records3, direct3):
+    """Every order L, forward (more packets than the tail takes: the main loop runs too) and adjoint: the same
+    coefficients, bit for bit, and the same paths."""
+    for (g, L), (fwd, adj, counts, info) in by_records3.items():
+        assert info[0] > 0 and info[1] == 0, (g, L)
+        d_fwd, d_adj, d_counts, d_info = _runs3(*GRIDS3[g], L)
+        assert d_info == (0, -1)
+        assert torch.equal(fwd, d_fwd) and torch.equal(adj, d_adj) and counts == d_counts, (g, L)
