@@ -50,8 +50,9 @@ typedef struct {
 /* Forward run: coeff device out [(L+1)^2][nz][ny][nx], L = run->K <= MCR3_MAX_L, n_packets <= 2^26
  * per call (use first_packet and run->accumulate to add further ranges); run->sectors and
  * run->time_bins must be 0.  The run deposits by records of 20 bytes as mcr.h's record deposit does (two
- * buffers of 2^22 to 2^28 of them, 1024 per packet); during a capture, or where they cannot be allocated,
- * directly.  The sums are the same integers either way. */
+ * buffers of 2^22 to 2^28 of them, 1024 per packet, with the same rules where there is little memory), or
+ * directly where there is no room for them.  The sums are the same integers either way.  The call synchronises
+ * the stream to read its counters, so it cannot be captured into a graph (MCR_ERR_CUDA). */
 int mc3_forward(const mcr3_medium *med, const mcr3_source *src, const mcr_run *run, float *coeff, mcr_stats *stats,
                 void *stream);
 /* Adjoint run from qstar (device [nz][ny][nx], signed, per unit volume and solid angle). */

@@ -521,6 +521,10 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
   } else {
     p.kind = -1;
   }
+  // the run reads its counters back at the end, which a capture does not allow
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  MCR3_TRY(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return MCR_ERR_CUDA;
   const int L = run->K, C = (L + 1) * (L + 1), Cpad = tally_row_words3(C);
   const int64_t nvox = (int64_t)med->nx * med->ny * med->nz;
   std::lock_guard<std::mutex> lock(g_mu3);
@@ -577,12 +581,10 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
   p.stats = dstats;
   p.flags = flags;
   // The record deposit (mcr3_records.cu), then the direct transport for packets it leaves; the direct
-  // transport alone when the record buffers cannot be allocated or a graph is being captured.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  MCR3_TRY(cudaStreamIsCapturing(s, &cap));
+  // transport alone when there is no room for record buffers.
   RecordPlan plan{};
   w->rec_info = RecordInfo{};
-  if (run->n_packets && cap == cudaStreamCaptureStatusNone && rec_plan3(p, nvox, &plan) == cudaSuccess) {
+  if (run->n_packets && rec_plan3(p, nvox, &plan) == cudaSuccess) {
     if (rec_store(w->rec, 20, run->n_packets, &plan, [](void *) { return false; }) &&
         grow3((void **)&w->rec_scratch, &w->rec_scratch_bytes, rec_scratch_bytes(plan)) == MCR_OK) {
       MCR3_TRY(launch_records3(p, plan, w->rec.a, w->rec.b, w->rec_scratch, &p, &w->rec_info, s));

@@ -222,3 +222,21 @@ def test_records_equal_the_direct_deposit_in_3d(by_records3, direct3):
         d_fwd, d_adj, d_counts, d_info = _runs3(*GRIDS3[g], L)
         assert d_info == (0, -1)
         assert torch.equal(fwd, d_fwd) and torch.equal(adj, d_adj) and counts == d_counts, (g, L)
+
+
+def test_3d_runs_refuse_a_capture_and_leave_it_whole():
+    """A 3D run synchronises, so it is refused under capture, before it has enqueued anything: the capture goes on."""
+    med = mcr3.Medium3(torch.full((8, 8, 8), 0.02, device="cuda"), torch.full((8, 8, 8), 8.0, device="cuda"), 0.2, 0.5)
+    src, run = mcr3.Source3(mcr.ISO_POINT, x0=0.8, y0=0.8, z0=0.8), mcr.Run(K=2, n_packets=1_000)
+    ref = mcr3.forward(med, src, run)
+    x = torch.zeros(4, device="cuda")
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream), torch.cuda.graph(graph, stream=stream):
+        x += 1.0
+        with pytest.raises(mcr.McrError):
+            mcr3.forward(med, src, run, stream=stream, out=ref)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [1.0] * 4
+    assert torch.equal(mcr3.forward(med, src, run), ref)
