@@ -36,24 +36,12 @@ UNIT = "photons/s"
 # kernels of libmcr per step beside the record launches: forward (pack, closing transport, finalize, H) | eps
 # (residual, reduction) | backward (adjoint source | pack, 4 CDF, closing transport, finalize | gradient)
 KERNELS_PER_STEP = 15
-# Algorithmic DRAM bytes per pixel segment of the record deposit: a 16-byte record written, read and rewritten
-# by the sort, read by the deposit; a second sorting pass (over 131,072 tally rows) counts, reads and rewrites
-# it once more.
-RECORD_BYTES_PER_SEGMENT = (64, 112)
-RECORD_ONE_PASS_ROWS = 131_072
 
 
-def record_kernels(packets, rows, deposits=1):
-    """Kernels that the record launches of one run enqueue (152 SMs): a launch per full buffer (4,096 segments a
-    packet), one per halving of the packets in use down to what the tail takes, one for a part-full buffer."""
-    buffer = min(max(packets * 1024, 1 << 22), 1 << 28)
-    n = max(4, -(-packets * 4096 // buffer)) + 1
-    in_use = min(packets, 152 * 4 * 256)
-    while in_use > 152 * 2 * 8 * 4:
-        in_use //= 2
-        n += 1
-    # transport, tail, scan, sort, deposit; a second sorting pass: count, scan, sort
-    return min(n, 1024) * (4 + deposits + (3 if rows > RECORD_ONE_PASS_ROWS else 0))
+def record_bytes(passes, record=16):
+    """Algorithmic DRAM bytes per pixel segment of the record deposit: a record written, read and rewritten by the
+    sort, read by the deposit; a second sorting pass counts, reads and rewrites it once more."""
+    return record * (4 if passes < 2 else 7)
 
 
 def _args():
@@ -342,7 +330,7 @@ def _gpu(args):
     sharded = world > 1 and not args.replicas
     share = world if sharded else 1
 
-    def step(k, a=leaf_a, s=leaf_s, hm=Hmeas, scale=1):
+    def step(k, a=leaf_a, s=leaf_s, hm=Hmeas, scale=1, info=None):
         # one gradient evaluation through the autograd.Function: H(mu) -> eps -> backward
         base = replica_seed(0 if sharded else rank, k)
         spec = MCSpec(dx=dx, g=g, sources=srcs, K=w.K, n_packets=scale * per_src * share,
@@ -350,12 +338,17 @@ def _gpu(args):
         a.grad = None
         s.grad = None
         H = HFromMu.apply(a, s, spec)
+        if info is not None:
+            info["forward"] = mcr.record_info()[0]  # of the last source's run; the others are like it
         eps = EpsFromH.apply(H, hm, dx)
         eps.backward()
+        if info is not None:
+            info["adjoint"], info["passes"] = mcr.record_info()[0], mcr.record_passes()
         return (a.grad, s.grad), eps
 
-    for k in range(args.warmup):
-        step(-1 - k)
+    record = {}  # kernels that the runs' record launches enqueue, as the library counts them
+    for k in range(max(1, args.warmup)):
+        step(-1 - k, info=record)
     torch.cuda.synchronize()
     mcr.check()
 
@@ -445,7 +438,7 @@ def _gpu(args):
     except Exception:
         pass
     hbm = float(peaks.get("hbm_gbs", 6800.0))
-    rec_bytes = RECORD_BYTES_PER_SEGMENT[w.nx * w.nz > RECORD_ONE_PASS_ROWS]
+    rec_bytes = record_bytes(record["passes"])
     achieved_gbs = rec_bytes * avg_segs / (avg_ms * 1e-3) / 1e9
     roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm, "unit": "GB/s", "frac": achieved_gbs / hbm,
                 "traffic": None, "kernel": "k_transport_rec + k_rec_sort + k_rec_deposit", "launch_ms": avg_ms,
@@ -485,8 +478,7 @@ def _gpu(args):
                # sharded runs add one raw export per run and, for the adjoint, the source strength
                # (4 CDF kernels) in the finalisation
                "gpu_launches": (KERNELS_PER_STEP + 3 * (len(srcs) - 1) + (len(srcs) + 5 if sharded else 0)
-                                + len(srcs) * record_kernels(per_src, w.nx * w.nz)
-                                + record_kernels(n, w.nx * w.nz)) * args.steps, "roofline": roofline,
+                                + len(srcs) * record["forward"] + record["adjoint"]) * args.steps, "roofline": roofline,
                "cpu_baseline": cpu}
         print(json.dumps(out), flush=True)
     if world > 1:
@@ -1195,15 +1187,20 @@ def _grad3d(args):
                                                                                              seed=999)))
     flush = torch.empty(256 * 2 ** 20 // 4, dtype=torch.float32, device="cuda")
 
-    def step(k):
+    def step(k, record=None):
         c, sf = mcr3.forward(med, s3, mcr.Run(K=L, n_packets=N, seed=2 * k), stats=True)
+        if record is not None:
+            record["forward"] = mcr.record_info(3)[0]
         H, v, eps = mcr3.h_eps(med, c, Hm)
         q = mcr3.adjoint_source(med, v)
         ca, sa = mcr3.adjoint(med, q, mcr.Run(K=L, n_packets=N, seed=2 * k + 1, stream_id=1), stats=True)
+        if record is not None:
+            record["adjoint"], record["passes"] = mcr.record_info(3)[0], mcr.record_passes(3)
         return mcr3.gradient(med, c, ca, v), sf, sa
 
-    for k in range(args.warmup):
-        step(k)
+    record = {}  # kernels that the runs' record launches enqueue, as the library counts them
+    for k in range(max(1, args.warmup)):
+        step(k, record)
     torch.cuda.synchronize()
     clk = ClockSampler(0)
     clk.start()
@@ -1232,7 +1229,7 @@ def _grad3d(args):
     C = (L + 1) ** 2
     ms = float(np.mean([t for t, _ in tr]))
     seg = float(np.mean([s for _, s in tr]))
-    rec_bytes = RECORD_BYTES_PER_SEGMENT[n ** 3 > RECORD_ONE_PASS_ROWS] // 16 * 20
+    rec_bytes = record_bytes(record["passes"], 20)
     achieved = rec_bytes * seg / (ms * 1e-3) / 1e9
     peaks = {}
     try:
@@ -1265,7 +1262,7 @@ def _grad3d(args):
                                   f"{N:.0e} forward + {N:.0e} adjoint packets per step",
                       "segments_per_photon": float(np.mean(segs)) / N, "l2": "flushed between timed steps (256 MB write)"},
            "clocks": clocks,
-           "gpu_launches": (14 + 2 * record_kernels(N, n ** 3, 2 if L > 6 else 1)) * args.steps, "roofline": roofline,
+           "gpu_launches": (14 + record["forward"] + record["adjoint"]) * args.steps, "roofline": roofline,
            "cpu_baseline": cpu}
     print(json.dumps(out), flush=True)
     return 0

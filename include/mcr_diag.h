@@ -42,10 +42,10 @@ int mc_philox_blocks(const uint32_t *ctr, const uint32_t *key, int32_t n, uint32
 /*
  * mc_record_info -- what the last 2D (dim 2) or 3D (dim 3) run on the current device enqueued by its record
  * deposit: *kernels kernels of its record launches (0 for a direct run), and *closing packets that they left to
- * the closing direct launch (of the last 2^26 packets of a longer run; -1 for a direct run).  Both host.
- * Synchronises the device after a run by records.  MCR_ERR_ARG for another dim or a null pointer.
+ * the closing direct launch (of the last 2^26 packets of a longer run; -1 for a direct run), *passes sorting
+ * passes over the records (0 for a direct run).  All host.  Synchronises the device after a run by records.  MCR_ERR_ARG for another dim or a null pointer.
  */
-int mc_record_info(int32_t dim, int64_t *kernels, int64_t *closing);
+int mc_record_info(int32_t dim, int64_t *kernels, int64_t *closing, int32_t *passes);
 
 /*
  * dn_wait_probe -- test hook (the paper has no counterpart): the denoiser kernels' bounded

@@ -650,11 +650,10 @@ int run3(const mcr3_medium *med, const mcr3_source *src, const float *qstar, con
 
 }  // namespace
 
-int record_info3(int dev, int64_t *kernels, int64_t *closing) {
+int record_info3(int dev, int64_t *kernels, int64_t *closing, int32_t *passes) {
   if (dev < 0 || dev >= 64) return MCR_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mu3);
-  *kernels = g_w3[dev].rec_info.kernels;
-  return closing_packets(g_w3[dev].rec_info, closing);
+  return describe(g_w3[dev].rec_info, kernels, closing, passes);
 }
 
 // Frees this device's 3D workspace (called by mc_release_workspace).

@@ -208,8 +208,9 @@ int enqueue(const std::vector<HostProblem> &probs, const mcr_run *common, const 
   p.n_problems = np;
   // record deposit: the harmonic tallies, unless an option of the direct deposit is asked for (256 x 256,
   // 2e6 packets, direct / records: K = 0 38.1 / 26.9 ms, K = 16 47.9 / 32.7, K = 64 134 / 74; 1e3 packets
-  // at K = 16: 6.6 / 3.1 ms -- there is no size at which the direct deposit is the faster one).  While a
-  // graph is being captured nothing may be allocated: then only if the workspace holds the buffers.
+  // at K = 16: 6.6 / 3.1 ms.  What the direct deposit would do faster has next to nothing to do: one packet
+  // 75 / 133 us, 1e5 packets that end after about a millimetre in 32 x 32 pixels, K = 0, 361 / 396 us).  While
+  // a graph is being captured nothing may be allocated: then only if the workspace holds the buffers.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   MCR_TRY_CUDA(cudaStreamIsCapturing(s, &cap));
   const bool timed = cap == cudaStreamCaptureStatusNone;
@@ -571,14 +572,13 @@ int mc_last_run_info(int32_t which, mcr_stats *stats, float *transport_ms) {
   return MCR_OK;
 }
 
-int mc_record_info(int32_t dim, int64_t *kernels, int64_t *closing) {
+int mc_record_info(int32_t dim, int64_t *kernels, int64_t *closing, int32_t *passes) {
   int dev = 0;
-  if ((dim != 2 && dim != 3) || !kernels || !closing) return MCR_ERR_ARG;
+  if ((dim != 2 && dim != 3) || !kernels || !closing || !passes) return MCR_ERR_ARG;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MCR_ERR_CUDA;
-  if (dim == 3) return record_info3(dev, kernels, closing);
+  if (dim == 3) return record_info3(dev, kernels, closing, passes);
   std::lock_guard<std::mutex> lock(g_mu);
-  *kernels = g_ws[dev].rec_info.kernels;
-  return closing_packets(g_ws[dev].rec_info, closing);
+  return describe(g_ws[dev].rec_info, kernels, closing, passes);
 }
 
 int mc_release_workspace(void) {
@@ -628,7 +628,9 @@ const char *mc_version(void) { return "mcr 1.1 sm_103a"; }
 
 namespace mcr {
 
-int closing_packets(const RecordInfo &info, int64_t *closing) {
+int describe(const RecordInfo &info, int64_t *kernels, int64_t *closing, int32_t *passes) {
+  *kernels = info.kernels;
+  *passes = info.passes;
   *closing = -1;
   if (!info.last) return MCR_OK;
   RecordHeader h;

@@ -137,6 +137,7 @@ struct RecordHeader {                           // one per record launch of a ca
 // What the last run by records was (mc_record_info).
 struct RecordInfo {
   int64_t kernels = 0;                 // enqueued by its record launches
+  int passes = 0;                      // of the sort
   const RecordHeader *last = nullptr;  // of its last record launch (null: a direct run)
 };
 // How a call's records are laid out and sorted (rec_plan).
@@ -341,8 +342,8 @@ int noalloc_take_flags(cudaStream_t s);
 
 // Frees the 3D transport's workspace on device dev (mcr3.cu).
 int release_workspace3(int dev);
-// The 3D part of mc_record_info, and the packets that `info`'s record launches left.
-int record_info3(int dev, int64_t *kernels, int64_t *closing);
-int closing_packets(const RecordInfo &info, int64_t *closing);
+// The 3D part of mc_record_info, and what it says of `info`.
+int record_info3(int dev, int64_t *kernels, int64_t *closing, int32_t *passes);
+int describe(const RecordInfo &info, int64_t *kernels, int64_t *closing, int32_t *passes);
 
 }  // namespace mcr

@@ -717,6 +717,7 @@ cudaError_t record_chain(const RecordPlan &pl, const Scratch &sc, const RecordBu
   }
   q.rec_prev = sc.hdr + pl.launches - 1;
   info->last = q.rec_prev;
+  info->passes = two ? 2 : 1;
   return cudaSuccess;
 }
 

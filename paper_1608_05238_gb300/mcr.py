@@ -140,7 +140,7 @@ def _declare(lib: C.CDLL) -> C.CDLL:
     lib.mc_philox_blocks.argtypes = [C.POINTER(C.c_uint32), C.POINTER(C.c_uint32), C.c_int32,
                                      C.POINTER(C.c_uint32)]
     lib.mc_philox_blocks.restype = C.c_int
-    lib.mc_record_info.argtypes = [C.c_int32, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]
+    lib.mc_record_info.argtypes = [C.c_int32, C.POINTER(C.c_int64), C.POINTER(C.c_int64), C.POINTER(C.c_int32)]
     lib.mc_record_info.restype = C.c_int
     lib.mc_last_run_info.argtypes = [C.c_int32, C.POINTER(_Stats), C.POINTER(C.c_float)]
     lib.mc_release_workspace.argtypes = []
@@ -510,9 +510,18 @@ def last_run_info(which: str = "forward"):
 def record_info(dim: int = 2):
     """(kernels that the record launches of the last 2D or 3D run enqueued, packets that they left to the closing
     direct launch); (0, -1) after a direct run (``mc_record_info``)."""
-    k, c = C.c_int64(0), C.c_int64(0)
-    _check(load().mc_record_info(dim, C.byref(k), C.byref(c)), "mc_record_info")
-    return k.value, c.value
+    return _record_info(dim)[:2]
+
+
+def record_passes(dim: int = 2):
+    """Sorting passes over the records of the last 2D or 3D run, 0 after a direct one (``mc_record_info``)."""
+    return _record_info(dim)[2]
+
+
+def _record_info(dim):
+    k, c, n = C.c_int64(0), C.c_int64(0), C.c_int32(0)
+    _check(load().mc_record_info(dim, C.byref(k), C.byref(c), C.byref(n)), "mc_record_info")
+    return k.value, c.value, n.value
 
 
 def release_workspace():

@@ -52,6 +52,7 @@ def test_both_sides_of_the_second_sorting_pass(nz, nx):
     med = _medium(nz, nx, 0.05, nx)
     src = mcr.Source(mcr.LINE, x0=0.0, z0=0.0, x1=f32(nx * 0.05), z1=0.0, dir_x=0.2, dir_z=1.0)
     _same([mcr.Problem(med, 40_000, seed=2, source=src)], mcr.Run(K=7, n_packets=0))
+    assert mcr.record_passes() == (1 if nz * nx <= 131_072 else 2)
 
 
 @pytest.mark.parametrize("launch", [None, DIRECT])
