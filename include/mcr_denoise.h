@@ -120,6 +120,21 @@ int dn_wgrad_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W, int3
 int dn_wgrad_bias_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W, int32_t taps, int32_t cout,
                        int32_t cin, float *dw, float *db, void *stream);
 
+/*
+ * dn_wgrad_begin, dn_wgrad_end -- dn_wgrad_bias_nhwc in two steps: the first leaves partial sums in scratch, the
+ * second adds them to dw and db, which may be read after that.  With beside_conv != 0 the second runs beside the
+ * kernel before it in the stream, which must be a dn_conv (or dn_conv_head) that was launched after the first and
+ * does not touch dw or db -- in a backward pass the layer's input gradient -- instead of after it; the results are
+ * the same.  Both on one stream; `pending` is the caller's and holds the scratch from the one to the other, so that
+ * a begun call has to be ended (once; a second end does nothing).
+ */
+typedef struct {
+  uint64_t opaque[24];
+} dn_wgrad_pending;
+int dn_wgrad_begin(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W, int32_t taps, int32_t cout, int32_t cin,
+                   float *dw, float *db, dn_wgrad_pending *pending, void *stream);
+int dn_wgrad_end(dn_wgrad_pending *pending, int32_t beside_conv, void *stream);
+
 /* dst[c][b][p] = src[b][p][off + c] for c < C (bf16); shifted = 1 writes three copies
  * (dst + k*C*B*HW) with x shifted by k - 1 and zeros outside the row. */
 int dn_to_ct(dn_slice src, int32_t B, int32_t H, int32_t W, int32_t C, int32_t shifted, void *dst, void *stream);

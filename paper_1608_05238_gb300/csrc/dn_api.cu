@@ -1,6 +1,9 @@
 // dn_api.cu -- C ABI of the denoiser kernels (include/mcr_denoise.h): argument checks, TMA
 // tensor-map encoding and launches.
+#include <string.h>
+
 #include <mutex>
+#include <type_traits>
 
 #include "../../include/mcr.h"
 #include "../../include/mcr_denoise.h"
@@ -118,12 +121,28 @@ struct Scratch {
       p = nullptr;
     }
   }
+  Scratch(void *held, cudaStream_t stream) : p(held), s(stream) {}
+  void *release() {
+    void *q = p;
+    p = nullptr;
+    return q;
+  }
   Scratch(const Scratch &) = delete;
   Scratch &operator=(const Scratch &) = delete;
   ~Scratch() {
     if (p) cudaFreeAsync(p, s);
   }
 };
+
+// What dn_wgrad_begin leaves to dn_wgrad_end.
+struct Pending {
+  WgradArgs a;
+  void *scratch;  // null: nothing
+  const float *bias;
+  int rows;
+  bool halo;
+};
+static_assert(sizeof(Pending) <= sizeof(dn_wgrad_pending) && std::is_trivially_copyable<Pending>::value, "opaque words");
 
 // db[c] += sums of dz over pixels, in a fixed order
 cudaError_t bias_sums(const dn_slice &dz, long long P, int C, float *db, cudaStream_t s) {
@@ -136,7 +155,7 @@ cudaError_t bias_sums(const dn_slice &dz, long long P, int C, float *db, cudaStr
   WgradArgs a{};
   a.cout = C;
   a.db = db;
-  return launch_wgrad_sum(a, false, static_cast<float *>(sc.p), rows, s);
+  return launch_wgrad_sum(a, false, static_cast<float *>(sc.p), rows, false, s);
 }
 
 bool conv_shape_ok(int B, int H, int W) {
@@ -340,7 +359,7 @@ int dn_wgrad(int32_t B, int32_t H, int32_t W, int32_t taps, int32_t cout, int32_
   a.part = static_cast<float4 *>(sc.p);
   if (!a.part) a.splits = 1;
   if (launch_wgrad_tc(tmA, tmB, a, s) != cudaSuccess) return MCR_ERR_CUDA;
-  if (a.part && launch_wgrad_sum(a, false, nullptr, 0, s) != cudaSuccess) return MCR_ERR_CUDA;
+  if (a.part && launch_wgrad_sum(a, false, nullptr, 0, false, s) != cudaSuccess) return MCR_ERR_CUDA;
   return MCR_OK;
 }
 
@@ -355,6 +374,26 @@ int dn_wgrad_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W, int3
 
 int dn_wgrad_bias_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W, int32_t taps, int32_t cout,
                        int32_t cin, float *dw, float *db, void *stream) {
+  dn_wgrad_pending p;
+  const int rc = dn_wgrad_begin(dz, x, B, H, W, taps, cout, cin, dw, db, &p, stream);
+  return rc ? rc : dn_wgrad_end(&p, 0, stream);
+}
+
+int dn_wgrad_end(dn_wgrad_pending *pending, int32_t beside_conv, void *stream) {
+  Pending p;
+  if (!pending) return MCR_ERR_ARG;
+  memcpy(&p, pending, sizeof(p));
+  memset(pending, 0, sizeof(*pending));
+  if (!p.scratch) return MCR_OK;  // nothing was left to add (or it has been)
+  Scratch sc(p.scratch, (cudaStream_t)stream);
+  return launch_wgrad_sum(p.a, p.halo, p.bias, p.rows, beside_conv != 0, (cudaStream_t)stream) == cudaSuccess ? MCR_OK
+                                                                                                               : MCR_ERR_CUDA;
+}
+
+int dn_wgrad_begin(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W, int32_t taps, int32_t cout, int32_t cin,
+                   float *dw, float *db, dn_wgrad_pending *pending, void *stream) {
+  if (!pending) return MCR_ERR_ARG;
+  memset(pending, 0, sizeof(*pending));
   if (!slice_ok(dz, cout) || !slice_ok(x, cin) || !dw || (taps != 9 && taps != 1)) return MCR_ERR_ARG;
   if (B <= 0 || H <= 0 || W < 16 || (W & (W - 1)) || ((long long)H * W) % 64) return MCR_ERR_ARG;
   if (cout < 1 || cin < 1 || cout > 512 || cin > 512) return MCR_ERR_ARG;
@@ -415,7 +454,8 @@ int dn_wgrad_bias_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W,
     a.part = static_cast<float4 *>(sc.p);
     if (!a.part) a.splits = 1;
     if (launch_wgrad_halo(tmA, tmH, a, s) != cudaSuccess) return MCR_ERR_CUDA;
-    if (a.part && launch_wgrad_sum(a, true, nullptr, 0, s) != cudaSuccess) return MCR_ERR_CUDA;
+    const Pending p{a, sc.release(), nullptr, 0, true};
+    memcpy(pending, &p, sizeof(p));
     return MCR_OK;
   }
   a.N = cin > 128 ? 128 : ((cin + 15) / 16) * 16;  // MMA N; B arrives in whole 64-channel boxes
@@ -442,7 +482,8 @@ int dn_wgrad_bias_nhwc(dn_slice dz, dn_slice x, int32_t B, int32_t H, int32_t W,
   if (db && bias_grad(z, (long long)B * HW, dz.stride, dz.off, cout, bias ? rows : 1, !bias, bias ? bias : db, true,
                       s) != cudaSuccess)
     return MCR_ERR_CUDA;
-  if (sc.p && launch_wgrad_sum(a, false, db ? bias : nullptr, rows, s) != cudaSuccess) return MCR_ERR_CUDA;
+  const Pending p{a, sc.release(), db ? bias : nullptr, rows, false};
+  memcpy(pending, &p, sizeof(p));
   return MCR_OK;
 }
 

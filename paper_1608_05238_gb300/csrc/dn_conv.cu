@@ -16,8 +16,6 @@
 //     offset/stride, so concatenations are free).
 #include <cuda_bf16.h>
 
-#include <type_traits>
-
 #include "dn_internal.h"
 #include "dn_sm100.cuh"
 
@@ -329,6 +327,7 @@ template <int SUB, bool HEAD>
 __global__ void __launch_bounds__(ws_threads<SUB>(), 1)
     k_conv_ws(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, const ConvArgs a,
               int stages, int num_tiles) {
+  cudaTriggerProgrammaticLaunchCompletion();  // (a k_wgrad_sum may run beside; all else waits for this kernel's end)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t bTileBytes = (uint32_t)a.N * kBlockK * 2;
@@ -487,6 +486,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 int stages, int num_tiles) {
   static_assert(KB == 64 || KB == 32, "channel block of 64 (128-byte rows) or 32 (64-byte rows)");
   constexpr uint32_t kHaloBytes = halo_bytes<KB>(), kHaloStride = halo_stride<KB>();
+  cudaTriggerProgrammaticLaunchCompletion();  // (a k_wgrad_sum may run beside; all else waits for this kernel's end)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int cblocks = KB == 64 ? a.cin_pad / 64 : 1;
@@ -627,16 +627,18 @@ __device__ __forceinline__ void put_part(float4 *part, int tile, int split, int 
 
 // dW (and db) += the partial tiles, and db += the rows of k_bias_grad's partial sums (blocks from sum_blocks on).
 // A warp takes 32 rows of four columns; G warps share a tile's splits (ranges of them, added in order).  Bound by
-// the latency of its loads from L2 (the partials, 5 to 25 MB, have just been written): 5 to 9 us a layer under ncu,
-// of which the launch ahead hides a part; the training step at 8 x 256^2 takes what it took with atomics (1920 us).
+// the latency of its loads from L2 (the partials, 5 to 25 MB, have just been written): 5 to 9 us a layer under ncu.
+// Launched ahead.  beside: the kernel before it is a convolution that was launched after the kernels that write the
+// partials had ended, and does not touch dW or db, so the sum runs beside it and waits for it only to end; else it
+// waits first.  (A training step by atomics / with the sums on the way of the next convolution / beside it: at
+// 9 x 128^2 pixels 1045 / 1067 / 999 us, at 7 x 256^2 1760 / 1776 / 1718 us.)
 // HALO: rows (tap, input channel), columns output channels (k_wgrad_halo); else rows output channels,
 // columns input channels.
 template <bool HALO, int G>
-__global__ void __launch_bounds__(G > 8 ? 32 * G : 256) k_wgrad_sum(const WgradArgs a, int columns, int units, int sum_blocks,
-                                                   const float *bias_part, int bias_rows) {
-  constexpr int kWarps = G > 8 ? G : 8;
+__device__ __forceinline__ void wgrad_sum(const WgradArgs &a, int columns, int units, int sum_blocks,
+                                          const float *bias_part, int bias_rows) {
+  constexpr int kWarps = 8;
   __shared__ float4 red[kWarps][32];
-  cudaGridDependencySynchronize();  // launched ahead: the kernels that write the partials have ended from here on
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if ((int)blockIdx.x >= sum_blocks) {
     const int c = ((int)blockIdx.x - sum_blocks) * 32 + lane;
@@ -699,6 +701,13 @@ __global__ void __launch_bounds__(G > 8 ? 32 * G : 256) k_wgrad_sum(const WgradA
         if (c + j < a.cin) o[j] += t[j];
     }
   }
+}
+template <bool HALO, int G>
+__global__ void __launch_bounds__(256, 6) k_wgrad_sum(const WgradArgs a, int columns, int units, int sum_blocks,
+                                                      const float *bias_part, int bias_rows, bool beside) {
+  if (!beside) cudaGridDependencySynchronize();
+  wgrad_sum<HALO, G>(a, columns, units, sum_blocks, bias_part, bias_rows);
+  if (beside) cudaGridDependencySynchronize();
 }
 
 // k_wgrad_tc: weight gradient dW[n][tap][c] += sum_p dZ[p][n] X[p + tap][c] as a GEMM over pixels
@@ -798,12 +807,12 @@ __global__ void __launch_bounds__(128, 1)
     if (m >= a.cout) continue;
     if (a.part) {
       put_part(a.part, (int)blockIdx.z * a.taps + tap, split, a.splits, a.N, warp * 32 + lane, c0, v, have);
-    } else if (have) {
+    } else if (have) {  // one block to an element: reductions, which wait for nothing, in any order
       float *o = a.dw + ((size_t)m * a.taps + tap) * a.cin + n_tile * a.N + c0;
       const int cb = n_tile * a.N + c0;
 #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (cb + j < a.cin) o[j] += __uint_as_float(v[j]);
+        if (cb + j < a.cin) atomicAdd(o + j, __uint_as_float(v[j]));
     }
   }
   tc_fence_before();
@@ -917,12 +926,12 @@ __global__ void __launch_bounds__(128, 1)
     if (m >= a.cout) continue;
     if (a.part) {
       put_part(a.part, (int)blockIdx.z * a.taps + tap, split, a.splits, a.N, warp * 32 + lane, c0, v, have);
-    } else if (have) {
+    } else if (have) {  // one block to an element: reductions, which wait for nothing, in any order
       float *o = a.dw + ((size_t)m * a.taps + tap) * a.cin + n_tile * a.N + c0;
       const int cb = n_tile * a.N + c0;
 #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (cb + j < a.cin) o[j] += __uint_as_float(v[j]);
+        if (cb + j < a.cin) atomicAdd(o + j, __uint_as_float(v[j]));
     }
   }
   tc_fence_before();
@@ -1057,7 +1066,7 @@ __global__ void __launch_bounds__(128, 1)
         const size_t step = ones_row ? 1 : (size_t)9 * a.cin;
 #pragma unroll
         for (int j = 0; j < 16; ++j)
-          if (c0 + j < a.cout) o[(c0 + j) * step] += __uint_as_float(v[j]);
+          if (c0 + j < a.cout) atomicAdd(o + (c0 + j) * step, __uint_as_float(v[j]));
       }
     }
   }
@@ -1207,25 +1216,17 @@ size_t wgrad_part_bytes(const WgradArgs &a, bool halo) {
   return tiles * a.splits * wgrad_columns(a, halo) * kBlockM * sizeof(float);
 }
 
-cudaError_t launch_wgrad_sum(const WgradArgs &a, bool halo, const float *bias_part, int bias_rows, cudaStream_t s) {
+cudaError_t launch_wgrad_sum(const WgradArgs &a, bool halo, const float *bias_part, int bias_rows, bool beside,
+                             cudaStream_t s) {
   const int columns = wgrad_columns(a, halo);
   const int tiles = !a.part ? 0 : halo ? (a.cin + 63) / 64 * 5 : a.taps * a.m_tiles * a.n_tiles;
   const int units = tiles * columns;  // (columns / 4 x 4 blocks of 32 rows)
-  // a warp adds up to 16 splits alone; of more, several warps a range each: eight, or for many splits as many as
-  // leave the chip's warp slots some room (1x1 head, 304 splits, 32 units: 16.4 us with 8 warps, 8.2 with 32;
-  // 32 -> 64 channels at 8 x 128^2, 152 splits, 320 units: 9.1 with 8, 9.4 with 16, 14 with 32)
-  int G = a.splits > 16 ? 8 : 1;
-  while (a.splits > 64 && G < 32 && units * 2 * G <= 152 * 40) G *= 2;
-  const int warps = G > 8 ? G : 8;
-  const int sum_blocks = (units * G + warps - 1) / warps;
+  const bool many = a.splits > 16;    // a warp alone adds up to 16
+  const int sum_blocks = many ? units : (units + 7) / 8;
   const int blocks = sum_blocks + (bias_part ? (a.cout + 31) / 32 : 0);
-  auto pick = [&](auto h) {
-    constexpr bool H = decltype(h)::value;
-    return G == 32 ? k_wgrad_sum<H, 32> : G == 16 ? k_wgrad_sum<H, 16> : G == 8 ? k_wgrad_sum<H, 8> : k_wgrad_sum<H, 1>;
-  };
-  auto *k = halo ? pick(std::true_type{}) : pick(std::false_type{});
+  auto *k = halo ? (many ? k_wgrad_sum<true, 8> : k_wgrad_sum<true, 1>) : (many ? k_wgrad_sum<false, 8> : k_wgrad_sum<false, 1>);
   if (!blocks) return cudaSuccess;
-  return launch(k, dim3((unsigned)blocks), dim3(32u * warps), true, s, a, columns, units, sum_blocks, bias_part, bias_rows);
+  return launch(k, dim3((unsigned)blocks), dim3(256), true, s, a, columns, units, sum_blocks, bias_part, bias_rows, beside);
 }
 
 // ---------------------------------------------------------------- bounded-wait test hook

@@ -86,9 +86,11 @@ cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, bool ahead, cuda
 }
 
 // Scratch for the partial tiles of `a` (its splits and tiles set), and the sum of them into a.dw (and, k_wgrad_halo's,
-// a.db) in a fixed order; bias_part: rows [bias_rows][cout] of bias_grad's partial sums to add to a.db.
+// a.db) in a fixed order; bias_part: rows [bias_rows][cout] of bias_grad's partial sums to add to a.db; beside: the
+// kernel before it in the stream is a convolution launched after those that write the partials.
 size_t wgrad_part_bytes(const WgradArgs &a, bool halo);
-cudaError_t launch_wgrad_sum(const WgradArgs &a, bool halo, const float *bias_part, int bias_rows, cudaStream_t s);
+cudaError_t launch_wgrad_sum(const WgradArgs &a, bool halo, const float *bias_part, int bias_rows, bool beside,
+                             cudaStream_t s);
 
 // Test hook (dn_conv.cu): one warp waits, with the kernels' own bounded mbarrier wait limited to
 // `spins` polls, on an mbarrier that nothing arrives at; on the timeout it latches the kernels'

@@ -38,11 +38,15 @@ class _AdamLayer(C.Structure):
                 ("gb", C.c_void_p)]
 
 
+class _WgradPending(C.Structure):
+    _fields_ = [("opaque", C.c_uint64 * 24)]
+
+
 class _Slice(C.Structure):
     _fields_ = [("data", C.c_void_p), ("stride", C.c_int32), ("off", C.c_int32)]
 
 
-EXPORTS = ("dn_conv", "dn_conv_head", "dn_wgrad", "dn_wgrad_nhwc", "dn_wgrad_bias_nhwc", "dn_to_ct", "dn_pool2", "dn_pool2_bwd", "dn_up2", "dn_up2_bwd", "dn_bias_grad",
+EXPORTS = ("dn_conv", "dn_conv_head", "dn_wgrad", "dn_wgrad_nhwc", "dn_wgrad_bias_nhwc", "dn_wgrad_begin", "dn_wgrad_end", "dn_to_ct", "dn_pool2", "dn_pool2_bwd", "dn_up2", "dn_up2_bwd", "dn_bias_grad",
            "dn_mse", "dn_residual", "dn_adam", "dn_adam_bias", "dn_adam_multi", "dn_pack_input", "dn_sample_scale", "dn_pack_target", "dn_predict_output",
            "dn_unpack_output", "dn_check")
 
@@ -59,6 +63,8 @@ def lib():
             "dn_wgrad": [i32, i32, i32, i32, i32, i32, vp, vp, vp, vp],
             "dn_wgrad_nhwc": [S, S, i32, i32, i32, i32, i32, i32, vp, vp],
             "dn_wgrad_bias_nhwc": [S, S, i32, i32, i32, i32, i32, i32, vp, vp, vp],
+            "dn_wgrad_begin": [S, S, i32, i32, i32, i32, i32, i32, vp, vp, C.POINTER(_WgradPending), vp],
+            "dn_wgrad_end": [C.POINTER(_WgradPending), i32, vp],
             "dn_to_ct": [S, i32, i32, i32, i32, i32, vp, vp],
             "dn_pool2": [S, i32, i32, i32, i32, S, vp],
             "dn_pool2_bwd": [S, S, S, i32, i32, i32, i32, S, vp],
@@ -133,6 +139,19 @@ def wgrad_nhwc(dz: Act, x: Act, taps: int, dw: torch.Tensor, db: torch.Tensor | 
     else:
         assert db.is_cuda and db.dtype == torch.float32 and db.numel() >= dz.C
         _call("dn_wgrad_bias_nhwc", dz.s(), x.s(), x.B, x.H, x.W, taps, dz.C, x.C, _p(dw), _p(db), _stream(stream))
+
+
+def wgrad_begin(dz: Act, x: Act, taps: int, dw: torch.Tensor, db: torch.Tensor, stream=None) -> _WgradPending:
+    """``wgrad_nhwc`` with its sums left to ``wgrad_end`` (``dn_wgrad_begin``)."""
+    assert db.is_cuda and db.dtype == torch.float32 and db.numel() >= dz.C
+    p = _WgradPending()
+    _call("dn_wgrad_begin", dz.s(), x.s(), x.B, x.H, x.W, taps, dz.C, x.C, _p(dw), _p(db), C.byref(p), _stream(stream))
+    return p
+
+
+def wgrad_end(pending: _WgradPending, beside_conv: bool, stream=None):
+    """Adds what ``wgrad_begin`` left; beside_conv: beside the convolution launched since (``dn_wgrad_end``)."""
+    _call("dn_wgrad_end", C.byref(pending), int(beside_conv), _stream(stream))
 
 
 def to_ct(src: Act, shifted: bool, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
@@ -238,8 +257,9 @@ def _p(t):
 
 
 def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is None:  # the handle alone: a torch.cuda.Stream object costs as much host time as a small kernel
+        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return C.c_void_p(stream.cuda_stream)
 
 
 def conv(x: torch.Tensor, w: torch.Tensor, cout: int, out: torch.Tensor, *, taps: int = 9, bias=None,

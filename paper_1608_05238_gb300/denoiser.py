@@ -212,9 +212,18 @@ class UNet:
         L["d0a"].forward(a["cat0"], Act(a["d0a"], c[0]))
         L["d0b"].forward(a["d0a"], Act(a["d0b"], c[0]))
 
-    def _wgrad(self, lay: Conv, dz: torch.Tensor, x: Act):
+    def _grads(self, lay: Conv, dz: torch.Tensor, x: Act, dx: torch.Tensor | None = None, mask: torch.Tensor | None = None):
+        """The layer's weight and bias gradients, and its input gradient if dx is given (whose convolution the
+        weight gradient's sums run beside)."""
         # straight from the NHWC activations (MN-major operands, no transposed copies)
-        ops.wgrad_nhwc(Act(dz, lay.cout), x, lay.taps, lay.gw, db=lay.gb)  # + the bias gradient
+        pending = ops.wgrad_begin(Act(dz, lay.cout), x, lay.taps, lay.gw, lay.gb)
+        beside = False
+        try:
+            if dx is not None:
+                lay.input_grad(dz, dx, mask)
+                beside = True
+        finally:
+            ops.wgrad_end(pending, beside)
 
     def backward(self):
         """Gradients of the loss computed by the last ``loss()`` into every layer's gw, gb."""
@@ -225,40 +234,33 @@ class UNet:
             ("d0a", Act(a["cat0"], c[1] + c[0]), g["dcat0"], None),
         ]
         for name, x, dx, mask in chain:
-            self._wgrad(L[name], g[name], x)
-            L[name].input_grad(g[name], dx, mask)
+            self._grads(L[name], g[name], x, dx, mask)
         ops.up2_bwd(Act(g["dcat0"], c[1], 0), Act(a["d1b"], c[1]), Act(g["d1b"], c[1]))
         for name, x, dx, mask in [("d1b", Act(a["d1a"], c[1]), g["d1a"], a["d1a"]),
                                   ("d1a", Act(a["cat1"], c[2] + c[1]), g["dcat1"], None)]:
-            self._wgrad(L[name], g[name], x)
-            L[name].input_grad(g[name], dx, mask)
+            self._grads(L[name], g[name], x, dx, mask)
         ops.up2_bwd(Act(g["dcat1"], c[2], 0), Act(a["d2b"], c[2]), Act(g["d2b"], c[2]))
         for name, x, dx, mask in [("d2b", Act(a["d2a"], c[2]), g["d2a"], a["d2a"]),
                                   ("d2a", Act(a["cat2"], c[3] + c[2]), g["dcat2"], None)]:
-            self._wgrad(L[name], g[name], x)
-            L[name].input_grad(g[name], dx, mask)
+            self._grads(L[name], g[name], x, dx, mask)
         ops.up2_bwd(Act(g["dcat2"], c[3], 0), Act(a["mb"], c[3]), Act(g["mb"], c[3]))
         for name, x, dx, mask in [("mb", Act(a["ma"], c[3]), g["ma"], a["ma"]),
                                   ("ma", Act(a["p2"], c[2]), g["dp2"], None)]:
-            self._wgrad(L[name], g[name], x)
-            L[name].input_grad(g[name], dx, mask)
+            self._grads(L[name], g[name], x, dx, mask)
         ops.pool2_bwd(Act(g["dp2"], c[2]), Act(g["dcat2"], c[2], c[3]), Act(a["cat2"], c[2], c[3]),
                       Act(g["e2b"], c[2]))
         for name, x, dx, mask in [("e2b", Act(a["e2a"], c[2]), g["e2a"], a["e2a"]),
                                   ("e2a", Act(a["p1"], c[1]), g["dp1"], None)]:
-            self._wgrad(L[name], g[name], x)
-            L[name].input_grad(g[name], dx, mask)
+            self._grads(L[name], g[name], x, dx, mask)
         ops.pool2_bwd(Act(g["dp1"], c[1]), Act(g["dcat1"], c[1], c[2]), Act(a["cat1"], c[1], c[2]),
                       Act(g["e1b"], c[1]))
         for name, x, dx, mask in [("e1b", Act(a["e1a"], c[1]), g["e1a"], a["e1a"]),
                                   ("e1a", Act(a["p0"], c[0]), g["dp0"], None)]:
-            self._wgrad(L[name], g[name], x)
-            L[name].input_grad(g[name], dx, mask)
+            self._grads(L[name], g[name], x, dx, mask)
         ops.pool2_bwd(Act(g["dp0"], c[0]), Act(g["dcat0"], c[0], c[1]), Act(a["cat0"], c[0], c[1]),
                       Act(g["e0b"], c[0]))
-        self._wgrad(L["e0b"], g["e0b"], Act(a["e0a"], c[0]))
-        L["e0b"].input_grad(g["e0b"], g["e0a"], a["e0a"])
-        self._wgrad(L["e0a"], g["e0a"], Act(a["x0"], self.in_ch))
+        self._grads(L["e0b"], g["e0b"], Act(a["e0a"], c[0]), g["e0a"], a["e0a"])
+        self._grads(L["e0a"], g["e0a"], Act(a["x0"], self.in_ch))
 
     def loss_and_grad_seed(self):
         """Residual MSE of the last forward pass against the loaded target; seeds the backward pass."""

@@ -56,6 +56,41 @@ def test_weight_and_bias_gradients_repeat(B, H, W, cin, cout, taps):
         assert (b.double() - z.sum((0, 1, 2))).abs().max() <= tol
 
 
+@pytest.mark.parametrize("B,H,W,cin,cout,taps", [(1, 8, 32, 128, 128, 9), (1, 4, 16, 40, 33, 9), (1, 1, 64, 64, 32, 9)])
+def test_one_split_repeats(B, H, W, cin, cout, taps):
+    """Few pixels: one block sums a tile and adds it straight onto what stands there."""
+    x, dz = _act(B, H, W, cin, 6), _act(B, H, W, cout, 7)
+    out = []
+    for _ in range(4):
+        dw, db = torch.full((cout, taps, cin), 0.5, device="cuda"), torch.full((cout,), 0.25, device="cuda")
+        ops.wgrad_nhwc(Act(dz, cout), Act(x, cin), taps, dw, db=db)
+        out.append((dw, db))
+    ops.check()
+    assert all(torch.equal(a, b) for o in out[1:] for a, b in zip(out[0], o))
+
+
+@pytest.mark.parametrize("B,H,W,cin,cout", [(4, 64, 64, 128, 128), (2, 64, 128, 33, 32), (1, 8, 32, 64, 128)])
+def test_sums_beside_a_convolution_are_the_same(B, H, W, cin, cout):
+    """dn_wgrad_begin, a convolution, dn_wgrad_end beside it (many splits of both kernels, and one): the bits of the
+    one call, and the convolution's own result; a second end adds nothing."""
+    x, dz = _act(B, H, W, cin, 8), _act(B, H, W, cout, 9)
+    ref = [torch.zeros(cout, 9, cin, device="cuda"), torch.zeros(cout, device="cuda")]
+    ops.wgrad_nhwc(Act(dz, cout), Act(x, cin), 9, ref[0], db=ref[1])
+    g = torch.Generator(device="cuda").manual_seed(10)
+    wd = (0.05 * torch.randn((cin + 15) // 16 * 16, 9, r64(cout), generator=g, device="cuda")).bfloat16()
+    dx, dx2 = torch.zeros(B, H, W, r64(cin), dtype=torch.bfloat16, device="cuda"), None
+    ops.conv(dz, wd, cin, dx, cin=cout)
+    for _ in range(5):
+        got = [torch.zeros_like(r) for r in ref]
+        dx2 = torch.zeros_like(dx)
+        p = ops.wgrad_begin(Act(dz, cout), Act(x, cin), 9, got[0], got[1])
+        ops.conv(dz, wd, cin, dx2, cin=cout)
+        ops.wgrad_end(p, True)
+        ops.wgrad_end(p, False)
+        assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1]) and torch.equal(dx, dx2)
+    ops.check()
+
+
 def test_wgrad_of_transposed_copies_repeats():
     B, H, W, cin, cout = 4, 64, 64, 96, 128
     x, dz = _act(B, H, W, cin, 3), _act(B, H, W, cout, 4)
