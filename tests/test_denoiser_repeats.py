@@ -115,3 +115,36 @@ def test_training_steps_repeat(B, H, W, C):
         ops.check()
         runs.append(losses + [v for lay in net.layers.values() for v in (lay.w, lay.b, lay.m, lay.v)])
     assert all(torch.equal(a, b) for a, b in zip(*runs))
+
+
+def test_gradients_can_be_captured():
+    """The weight gradient's scratch and its launches ahead in a CUDA graph: replays give the eager bits, and each
+    adds once more."""
+    B, H, W, cin, cout = 4, 64, 64, 128, 128
+    x, dz = _act(B, H, W, cin, 12), _act(B, H, W, cout, 13)
+    wd = (0.05 * torch.randn(cin, 9, r64(cout), device="cuda")).bfloat16()
+    dx = torch.zeros(B, H, W, r64(cin), dtype=torch.bfloat16, device="cuda")
+    dw, db, one = (torch.zeros(cout, 9, cin, device="cuda"), torch.zeros(cout, device="cuda"),
+                   torch.zeros(cout, device="cuda"))
+
+    def grads():
+        p = ops.wgrad_begin(Act(dz, cout), Act(x, cin), 9, dw, db)
+        ops.conv(dz, wd, cin, dx, cin=cout)
+        ops.wgrad_end(p, True)
+        ops.bias_grad(Act(dz, cout), one)
+
+    grads()
+    ref = [t.clone() for t in (dw, db, one, dx)]
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream), torch.cuda.graph(graph, stream=stream):
+        grads()
+    torch.cuda.current_stream().wait_stream(stream)
+    for _ in range(3):
+        for t in (dw, db, one, dx):
+            t.zero_()
+        graph.replay()
+        assert all(torch.equal(a, b) for a, b in zip(ref, (dw, db, one, dx)))
+    graph.replay()
+    assert torch.equal(db, 2 * ref[1])
+    ops.check()
