@@ -950,8 +950,8 @@ def _invert1024(args):
     paper's, Sec. 6.1), each plain or with the fluence preconditioner (``_pre``: the diagonal
     1 / (dx^2 Phi^2) as L-BFGS's initial inverse Hessian, or as the descent's step scaling).  All use
     the gradient of the autograd Function (forward harmonics recomputed at K = 64) and the line
-    searches' FP64 inner products on the GPU (mc_dot); the tallies take the sorted-record deposit
-    (1.2 GB each).  Reports the mean relative mu_a error and eps per iteration and the time per
+    searches' FP64 inner products on the GPU (mc_dot); the runs deposit by records
+    (tallies of 1.2 GB).  Reports the mean relative mu_a error and eps per iteration and the time per
     iteration of each method; the headline is the first method's seconds per iteration."""
     import torch
     from paper_1608_05238_gb300 import _build, mcr, workloads

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(256, 2) k_transport_tail(const __grid_constant
 
 // ------------------------------------------------------------------------------------- deposit
 // Bound by instruction issue: 27 instructions per order and two records, 68 % of the issue slots with the 12 warps
-// an SM that the sums' registers leave (FMA pipe 45 %, ALU 27 %, XU 33 % of its cycles); at 256^2, K = 32 some
+// an SM that the sums' registers leave (FMA pipe 46 %, ALU 28 %, XU 34 % of its cycles); at 256^2, K = 32 some
 // 22 ps a record, of which 15 grow with K.
 // Orders n0+1 .. n0+KT per pass, coefficient 0 with the first; TWO: two passes, the second starting from
 // the powers that the first left in shared memory.
