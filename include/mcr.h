@@ -19,8 +19,8 @@
  * (a call with stats != NULL, or mc_check).
  *
  * The library keeps one grow-only workspace per device (fixed-point tallies, packed medium,
- * source CDF, counters, and two record buffers of up to 4 GB each, see mcr_launch.deposit), allocated with cudaMalloc on first use and freed by
- * mc_release_workspace().  Calls that share a device share that workspace: calls on different
+ * source CDF, counters, and two record buffers of up to 4 GB each, see mcr_launch.deposit), allocated
+ * with cudaMalloc on first use and freed by mc_release_workspace().  Calls that share a device share that workspace: calls on different
  * streams of one device must not overlap in time.  A graph captured from a call holds the addresses of the
  * workspace of that time: those buffers are kept when later calls grow past them, so that it can be replayed
  * until mc_release_workspace(), after which it must not be.
@@ -258,9 +258,10 @@ typedef struct {
                                 at most 2^28: two buffers of 64 MB to 4 GB, which take no more than a quarter
                                 of the memory free; where there is no room for that the buffers are smaller
                                 and the launches more, and without 2 x 64 MB the run deposits directly; a
-                                size that was not to be had is not tried again before mc_release_workspace()).  A launch whose buffer is full pauses and the next one
-                                goes on with its packets; packets left after all launches (some 4096 records per
-                                packet, at most 1024 launches) are finished by the direct deposit */
+                                size that was not to be had is not tried again before mc_release_workspace()).
+                                A launch whose buffer is full pauses and the next one goes on with its packets;
+                                packets left after all launches (some 4096 records per packet, at most 1024
+                                launches) are finished by the direct deposit */
 } mcr_launch;
 
 /*
